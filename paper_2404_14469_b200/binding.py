@@ -1,20 +1,25 @@
-"""ctypes binding of libsnapkv.so: argument marshalling only.
+"""Binding of libsnapkv.so: argument marshalling only.
 
 Every step of the compression path runs in the library's CUDA kernels; torch is
 used here for device memory (outputs, workspace) and for the current stream.  The
 functions carry the names of the C entry points declared in include/snapkv.h.
+The calls a serving loop makes for every layer or token (the whole-step calls and the
+decode call) are marshalled by the extension `_native` (csrc/native_binding.cpp), the
+others through ctypes; both reach the same copy of the library.
 If the library has not been built, or a call returns an error status, a
 RuntimeError is raised: there is no fallback path.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libsnapkv.so")
+NATIVE_PATH = os.path.join(HERE, "_native.so")
 
 POOL_MAX = 0
 POOL_AVG = 1
@@ -34,6 +39,7 @@ SYMBOLS = [
 ]
 
 _lib = None
+_native = None
 
 
 class SnapKVError(RuntimeError):
@@ -118,6 +124,20 @@ def lib() -> ctypes.CDLL:
     return L
 
 
+def _load_native():
+    """The extension, with the addresses of the library's functions handed to it (once)."""
+    global _native
+    L = lib()
+    if not os.path.exists(NATIVE_PATH):
+        raise SnapKVError(f"{NATIVE_PATH} is missing: build it with `python -m paper_2404_14469_b200.build`")
+    spec = importlib.util.spec_from_file_location("paper_2404_14469_b200._native", NATIVE_PATH)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    mod.bind({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in SYMBOLS}, SnapKVError)
+    _native = mod
+    return mod
+
+
 def status_string(code: int) -> str:
     return lib().snapkv_status_string(int(code)).decode()
 
@@ -134,13 +154,6 @@ def _stream_ptr() -> int:
 def _dev_bf16(t: torch.Tensor, name: str) -> torch.Tensor:
     if not (t.is_cuda and t.dtype == torch.bfloat16 and t.is_contiguous()):
         raise SnapKVError(f"{name} must be a contiguous CUDA bf16 tensor")
-    return t
-
-
-def _dev_bf16_rows(t: torch.Tensor, name: str) -> torch.Tensor:
-    """A 4-D [B, Hkv, L, d] view whose rows of d elements are contiguous; the other strides are free."""
-    if not (t.is_cuda and t.dtype == torch.bfloat16 and t.dim() == 4 and t.stride(3) == 1):
-        raise SnapKVError(f"{name} must be a CUDA bf16 [B, Hkv, L, d] view with contiguous rows")
     return t
 
 
@@ -196,45 +209,8 @@ def snapkv_compress(q_obs, k, v, pool_kernel: int, pool_type: int, budget: int,
 
     out_k/out_v: bf16 [B, Hq, min(budget, L), d]; out_idx: int32 [B, Hq, rows - W].
     """
-    _dev_bf16(q_obs, "q_obs"), _dev_bf16_rows(k, "k"), _dev_bf16_rows(v, "v")
-    if tuple(v.shape) != tuple(k.shape):
-        raise SnapKVError("k and v must have the same shape")
-    strided = not (k.is_contiguous() and v.is_contiguous())
-    B, Hq, Hkv, L, d, W = _shapes(q_obs, k)
-    L_ = lib()
-    rows = L_.snapkv_out_rows(L, budget)
-    # the library addresses outputs with `budget` rows per head; on the identity path we
-    # call it with budget = L so that the tensors stay dense
-    eff_budget = rows
-    dev = k.device
-    Ho = Hkv if grouped else Hq
-    if out_k is None:
-        out_k = torch.empty(B, Ho, rows, d, dtype=torch.bfloat16, device=dev)
-    if out_v is None:
-        out_v = torch.empty(B, Ho, rows, d, dtype=torch.bfloat16, device=dev)
-    if out_idx is None:
-        out_idx = torch.empty(B, Ho, rows - W, dtype=torch.int32, device=dev)
-    need = L_.snapkv_workspace_size(B, Hq, Hkv, L, d, W, pool_kernel, pool_type, eff_budget)
-    if workspace is None or workspace.numel() < need:
-        workspace = _alloc_ws(need, dev)
-    tail = (B, Hq, Hkv, L, d, W, pool_kernel, pool_type, eff_budget, out_k.data_ptr(),
-            out_v.data_ptr(), out_idx.data_ptr(), workspace.data_ptr(), workspace.numel(),
-            _stream_ptr())
-    if strided or grouped:
-        # any [B, Hkv, L, d] view with contiguous rows, e.g. a permuted [B, L, Hkv, d] cache
-        st = ctypes.c_int64 * 3
-        fn = L_.snapkv_compress_grouped if grouped else L_.snapkv_compress_strided
-        code = fn(
-            q_obs.data_ptr(), k.data_ptr(), v.data_ptr(),
-            st(*k.stride()[:3]) if strided else None, st(*v.stride()[:3]) if strided else None,
-            None if lse_obs is None else _lse_arg(lse_obs, B, Hq, W), *tail)
-    elif lse_obs is None:
-        code = L_.snapkv_compress(q_obs.data_ptr(), k.data_ptr(), v.data_ptr(), *tail)
-    else:
-        code = L_.snapkv_compress_lse(q_obs.data_ptr(), k.data_ptr(), v.data_ptr(),
-                                      _lse_arg(lse_obs, B, Hq, W), *tail)
-    _check(code, "snapkv_compress")
-    return out_k, out_v, out_idx, workspace
+    return (_native or _load_native()).compress(q_obs, k, v, pool_kernel, pool_type, budget, out_k, out_v,
+                                                out_idx, workspace, lse_obs, grouped)
 
 
 def snapkv_compress_varlen(q_obs, k, v, seq_lens, pool_kernel: int, pool_type: int, budget: int,
@@ -247,38 +223,8 @@ def snapkv_compress_varlen(q_obs, k, v, seq_lens, pool_kernel: int, pool_type: i
     out_idx [B, Hq, budget - W] filled with -1, workspace); a sequence with budget >= its
     length fills only its first rows.
     """
-    _dev_bf16(q_obs, "q_obs")
-    B, Hq, W, d = q_obs.shape
-    lens = [int(x) for x in seq_lens]
-    st = ctypes.c_int64 * 3
-    if cu_seqlens is None:
-        _dev_bf16_rows(k, "k"), _dev_bf16_rows(v, "v")
-        Hkv, Lmax = k.shape[1], k.shape[2]
-        ks, vs, ko, vo = st(*k.stride()[:3]), st(*v.stride()[:3]), None, None
-    else:
-        if not (k.is_cuda and k.dtype == torch.bfloat16 and k.dim() == 3 and k.is_contiguous()
-                and v.shape == k.shape and v.is_contiguous() and v.dtype == torch.bfloat16):
-            raise SnapKVError("packed k and v must be contiguous CUDA bf16 [total_tokens, Hkv, d]")
-        Hkv, Lmax = k.shape[1], max(lens)
-        row = Hkv * d
-        ks = vs = st(row * 8, d, row)       # the batch stride is not used: offsets are given
-        ko = vo = (ctypes.c_int64 * B)(*[int(c) * row for c in cu_seqlens])
-    L_ = lib()
-    dev = k.device
-    out_k = torch.zeros(B, Hq, budget, d, dtype=torch.bfloat16, device=dev)
-    out_v = torch.zeros_like(out_k)
-    out_idx = torch.full((B, Hq, budget - W), -1, dtype=torch.int32, device=dev)
-    need = max([L_.snapkv_workspace_size(1, Hq, Hkv, x, d, W, pool_kernel, pool_type, budget)
-                for x in set(lens) if x > budget] + [256])
-    if workspace is None or workspace.numel() < need:
-        workspace = _alloc_ws(need, dev)
-    code = L_.snapkv_compress_varlen(
-        q_obs.data_ptr(), k.data_ptr(), v.data_ptr(), ks, vs, ko, vo, (ctypes.c_int32 * B)(*lens),
-        None if lse_obs is None else _lse_arg(lse_obs, B, Hq, W), B, Hq, Hkv, Lmax, d, W,
-        pool_kernel, pool_type, budget, out_k.data_ptr(), out_v.data_ptr(), out_idx.data_ptr(),
-        workspace.data_ptr(), workspace.numel(), _stream_ptr())
-    _check(code, "snapkv_compress_varlen")
-    return out_k, out_v, out_idx, workspace
+    return (_native or _load_native()).varlen(q_obs, k, v, seq_lens, pool_kernel, pool_type, budget, cu_seqlens,
+                                              lse_obs, workspace)
 
 
 def snapkv_compress_paged(q_obs, k_pool, v_pool, page_table, L, pool_kernel: int, pool_type: int,
@@ -288,44 +234,8 @@ def snapkv_compress_paged(q_obs, k_pool, v_pool, page_table, L, pool_kernel: int
     pool); page_table: int32 CUDA [B, pages_per_seq]; L: prompt length (the longest one when
     seq_lens, a list of B lengths, is given).  Returns (out_k, out_v, out_idx, workspace) as
     snapkv_compress does, or, with seq_lens, as snapkv_compress_varlen does."""
-    _dev_bf16(q_obs, "q_obs"), _dev_bf16_rows(k_pool, "k_pool"), _dev_bf16_rows(v_pool, "v_pool")
-    if not (page_table.is_cuda and page_table.dtype == torch.int32 and page_table.is_contiguous()
-            and page_table.dim() == 2 and page_table.shape[0] == q_obs.shape[0]):
-        raise SnapKVError("page_table must be a contiguous CUDA int32 [B, pages_per_seq] tensor")
-    if tuple(v_pool.shape) != tuple(k_pool.shape):
-        raise SnapKVError("k_pool and v_pool must have the same shape")
-    B, Hq, W, d = q_obs.shape
-    num_pages, Hkv, page_size, dk = k_pool.shape
-    if dk != d:
-        raise SnapKVError("q_obs and k_pool disagree on the head dimension")
-    L_ = lib()
-    dev = k_pool.device
-    st = ctypes.c_int64 * 3
-    if seq_lens is None:
-        rows = L_.snapkv_out_rows(L, budget)
-        out_k = torch.empty(B, Hq, rows, d, dtype=torch.bfloat16, device=dev)
-        out_v = torch.empty_like(out_k)
-        out_idx = torch.empty(B, Hq, rows - W, dtype=torch.int32, device=dev)
-        eff_budget, lens_arg = rows, None
-        need = L_.snapkv_workspace_size(B, Hq, Hkv, L, d, W, pool_kernel, pool_type, eff_budget)
-    else:
-        lens = [int(x) for x in seq_lens]
-        out_k = torch.zeros(B, Hq, budget, d, dtype=torch.bfloat16, device=dev)
-        out_v = torch.zeros_like(out_k)
-        out_idx = torch.full((B, Hq, budget - W), -1, dtype=torch.int32, device=dev)
-        eff_budget, lens_arg = budget, (ctypes.c_int32 * B)(*lens)
-        need = max([L_.snapkv_workspace_size(1, Hq, Hkv, x, d, W, pool_kernel, pool_type, budget)
-                    for x in set(lens) if x > budget] + [256])
-    if workspace is None or workspace.numel() < need:
-        workspace = _alloc_ws(need, dev)
-    code = L_.snapkv_compress_paged(
-        q_obs.data_ptr(), k_pool.data_ptr(), v_pool.data_ptr(), st(*k_pool.stride()[:3]),
-        st(*v_pool.stride()[:3]), page_table.data_ptr(), page_table.shape[1], page_size, num_pages,
-        lens_arg, None if lse_obs is None else _lse_arg(lse_obs, B, Hq, W), B, Hq, Hkv, L, d, W,
-        pool_kernel, pool_type, eff_budget, out_k.data_ptr(), out_v.data_ptr(), out_idx.data_ptr(),
-        workspace.data_ptr(), workspace.numel(), _stream_ptr())
-    _check(code, "snapkv_compress_paged")
-    return out_k, out_v, out_idx, workspace
+    return (_native or _load_native()).paged(q_obs, k_pool, v_pool, page_table, L, pool_kernel, pool_type, budget,
+                                             seq_lens, lse_obs, workspace)
 
 
 def snapkv_shard_lse(q_obs, k_shard, mask_n: int, workspace=None):
@@ -407,22 +317,7 @@ def snapkv_hit_counts(a_cur, idx, theta: float):
 def snapkv_decode_attention(q_cur, cache_k, cache_v, workspace=None, want_lse: bool = True):
     """q_cur bf16 [B, Hq, d], cache_k/v bf16 [B, Hc, rows, d] (CUDA, contiguous) ->
     (out fp32 [B, Hq, d], lse fp32 [B, Hq] or None, workspace)."""
-    _dev_bf16(q_cur, "q_cur"), _dev_bf16(cache_k, "cache_k"), _dev_bf16(cache_v, "cache_v")
-    B, Hq, d = q_cur.shape
-    Bc, Hc, rows, dc = cache_k.shape
-    if Bc != B or dc != d or tuple(cache_v.shape) != tuple(cache_k.shape):
-        raise SnapKVError("q_cur, cache_k and cache_v disagree on their shapes")
-    L_ = lib()
-    need = L_.snapkv_decode_workspace_size(B, Hq, rows, d)
-    if workspace is None or workspace.numel() < need:
-        workspace = _alloc_ws(need, q_cur.device)
-    out = torch.empty(B, Hq, d, dtype=torch.float32, device=q_cur.device)
-    lse = torch.empty(B, Hq, dtype=torch.float32, device=q_cur.device) if want_lse else None
-    code = L_.snapkv_decode_attention(q_cur.data_ptr(), cache_k.data_ptr(), cache_v.data_ptr(), B, Hq, Hc,
-                                      rows, d, out.data_ptr(), lse.data_ptr() if want_lse else None,
-                                      workspace.data_ptr(), workspace.numel(), _stream_ptr())
-    _check(code, "snapkv_decode_attention")
-    return out, lse, workspace
+    return (_native or _load_native()).decode(q_cur, cache_k, cache_v, workspace, want_lse)
 
 
 def snapkv_window_scores_lse(q_obs, k, lse_obs, out_vote=None, workspace=None):
