@@ -319,9 +319,10 @@ snapkv_status_t snapkv_hit_counts(const float* a_cur, const int32_t* idx, int ro
  *   out_lse   fp32 [B, Hq] device or NULL: natural-log sum-exp of the logits (lets the
  *             caller merge with attention over rows kept elsewhere, e.g. newly generated ones)
  * bf16 products accumulated in fp32; the rows are split over many blocks and merged in a
- * fixed order, so results are reproducible run to run.  `workspace`: device scratch of
+ * fixed order, so results are reproducible run to run.  `workspace`: device memory of
  * snapkv_decode_workspace_size(B, Hq, rows, d) bytes, 256-byte aligned (0 from the size
- * query means unacceptable arguments).  Enqueued on `stream`: two kernels, no allocation.
+ * query means unacceptable arguments); checked, not written.  Enqueued on `stream`: one kernel,
+ * no allocation.  Should a wait of the kernel exceed its time limit, the affected outputs are NaN.
  * d must be 64 or 128 (SNAPKV_ERR_UNSUPPORTED otherwise), B * Hq <= 65535.
  */
 size_t snapkv_decode_workspace_size(int B, int Hq, int rows, int d);

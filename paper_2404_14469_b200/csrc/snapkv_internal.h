@@ -1,5 +1,6 @@
 // Internal interfaces between the translation units of libsnapkv (not part of the ABI).
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -118,6 +119,14 @@ int list_schedule_items(const ScorePlan& plan, int L, int W, int Hkv, int votes_
 // Time limit, in nanoseconds, that kernels launched from now on give each of their device-side
 // waits (process-wide; one second unless snapkv_set_wait_limit_ns changed it).
 unsigned long long wait_limit_setting();
+
+// A bf16 tensor map with the 128-byte swizzle (boxes of 64 elements in the innermost dimension);
+// `strides_bytes` has rank - 1 entries.
+bool encode_tensor_map(CUtensorMap* m, const void* base, int rank, const unsigned long long* dims,
+                       const unsigned long long* strides_bytes, const unsigned* box);
+
+// SM count of the current device (asked once per device).
+int sm_count();
 
 // `n_vote` < 0: the keys that get a vote are the L - W prefix keys (the whole prompt is here).
 bool make_score_plan(int B, int Hq, int Hkv, int L, int d, int W, ScorePlan* plan, int n_vote = -1);

@@ -783,14 +783,19 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
-bool encode_map(CUtensorMap* m, const void* base, int rank, const cuuint64_t* dims,
-                const cuuint64_t* strides_bytes, const cuuint32_t* box) {
+}  // namespace
+
+bool encode_tensor_map(CUtensorMap* m, const void* base, int rank, const unsigned long long* dims,
+                       const unsigned long long* strides_bytes, const unsigned* box) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
-  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims,
-            strides_bytes, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  cuuint64_t d64[5] = {}, s64[5] = {};
+  for (int i = 0; i < rank; ++i) d64[i] = dims[i];
+  for (int i = 0; i + 1 < rank; ++i) s64[i] = strides_bytes[i];
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), d64, s64, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 int sm_count() {
@@ -805,6 +810,8 @@ int sm_count() {
   }
   return cached[dev];
 }
+
+namespace {
 
 // Supplied-normaliser variant: the caller hands in each window row's natural-log sum-exp
 // (what a prefill attention kernel keeps per query row).  This kernel puts it where the vote
@@ -1001,20 +1008,19 @@ cudaError_t launch_window_scores(const void* q_obs, const void* k, const KVStrid
     // elements are contiguous is one tensor map, e.g. [B, L, Hkv, d] as well as [B, Hkv, L, d].
     // A paged cache is the same map over the pool: (d, position in page, KV head, page); rows
     // past a page's end or pages outside the pool read as zeros.
-    cuuint64_t dims[4] = {static_cast<cuuint64_t>(d),
-                          static_cast<cuuint64_t>(paged ? paged->page_size : L),
-                          static_cast<cuuint64_t>(Hkv),
-                          static_cast<cuuint64_t>(paged ? paged->num_pages : B)};
-    cuuint64_t strides[3] = {static_cast<cuuint64_t>(ks.l) * 2, static_cast<cuuint64_t>(ks.h) * 2,
-                             static_cast<cuuint64_t>(ks.b) * 2};
-    cuuint32_t box[4] = {64, TILE_KEYS, 1, 1};
-    if (!encode_map(&tmK, k, 4, dims, strides, box)) return cudaErrorInvalidValue;
+    using u64 = unsigned long long;
+    const u64 dims[4] = {static_cast<u64>(d), static_cast<u64>(paged ? paged->page_size : L),
+                         static_cast<u64>(Hkv), static_cast<u64>(paged ? paged->num_pages : B)};
+    const u64 strides[3] = {static_cast<u64>(ks.l) * 2, static_cast<u64>(ks.h) * 2, static_cast<u64>(ks.b) * 2};
+    const unsigned box[4] = {64, TILE_KEYS, 1, 1};
+    if (!encode_tensor_map(&tmK, k, 4, dims, strides, box)) return cudaErrorInvalidValue;
   }
   {
-    cuuint64_t dims[2] = {static_cast<cuuint64_t>(d), static_cast<cuuint64_t>(B) * Hq * W};
-    cuuint64_t strides[1] = {static_cast<cuuint64_t>(d) * 2};
-    cuuint32_t box[2] = {64, static_cast<cuuint32_t>(plan.npad)};
-    if (!encode_map(&tmQ, q_obs, 2, dims, strides, box)) return cudaErrorInvalidValue;
+    using u64 = unsigned long long;
+    const u64 dims[2] = {static_cast<u64>(d), static_cast<u64>(B) * Hq * W};
+    const u64 strides[1] = {static_cast<u64>(d) * 2};
+    const unsigned box[2] = {64, static_cast<unsigned>(plan.npad)};
+    if (!encode_tensor_map(&tmQ, q_obs, 2, dims, strides, box)) return cudaErrorInvalidValue;
   }
   ScoreArgs a = schedule_args(plan, L, W, Hkv, (lse_obs || never_ready) ? 1 : 0);
   a.wait_ns = wait_limit_setting();

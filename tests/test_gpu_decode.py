@@ -60,3 +60,18 @@ def test_decode_over_the_steps_own_output_and_runs_are_bit_identical():
     a = sk.snapkv_decode_attention(q_cur, ok, ov)
     b = sk.snapkv_decode_attention(q_cur, ok, ov)
     assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("B,Hq,Hc,rows,d", [
+    (1, 2, 2, 15, 128), (1, 4, 2, 16, 128), (2, 6, 2, 17, 128),     # one tile of 16 rows; groups of 1, 2, 3
+    (1, 8, 2, 31, 64), (1, 5, 1, 32, 64), (1, 8, 1, 33, 64),        # one tile of 32 rows; groups of 4, 5, 8
+    (1, 9, 1, 129, 128), (1, 17, 1, 300, 64),                       # more than one CTA's eight query heads
+    (1, 32, 8, 500, 128), (3, 32, 8, 2777, 128), (1, 4, 2, 8000, 128),  # clusters of 2 to 16 CTAs
+    (38, 8, 4, 100, 128),                                           # more cache heads than SMs
+])
+def test_decode_at_tile_group_and_cluster_edges(B, Hq, Hc, rows, d):
+    g = torch.Generator().manual_seed(7 * rows + Hq)
+    q = (2.0 * torch.randn(B, Hq, d, generator=g)).to(torch.bfloat16)
+    ck = torch.randn(B, Hc, rows, d, generator=g).to(torch.bfloat16)
+    cv = torch.randn(B, Hc, rows, d, generator=g).to(torch.bfloat16)
+    assert _check(q, ck, cv) < 2e-5  # fp32 probabilities and sums, not bf16 ones
