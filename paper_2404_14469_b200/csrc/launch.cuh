@@ -2,12 +2,13 @@
 // resident while the previous kernel of the stream is still running, which hides its launch
 // latency and prologue.  A kernel launched this way calls pdl_wait() before its first access
 // to global memory (it returns once the previous kernel has completed and its writes are
-// visible) and pdl_launch_dependents() at the top.  Used for the clear kernel and the scoring
-// kernel behind it (202 instead of 207 us per layer on the 32K GQA workload, 93 instead of
-// 97 us on the 16K MHA one) and for the gather kernel behind the one-CTA select kernel (another
-// 1.5 us per layer).  The select kernel itself is launched the plain way: launched early as
-// well it gains 0.6-1 us alone, but with both early the layer takes 7.5 us longer, and a gather
-// kernel that lets the next call's kernels in early costs 1.5 us (both measured).
+// visible).  A kernel that calls pdl_launch_dependents() lets the next one in early; without it
+// the next one is let in when the kernel ends, which still saves most of the launch latency (the
+// select kernel behind the scoring kernel starts 2.5 us earlier than with a plain launch).
+// Only the small kernels in front of the scoring kernel let it in early (202 instead of 207 us per
+// layer on the 32K GQA workload, 93 instead of 97 us on the 16K MHA one).  The scoring kernel does
+// not let the select kernel in: CTAs that wait on the SMs that come free first cost 1-2 us; nor
+// the select kernel the gather kernel, whose blocks would crowd there (68 instead of 60 us).
 #pragma once
 #include <cuda_runtime.h>
 

@@ -54,7 +54,7 @@ gather_kernel(const uint4* __restrict__ k, const uint4* __restrict__ v, const Ga
               int W, int ksel, int out_stride, uint4* __restrict__ out_k, uint4* __restrict__ out_v) {
   constexpr int RPT = GATHER_THREADS / VPR;      // rows covered by the block per unrolled step
   constexpr int RPB = RPT * GATHER_UNROLL;       // rows per block
-  pdl_wait();  // launched early behind the select kernel: idx is complete only from here on
+  pdl_wait();  // idx is complete only from here on
   const int rows = ksel + W;
   const int n = L - W;
   const int bh = h0 + blockIdx.y;

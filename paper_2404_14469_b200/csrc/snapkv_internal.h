@@ -165,7 +165,7 @@ cudaError_t launch_pool_topk(const float* vote, int rows, int n, int pool_kernel
 bool select_cluster_applies(int rows, int n, int pool_kernel);
 cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int pool_kernel,
                                      int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream,
-                                     int* launches, int gsum);
+                                     int* launches, int gsum, bool vote_is_scratch);
 
 // Gather + append.  idx == nullptr copies rows 0..ksel-1 (identity path).
 cudaError_t launch_gather(const void* k, const void* v, const KVStrides& ks, const KVStrides& vs,

@@ -222,7 +222,6 @@ template <int D, int NCH, bool SPLIT>
 __global__ void __launch_bounds__(threads_for(SPLIT), 1)
 score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ,
              const ScoreArgs a) {
-  pdl_launch_dependents();
   using SM = Smem<D>;
   constexpr int SUBT = SM::SUBT;
   constexpr int NPAD = NCH * 32;

@@ -1,7 +1,7 @@
-// Pooling and per-head top-k (Listing 1's pool1d and topk; Eq. 2), one CTA per row.
-//
-// Two kernels: a fast one for rows that fit in shared memory (below) and this generic
-// one, which also handles rows of any length through global scratch.
+// Pooling and per-head top-k (Listing 1's pool1d and topk; Eq. 2) for what the cluster kernel does
+// not take: pooling radii of 8 to 31, rows beyond 524288 positions, and the entry point that keeps
+// its keys in an array of the library.  Rows of up to 49152 positions take one CTA each (below),
+// longer ones many.
 //
 //  1. pooled[j] = max or mean of vote[j-r .. j+r] (stride 1, same length; the mean
 //     divides by pool_kernel, positions outside the row count as zero), turned into a
@@ -21,12 +21,6 @@
 namespace snapkv {
 
 namespace {
-
-// Tells L2 that a 128-byte line (global memory, 128-byte aligned) holds nothing worth keeping:
-// a dirty line may then be dropped instead of written back.  Its contents are undefined afterwards.
-__device__ __forceinline__ void discard_l2_line(const void* p) {
-  asm volatile("discard.global.L2 [%0], 128;" ::"l"(__cvta_generic_to_global(p)) : "memory");
-}
 
 constexpr int SEL_THREADS = 1024;
 constexpr int SEL_WARPS = SEL_THREADS / 32;
@@ -193,423 +187,9 @@ pool_topk_kernel(const float* __restrict__ vote, int n, int gsum, int pool_kerne
   }
 }
 
-// ---------------------------------------------------------------------------------------
-// Fast path for rows that fit in shared memory and pooling radii up to RMAX.
-// Thread t owns the EPT consecutive positions [t*EPT, (t+1)*EPT): pooling is a sliding
-// window over registers, histogram updates are run-length aggregated (pooled neighbours
-// fall into the same bin), and the ordered compaction is a single block scan.  Keys sit
-// in shared memory at slot j + j/32, which keeps the strided per-thread sweeps free of
-// bank conflicts.  The first histogram pass bins (key - min) >> shift with the shift
-// chosen from the row's key range, so the bins are spread over the values that occur.
+// Keys of a staged chunk sit at slot j + j/32, which keeps the strided per-thread sweeps free of
+// bank conflicts.
 __device__ __forceinline__ int key_slot(int j) { return j + (j >> 5); }
-// Layout of the one-CTA-per-row kernel: four pad words after every 32 keys.  A thread's run
-// starts at a multiple of 8 keys, so it reads and writes its keys four at a time as aligned
-// 16-byte vectors, and the runs of eight neighbouring threads fall into different banks.
-__device__ __forceinline__ int key_slot4(int j) { return j + ((j >> 5) << 2); }
-__device__ __forceinline__ uint4 ld_keys4(const uint32_t* keys, int j) {
-  return *reinterpret_cast<const uint4*>(keys + key_slot4(j));
-}
-constexpr int FAST_MAX_KEYS = 40960;  // 40 keys per thread: what fits with the padding
-constexpr int CAND_CAP = 2048;   // keys of the first-pass bin that are refined from a list
-constexpr int MASK_WORDS = 2;    // a thread owns at most 64 positions (SEL_SMEM_KEYS / SEL_THREADS = 48)
-
-// PT = -1: pooling radius r <= RMAX and pool type are run-time values.  PT = 0 (max) or 1
-// (avg): the radius is exactly RMAX, so the window loop has no per-element tests.
-template <int RMAX, int PT>
-__global__ void __launch_bounds__(SEL_THREADS, 1)
-pool_topk_fast_kernel(const float* __restrict__ vote, int n, int gsum, int r, int pool_type,
-                      int ept, int ksel, int32_t* __restrict__ out_idx, int discard_votes) {
-  extern __shared__ __align__(16) uint32_t keys[];
-  __shared__ int hist[NBINS];
-  __shared__ int warp_sums[SEL_WARPS];
-  __shared__ int scan_total;
-  __shared__ int sel_bin, sel_above, sel_count, ncand_s;
-  __shared__ int above_s, br_lo, br_hi;
-  __shared__ uint32_t red_min[SEL_WARPS], red_max[SEL_WARPS];
-  __shared__ uint32_t cand[CAND_CAP];
-  int ncand = 0;
-
-  const int row = blockIdx.x;
-  const float* vrow = vote + static_cast<size_t>(row) * gsum * n;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int base = threadIdx.x * ept;
-  // the gather kernel behind this one may become resident now; it waits for this kernel's end
-  pdl_launch_dependents();
-
-  // ---- 1. pooling
-  // The row is first copied into the key slots with coalesced loads (raw fp32 bits), then
-  // every thread pools its own positions in place over a rolling register window.  The
-  // values it needs from its neighbours' positions are saved before anybody overwrites.
-  uint32_t kmin = 0xffffffffu, kmax = 0u;
-  {
-    const int total = SEL_THREADS * ept;
-    if (gsum == 1) {
-      // eight loads in flight per thread before the first store: the votes come from L2, and
-      // one load per loop turn would pay that latency once per element (ept is a multiple of 8)
-      for (int j0 = threadIdx.x; j0 < total; j0 += 8 * SEL_THREADS) {
-        uint32_t x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int j = j0 + u * SEL_THREADS;
-          x[u] = (j < n) ? __float_as_uint(__ldg(vrow + j)) : 0u;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) keys[key_slot4(j0 + u * SEL_THREADS)] = x[u];
-      }
-    } else {
-      // group sum: four positions per thread and step, so that the loads of a step are
-      // independent of one another; heads are added in ascending order
-      for (int j0 = threadIdx.x; j0 < total; j0 += 4 * SEL_THREADS) {
-        float x[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int t = 0; t < gsum; ++t) {
-          const float* src = vrow + static_cast<size_t>(t) * n;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int j = j0 + u * SEL_THREADS;
-            if (j < n) x[u] += __ldg(src + j);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int j = j0 + u * SEL_THREADS;
-          if (j < total) keys[key_slot4(j)] = __float_as_uint(x[u]);
-        }
-      }
-    }
-    __syncthreads();
-    if (discard_votes && gsum == 1) {
-      // The row is in shared memory and its votes are scratch that nobody reads again: drop the
-      // whole 128-byte lines inside the row from L2, so that they are not written back to HBM
-      // while the gather kernel needs the bandwidth (16.8 MB per layer of the 32K GQA workload).
-      // Lines that the row shares with its neighbours stay.
-      const uintptr_t b0 = (reinterpret_cast<uintptr_t>(vrow) + 127) & ~static_cast<uintptr_t>(127);
-      const uintptr_t b1 = reinterpret_cast<uintptr_t>(vrow + n) & ~static_cast<uintptr_t>(127);
-      for (uintptr_t a = b0 + static_cast<uintptr_t>(threadIdx.x) * 128; a < b1;
-           a += static_cast<uintptr_t>(SEL_THREADS) * 128)
-        discard_l2_line(reinterpret_cast<const void*>(a));
-    }
-    // a[]: the last RMAX values before the current block of 8, the block, the next block
-    float a[RMAX + 16];
-    float halo_r[RMAX > 0 ? RMAX : 1];
-#pragma unroll
-    for (int i = 0; i < RMAX; ++i) {
-      const int jl = base - RMAX + i;             // left neighbours
-      a[i] = (jl >= 0) ? __uint_as_float(keys[key_slot4(jl)]) : 0.f;
-      const int jr = base + ept + i;              // right neighbours
-      halo_r[i] = (jr < total) ? __uint_as_float(keys[key_slot4(jr)]) : 0.f;
-    }
-    auto load8 = [&](int pos, float* dst) {       // own positions pos .. pos + 7
-      const uint4 x = ld_keys4(keys, pos), y = ld_keys4(keys, pos + 4);
-      dst[0] = __uint_as_float(x.x); dst[1] = __uint_as_float(x.y);
-      dst[2] = __uint_as_float(x.z); dst[3] = __uint_as_float(x.w);
-      dst[4] = __uint_as_float(y.x); dst[5] = __uint_as_float(y.y);
-      dst[6] = __uint_as_float(y.z); dst[7] = __uint_as_float(y.w);
-    };
-    auto next8 = [&](int sb_next, float* dst) {   // the block after sb_next - 8, or the halo
-      if (sb_next < ept) {
-        load8(base + sb_next, dst);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) dst[i] = (i < RMAX) ? halo_r[i < RMAX ? i : 0] : 0.f;
-      }
-    };
-    load8(base, a + RMAX);
-    __syncthreads();  // every neighbour value is in registers before anybody overwrites
-    next8(8, a + RMAX + 8);
-    for (int sb = 0; sb < ept; sb += 8) {
-      uint32_t out[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        float p = 0.f;  // votes are >= 0: zero is neutral for max and is the avg padding
-#pragma unroll
-        for (int t = 0; t <= 2 * RMAX; ++t) {
-          const int off = t - RMAX;
-          if (PT >= 0 || (off >= -r && off <= r))
-            p = ((PT >= 0) ? (PT == 0) : (pool_type == 0)) ? fmaxf(p, a[i + t]) : p + a[i + t];
-        }
-        const int j = base + sb + i;
-        uint32_t key = 0u;  // positions past the row end rank below every real key
-        if (j < n) {
-          key = float_to_key(p);
-          kmin = min(kmin, key);
-          kmax = max(kmax, key);
-        }
-        out[i] = key;
-      }
-#pragma unroll
-      for (int i = 0; i < RMAX + 8; ++i) a[i] = a[i + 8];
-      // the block after the next one is still untouched; the current one is done with
-      next8(sb + 16, a + RMAX + 8);
-      *reinterpret_cast<uint4*>(keys + key_slot4(base + sb)) = make_uint4(out[0], out[1], out[2], out[3]);
-      *reinterpret_cast<uint4*>(keys + key_slot4(base + sb + 4)) =
-          make_uint4(out[4], out[5], out[6], out[7]);
-    }
-  }
-  kmin = __reduce_min_sync(0xffffffffu, kmin);
-  kmax = __reduce_max_sync(0xffffffffu, kmax);
-  if (lane == 0) {
-    red_min[warp] = kmin;
-    red_max[warp] = kmax;
-  }
-  __syncthreads();
-  kmin = red_min[lane];
-  kmax = red_max[lane];
-  kmin = __reduce_min_sync(0xffffffffu, kmin);
-  kmax = __reduce_max_sync(0xffffffffu, kmax);
-
-  // ---- 2. threshold
-  // One histogram pass over all keys picks the bin that holds the ksel-th largest key.  A
-  // second sweep notes, per thread, which of its keys lie above that bin (kept for sure,
-  // one bit each) and which lie inside it, and copies the latter to a small candidate
-  // list; the remaining passes refine the threshold on that list alone.
-  uint32_t lo = kmin;
-  int krem = ksel;
-  uint32_t T = kmin;
-  uint32_t m_gt[MASK_WORDS], m_in[MASK_WORDS];  // bit i: own key i above / inside the bin
-#pragma unroll
-  for (int wd = 0; wd < MASK_WORDS; ++wd) { m_gt[wd] = 0u; m_in[wd] = 0u; }
-  bool use_list = false;
-  if (kmax != kmin) {
-    const uint32_t range = kmax - kmin;
-    int shift = 32 - __clz(range) - 11;
-    if (shift < 0) shift = 0;
-    uint32_t width_m1 = range;  // candidates are keys with key - lo <= width_m1
-    bool first = true;
-    // 2a. A guess from a sample.  Every fourth key goes into the histogram (a quarter of the
-    // shared-memory atomics of a full pass, which is what that pass spends its time on); the
-    // sample's cumulative counts give a RANGE of bins that should hold the ksel-th key: the
-    // bins between the sample ranks 4 standard deviations to either side of ksel/4.  One sweep
-    // then counts, exactly, the keys above that range and collects the keys inside it.  If the
-    // exact counts confirm that the ksel-th key is inside and the range fits the candidate list,
-    // the threshold is refined on the list; otherwise nothing of this is used and the full
-    // histogram pass below decides (exactness never rests on the sample).
-    {
-      for (int b = threadIdx.x; b < NBINS; b += SEL_THREADS) hist[b] = 0;
-      if (threadIdx.x == 0) { ncand_s = 0; above_s = 0; br_lo = 0; br_hi = NBINS - 1; }
-      __syncthreads();
-      for (int i0 = 0; i0 < ept; i0 += 4) {
-        const uint32_t key = keys[key_slot4(base + i0)];
-        if (key >= kmin) atomicAdd(&hist[(key - kmin) >> shift], 1);  // (padding keys are below kmin)
-      }
-      __syncthreads();
-      int c0 = 0, c1 = 0;
-      const int b0 = NBINS - 1 - 2 * static_cast<int>(threadIdx.x);
-      if (b0 >= 0) c0 = hist[b0];
-      if (b0 - 1 >= 0) c1 = hist[b0 - 1];
-      const int before = block_exclusive_scan(c0 + c1, warp_sums, &scan_total);
-      const int m_s = scan_total;  // samples in the row
-      const float pfrac = static_cast<float>(ksel) / static_cast<float>(n);
-      const int delta = static_cast<int>(4.f * sqrtf(static_cast<float>(m_s) * pfrac * (1.f - pfrac))) + 2;
-      const int r_mid = static_cast<int>(static_cast<long long>(ksel) * m_s / n);
-      const int r_hi = max(1, r_mid - delta);  // sample rank that bounds the range from above
-      const int r_lo = r_mid + delta;          // ... from below; beyond the sample: down to the lowest bin
-      if (c0 > 0 && before < r_hi && r_hi <= before + c0) br_hi = b0;
-      else if (c1 > 0 && before + c0 < r_hi && r_hi <= before + c0 + c1) br_hi = b0 - 1;
-      if (c0 > 0 && before < r_lo && r_lo <= before + c0) br_lo = b0;
-      else if (c1 > 0 && before + c0 < r_lo && r_lo <= before + c0 + c1) br_lo = b0 - 1;
-      __syncthreads();
-      const int b_hi = br_hi, b_lo = r_lo > m_s ? 0 : br_lo;
-      int cntg = 0, cnti = 0;
-      for (int i0 = 0; i0 < ept; i0 += 4) {
-        const uint4 kv = ld_keys4(keys, base + i0);
-        const uint32_t k4[4] = {kv.x, kv.y, kv.z, kv.w};
-        uint32_t bg = 0u, bi = 0u;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const uint32_t key = k4[u];
-          const int bin = static_cast<int>((key - kmin) >> shift);
-          const bool real = key >= kmin;
-          const bool gt = real && bin > b_hi;
-          const bool inb = real && bin >= b_lo && bin <= b_hi;
-          bg |= static_cast<uint32_t>(gt) << u;
-          bi |= static_cast<uint32_t>(inb) << u;
-          cntg += gt;
-          cnti += inb;
-        }
-        if (i0 < 32) { m_gt[0] |= bg << i0; m_in[0] |= bi << i0; }
-        else { m_gt[1] |= bg << (i0 - 32); m_in[1] |= bi << (i0 - 32); }
-      }
-      // the keys inside the range go to the candidate list: one atomic per warp reserves the
-      // warp's slots (a thousand single appends to one counter would take as long as the pass
-      // this replaces), a warp scan places each thread's keys
-      {
-        int inc = cnti;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, inc, o);
-          if (lane >= o) inc += y;
-        }
-        int wbase = 0;
-        if (lane == 31 && inc > 0) wbase = atomicAdd(&ncand_s, inc);
-        wbase = __shfl_sync(0xffffffffu, wbase, 31);
-        int at = wbase + inc - cnti;
-#pragma unroll
-        for (int wd = 0; wd < MASK_WORDS; ++wd) {
-          uint32_t rest = m_in[wd];
-          while (rest) {
-            const int i = wd * 32 + __ffs(rest) - 1;
-            rest &= rest - 1;
-            if (at < CAND_CAP) cand[at] = keys[key_slot4(base + i)];
-            ++at;
-          }
-        }
-      }
-      cntg = __reduce_add_sync(0xffffffffu, cntg);
-      if (lane == 0 && cntg) atomicAdd(&above_s, cntg);
-      __syncthreads();
-      const int above = above_s, inside = ncand_s;
-      __syncthreads();  // everybody has read the counts before anybody starts the next pass
-      if (above < ksel && ksel <= above + inside && inside <= CAND_CAP) {
-        first = false;
-        use_list = true;
-        ncand = inside;
-        krem = ksel - above;
-        lo = kmin + (static_cast<uint32_t>(b_lo) << shift);
-        const unsigned long long top =
-            static_cast<unsigned long long>(kmin) + (static_cast<unsigned long long>(b_hi + 1) << shift) - 1ull;
-        const uint32_t hi_key = top > kmax ? kmax : static_cast<uint32_t>(top);
-        width_m1 = hi_key - lo;
-        shift = 32 - __clz(width_m1 | 1u) - 11;
-        if (shift < 0) shift = 0;
-      } else {
-#pragma unroll
-        for (int wd = 0; wd < MASK_WORDS; ++wd) { m_gt[wd] = 0u; m_in[wd] = 0u; }
-      }
-    }
-#pragma unroll 1
-    for (;;) {
-      for (int b = threadIdx.x; b < NBINS; b += SEL_THREADS) hist[b] = 0;
-      __syncthreads();
-      if (!use_list) {
-        int cur = -1, cnt = 0;
-        for (int i0 = 0; i0 < ept; i0 += 4) {
-          const uint4 kv = ld_keys4(keys, base + i0);
-          const uint32_t k4[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const uint32_t key = k4[u];
-            const uint32_t rel = key - lo;
-            if (key >= lo && rel <= width_m1) {
-              const int b = static_cast<int>(rel >> shift);
-              if (b != cur) {
-                if (cnt) atomicAdd(&hist[cur], cnt);
-                cur = b;
-                cnt = 0;
-              }
-              ++cnt;
-            }
-          }
-        }
-        if (cnt) atomicAdd(&hist[cur], cnt);
-      } else {
-        for (int c = threadIdx.x; c < ncand; c += SEL_THREADS) {
-          const uint32_t rel = cand[c] - lo;  // wraps to a huge value for keys below lo
-          if (rel <= width_m1) atomicAdd(&hist[rel >> shift], 1);
-        }
-      }
-      __syncthreads();
-      int c0 = 0, c1 = 0;
-      const int b0 = NBINS - 1 - 2 * static_cast<int>(threadIdx.x);
-      if (b0 >= 0) c0 = hist[b0];
-      if (b0 - 1 >= 0) c1 = hist[b0 - 1];
-      const int before = block_exclusive_scan(c0 + c1, warp_sums, &scan_total);
-      if (c0 > 0 && before < krem && krem <= before + c0) {
-        sel_bin = b0;
-        sel_above = before;
-        sel_count = c0;
-      } else if (c1 > 0 && before + c0 < krem && krem <= before + c0 + c1) {
-        sel_bin = b0 - 1;
-        sel_above = before + c0;
-        sel_count = c1;
-      }
-      if (threadIdx.x == 0) ncand_s = 0;
-      __syncthreads();
-      krem -= sel_above;
-      lo += static_cast<uint32_t>(sel_bin) << shift;
-      const int in_bin = sel_count;
-      const int done = (shift == 0);
-      __syncthreads();
-      if (first) {
-        // classify own keys against the chosen bin; gather the bin's keys if they fit
-        first = false;
-        const uint32_t hi_m1 = done ? 0u : ((1u << shift) - 1u);
-        use_list = !done && in_bin <= CAND_CAP;
-        for (int i0 = 0; i0 < ept; i0 += 4) {
-          const uint4 kv = ld_keys4(keys, base + i0);
-          const uint32_t k4[4] = {kv.x, kv.y, kv.z, kv.w};
-          uint32_t bg = 0u, bi = 0u;  // four bits each
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const uint32_t key = k4[u];
-            const bool inb = key >= lo && key - lo <= hi_m1;
-            const bool gt = key >= lo && key - lo > hi_m1;
-            bg |= static_cast<uint32_t>(gt) << u;
-            bi |= static_cast<uint32_t>(inb) << u;
-            if (inb && use_list) cand[atomicAdd(&ncand_s, 1)] = key;
-          }
-          // i0 is a multiple of 4: the four bits never straddle a mask word
-          if (i0 < 32) { m_gt[0] |= bg << i0; m_in[0] |= bi << i0; }
-          else { m_gt[1] |= bg << (i0 - 32); m_in[1] |= bi << (i0 - 32); }
-        }
-        __syncthreads();
-        ncand = ncand_s;
-      }
-      if (done) break;
-      width_m1 = (1u << shift) - 1u;
-      shift = shift > 11 ? shift - 11 : 0;
-    }
-    T = lo;
-  } else {
-    // every key equals T
-#pragma unroll
-    for (int wd = 0; wd < MASK_WORDS; ++wd)
-      for (int i = wd * 32; i < min(ept, wd * 32 + 32); ++i)
-        if (base + i < n) m_in[wd] |= 1u << (i & 31);
-  }
-  const int need_eq = krem;
-
-  // ---- 3. ordered compaction
-  // Keys inside the first bin are compared with the final threshold (few per thread), the
-  // rest is known from the bit masks; one block scan gives every thread its output offset.
-  uint32_t m_eq[MASK_WORDS];
-  int cg = 0, ce = 0;
-#pragma unroll
-  for (int wd = 0; wd < MASK_WORDS; ++wd) {
-    m_eq[wd] = 0u;
-    uint32_t rest = m_in[wd];
-    while (rest) {
-      const int i = wd * 32 + __ffs(rest) - 1;
-      rest &= rest - 1;
-      const uint32_t key = keys[key_slot4(base + i)];
-      if (key > T) m_gt[wd] |= 1u << (i & 31);
-      else if (key == T) m_eq[wd] |= 1u << (i & 31);
-    }
-    cg += __popc(m_gt[wd]);
-    ce += __popc(m_eq[wd]);
-  }
-  // Two counts in one scan: keys above the threshold in the high half, keys equal to it in
-  // the low half.  Either total is at most n <= FAST_MAX_KEYS < 65536, so the low half never
-  // carries into the high one, and the word is unsigned so that a high half of 32768 or more
-  // (ksel that large is valid) stays a count after the shift.
-  static_assert(FAST_MAX_KEYS < 65536, "two 16-bit counts share one scan word");
-  uint32_t* scan_u = reinterpret_cast<uint32_t*>(warp_sums);
-  const uint32_t packed =
-      block_exclusive_scan<uint32_t>((static_cast<uint32_t>(cg) << 16) | static_cast<uint32_t>(ce),
-                                     scan_u, reinterpret_cast<uint32_t*>(&scan_total));
-  int eq_before = static_cast<int>(packed & 0xffffu);
-  int out_pos = static_cast<int>(packed >> 16) + min(eq_before, need_eq);
-  int32_t* orow = out_idx + static_cast<size_t>(row) * ksel;
-#pragma unroll
-  for (int wd = 0; wd < MASK_WORDS; ++wd) {
-    uint32_t rest = m_gt[wd] | m_eq[wd];
-    while (rest) {
-      const int bit = __ffs(rest) - 1;
-      rest &= rest - 1;
-      const bool is_eq = (m_eq[wd] >> bit) & 1u;
-      if (!is_eq || eq_before++ < need_eq) orow[out_pos++] = base + wd * 32 + bit;
-    }
-  }
-}
 
 // ---------------------------------------------------------------------------------------
 // Rows too long for one CTA's shared memory: the same radix select spread over many CTAs.
@@ -882,9 +462,6 @@ static DeviceOnce& select_attr_once() {
   return once;
 }
 
-static inline int key_slot4_host(int j) { return j + ((j >> 5) << 2); }
-constexpr int FAST_SMEM_BYTES = (FAST_MAX_KEYS + FAST_MAX_KEYS / 8 + 64) * 4;
-
 bool select_needs_scratch(int n) { return n > SEL_SMEM_KEYS; }
 
 static inline size_t up256(size_t x) { return (x + 255) / 256 * 256; }
@@ -907,44 +484,11 @@ cudaError_t launch_pool_topk(const float* vote, int rows, int n, int pool_kernel
     cudaError_t e = cudaFuncSetAttribute(pool_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          SEL_SMEM_KEYS * 4);
     if (e != cudaSuccess) return e;
-#define SNAPKV_FAST_ATTR(RM, P)                                                              \
-  e = cudaFuncSetAttribute(pool_topk_fast_kernel<RM, P>,                                     \
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, FAST_SMEM_BYTES);    \
-  if (e != cudaSuccess) return e;
-    SNAPKV_FAST_ATTR(3, -1) SNAPKV_FAST_ATTR(7, -1)
-    SNAPKV_FAST_ATTR(2, 0) SNAPKV_FAST_ATTR(2, 1) SNAPKV_FAST_ATTR(3, 0) SNAPKV_FAST_ATTR(3, 1)
-    SNAPKV_FAST_ATTR(6, 0) SNAPKV_FAST_ATTR(6, 1)
-#undef SNAPKV_FAST_ATTR
     once.set();
   }
-  const int r = pool_kernel >> 1;
-  // One cluster of small CTAs per row: for rows too long for the one-CTA kernel below, and
-  // whenever there are too few rows to fill the GPU with one CTA each.  The cluster kernel's
-  // chain of cluster barriers takes about 17-21 us whatever the row count (measured: 32 rows
-  // of 32736 in 21 us, 64 in 25 us, 128 in 45 us); the one-CTA kernel takes about 26-28 us for
-  // any number of rows up to the SM count.
-  const bool one_cta_fits = n <= FAST_MAX_KEYS && r <= 7;
-  if ((!one_cta_fits || rows <= 48) && select_cluster_applies(rows, n, pool_kernel))
+  if (select_cluster_applies(rows, n, pool_kernel))
     return launch_pool_topk_cluster(vote, rows, n, pool_kernel, pool_type, ksel, out_idx, stream,
-                                    launches, gsum);
-  if (one_cta_fits) {
-    const int ept = (((n + SEL_THREADS - 1) / SEL_THREADS) + 7) & ~7;
-    const int words = key_slot4_host(SEL_THREADS * ept) + 4;
-#define SNAPKV_FAST_LAUNCH(RM, P)                                                            \
-  pool_topk_fast_kernel<RM, P><<<rows, SEL_THREADS, words * 4, stream>>>(vote, n, gsum, r,    \
-                                                                        pool_type, ept, ksel, out_idx, \
-                                                                        vote_is_scratch ? 1 : 0)
-    // the paper's kernel sizes 5, 7 and 13 have instantiations of their own
-    const bool mx = pool_type == 0;
-    if (r == 2) { if (mx) SNAPKV_FAST_LAUNCH(2, 0); else SNAPKV_FAST_LAUNCH(2, 1); }
-    else if (r == 3) { if (mx) SNAPKV_FAST_LAUNCH(3, 0); else SNAPKV_FAST_LAUNCH(3, 1); }
-    else if (r == 6) { if (mx) SNAPKV_FAST_LAUNCH(6, 0); else SNAPKV_FAST_LAUNCH(6, 1); }
-    else if (r <= 3) SNAPKV_FAST_LAUNCH(3, -1);
-    else SNAPKV_FAST_LAUNCH(7, -1);
-#undef SNAPKV_FAST_LAUNCH
-    *launches += 1;
-    return cudaGetLastError();
-  }
+                                    launches, gsum, vote_is_scratch);
   if (!select_needs_scratch(n)) {  // fits one CTA, but the radius is beyond the fast path
     pool_topk_kernel<<<rows, SEL_THREADS, static_cast<size_t>(n) * 4, stream>>>(
         vote, n, gsum, pool_kernel, pool_type, ksel, out_idx, nullptr);

@@ -1,88 +1,82 @@
-// Pooling and per-head top-k (Listing 1's pool1d and topk; Eq. 2) for rows of a few thousand to
-// 131072 positions: one thread-block CLUSTER per row.
+// Pooling and per-head top-k (Listing 1's pool1d and topk; Eq. 2): one thread-block CLUSTER of 1
+// to 16 CTAs per row, pooling radii up to 7, rows of up to 524288 positions.
 //
-// A row is cut into C chunks, one CTA of 256 threads each; a thread keeps its EPT consecutive
-// pooled keys in registers for the whole kernel.  The CTAs of a row talk through distributed
-// shared memory only:
-//   1. votes of the chunk (plus the pooling halo) go to shared memory with coalesced loads,
-//      each thread pools its own positions and turns them into order-preserving 32-bit keys;
-//   2. radix select of the ksel-th largest key, most significant byte first: every CTA
-//      histograms its keys that match the prefix found so far (256 bins), the cluster meets at
-//      a barrier, every CTA adds up the C histograms (thread t owns bin t, one remote read per
-//      peer) and walks the bins from the top - all CTAs get the same digit without a second
-//      exchange.  Two histogram buffers alternate, so that a CTA may clear the next one while
-//      its peers still read the current one;
-//   3. ordered compaction: keys above the threshold, plus the lowest-position keys equal to
-//      it until ksel are out; a block scan gives the offset inside the CTA, the CTA totals go
-//      round the cluster for the offset of the chunk.
-// Ties go to the lower position by construction.  The only waits are cluster barriers (every
-// CTA of a cluster is resident by definition and reaches every barrier); a last barrier
-// keeps a CTA's shared memory alive until its peers have finished reading it.
-//
-// Small CTAs with few registers spread a row over up to 16 SMs and fill all of them, where
-// one CTA per row leaves SMs idle whenever there are fewer rows than SMs and pays a whole
-// row's latency on a single SM.
+// The votes come from L2 and are few (17 MB for 128 rows of 32K); what a row costs is the chain of
+// steps that its threads take together.  So the chain is kept short:
+//   1. a CTA's chunk of votes (plus the pooling halo) goes to shared memory with coalesced loads;
+//      every thread pools its own EPT consecutive positions and keeps them, as order-preserving
+//      32-bit keys, in registers for the rest of the kernel;
+//   2. a small histogram of 256 pooled values sampled over the whole row, the same in every CTA,
+//      gives the bins that lie four standard deviations to either side of the rank that ksel maps
+//      to; they bound a window of keys which should hold the ksel-th largest;
+//   3. the keys inside the window (a sixth of a row, a few per cent when ksel << n) are histogrammed
+//      into 1024 bins, those above it counted; the CTAs of the cluster add up one another's
+//      histograms through distributed shared memory, and all find the same bin;
+//   4. that bin's few keys (about five for a row of 32K) are pushed, with the CTA's counts, into
+//      every CTA's memory: each CTA ranks them by counting and knows the threshold, and how many
+//      selected positions come before its chunk;
+//   5. ordered compaction: a block scan, positions staged in shared memory, coalesced stores.
+// The sample only guesses.  Counts are exact: when the ksel-th key turns out to lie outside the
+// window the histogram is taken over the whole key range, and a bin with more keys than the list
+// holds is refined by a further histogram; ties go to the lower position by construction.
+// Two cluster barriers on the usual path (a byte-wise radix select took five), one histogram
+// update for every sixth key.  Back to back: 4 rows of 992 in 6.0 us (one CTA per row with all keys
+// in shared memory and five passes over them: 12.4 us), 32 rows of 16352 in 11.6 us (14.4), 128 rows
+// of 32736 in 16.8 us (20.6), 32 rows of 131008 in 22.7 us (49.9), 32 rows of 379968 in 118 us (177:
+// eight launches with the keys in global memory).
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <atomic>
 
+#include "launch.cuh"
+#include "sm100_ptx.cuh"
 #include "snapkv_internal.h"
 
 namespace snapkv {
 
 namespace {
 
-constexpr int CL_THREADS = 256;
-constexpr int CL_WARPS = CL_THREADS / 32;
-constexpr int CL_RMAX = 7;          // largest pooling radius this kernel takes
-constexpr int CL_MAX_CLUSTER = 16;  // 16 needs the non-portable cluster size
-constexpr int CL_BINS = 256;
-constexpr int CL_COPIES = 4;        // private histogram copies per CTA (two warps share one)
+constexpr int CL_RMAX = 7;           // largest pooling radius this kernel takes
+constexpr int CL_MAX_CLUSTER = 16;   // above 8: non-portable cluster size
+constexpr int CL_BINS = 1024;
+constexpr int CL_SAMPLES = 256;
+constexpr int CL_SAMPLE_BINS = 512;
+constexpr int CL_LIST = 2048;        // candidates in all of a cluster's lists
+constexpr uint32_t KEY_MIN = 0x80000000u;  // key of a vote of zero; below it: no position
 
 __device__ __forceinline__ uint32_t float_to_key(float x) {
   const uint32_t b = __float_as_uint(x);
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank) {
   uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
   return r;
 }
-__device__ __forceinline__ uint32_t cluster_size() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-  return r;
+__device__ __forceinline__ void st_peer2(uint32_t addr, uint32_t a, uint32_t b) {
+  asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
-// All threads of all CTAs of the cluster; orders shared-memory accesses across the cluster.
-__device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Address of the same shared-memory variable in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ int ld_peer(uint32_t addr) {
-  int v;
-  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_peer(uint32_t addr, int v) {
-  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// Tells L2 that a 128-byte line (global memory, 128-byte aligned) holds nothing worth keeping:
+// a dirty line may then be dropped instead of written back.  Its contents are undefined afterwards.
+__device__ __forceinline__ void discard_l2_line(const void* p) {
+  asm volatile("discard.global.L2 [%0], 128;" ::"l"(__cvta_generic_to_global(p)) : "memory");
 }
 
-// slot of position t of the staged chunk: one pad word per 32, so that threads reading
-// consecutive runs of EPT positions do not meet in a bank
-__device__ __forceinline__ int slot(int t) { return t + (t >> 5); }
+// Slot of position t of the staged chunk: four pad words after every 32, so that a thread reads
+// its run (a multiple of 8 positions) as aligned 16-byte vectors and the runs of neighbouring
+// threads fall into different banks.
+__device__ __forceinline__ int slot(int t) { return t + ((t >> 5) << 2); }
+constexpr int slots_for(int n) { return n + n / 8 + 8; }
 
-// Exclusive prefix sum over the CTA's 256 threads (8 warps); *total_s holds the sum after the
-// second barrier inside.
-__device__ __forceinline__ uint32_t cta_exclusive_scan(uint32_t x, uint32_t* warp_sums_s, uint32_t* total_s) {
+// Exclusive prefix sum over the CTA's threads; *total_s holds the sum afterwards.  Two barriers.
+template <int THREADS>
+__device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t* warp_sums_s, uint32_t* total_s) {
+  constexpr int WARPS = THREADS / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t inc = x;
 #pragma unroll
@@ -93,255 +87,546 @@ __device__ __forceinline__ uint32_t cta_exclusive_scan(uint32_t x, uint32_t* war
   if (lane == 31) warp_sums_s[warp] = inc;
   __syncthreads();
   if (warp == 0) {
-    const uint32_t w = lane < CL_WARPS ? warp_sums_s[lane] : 0u;
+    const uint32_t w = lane < WARPS ? warp_sums_s[lane] : 0u;
     uint32_t winc = w;
 #pragma unroll
-    for (int o = 1; o < CL_WARPS; o <<= 1) {
+    for (int o = 1; o < WARPS; o <<= 1) {
       const uint32_t y = __shfl_up_sync(0xffffffffu, winc, o);
       if (lane >= o) winc += y;
     }
-    if (lane < CL_WARPS) warp_sums_s[lane] = winc - w;
-    if (lane == CL_WARPS - 1) *total_s = winc;
+    if (lane < WARPS) warp_sums_s[lane] = winc - w;
+    if (lane == WARPS - 1) *total_s = winc;
   }
   __syncthreads();
   return warp_sums_s[warp] + inc - x;
 }
 
-// R, PT >= 0: the pooling radius is exactly R and the type PT (0 max, 1 avg), no per-tap tests.
-// PT = -1: radius r <= R and pool_type are run-time values.
-template <int EPT, int R, int PT>
-__global__ void __launch_bounds__(CL_THREADS)
-pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r, int pool_type,
-                         int ksel, int32_t* __restrict__ out_idx) {
-  constexpr int CHUNK = CL_THREADS * EPT;
-  constexpr int STAGED = CHUNK + 2 * CL_RMAX;
-  __shared__ float raw[STAGED + STAGED / 32 + 1];
-  __shared__ int hist[2][CL_BINS];        // the CTA's histogram of a round, read by the peers
-  __shared__ int hist_w[CL_COPIES][CL_BINS];  // private histograms, one per pair of warps
-  __shared__ int totals[CL_MAX_CLUSTER][2];  // per CTA of the cluster: keys above / equal to the threshold
-  __shared__ uint32_t warp_sums[CL_WARPS];
-  __shared__ uint32_t scan_total;
-  __shared__ int sel_bin, sel_above;
+// Sliding pooling of eight positions: out[i] over a[i .. i + 2R].  The maximum is taken over
+// doubling spans (three or four operations per position instead of 2R + 1; a maximum is the same
+// in any order), the sum in ascending order.
+template <int R, int PT>
+__device__ __forceinline__ void pool8(const float* a, float (&out)[8], int r, int pool_type, float divisor) {
+  if constexpr (PT == 0 && (R == 2 || R == 3 || R == 6)) {
+    float m2[2 * R + 7], m4[2 * R + 5];
+#pragma unroll
+    for (int i = 0; i < 2 * R + 7; ++i) m2[i] = fmaxf(a[i], a[i + 1]);
+#pragma unroll
+    for (int i = 0; i < 2 * R + 5; ++i) m4[i] = fmaxf(m2[i], m2[i + 2]);
+    if constexpr (R == 6) {
+      float m8[13];
+#pragma unroll
+      for (int i = 0; i < 13; ++i) m8[i] = fmaxf(m4[i], m4[i + 4]);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) out[i] = fmaxf(fmaxf(m8[i], m8[i + 5]), 0.f);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) out[i] = fmaxf(fmaxf(m4[i], m4[i + 2 * R - 3]), 0.f);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float p = 0.f;  // votes are >= 0: zero is neutral for max and is the padding of avg
+#pragma unroll
+      for (int t = 0; t <= 2 * R; ++t)
+        if (PT >= 0 || (t - R >= -r && t - R <= r))
+          p = (PT >= 0 ? PT == 0 : pool_type == 0) ? fmaxf(p, a[i + t]) : p + a[i + t];
+      if (PT < 0 && divisor != 0.f) p = p / divisor;
+      out[i] = p;
+    }
+  }
+}
 
-  const uint32_t C = cluster_size(), rank = cluster_rank();
-  const int row = blockIdx.x / C;
+// R, PT >= 0: the pooling radius is exactly R and the type PT (0 max, 1 avg), no per-tap tests.
+// PT = -1: radius r <= R and pool_type are run-time values, and with `divisor` != 0 average pooling
+// divides the window sum by it (otherwise rows are ranked by the sum, which orders the same way up
+// to rounding).  `want`: the sample ranks (from the top) that bound the window.
+template <int THREADS, int EPT, int R, int PT>
+__global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 1024 / THREADS)
+pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r, int pool_type, float divisor,
+                         int ksel, int2 want, int32_t* __restrict__ out_idx, int ctas, int discard_votes) {
+  constexpr int CHUNK = THREADS * EPT;
+  constexpr int BPT = CL_BINS / THREADS;      // bins a thread owns in the scans
+  extern __shared__ __align__(16) uint32_t stage[];  // votes of the chunk, later the selected positions
+  __shared__ float halo[2][CL_RMAX + 1];      // CL_RMAX positions before the chunk and behind it
+  __shared__ __align__(16) uint32_t hist[2][CL_BINS + 4];  // word CL_BINS: keys above the window
+  __shared__ __align__(16) uint32_t samp_hist[CL_SAMPLE_BINS];
+  __shared__ uint32_t samp_min[CL_SAMPLES / 32], samp_max[CL_SAMPLES / 32];
+  __shared__ __align__(8) uint2 list[CL_LIST];           // {key, position}, a region per CTA of the cluster
+  __shared__ __align__(8) uint2 totals[CL_MAX_CLUSTER];  // per CTA: keys above the bin, keys inside it
+  __shared__ uint32_t warp_sums[32];
+  __shared__ uint32_t scan_total, sel_bin, sel_above, sel_count, win_hi, win_lo, n_list, n_gt;
+  __shared__ uint32_t thr_key, thr_eq, thr_all, before_gt, before_eq;
+
+  const uint32_t C = ctas, rank = blockIdx.x % ctas;
+  const int row = blockIdx.x / ctas;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int c0 = static_cast<int>(rank) * CHUNK;  // first position of this CTA's chunk
   const float* vrow = vote + static_cast<size_t>(row) * gsum * n;
+  pdl_wait();
+  if (C > 1) cluster_arrive();  // waited for before the first access to a peer's memory
 
-  // ---- 1. stage the chunk and its halo: position c0 - CL_RMAX + t at slot(t); zero outside the row.
-  // All of a thread's loads are issued before the first value is stored: the votes come from
-  // L2, and a loop of load-then-store would pay that latency once per element.
+  // ---- 1. the sample (pooled values at 256 positions spread over the whole row), the chunk and its
+  // halo: all loads are issued before the first value is used.  Positions outside the row are zero.
+  // A group's votes are summed in ascending head order.
+  float tap[2 * R + 1];
+  const int js = static_cast<int>((static_cast<long long>(tid) * n + n / 2) / CL_SAMPLES);
+  if (tid < CL_SAMPLES) {
+#pragma unroll
+    for (int t = 0; t <= 2 * R; ++t) {
+      const int j = js + t - R;
+      tap[t] = static_cast<unsigned>(j) < static_cast<unsigned>(n) ? __ldg(vrow + j) : 0.f;
+    }
+    for (int g = 1; g < gsum; ++g) {
+      const float* src = vrow + static_cast<size_t>(g) * n;
+#pragma unroll
+      for (int t = 0; t <= 2 * R; ++t) {
+        const int j = js + t - R;
+        if (static_cast<unsigned>(j) < static_cast<unsigned>(n)) tap[t] += __ldg(src + j);
+      }
+    }
+  }
+  float h_val = 0.f;
+  if (tid >= THREADS - 2 * CL_RMAX) {
+    const int i = tid - (THREADS - 2 * CL_RMAX);
+    const int j = i < CL_RMAX ? c0 - CL_RMAX + i : c0 + CHUNK + i - CL_RMAX;
+    if (static_cast<unsigned>(j) < static_cast<unsigned>(n)) {
+      h_val = __ldg(vrow + j);
+      for (int g = 1; g < gsum; ++g) h_val += __ldg(vrow + static_cast<size_t>(g) * n + j);
+    }
+  }
   {
     float x[EPT];
 #pragma unroll
-    for (int i = 0; i < EPT; ++i) {
-      const int j = c0 + static_cast<int>(threadIdx.x) + CL_THREADS * i;
-      x[i] = (j < n) ? __ldg(vrow + j) : 0.f;
+    for (int u = 0; u < EPT; ++u) {
+      const int j = c0 + tid + THREADS * u;
+      x[u] = j < n ? __ldg(vrow + j) : 0.f;
     }
-    for (int g = 1; g < gsum; ++g) {  // ascending head order
+    for (int g = 1; g < gsum; ++g) {
       const float* src = vrow + static_cast<size_t>(g) * n;
 #pragma unroll
-      for (int i = 0; i < EPT; ++i) {
-        const int j = c0 + static_cast<int>(threadIdx.x) + CL_THREADS * i;
-        if (j < n) x[i] += __ldg(src + j);
+      for (int u = 0; u < EPT; ++u) {
+        const int j = c0 + tid + THREADS * u;
+        if (j < n) x[u] += __ldg(src + j);
       }
     }
 #pragma unroll
-    for (int i = 0; i < EPT; ++i) raw[slot(CL_RMAX + static_cast<int>(threadIdx.x) + CL_THREADS * i)] = x[i];
-    if (threadIdx.x < 2 * CL_RMAX) {  // the halo: CL_RMAX positions before the chunk, CL_RMAX after
-      const int t = threadIdx.x < CL_RMAX ? static_cast<int>(threadIdx.x)
-                                          : CHUNK + static_cast<int>(threadIdx.x);
-      const int j = c0 - CL_RMAX + t;
-      float h = 0.f;
-      if (j >= 0 && j < n) {
-        h = __ldg(vrow + j);
-        for (int g = 1; g < gsum; ++g) h += __ldg(vrow + static_cast<size_t>(g) * n + j);
-      }
-      raw[slot(t)] = h;
+    for (int u = 0; u < EPT; ++u) stage[slot(tid + THREADS * u)] = __float_as_uint(x[u]);
+  }
+  if (tid >= THREADS - 2 * CL_RMAX) {
+    const int i = tid - (THREADS - 2 * CL_RMAX);
+    halo[i >= CL_RMAX][i >= CL_RMAX ? i - CL_RMAX : i] = h_val;
+  }
+  uint32_t s_key = 0u;
+  if (tid < CL_SAMPLES) {
+    float p = 0.f;
+#pragma unroll
+    for (int t = 0; t <= 2 * R; ++t)
+      if (PT >= 0 || (t - R >= -r && t - R <= r))
+        p = (PT >= 0 ? PT == 0 : pool_type == 0) ? fmaxf(p, tap[t]) : p + tap[t];
+    if (PT < 0 && divisor != 0.f) p = p / divisor;
+    s_key = float_to_key(p);
+    const uint32_t lo = __reduce_min_sync(0xffffffffu, s_key), hi = __reduce_max_sync(0xffffffffu, s_key);
+    if (lane == 0) {
+      samp_min[warp] = lo;
+      samp_max[warp] = hi;
     }
   }
+  for (int b = tid; b < CL_SAMPLE_BINS; b += THREADS) samp_hist[b] = 0u;
+  for (int b = tid; b < CL_BINS + 4; b += THREADS) hist[0][b] = 0u;
+  if (tid == 0) {
+    sel_bin = ~0u;
+    n_list = n_gt = before_gt = before_eq = 0u;
+  }
   __syncthreads();
+
+  // ---- 2. the window, from a histogram of the sample: the bins that hold the sample ranks four
+  // standard deviations to either side of the rank that ksel maps to
+  uint32_t smin = ~0u, smax = 0u;
+  if (tid < CL_SAMPLES) {
+#pragma unroll
+    for (int w = 0; w < CL_SAMPLES / 32; ++w) {
+      smin = min(smin, samp_min[w]);
+      smax = max(smax, samp_max[w]);
+    }
+  }
+  const int sshift = max(0, 23 - __clz(smax - smin));  // (range >> sshift) < CL_SAMPLE_BINS
+  if (tid < CL_SAMPLES) atomicAdd(&samp_hist[(s_key - smin) >> sshift], 1u);
+  __syncthreads();
+  if (warp == 0) {  // lane t owns the 16 bins CL_SAMPLE_BINS - 16 t - 1 and down
+    static_assert(CL_SAMPLE_BINS == 512, "16 bins per lane");
+    const uint32_t want_hi = static_cast<uint32_t>(max(1, want.x + 1));
+    const uint32_t want_lo = static_cast<uint32_t>(min(CL_SAMPLES, want.y + 1));
+    uint32_t c[16], sum = 0u;
+#pragma unroll
+    for (int i = 0; i < 16; i += 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(samp_hist + CL_SAMPLE_BINS - 16 * (lane + 1) + i);
+      c[i] = v.x; c[i + 1] = v.y; c[i + 2] = v.z; c[i + 3] = v.w;
+      sum += v.x + v.y + v.z + v.w;
+    }
+    uint32_t above = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, above, o);
+      if (lane >= o) above += y;
+    }
+    above -= sum;
+#pragma unroll
+    for (int i = 15; i >= 0; --i) {
+      const uint32_t edge = smin + (static_cast<uint32_t>(CL_SAMPLE_BINS - 16 * (lane + 1) + i) << sshift);
+      if (above < want_hi && want_hi <= above + c[i]) win_hi = min(edge + ((1u << sshift) - 1u), smax);
+      if (above < want_lo && want_lo <= above + c[i]) win_lo = want.y >= CL_SAMPLES ? KEY_MIN : edge;
+      above += c[i];
+    }
+  }
 
   // ---- pooling: thread owns positions c0 + base .. c0 + base + EPT - 1
-  const int base = threadIdx.x * EPT;
+  const int base = tid * EPT;
   uint32_t key[EPT];
   {
-    float a[EPT + 2 * R];
+    auto own8 = [&](int i, float* dst) {  // positions base + i .. + 7 of the chunk
 #pragma unroll
-    for (int i = 0; i < EPT + 2 * R; ++i) a[i] = raw[slot(base + (CL_RMAX - R) + i)];
+      for (int q = 0; q < 8; q += 4) {
+        const uint4 v = *reinterpret_cast<const uint4*>(stage + slot(base + i + q));
+        dst[q] = __uint_as_float(v.x);
+        dst[q + 1] = __uint_as_float(v.y);
+        dst[q + 2] = __uint_as_float(v.z);
+        dst[q + 3] = __uint_as_float(v.w);
+      }
+    };
+    auto at = [&](int t) {  // position t of the chunk or its halo
+      return t < 0 ? halo[0][CL_RMAX + t] : (t >= CHUNK ? halo[1][t - CHUNK] : __uint_as_float(stage[slot(t)]));
+    };
+    // a[]: the R values before the current block of eight, the block, the next block
+    float a[R + 16];
+#pragma unroll
+    for (int i = 0; i < R; ++i) a[i] = at(base - R + i);
+    own8(0, a + R);
+#pragma unroll
+    for (int sb = 0; sb < EPT; sb += 8) {
+      if (sb + 8 < EPT) {
+        own8(sb + 8, a + R + 8);
+      } else {
+#pragma unroll
+        for (int i = 0; i < R; ++i) a[R + 8 + i] = at(base + EPT + i);
+      }
+      float p[8];
+      pool8<R, PT>(a, p, r, pool_type, divisor);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) key[sb + i] = (c0 + base + sb + i < n) ? float_to_key(p[i]) : 0u;
+#pragma unroll
+      for (int i = 0; i < R + 8; ++i) a[i] = a[i + 8];
+    }
+  }
+  __syncthreads();
+
+  // ---- 3. histogram rounds: the usual path takes one.  Keys lo .. lo + width take part, `top`
+  // counts those above.
+  uint32_t lo = win_lo, width = win_hi - win_lo;
+  int shift = max(0, 22 - __clz(width));  // (width >> shift) < CL_BINS
+  uint32_t krem = static_cast<uint32_t>(ksel);
+  const uint32_t cap = min(CL_LIST / C, static_cast<uint32_t>(CL_SAMPLES));  // a thread per entry
+  bool guess = true;
+  uint32_t bin_lo = 0u, bin_w = 0u, in_bin = 0u;
+#pragma unroll 1
+  for (int round = 0;; ++round) {
+    uint32_t* h = hist[round & 1];
+    if (round > 0) {
+      for (int b = tid; b < CL_BINS + 4; b += THREADS) h[b] = 0u;
+      if (tid == 0) sel_bin = ~0u;
+      __syncthreads();
+    }
+    uint32_t top = 0u;
+    const uint32_t hi = lo + width;
 #pragma unroll
     for (int i = 0; i < EPT; ++i) {
-      float p = 0.f;  // votes are >= 0: zero is neutral for max and is the avg padding
-#pragma unroll
-      for (int t = 0; t <= 2 * R; ++t) {
-        const int off = t - R;
-        if (PT >= 0 || (off >= -r && off <= r))
-          p = ((PT >= 0) ? (PT == 0) : (pool_type == 0)) ? fmaxf(p, a[i + t]) : p + a[i + t];
-      }
-      // average pooling ranks by the window sum: dividing by the kernel size is monotone.
-      // Positions past the row's end rank below every real key (votes >= 0 set the top bit).
-      key[i] = (c0 + base + i < n) ? float_to_key(p) : 0u;
+      const uint32_t rel = key[i] - lo;  // wraps for keys below lo
+      if (rel <= width) atomicAdd(&h[rel >> shift], 1u);
+      top += key[i] > hi;
     }
-  }
-
-  // ---- 2. radix select, one byte per round from the top
-  // Pairs of warps count into a histogram of their own (pooled neighbours mostly share a bin,
-  // and in the first rounds so do most keys of the row: one shared histogram would serialise
-  // the whole CTA on a few words); thread t then adds the copies of bin t, publishes the sum
-  // in the CTA's histogram of this round and clears the copies for the next round.
-  uint32_t prefix = 0u, mask = 0u;
-  int krem = ksel;
-  const uint32_t hist_base = smem_addr(&hist[0][0]);
-  const int warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int w = 0; w < CL_COPIES; ++w) hist_w[w][threadIdx.x] = 0;  // CL_BINS == CL_THREADS
-  __syncthreads();
-#pragma unroll 1
-  for (int round = 0; round < 4; ++round) {
-    const int shift = 24 - 8 * round;
+    if (guess) {
+      top = __reduce_add_sync(0xffffffffu, top);
+      if (lane == 0 && top) atomicAdd(&h[CL_BINS], top);
+    }
+    if (C > 1) {
+      if (round == 0) cluster_wait();
+      cluster_arrive();  // the cluster's barrier stands in for the CTA's
+      cluster_wait();
+    } else {
+      __syncthreads();
+    }
+    // thread t owns the bins CL_BINS - 1 - BPT t and down; thread 0 also the keys above the window
+    uint32_t c[BPT], sum = 0u;
+    top = 0u;
     {
-      int* h = hist_w[warp % CL_COPIES];
-      int cur = -1, cnt = 0;  // count runs of equal bins
+      const int b0 = CL_BINS - BPT * (tid + 1);
 #pragma unroll
-      for (int i = 0; i < EPT; ++i) {
-        if ((key[i] & mask) == prefix) {
-          const int b = static_cast<int>((key[i] >> shift) & 255u);
-          if (b != cur) {
-            if (cnt) atomicAdd(&h[cur], cnt);
-            cur = b;
-            cnt = 0;
+      for (int u = 0; u < BPT; ++u) c[u] = 0u;
+      if (C == 1) {
+#pragma unroll
+        for (int u = 0; u < BPT; ++u) c[u] = h[b0 + u];
+        if (tid == 0) top = h[CL_BINS];
+      } else {
+        // the peers' reads are in flight four at a time
+#pragma unroll 1
+        for (uint32_t p0 = 0; p0 < C; p0 += 4) {
+          uint32_t x[4][BPT];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint32_t addr = peer_addr(h + b0, min(p0 + q, C - 1));
+            if constexpr (BPT == 4)
+              asm volatile("ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [%4];"
+                           : "=r"(x[q][0]), "=r"(x[q][1]), "=r"(x[q][2]), "=r"(x[q][3]) : "r"(addr) : "memory");
+            else if constexpr (BPT == 2)
+              asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(x[q][0]), "=r"(x[q][1]) : "r"(addr) : "memory");
+            else
+              asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x[q][0]) : "r"(addr) : "memory");
           }
-          ++cnt;
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int u = 0; u < BPT; ++u) c[u] += p0 + q < C ? x[q][u] : 0u;
+        }
+        if (warp == 0) {
+          uint32_t x = 0u;
+          if (static_cast<uint32_t>(lane) < C)
+            asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x) : "r"(peer_addr(h + CL_BINS, lane)) : "memory");
+          x = __reduce_add_sync(0xffffffffu, x);
+          if (lane == 0) top = x;
         }
       }
-      if (cnt) atomicAdd(&h[cur], cnt);
-    }
-    __syncthreads();
-    {
-      int sum = 0;
 #pragma unroll
-      for (int w = 0; w < CL_COPIES; ++w) {
-        sum += hist_w[w][threadIdx.x];
-        hist_w[w][threadIdx.x] = 0;
+      for (int u = 0; u < BPT; ++u) sum += c[u];
+    }
+    uint32_t above = block_scan<THREADS>(sum + top, warp_sums, &scan_total) + top;
+#pragma unroll
+    for (int u = BPT - 1; u >= 0; --u) {
+      if (above < krem && krem <= above + c[u]) {
+        sel_bin = static_cast<uint32_t>(CL_BINS - BPT * (tid + 1) + u);
+        sel_above = above;
+        sel_count = c[u];
       }
-      hist[round & 1][threadIdx.x] = sum;
-    }
-    cluster_barrier();  // every CTA's histogram of this round is complete
-    int cnt_bin = 0;    // thread t owns bin 255 - t: the scan below then runs from the top bin down
-    {
-      const uint32_t my = hist_base + static_cast<uint32_t>(((round & 1) * CL_BINS + (255 - static_cast<int>(threadIdx.x))) * 4);
-      // all remote reads are issued before the first one is used
-      int part[CL_MAX_CLUSTER];
-#pragma unroll
-      for (uint32_t p = 0; p < CL_MAX_CLUSTER; ++p) part[p] = p < C ? ld_peer(peer_addr(my, p)) : 0;
-#pragma unroll
-      for (uint32_t p = 0; p < CL_MAX_CLUSTER; ++p) cnt_bin += part[p];
-    }
-    const int above = static_cast<int>(cta_exclusive_scan(static_cast<uint32_t>(cnt_bin), warp_sums, &scan_total));
-    if (cnt_bin > 0 && above < krem && krem <= above + cnt_bin) {
-      sel_bin = 255 - static_cast<int>(threadIdx.x);
-      sel_above = above;
+      above += c[u];
     }
     __syncthreads();
-    prefix |= static_cast<uint32_t>(sel_bin) << shift;
-    mask |= 255u << shift;
+    const uint32_t b = sel_bin;
+    if (b == ~0u) {  // above the guessed window or below it: the whole range decides
+      guess = false;
+      lo = KEY_MIN;
+      width = ~KEY_MIN;
+      shift = 21;
+      __syncthreads();  // everybody has read sel_bin before it is written again
+      continue;
+    }
+    guess = false;
     krem -= sel_above;
-    // (sel_bin and the warps' histograms are written again only behind the next barriers; a
-    // peer reads hist[round & 1] until it arrives at the next cluster barrier, and this CTA
-    // writes that buffer again two rounds on)
+    in_bin = sel_count;
+    bin_lo = lo + (b << shift);
+    bin_w = (1u << shift) - 1u;
+    if (shift == 0 || in_bin <= cap) break;
+    lo = bin_lo;
+    width = bin_w;
+    shift = max(0, shift - 10);
+    __syncthreads();
   }
-  const uint32_t T = prefix;  // key of the ksel-th largest pooled vote of the row
-  const int need_eq = krem;   // how many positions equal to it are kept (the lowest ones)
+  const bool listed = shift > 0;  // else every key of the bin equals bin_lo
 
-  // ---- 3. ordered compaction
-  uint32_t m_gt = 0u, m_eq = 0u;  // EPT <= 32
+  // ---- 4. the bin's keys and this CTA's counts go to every CTA of the cluster
+  {
+    const uint32_t bin_hi = bin_lo + bin_w;
+    uint32_t m_in = 0u;
 #pragma unroll
-  for (int i = 0; i < EPT; ++i) {
-    m_gt |= static_cast<uint32_t>(key[i] > T) << i;
-    m_eq |= static_cast<uint32_t>(key[i] == T) << i;
-  }
-  // two counts of at most CHUNK <= 8192 each in one unsigned word: no carry between the halves
-  static_assert(CHUNK < 65536, "two 16-bit counts share one scan word");
-  const uint32_t packed = cta_exclusive_scan((static_cast<uint32_t>(__popc(m_gt)) << 16) | __popc(m_eq),
-                                             warp_sums, &scan_total);
-  if (threadIdx.x == 0) {
-    const uint32_t mine = smem_addr(&totals[rank][0]);
-    for (uint32_t p = 0; p < C; ++p) {
-      st_peer(peer_addr(mine, p), static_cast<int>(scan_total >> 16));
-      st_peer(peer_addr(mine + 4, p), static_cast<int>(scan_total & 0xffffu));
+    for (int i = 0; i < EPT; ++i) m_in |= static_cast<uint32_t>(key[i] - bin_lo <= bin_w) << i;
+    if (C > 1) {  // the keys above the bin matter to the CTAs behind this one
+      uint32_t gt = 0u;
+#pragma unroll
+      for (int i = 0; i < EPT; ++i) gt += key[i] > bin_hi;
+      gt = __reduce_add_sync(0xffffffffu, gt);
+      if (lane == 0 && gt) atomicAdd(&n_gt, gt);
+    }
+    if (listed) {
+      while (m_in) {  // a few keys per row: the register is picked by comparison
+        const int bit = __ffs(m_in) - 1;
+        m_in &= m_in - 1;
+        uint32_t k = key[0];
+#pragma unroll
+        for (int i = 1; i < EPT; ++i) k = i == bit ? key[i] : k;
+        const uint32_t at = rank * cap + atomicAdd(&n_list, 1u);
+        for (uint32_t p = 0; p < C; ++p) st_peer2(peer_addr(&list[at], p), k, static_cast<uint32_t>(c0 + base + bit));
+      }
+    } else {
+      const uint32_t in = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(__popc(m_in)));
+      if (lane == 0 && in) atomicAdd(&n_list, in);
     }
   }
-  cluster_barrier();  // every CTA has every CTA's totals
-  int gt_before = 0, eq_before = 0;
-  for (uint32_t p = 0; p < rank; ++p) {
-    gt_before += totals[p][0];
-    eq_before += totals[p][1];
+  __syncthreads();
+  if (tid < static_cast<int>(C)) st_peer2(peer_addr(&totals[rank], tid), n_gt, n_list);
+  if (C > 1) {
+    cluster_arrive();
+    cluster_wait();
+  } else {
+    __syncthreads();
   }
-  int eq_seen = eq_before + static_cast<int>(packed & 0xffffu);
-  int out_pos = gt_before + static_cast<int>(packed >> 16) + min(eq_seen, need_eq);
-  int32_t* orow = out_idx + static_cast<size_t>(row) * ksel;
-  uint32_t rest = m_gt | m_eq;
-  while (rest) {
-    const int bit = __ffs(rest) - 1;
-    rest &= rest - 1;
-    const bool is_eq = (m_eq >> bit) & 1u;
-    if (!is_eq || eq_seen++ < need_eq) orow[out_pos++] = c0 + base + bit;
+  if (discard_votes) {
+    // Every CTA of the row has its votes, and nobody reads them again: drop the whole 128-byte
+    // lines inside the row from L2, so that they are not written back to HBM while the gather
+    // kernel needs the bandwidth.  Lines that the row shares with its neighbours stay.
+    const uintptr_t b0 = (reinterpret_cast<uintptr_t>(vrow) + 127) & ~static_cast<uintptr_t>(127);
+    const uintptr_t b1 = reinterpret_cast<uintptr_t>(vrow + static_cast<size_t>(gsum) * n) & ~static_cast<uintptr_t>(127);
+    for (uintptr_t a = b0 + (static_cast<uintptr_t>(rank) * THREADS + tid) * 128; a < b1;
+         a += static_cast<uintptr_t>(C) * THREADS * 128)
+      discard_l2_line(reinterpret_cast<const void*>(a));
   }
-  // nobody leaves while a peer may still read its histograms
-  cluster_barrier();
+  if (listed) {
+    // entry e of the lists: rank it among all (keys only), find the threshold
+    uint32_t my_key = 0u, my_cta = C;
+    if (static_cast<uint32_t>(tid) < in_bin) {
+      uint32_t e = tid;
+      my_cta = 0u;
+      while (e >= totals[my_cta].y) e -= totals[my_cta++].y;
+      my_key = list[my_cta * cap + e].x;
+      uint32_t gt = 0u, eq = 0u;
+      for (uint32_t p = 0; p < C; ++p)
+        for (uint32_t i = 0; i < totals[p].y; ++i) {
+          const uint32_t k = list[p * cap + i].x;
+          gt += k > my_key;
+          eq += k == my_key;
+        }
+      if (gt < krem && krem <= gt + eq) {
+        thr_key = my_key;
+        thr_eq = krem - gt;
+        thr_all = eq;
+      }
+    }
+    __syncthreads();
+    if (my_cta < rank) {
+      if (my_key > thr_key) atomicAdd(&before_gt, 1u);
+      if (my_key == thr_key) atomicAdd(&before_eq, 1u);
+    }
+  } else if (tid == 0) {
+    thr_key = bin_lo;
+    thr_eq = krem;
+    thr_all = in_bin;
+  }
+  if (tid < static_cast<int>(rank)) {
+    atomicAdd(&before_gt, totals[tid].x);
+    if (!listed) atomicAdd(&before_eq, totals[tid].y);
+  }
+  __syncthreads();
+
+  // ---- 5. ordered compaction: keys above the threshold, plus the lowest positions equal to it
+  const uint32_t T = thr_key, need_eq = thr_eq, gt0 = before_gt, eq0 = before_eq;
+  const bool all_eq = need_eq == thr_all;  // every key equal to the threshold is kept (the usual case)
+  uint32_t m_keep = 0u, m_eq = 0u;         // EPT <= 32
+  const uint32_t T_keep = all_eq ? T : T + 1u;
+#pragma unroll
+  for (int i = 0; i < EPT; ++i) m_keep |= static_cast<uint32_t>(key[i] >= T_keep) << i;
+  if (!all_eq) {
+#pragma unroll
+    for (int i = 0; i < EPT; ++i) m_eq |= static_cast<uint32_t>(key[i] == T) << i;
+  }
+  static_assert(CHUNK < 65536, "two 16-bit counts share one scan word");
+  const uint32_t packed = block_scan<THREADS>((static_cast<uint32_t>(__popc(m_keep)) << 16) | __popc(m_eq),
+                                              warp_sums, &scan_total);
+  const uint32_t kept0 = min(eq0, need_eq);  // equal positions kept before this chunk
+  uint32_t eq_seen = eq0 + (packed & 0xffffu);
+  uint32_t at = packed >> 16;
+  if (!all_eq) {
+    at += min(eq_seen, need_eq) - kept0;
+    while (m_eq && eq_seen < need_eq) {  // the lowest ones
+      m_keep |= m_eq & (0u - m_eq);
+      m_eq &= m_eq - 1;
+      ++eq_seen;
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < EPT; ++i) {  // no loop over set bits: its length would be that of the fullest lane
+    if ((m_keep >> i) & 1u) stage[at] = static_cast<uint32_t>(c0 + base + i);
+    at += (m_keep >> i) & 1u;
+  }
+  const uint32_t mine = (scan_total >> 16) + (all_eq ? 0u : min(eq0 + (scan_total & 0xffffu), need_eq) - kept0);
+  __syncthreads();
+  int32_t* orow = out_idx + static_cast<size_t>(row) * ksel + gt0 + kept0;
+  for (uint32_t i = tid; i < mine; i += THREADS) orow[i] = static_cast<int32_t>(stage[i]);
 }
 
 struct ClusterShape {
-  int ept, clusters;  // keys per thread, CTAs per row
+  int threads, ept, ctas;  // threads per CTA, keys per thread, CTAs per row
 };
 
-// How a row of n positions is cut: as many CTAs as the portable cluster size allows, the
-// smallest per-thread run that covers the row; rows beyond 8 x 8192 take 16 CTAs.
-bool cluster_shape(int n, ClusterShape* s) {
-  if (n < 4096 || n > CL_MAX_CLUSTER * CL_THREADS * 32) return false;
-  if (n > 8 * CL_THREADS * 32) {
-    s->ept = 32;
-    s->clusters = 16;
-    return true;
-  }
-  const int per = (n + 7) / 8;
-  s->ept = per <= CL_THREADS * 8 ? 8 : (per <= CL_THREADS * 16 ? 16 : 32);
-  s->clusters = (n + CL_THREADS * s->ept - 1) / (CL_THREADS * s->ept);
-  return true;
-}
-
-template <int EPT, int R, int PT>
-cudaError_t launch_one(const float* vote, int rows, int n, int gsum, int r, int pool_type, int ksel,
-                       int32_t* out_idx, int clusters, cudaStream_t stream) {
-  auto kernel = pool_topk_cluster_kernel<EPT, R, PT>;
-  if (clusters > 8) {
-    static DeviceOnce once;
-    if (!once.done()) {
-      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e != cudaSuccess) return e;
-      once.set();
+// How rows of n positions are cut: the shape with the smallest estimated time.  Up to 4096
+// positions small CTAs have the shortest chain, and clusters of them while every CTA has an SM to
+// itself (79.6 against 84.2 us for the whole step of 32 rows of 16352).  Beyond, CTAs of 1024 threads
+// (one per SM) with 8, 16 or 32 keys a thread take about 8, 10.5 and 16.5 us, 2 to 4 us more when a
+// cluster shares a row, and come in rounds when they do not all find a place at once (clusters fit
+// less well the larger they are).
+ClusterShape cluster_shape(int rows, int n) {
+  if (n <= 2048) return {256, 8, 1};
+  const int small = (n + 4095) / 4096;
+  if (small <= 8 && rows * small <= 148) return {512, 8, small};
+  const int ept[3] = {8, 16, 32};
+  const double alone[3] = {8.0, 10.5, 16.5}, shared[3] = {10.2, 12.5, 20.0};
+  ClusterShape best = {1024, 32, (n + 32767) / 32768};
+  double best_us = 1e30;
+  for (int i = 0; i < 3; ++i) {
+    const int c = (n + 1024 * ept[i] - 1) / (1024 * ept[i]);
+    if (c > CL_MAX_CLUSTER) continue;
+    const int fit = c == 1 ? 148 : (c <= 2 ? 74 : (c <= 4 ? 132 / c : (c <= 8 ? 120 / c : 7)));  // clusters at once
+    const double us = static_cast<double>((rows + fit - 1) / fit) * (c == 1 ? alone[i] : shared[i] + 0.35 * c);
+    if (us < best_us) {
+      best_us = us;
+      best = {1024, ept[i], c};
     }
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(rows) * clusters);
-  cfg.blockDim = dim3(CL_THREADS);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = clusters;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, vote, n, gsum, r, pool_type, ksel, out_idx);
+  return best;
 }
 
-template <int EPT>
-cudaError_t launch_ept(const float* vote, int rows, int n, int gsum, int r, int pool_type, int ksel,
-                       int32_t* out_idx, int clusters, cudaStream_t stream) {
+template <int THREADS, int EPT, int R, int PT>
+cudaError_t launch_one(const float* vote, int rows, int n, int gsum, int r, int pool_type, float divisor, int ksel,
+                       int32_t* out_idx, int ctas, int discard, cudaStream_t stream) {
+  auto kernel = pool_topk_cluster_kernel<THREADS, EPT, R, PT>;
+  // CTAs of this kernel take their places while the scoring CTAs leave the SMs one by one.  Asking
+  // for so much shared memory that no SM takes more than its even share keeps them from crowding
+  // on the SMs that come free first.
+  constexpr int SMEM_MOST = 192 * 1024;
+  const int per_sm = (rows * ctas + sm_count() - 1) / sm_count();
+  int smem = slots_for(THREADS * EPT) * 4;
+  if (smem < SMEM_MOST / per_sm) smem = SMEM_MOST / per_sm;
+  static DeviceOnce once;
+  if (!once.done()) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MOST);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    once.set();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(rows) * ctas);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = ctas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  // four standard deviations of a sample rank to either side of the rank that ksel maps to
+  const double frac = static_cast<double>(ksel) / n;
+  const int delta = static_cast<int>(4.0 * sqrt(CL_SAMPLES * frac * (1.0 - frac))) + 2;
+  const int mid = static_cast<int>(frac * CL_SAMPLES);
+  const int2 want = make_int2(mid - delta, mid + delta);
+  return cudaLaunchKernelEx(&cfg, kernel, vote, n, gsum, r, pool_type, divisor, ksel, want, out_idx, ctas, discard);
+}
+
+template <int THREADS, int EPT>
+cudaError_t launch_shape(const float* vote, int rows, int n, int gsum, int r, int pool_type, float divisor, int ksel,
+                         int32_t* out_idx, int ctas, int discard, cudaStream_t stream) {
   const bool mx = pool_type == 0;
-#define SNAPKV_CL(RR, PP) launch_one<EPT, RR, PP>(vote, rows, n, gsum, r, pool_type, ksel, out_idx, clusters, stream)
+#define SNAPKV_CL(RR, PP) \
+  launch_one<THREADS, EPT, RR, PP>(vote, rows, n, gsum, r, pool_type, divisor, ksel, out_idx, ctas, discard, stream)
+  if (divisor != 0.f) return SNAPKV_CL(CL_RMAX, -1);
   // the paper's kernel sizes 5, 7 and 13 have instantiations of their own
   if (r == 2) return mx ? SNAPKV_CL(2, 0) : SNAPKV_CL(2, 1);
   if (r == 3) return mx ? SNAPKV_CL(3, 0) : SNAPKV_CL(3, 1);
@@ -352,7 +637,7 @@ cudaError_t launch_ept(const float* vote, int rows, int n, int gsum, int r, int 
 
 }  // namespace
 
-// Whether this device can hold a cluster of 16 of these CTAs (asked once per device).
+// Whether this device can hold a cluster of 16 CTAs of the largest shape (asked once per device).
 static bool cluster16_ok() {
   constexpr int MAX_DEV = 64;
   static std::atomic<int> state[MAX_DEV] = {};  // 0 unknown, 1 yes, 2 no
@@ -360,13 +645,16 @@ static bool cluster16_ok() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return false;
   int st = state[dev].load(std::memory_order_acquire);
   if (st == 0) {
-    auto kernel = pool_topk_cluster_kernel<32, CL_RMAX, -1>;
+    auto kernel = pool_topk_cluster_kernel<1024, 32, CL_RMAX, -1>;
+    constexpr int SMEM = slots_for(1024 * 32) * 4;
     int n_clusters = 0;
-    bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+              cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) == cudaSuccess;
     if (ok) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(16);
-      cfg.blockDim = dim3(CL_THREADS);
+      cfg.blockDim = dim3(1024);
+      cfg.dynamicSmemBytes = SMEM;
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeClusterDimension;
       attr[0].val.clusterDim.x = 16;
@@ -384,23 +672,22 @@ static bool cluster16_ok() {
 }
 
 bool select_cluster_applies(int rows, int n, int pool_kernel) {
-  ClusterShape s;
-  if ((pool_kernel >> 1) > CL_RMAX || !cluster_shape(n, &s)) return false;
-  if (s.clusters > 8 && !cluster16_ok()) return false;
-  // the grid is rows x CTAs per row in one dimension
-  return static_cast<long long>(rows) * s.clusters < 2147483647ll;
+  if ((pool_kernel >> 1) > CL_RMAX || n > CL_MAX_CLUSTER * 1024 * 32) return false;
+  const int ctas = cluster_shape(rows, n).ctas;
+  return static_cast<long long>(rows) * ctas < 2147483647ll && (ctas <= 8 || cluster16_ok());
 }
 
 cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int pool_kernel,
                                      int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream,
-                                     int* launches, int gsum) {
-  ClusterShape s;
-  if (!cluster_shape(n, &s)) return cudaErrorInvalidValue;
-  const int r = pool_kernel >> 1;
-  cudaError_t e;
-  if (s.ept == 8) e = launch_ept<8>(vote, rows, n, gsum, r, pool_type, ksel, out_idx, s.clusters, stream);
-  else if (s.ept == 16) e = launch_ept<16>(vote, rows, n, gsum, r, pool_type, ksel, out_idx, s.clusters, stream);
-  else e = launch_ept<32>(vote, rows, n, gsum, r, pool_type, ksel, out_idx, s.clusters, stream);
+                                     int* launches, int gsum, bool vote_is_scratch) {
+  const ClusterShape s = cluster_shape(rows, n);
+  const int r = pool_kernel >> 1, discard = vote_is_scratch ? 1 : 0;
+  // rows beyond 131072 positions rank average-pooled votes by the mean, shorter ones by the sum
+  const float divisor = n > 131072 && pool_type == 1 ? static_cast<float>(pool_kernel) : 0.f;
+  auto f = s.threads == 256 ? launch_shape<256, 8>
+           : s.threads == 512 ? launch_shape<512, 8>
+           : s.ept == 8 ? launch_shape<1024, 8> : (s.ept == 16 ? launch_shape<1024, 16> : launch_shape<1024, 32>);
+  const cudaError_t e = f(vote, rows, n, gsum, r, pool_type, divisor, ksel, out_idx, s.ctas, discard, stream);
   if (e != cudaSuccess) return e;
   *launches += 1;
   return cudaGetLastError();

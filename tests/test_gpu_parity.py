@@ -140,6 +140,33 @@ def test_pool_topk_matches_oracle(rows, n, kernel, ptype, ksel):
 
 
 @pytest.mark.parametrize("rows,n,kernel,ptype,ksel", [
+    (3, 1, 7, "max", 1), (2, 255, 5, "avg", 254), (2, 2048, 15, "avg", 2048),  # 256 threads per row
+    (2, 2049, 3, "max", 1), (3, 4096, 13, "avg", 4095),                        # 512 threads per row
+    (3, 4097, 5, "avg", 300), (2, 32768, 13, "max", 320),                      # clusters of 2 and 8 of them
+    (80, 4097, 7, "max", 64), (149, 8193, 5, "avg", 999),                      # 1024 threads, 8 and 16 keys each
+    (75, 32769, 13, "max", 5000), (3, 262145, 7, "max", 262144),               # clusters of 2 and more CTAs
+    (1, 131073, 5, "avg", 2000), (1, 524288, 7, "avg", 3),                     # ranked by the mean; the longest row
+    (1, 524289, 7, "max", 100),                                                # one more: many-launch path
+])
+def test_pool_topk_at_the_edges_of_its_shapes(rows, n, kernel, ptype, ksel):
+    # votes of few distinct values make plateaus wider than a candidate list, scaled ones spread
+    # over 60 octaves, and one row is constant: the guessed window must not decide anything
+    g = torch.Generator().manual_seed(n + ksel)
+    vote = torch.rand(rows, n, generator=g)
+    vote[0] = torch.floor(vote[0] * 3) / 4
+    if rows > 1:
+        vote[1] = torch.exp2(60 * (vote[1] - 0.5))
+    if rows > 2:
+        vote[2] = 0.25
+    idx = sk.snapkv_pool_topk(vote.cuda(), kernel, PT[ptype], ksel).cpu().numpy()
+    for r in range(min(rows, 4)):
+        pooled = orc.pool1d(vote[r].numpy().astype(np.float64), kernel, PT[ptype])
+        same = parity.check_indices(idx[r], pooled, ksel, orc.topk_positions(pooled, ksel))
+        if ptype == "max":
+            assert same
+
+
+@pytest.mark.parametrize("rows,n,kernel,ptype,ksel", [
     (2, 40960, 7, "max", 32767),    # one below / at the point where a 16-bit count reaches bit 15
     (2, 40960, 7, "max", 32768),
     (2, 40000, 5, "avg", 39000),
