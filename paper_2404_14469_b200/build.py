@@ -19,7 +19,7 @@ LIB = os.path.join(HERE, "libsnapkv.so")
 NATIVE = os.path.join(HERE, "_native.so")
 SOURCES = ["snapkv_api.cu", "snapkv_score.cu", "snapkv_select.cu", "snapkv_select_cluster.cu", "snapkv_gather.cu",
            "snapkv_metrics.cu", "snapkv_decode.cu"]
-HEADERS = ["sm100_ptx.cuh", "snapkv_internal.h", "launch.cuh", os.path.join("..", "..", "include", "snapkv.h")]
+HEADERS = ["sm100_ptx.cuh", "score_kernel.cuh", "snapkv_internal.h", "launch.cuh", os.path.join("..", "..", "include", "snapkv.h")]
 NATIVE_SOURCE = "native_binding.cpp"
 NATIVE_HEADERS = [os.path.join("..", "..", "include", "snapkv.h")]
 

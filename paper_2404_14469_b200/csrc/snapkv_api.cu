@@ -14,24 +14,28 @@ namespace snapkv {
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Clears the status block and the unit counters behind it (a multiple of 256 bytes).  A
-// kernel rather than a memset so that the scoring kernel behind it can be made resident early.
-__global__ void clear_kernel(uint4* p, int n16) {
+// Clears the status block and the unit counters behind it (n16 vectors) and marks the partial
+// slots that follow as not written (up to n16_all).  A kernel rather than memsets so that the
+// scoring kernel behind it can be made resident early.
+__global__ void clear_kernel(uint4* p, int n16, int n16_all) {
   pdl_launch_dependents();
   pdl_wait();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += gridDim.x * blockDim.x)
-    p[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n16_all; i += gridDim.x * blockDim.x) {
+    const uint32_t x = i < n16 ? 0u : NO_PARTIAL;
+    p[i] = make_uint4(x, x, x, x);
+  }
 }
 
 // `keep_status`: leave the status block alone (a later part of one logical call must not wipe
-// an error an earlier part recorded) and clear the counters only.
+// an error an earlier part recorded).
 static cudaError_t launch_clear(uint8_t* ws, const WorkspaceLayout& w, cudaStream_t s,
                                 bool keep_status = false) {
   const size_t from = keep_status ? w.off_counters : w.off_status;
   const int n16 = static_cast<int>((w.off_partials - from) / 16);
-  const int blocks = n16 > 256 * 64 ? 64 : (n16 + 255) / 256;
+  const int n16_all = static_cast<int>((w.off_lse - from) / 16);
+  const int blocks = n16_all > 256 * 148 ? 148 : (n16_all + 255) / 256;
   return launch_pdl(clear_kernel, dim3(blocks), dim3(256), 0, s,
-                    reinterpret_cast<uint4*>(ws + from), n16);
+                    reinterpret_cast<uint4*>(ws + from), n16, n16_all);
 }
 
 // Zeroes the status block alone.  Entry points that run several single-sequence steps on one

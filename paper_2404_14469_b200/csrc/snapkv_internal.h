@@ -15,6 +15,9 @@ constexpr int STATUS_BYTES = 256;   // status block at the start of every worksp
 constexpr int SM_COUNT_HINT = 148;  // B200
 constexpr int MAX_GRID = 192;       // the scoring kernel runs one CTA per SM, at most this many
 
+constexpr uint32_t NO_PARTIAL = 0xffffffffu;  // a partial-statistics slot that has not been written
+constexpr int RAGGED_MAX = 32;      // sequences of a ragged batch that share a launch
+
 // Codes stored in the workspace status block's second word when a wait gives up.
 enum WaitCode {
   WAIT_NONE = 0,
@@ -29,7 +32,6 @@ enum WaitCode {
   WAIT_PART_FULL = 9,
   WAIT_LSE_FULL = 10,
   WAIT_LSE_EMPTY = 11,
-  WAIT_MERGE_COPY = 12,
 };
 
 // How the scoring passes split the work.  A "unit" is one (batch, KV head, head
@@ -105,6 +107,17 @@ struct ShardMode {
   float* lse_out;
 };
 
+// A ragged batch: the sequences (at most RAGGED_MAX) that are compressed in one set of launches.
+struct RaggedBatch {
+  int count;
+  int batch[RAGGED_MAX];        // index in the caller's batch
+  int L[RAGGED_MAX];            // prompt length (more than the budget)
+  long long k_off[RAGGED_MAX];  // element offset of the sequence's first key (0 with a block table)
+  ScorePlan plan[RAGGED_MAX];   // as for a call of its own
+  long long part0[RAGGED_MAX], vote0[RAGGED_MAX];  // first partial slot, first vote
+  size_t off_counters, off_partials, off_lse, off_vote, total;  // workspace, status block in front
+};
+
 struct WorkspaceLayout {
   size_t off_status, off_counters, off_partials, off_lse, off_vote, off_pooled, total;
 };
@@ -135,8 +148,8 @@ WorkspaceLayout make_layout(const ScorePlan& p, int B, int Hq, int n, bool need_
 bool select_needs_scratch(int n);
 size_t select_scratch_bytes(int rows, int n);  // 0 when the rows fit one CTA
 
-// Enqueue both scoring passes.  `vote` is fp32 [B*Hq, n].  `counters` must be zero when the
-// kernel starts (the callers clear it together with the status block).  With `lse_obs`
+// Enqueue both scoring passes.  `vote` is fp32 [B*Hq, n].  `counters` must be zero and the
+// partial slots NO_PARTIAL when the kernel starts (the callers' clear kernel).  With `lse_obs`
 // (device fp32 [B*Hq, W], natural-log sum-exp of every window row) the statistics pass is
 // skipped: a small kernel converts the rows first, then only the vote pass runs; that kernel
 // also zeroes the status block unless `keep_status` is set.  `never_ready` (self-test of the
@@ -166,6 +179,24 @@ bool select_cluster_applies(int rows, int n, int pool_kernel);
 cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int pool_kernel,
                                      int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream,
                                      int* launches, int gsum, bool vote_is_scratch);
+
+// The same two steps for the sequences of a ragged batch.
+cudaError_t launch_ragged_scores(const RaggedBatch& rb, const void* q_obs, const void* k, const KVStrides& ks,
+                                 int B, int Hq, int Hkv, int d, int W, uint8_t* ws, cudaStream_t stream,
+                                 int* launches, const float* lse_obs, bool keep_status, const PagedKV* paged);
+bool ragged_select_applies(int n_max, int pool_kernel, int pool_type);
+cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int Hq, int W, int pool_kernel,
+                                 int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream, int* launches);
+
+// Gather + append for `count` (up to RAGGED_MAX) consecutive sequences of a batch, from sequence b0
+// on; lens, k_off and v_off begin with that sequence.  A sequence with budget >= its length is
+// copied through and its positions 0 .. n - 1 are written; with `fill` rows behind a sequence's end
+// become zero and positions -1, else they are left untouched.  k_off / v_off: element offsets of the
+// sequences' first rows (ignored with a block table).
+cudaError_t launch_ragged_gather(const void* k, const void* v, const KVStrides& ks, const KVStrides& vs,
+                                 const int* lens, const long long* k_off, const long long* v_off, int b0, int count,
+                                 int Hq, int Hkv, int d, int W, int budget, bool fill, int32_t* idx, void* out_k,
+                                 void* out_v, cudaStream_t stream, int* launches, const PagedKV* paged);
 
 // Gather + append.  idx == nullptr copies rows 0..ksel-1 (identity path).
 cudaError_t launch_gather(const void* k, const void* v, const KVStrides& ks, const KVStrides& vs,
