@@ -241,7 +241,8 @@ snapkv_status_t snapkv_compress_grouped(const void* q_obs, const void* k, const 
 /*
  * The whole step (Listing 1) on a batch whose prompts differ in length.  Listing 1 has one
  * q_len for the batch; the sequences are independent of one another (Sec. 4.1), so each is
- * compressed as a single-sequence step of its own length, one after the other on `stream`.
+ * compressed as a single-sequence step of its own length.  Up to 32 of them share each launch when
+ * the workspace has room for them all (the more it holds, the fewer launches).
  *   seq_lens       HOST int32 [B]: L_b, W <= L_b <= Lmax.  Sequence b's window is its last W
  *                  positions, its prefix the L_b - W before them.
  *   k, v           as in snapkv_compress_strided (k_strides / v_strides NULL: dense
@@ -354,7 +355,7 @@ snapkv_status_t snapkv_device_status(const void* workspace, void* stream, int* d
  *   page_size       positions per page: a multiple of 128, so that a tile of 128 keys lies in
  *                   one page (SNAPKV_ERR_INVALID_ARG otherwise); pages_per_seq * page_size >= L.
  *   seq_lens        host int32[B] or NULL.  NULL: every sequence has L positions.  Otherwise
- *                   sequence b has seq_lens[b] in [W, L] positions and the call runs one
+ *                   sequence b has seq_lens[b] in [W, L] positions and the call does one
  *                   single-sequence step per prompt (as snapkv_compress_varlen does), a
  *                   sequence with budget >= its length being copied through.
  *   lse_obs         optional, as in snapkv_compress_lse.

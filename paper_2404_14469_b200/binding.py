@@ -38,6 +38,9 @@ SYMBOLS = [
     "snapkv_shard_lse", "snapkv_lse_merge", "snapkv_shard_votes", "snapkv_gather_range",
 ]
 
+# entry points for the extension alone (csrc/snapkv_binding.h)
+BINDING_SYMBOLS = ["snapkv_binding_ragged_workspace", "snapkv_binding_varlen", "snapkv_binding_paged"]
+
 _lib = None
 _native = None
 
@@ -133,7 +136,8 @@ def _load_native():
     spec = importlib.util.spec_from_file_location("paper_2404_14469_b200._native", NATIVE_PATH)
     mod = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(mod)
-    mod.bind({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in SYMBOLS}, SnapKVError)
+    mod.bind({name: ctypes.cast(getattr(L, name), ctypes.c_void_p).value for name in SYMBOLS + BINDING_SYMBOLS},
+             SnapKVError)
     _native = mod
     return mod
 

@@ -18,10 +18,10 @@ OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libsnapkv.so")
 NATIVE = os.path.join(HERE, "_native.so")
 SOURCES = ["snapkv_api.cu", "snapkv_score.cu", "snapkv_select.cu", "snapkv_select_cluster.cu", "snapkv_gather.cu",
-           "snapkv_metrics.cu", "snapkv_decode.cu"]
-HEADERS = ["sm100_ptx.cuh", "score_kernel.cuh", "snapkv_internal.h", "launch.cuh", os.path.join("..", "..", "include", "snapkv.h")]
+           "snapkv_metrics.cu", "snapkv_decode.cu", "snapkv_score_ragged.cu"]
+HEADERS = ["sm100_ptx.cuh", "score_kernel.cuh", "snapkv_internal.h", "launch.cuh", "snapkv_binding.h", os.path.join("..", "..", "include", "snapkv.h")]
 NATIVE_SOURCE = "native_binding.cpp"
-NATIVE_HEADERS = [os.path.join("..", "..", "include", "snapkv.h")]
+NATIVE_HEADERS = ["snapkv_binding.h", os.path.join("..", "..", "include", "snapkv.h")]
 
 
 def _nvcc() -> str:

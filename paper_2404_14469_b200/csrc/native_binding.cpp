@@ -17,7 +17,7 @@
 #include <string>
 #include <vector>
 
-#include "../../include/snapkv.h"
+#include "snapkv_binding.h"
 
 namespace {
 
@@ -34,8 +34,9 @@ struct Library {
   decltype(&snapkv_compress_lse) compress_lse;
   decltype(&snapkv_compress_strided) compress_strided;
   decltype(&snapkv_compress_grouped) compress_grouped;
-  decltype(&snapkv_compress_varlen) compress_varlen;
-  decltype(&snapkv_compress_paged) compress_paged;
+  decltype(&snapkv_binding_ragged_workspace) binding_ragged_workspace;
+  decltype(&snapkv_binding_varlen) binding_varlen;
+  decltype(&snapkv_binding_paged) binding_paged;
   decltype(&snapkv_decode_workspace_size) decode_workspace_size;
   decltype(&snapkv_decode_attention) decode_attention;
 } g_lib;
@@ -227,26 +228,32 @@ PyObject* py_compress(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   });
 }
 
-// What a batch of `lens` needs when its sequences go one after the other.
-size_t ragged_need(const std::vector<int32_t>& lens, int Hq, int Hkv, int d, int W, int pk, int pt, int budget) {
-  size_t need = 256;
-  for (int32_t x : lens)
-    if (x > budget) {
-      const size_t one = g_lib.workspace_size(1, Hq, Hkv, x, d, W, pk, pt, budget);
-      if (one > need) need = one;
-    }
-  return need;
+// The caller's workspace if it meets the requirement (the largest single sequence), else a new one
+// with which the whole batch goes through in one set of launches.
+Out ragged_workspace(PyObject* given, const std::vector<int32_t>& lens, int Hq, int Hkv, int d, int W, int pk, int pt,
+                     int budget, const at::Device& dev) {
+  if (given != Py_None) {
+    size_t need = 256;
+    for (int32_t x : lens)
+      if (x > budget) {
+        const size_t one = g_lib.workspace_size(1, Hq, Hkv, x, d, W, pk, pt, budget);
+        if (one > need) need = one;
+      }
+    if (static_cast<size_t>(tensor(given, "workspace").numel()) >= need) return workspace_for(given, need, dev);
+  }
+  const int B = static_cast<int>(lens.size());
+  return workspace_for(Py_None, g_lib.binding_ragged_workspace(lens.data(), B, Hq, Hkv, d, W, pk, pt, budget), dev);
 }
 
 struct RaggedOut {
   Out ok, ov, oi;
 };
-// rows behind a sequence's own are zero, positions -1
+// the library writes all of it: rows behind a sequence's own become zero, positions -1
 RaggedOut ragged_outputs(int64_t B, int64_t Hq, int64_t budget, int64_t W, int64_t d, const at::Device& dev) {
   RaggedOut r;
-  r.ok.t = empty({B, Hq, budget, d}, at::kBFloat16, dev).zero_();
-  r.ov.t = empty({B, Hq, budget, d}, at::kBFloat16, dev).zero_();
-  r.oi.t = empty({B, Hq, budget - W}, at::kInt, dev).fill_(-1);
+  r.ok.t = empty({B, Hq, budget, d}, at::kBFloat16, dev);
+  r.ov.t = empty({B, Hq, budget, d}, at::kBFloat16, dev);
+  r.oi.t = empty({B, Hq, budget - W}, at::kInt, dev);
   return r;
 }
 
@@ -289,17 +296,17 @@ PyObject* py_varlen(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     const int iHq = static_cast<int>(Hq), iHkv = static_cast<int>(Hkv), id = static_cast<int>(d),
               iW = static_cast<int>(W);
     RaggedOut out = ragged_outputs(B, Hq, budget, W, d, dev);
-    Out ws = workspace_for(a[9], ragged_need(lens, iHq, iHkv, id, iW, pk, pt, budget), dev);
+    Out ws = ragged_workspace(a[9], lens, iHq, iHkv, id, iW, pk, pt, budget, dev);
     const float* lse = lse_arg(a[8], B, Hq, W);
     const int64_t* offp = off.empty() ? nullptr : off.data();
     int code;
     {
       void* s = stream();
       NoGil unlocked;
-      code = g_lib.compress_varlen(q.data_ptr(), k.data_ptr(), v.data_ptr(), ks, vs, offp, offp, lens.data(), lse,
-                                   static_cast<int>(B), iHq, iHkv, static_cast<int>(Lmax), id, iW, pk, pt, budget,
-                                   out.ok.data(), out.ov.data(), static_cast<int32_t*>(out.oi.data()), ws.data(),
-                                   static_cast<size_t>(ws.t.numel()), s);
+      code = g_lib.binding_varlen(q.data_ptr(), k.data_ptr(), v.data_ptr(), ks, vs, offp, offp, lens.data(), lse,
+                                  static_cast<int>(B), iHq, iHkv, static_cast<int>(Lmax), id, iW, pk, pt, budget,
+                                  out.ok.data(), out.ov.data(), static_cast<int32_t*>(out.oi.data()), ws.data(),
+                                  static_cast<size_t>(ws.t.numel()), s, 1);
     }
     check(code, "snapkv_compress_varlen");
     return tuple4(out.ok, out.ov, out.oi, ws);
@@ -327,32 +334,27 @@ PyObject* py_paged(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     const bool ragged = a[8] != Py_None;
     const int budget = ragged || want < L ? want : L;
     std::vector<int32_t> lens;
-    RaggedOut out;
-    size_t need;
+    RaggedOut out = ragged_outputs(B, Hq, budget, W, d, dev);
+    Out ws;
     if (ragged) {
       lens = whole_numbers<int32_t>(a[8], "seq_lens");
       if (static_cast<int64_t>(lens.size()) != B) throw Fail{"one length per sequence is needed"};
-      out = ragged_outputs(B, Hq, budget, W, d, dev);
-      need = ragged_need(lens, iHq, iHkv, id, iW, pk, pt, budget);
+      ws = ragged_workspace(a[10], lens, iHq, iHkv, id, iW, pk, pt, budget, dev);
     } else {
-      out.ok.t = empty({B, Hq, budget, d}, at::kBFloat16, dev);
-      out.ov.t = empty({B, Hq, budget, d}, at::kBFloat16, dev);
-      out.oi.t = empty({B, Hq, budget - W}, at::kInt, dev);
-      need = g_lib.workspace_size(iB, iHq, iHkv, L, id, iW, pk, pt, budget);
+      ws = workspace_for(a[10], g_lib.workspace_size(iB, iHq, iHkv, L, id, iW, pk, pt, budget), dev);
     }
-    Out ws = workspace_for(a[10], need, dev);
     const float* lse = lse_arg(a[9], B, Hq, W);
     int code;
     {
       void* s = stream();
       const int64_t ks[3] = {k.stride(0), k.stride(1), k.stride(2)}, vs[3] = {v.stride(0), v.stride(1), v.stride(2)};
       NoGil unlocked;
-      code = g_lib.compress_paged(q.data_ptr(), k.data_ptr(), v.data_ptr(), ks, vs,
-                                  static_cast<const int32_t*>(table.data_ptr()), static_cast<int>(table.size(1)),
-                                  static_cast<int>(k.size(2)), static_cast<int>(k.size(0)),
-                                  ragged ? lens.data() : nullptr, lse, iB, iHq, iHkv, L, id, iW, pk, pt, budget,
-                                  out.ok.data(), out.ov.data(), static_cast<int32_t*>(out.oi.data()), ws.data(),
-                                  static_cast<size_t>(ws.t.numel()), s);
+      code = g_lib.binding_paged(q.data_ptr(), k.data_ptr(), v.data_ptr(), ks, vs,
+                                 static_cast<const int32_t*>(table.data_ptr()), static_cast<int>(table.size(1)),
+                                 static_cast<int>(k.size(2)), static_cast<int>(k.size(0)),
+                                 ragged ? lens.data() : nullptr, lse, iB, iHq, iHkv, L, id, iW, pk, pt, budget,
+                                 out.ok.data(), out.ov.data(), static_cast<int32_t*>(out.oi.data()), ws.data(),
+                                 static_cast<size_t>(ws.t.numel()), s, 1);
     }
     check(code, "snapkv_compress_paged");
     return tuple4(out.ok, out.ov, out.oi, ws);
@@ -418,8 +420,9 @@ PyObject* py_bind(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     SNAPKV_BIND(compress_lse);
     SNAPKV_BIND(compress_strided);
     SNAPKV_BIND(compress_grouped);
-    SNAPKV_BIND(compress_varlen);
-    SNAPKV_BIND(compress_paged);
+    SNAPKV_BIND(binding_ragged_workspace);
+    SNAPKV_BIND(binding_varlen);
+    SNAPKV_BIND(binding_paged);
     SNAPKV_BIND(decode_workspace_size);
     SNAPKV_BIND(decode_attention);
 #undef SNAPKV_BIND

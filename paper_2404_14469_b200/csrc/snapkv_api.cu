@@ -8,6 +8,7 @@
 
 #include "../../include/snapkv.h"
 #include "launch.cuh"
+#include "snapkv_binding.h"
 #include "snapkv_internal.h"
 
 namespace snapkv {
@@ -390,18 +391,192 @@ snapkv_status_t snapkv_compress_grouped(const void* q_obs, const void* k, const 
                        k_strides ? &ks : nullptr, v_strides ? &vs : nullptr, true);
 }
 
-snapkv_status_t snapkv_compress_varlen(const void* q_obs, const void* k, const void* v,
-                                       const int64_t* k_strides, const int64_t* v_strides,
-                                       const int64_t* k_seq_offsets, const int64_t* v_seq_offsets,
-                                       const int32_t* seq_lens, const float* lse_obs, int B,
-                                       int Hq, int Hkv, int Lmax, int d, int W, int pool_kernel,
-                                       int pool_type, int budget, void* out_k, void* out_v,
-                                       int32_t* out_idx, void* workspace, size_t workspace_bytes,
-                                       void* stream) {
+// ---- prompts of different lengths
+// The sequences are independent (Sec. 4.1).  Those longer than the budget are scored and selected
+// in groups of up to RAGGED_MAX, each group in one set of launches; a group is as large as the
+// workspace allows, one sequence always fits.  One gather launch then serves up to RAGGED_MAX
+// consecutive sequences, those that are copied through included.
+static void ragged_layout(RaggedBatch* rb, int Hq) {
+  size_t off = STATUS_BYTES;
+  const size_t units = static_cast<size_t>(rb->plan[0].units);
+  rb->off_counters = off;
+  off = align_up(off + sizeof(int) * units * rb->count, 256);
+  rb->off_partials = off;
+  long long slots = 0, votes = 0;
+  for (int i = 0; i < rb->count; ++i) {
+    rb->part0[i] = slots;
+    slots += static_cast<long long>(units) * rb->plan[i].maxseg;
+    rb->vote0[i] = votes;
+    votes += static_cast<long long>(Hq) * rb->plan[i].n_vote;
+  }
+  off = align_up(off + sizeof(float) * static_cast<size_t>(slots) * MAX_COLS, 256);
+  rb->off_lse = off;
+  off = align_up(off + sizeof(float) * units * rb->count * MAX_COLS, 256);
+  rb->off_vote = off;
+  rb->total = align_up(off + sizeof(float) * static_cast<size_t>(votes), 256);
+}
+
+// The group of sequences longer than the budget that starts at or behind sequence `b`; returns the
+// sequence behind it.
+static int ragged_group(const int32_t* lens, int B, int b, int Hq, int Hkv, int d, int W, int budget,
+                        size_t workspace_bytes, RaggedBatch* rb) {
+  rb->count = 0;
+  rb->total = 0;
+  for (; b < B; ++b) {
+    if (budget >= lens[b]) continue;
+    if (rb->count == RAGGED_MAX) break;
+    const int i = rb->count;
+    if (!make_score_plan(1, Hq, Hkv, lens[b], d, W, &rb->plan[i])) break;
+    rb->L[i] = lens[b];
+    rb->batch[i] = b;
+    rb->count = i + 1;
+    ragged_layout(rb, Hq);
+    if (i > 0 && rb->total > workspace_bytes) {
+      rb->count = i;
+      ragged_layout(rb, Hq);
+      break;
+    }
+  }
+  return b;
+}
+
+struct RaggedCall {
+  const void *q_obs, *k, *v;
+  KVStrides ks, vs;
+  const int64_t *k_off, *v_off;  // per sequence, or nullptr: b * stride
+  const int32_t* lens;
+  const float* lse_obs;
+  int B, Hq, Hkv, d, W, pool_kernel, pool_type, budget;
+  void *out_k, *out_v;
+  int32_t* out_idx;
+  void* workspace;
+  size_t workspace_bytes;
+  cudaStream_t stream;
+  const PagedKV* paged;
+  bool fill;
+};
+
+// Lengths and workspace, before anything is launched.
+static snapkv_status_t ragged_check(const RaggedCall& c, int Lmax) {
+  for (int b = 0; b < c.B; ++b) {
+    if (c.lens[b] < c.W || c.lens[b] > Lmax) return SNAPKV_ERR_INVALID_ARG;
+    if (c.k_off && (c.k_off[b] < 0 || (c.k_off[b] & 7))) return SNAPKV_ERR_INVALID_ARG;
+    if (c.v_off && (c.v_off[b] < 0 || (c.v_off[b] & 7))) return SNAPKV_ERR_INVALID_ARG;
+    if (!c.out_idx && c.lens[b] > c.W) return SNAPKV_ERR_INVALID_ARG;
+  }
+  for (int b = 0; b < c.B; ++b) {
+    if (c.budget >= c.lens[b]) continue;  // copied through: no scratch
+    const size_t need =
+        snapkv_workspace_size(1, c.Hq, c.Hkv, c.lens[b], c.d, c.W, c.pool_kernel, c.pool_type, c.budget);
+    if (need == 0) return SNAPKV_ERR_INVALID_ARG;
+    if (!workspace_ok(c.workspace, c.workspace_bytes, need)) return SNAPKV_ERR_WORKSPACE;
+  }
+  return SNAPKV_OK;
+}
+
+static snapkv_status_t ragged_impl(const RaggedCall& c) {
+  const size_t head_rows = static_cast<size_t>(c.Hq) * c.budget * c.d * 2;  // bytes of one sequence's out_k
+  const bool have_ws = workspace_ok(c.workspace, c.workspace_bytes, STATUS_BYTES);
+  int longest = 0;
+  for (int b = 0; b < c.B; ++b)
+    if (c.lens[b] > longest) longest = c.lens[b];
+  int launches = 0;
+  if (c.out_idx && c.Hq <= 65535 &&
+      ragged_select_applies(longest - c.W > 0 ? longest - c.W : 1, c.pool_kernel, c.pool_type)) {
+    uint8_t* ws = static_cast<uint8_t*>(c.workspace);
+    bool first = true;  // the first group's launches clear the status block, later ones leave it
+    for (int b = 0; b < c.B;) {
+      RaggedBatch rb;
+      b = ragged_group(c.lens, c.B, b, c.Hq, c.Hkv, c.d, c.W, c.budget, c.workspace_bytes, &rb);
+      if (rb.count == 0) {
+        if (b < c.B) return SNAPKV_ERR_UNSUPPORTED;  // no plan for sequence b
+        break;
+      }
+      for (int i = 0; i < rb.count; ++i)
+        rb.k_off[i] = c.paged ? 0 : (c.k_off ? c.k_off[rb.batch[i]] : rb.batch[i] * c.ks.b);
+      if (launch_ragged_scores(rb, c.q_obs, c.k, c.ks, c.B, c.Hq, c.Hkv, c.d, c.W, ws, c.stream, &launches,
+                               c.lse_obs, !first, c.paged) != cudaSuccess)
+        return SNAPKV_ERR_CUDA;
+      if (launch_ragged_select(rb, reinterpret_cast<const float*>(ws + rb.off_vote), c.Hq, c.W, c.pool_kernel,
+                               c.pool_type, c.budget - c.W, c.out_idx, c.stream, &launches) != cudaSuccess)
+        return SNAPKV_ERR_CUDA;
+      first = false;
+    }
+    if (first && have_ws && clear_status(c.workspace, c.stream) != cudaSuccess) return SNAPKV_ERR_CUDA;
+    const int most = 65535 / c.Hq < RAGGED_MAX ? 65535 / c.Hq : RAGGED_MAX;
+    for (int b0 = 0; b0 < c.B; b0 += most) {
+      const int count = c.B - b0 < most ? c.B - b0 : most;
+      long long ko[RAGGED_MAX], vo[RAGGED_MAX];
+      for (int i = 0; i < count; ++i) {
+        ko[i] = c.k_off ? c.k_off[b0 + i] : (b0 + i) * c.ks.b;
+        vo[i] = c.v_off ? c.v_off[b0 + i] : (b0 + i) * c.vs.b;
+      }
+      if (launch_ragged_gather(c.k, c.v, c.ks, c.vs, c.lens + b0, ko, vo, b0, count, c.Hq, c.Hkv, c.d, c.W, c.budget,
+                               c.fill, c.out_idx, c.out_k, c.out_v, c.stream, &launches, c.paged) != cudaSuccess)
+        return SNAPKV_ERR_CUDA;
+    }
+    g_last_launches = launches;
+    return SNAPKV_OK;
+  }
+  // pooling radii or lengths that the shared select launch does not take: one single-sequence step
+  // each, one after the other on the same stream and workspace; the status block keeps the first
+  // error of any of them
+  if (have_ws && clear_status(c.workspace, c.stream) != cudaSuccess) return SNAPKV_ERR_CUDA;
+  if (c.fill && (cudaMemsetAsync(c.out_k, 0, head_rows * c.B, c.stream) != cudaSuccess ||
+                 cudaMemsetAsync(c.out_v, 0, head_rows * c.B, c.stream) != cudaSuccess ||
+                 cudaMemsetAsync(c.out_idx, 0xff, sizeof(int32_t) * c.B * c.Hq * (c.budget - c.W), c.stream) != cudaSuccess))
+    return SNAPKV_ERR_CUDA;
+  for (int b = 0; b < c.B; ++b) {
+    const long long ko = c.paged ? 0 : (c.k_off ? c.k_off[b] : b * c.ks.b);
+    const long long vo = c.paged ? 0 : (c.v_off ? c.v_off[b] : b * c.vs.b);
+    PagedKV one = {};
+    if (c.paged) {
+      one = *c.paged;
+      one.table += static_cast<size_t>(b) * one.pages_per_seq;
+    }
+    const snapkv_status_t st = compress_impl(
+        static_cast<const uint8_t*>(c.q_obs) + static_cast<size_t>(b) * c.Hq * c.W * c.d * 2,
+        static_cast<const uint8_t*>(c.k) + ko * 2, static_cast<const uint8_t*>(c.v) + vo * 2, 1, c.Hq, c.Hkv,
+        c.lens[b], c.d, c.W, c.pool_kernel, c.pool_type, c.budget, static_cast<uint8_t*>(c.out_k) + b * head_rows,
+        static_cast<uint8_t*>(c.out_v) + b * head_rows,
+        c.out_idx ? c.out_idx + static_cast<size_t>(b) * c.Hq * (c.budget - c.W) : nullptr, c.workspace,
+        c.workspace_bytes, c.stream, /*keep_status=*/true,
+        c.lse_obs ? c.lse_obs + static_cast<size_t>(b) * c.Hq * c.W : nullptr, &c.ks, &c.vs, false,
+        c.paged ? &one : nullptr);
+    if (st != SNAPKV_OK) return st;
+    launches += g_last_launches;
+  }
+  g_last_launches = launches;
+  return SNAPKV_OK;
+}
+
+size_t snapkv_binding_ragged_workspace(const int32_t* lens, int B, int Hq, int Hkv, int d, int W, int pool_kernel,
+                                       int pool_type, int budget) {
+  size_t need = 0;
+  for (int b = 0; b < B; ++b) {
+    if (lens[b] <= budget) continue;
+    const size_t one = snapkv_workspace_size(1, Hq, Hkv, lens[b], d, W, pool_kernel, pool_type, budget);
+    if (one == 0) return 0;
+    if (one > need) need = one;
+  }
+  for (int b = 0; b < B;) {
+    RaggedBatch rb;
+    b = ragged_group(lens, B, b, Hq, Hkv, d, W, budget, ~static_cast<size_t>(0), &rb);
+    if (rb.count == 0) break;
+    if (rb.total > need) need = rb.total;
+  }
+  return need;
+}
+
+snapkv_status_t snapkv_binding_varlen(const void* q_obs, const void* k, const void* v, const int64_t* k_strides,
+                                      const int64_t* v_strides, const int64_t* k_seq_offsets,
+                                      const int64_t* v_seq_offsets, const int32_t* seq_lens, const float* lse_obs,
+                                      int B, int Hq, int Hkv, int Lmax, int d, int W, int pool_kernel, int pool_type,
+                                      int budget, void* out_k, void* out_v, int32_t* out_idx, void* workspace,
+                                      size_t workspace_bytes, void* stream, int fill) {
   snapkv_status_t st = check_common(B, Hq, Hkv, Lmax, d, W);
   if (st != SNAPKV_OK) return st;
-  if (!seq_lens || budget <= W || !q_obs || !k || !v || !out_k || !out_v)
-    return SNAPKV_ERR_INVALID_ARG;
+  if (!seq_lens || budget <= W || !q_obs || !k || !v || !out_k || !out_v) return SNAPKV_ERR_INVALID_ARG;
   KVStrides ks = dense_strides(Hkv, Lmax, d), vs = ks;
   if ((k_strides && !strides_ok(k_strides, d, &ks)) || (v_strides && !strides_ok(v_strides, d, &vs)))
     return SNAPKV_ERR_INVALID_ARG;
@@ -411,54 +586,33 @@ snapkv_status_t snapkv_compress_varlen(const void* q_obs, const void* k, const v
   if (st != SNAPKV_OK) return st;
   if (!aligned16(q_obs) || !aligned16(k) || !aligned16(v) || !aligned16(out_k) || !aligned16(out_v))
     return SNAPKV_ERR_INVALID_ARG;
-  for (int b = 0; b < B; ++b) {
-    if (seq_lens[b] < W || seq_lens[b] > Lmax) return SNAPKV_ERR_INVALID_ARG;
-    if (k_seq_offsets && (k_seq_offsets[b] < 0 || (k_seq_offsets[b] & 7))) return SNAPKV_ERR_INVALID_ARG;
-    if (v_seq_offsets && (v_seq_offsets[b] < 0 || (v_seq_offsets[b] & 7))) return SNAPKV_ERR_INVALID_ARG;
-    if (!out_idx && seq_lens[b] > W) return SNAPKV_ERR_INVALID_ARG;
-  }
-  for (int b = 0; b < B; ++b) {
-    if (budget >= seq_lens[b]) continue;  // copied through: no scratch
-    const size_t need =
-        snapkv_workspace_size(1, Hq, Hkv, seq_lens[b], d, W, pool_kernel, pool_type, budget);
-    if (need == 0) return SNAPKV_ERR_INVALID_ARG;
-    if (!workspace_ok(workspace, workspace_bytes, need)) return SNAPKV_ERR_WORKSPACE;
-  }
-  // one clear of the status block for the whole call, whichever path the first sequence takes
-  const bool have_ws = workspace_ok(workspace, workspace_bytes, STATUS_BYTES);
-  if (have_ws && clear_status(workspace, static_cast<cudaStream_t>(stream)) != cudaSuccess)
-    return SNAPKV_ERR_CUDA;
-  const size_t head_rows = static_cast<size_t>(Hq) * budget * d * 2;  // bytes of one sequence's out_k
-  int launches = 0;
-  for (int b = 0; b < B; ++b) {
-    const long long ko = k_seq_offsets ? k_seq_offsets[b] : b * ks.b;
-    const long long vo = v_seq_offsets ? v_seq_offsets[b] : b * vs.b;
-    // the sequences are independent (Sec. 4.1): one single-sequence step each, on the same
-    // stream and workspace; the status block keeps the first error of any of them
-    st = compress_impl(static_cast<const uint8_t*>(q_obs) + static_cast<size_t>(b) * Hq * W * d * 2,
-                       static_cast<const uint8_t*>(k) + ko * 2,
-                       static_cast<const uint8_t*>(v) + vo * 2, 1, Hq, Hkv, seq_lens[b], d, W,
-                       pool_kernel, pool_type, budget,
-                       static_cast<uint8_t*>(out_k) + b * head_rows,
-                       static_cast<uint8_t*>(out_v) + b * head_rows,
-                       out_idx ? out_idx + static_cast<size_t>(b) * Hq * (budget - W) : nullptr,
-                       workspace, workspace_bytes, stream, /*keep_status=*/true,
-                       lse_obs ? lse_obs + static_cast<size_t>(b) * Hq * W : nullptr, &ks, &vs);
-    if (st != SNAPKV_OK) return st;
-    launches += g_last_launches;
-  }
-  g_last_launches = launches;
-  return SNAPKV_OK;
+  const RaggedCall c = {q_obs, k, v, ks, vs, k_seq_offsets, v_seq_offsets, seq_lens, lse_obs, B, Hq, Hkv, d, W,
+                        pool_kernel, pool_type, budget, out_k, out_v, out_idx, workspace, workspace_bytes,
+                        static_cast<cudaStream_t>(stream), nullptr, fill != 0};
+  st = ragged_check(c, Lmax);
+  return st != SNAPKV_OK ? st : ragged_impl(c);
 }
 
-snapkv_status_t snapkv_compress_paged(const void* q_obs, const void* k_pool, const void* v_pool,
-                                      const int64_t* k_strides, const int64_t* v_strides,
-                                      const int32_t* page_table, int pages_per_seq, int page_size,
-                                      int num_pages, const int32_t* seq_lens, const float* lse_obs,
-                                      int B, int Hq, int Hkv, int L, int d, int W, int pool_kernel,
-                                      int pool_type, int budget, void* out_k, void* out_v,
-                                      int32_t* out_idx, void* workspace, size_t workspace_bytes,
-                                      void* stream) {
+snapkv_status_t snapkv_compress_varlen(const void* q_obs, const void* k, const void* v,
+                                       const int64_t* k_strides, const int64_t* v_strides,
+                                       const int64_t* k_seq_offsets, const int64_t* v_seq_offsets,
+                                       const int32_t* seq_lens, const float* lse_obs, int B,
+                                       int Hq, int Hkv, int Lmax, int d, int W, int pool_kernel,
+                                       int pool_type, int budget, void* out_k, void* out_v,
+                                       int32_t* out_idx, void* workspace, size_t workspace_bytes,
+                                       void* stream) {
+  return snapkv_binding_varlen(q_obs, k, v, k_strides, v_strides, k_seq_offsets, v_seq_offsets, seq_lens, lse_obs, B,
+                               Hq, Hkv, Lmax, d, W, pool_kernel, pool_type, budget, out_k, out_v, out_idx, workspace,
+                               workspace_bytes, stream, 0);
+}
+
+snapkv_status_t snapkv_binding_paged(const void* q_obs, const void* k_pool, const void* v_pool,
+                                     const int64_t* k_strides, const int64_t* v_strides, const int32_t* page_table,
+                                     int pages_per_seq, int page_size, int num_pages, const int32_t* seq_lens,
+                                     const float* lse_obs, int B, int Hq, int Hkv, int L, int d, int W,
+                                     int pool_kernel, int pool_type, int budget, void* out_k, void* out_v,
+                                     int32_t* out_idx, void* workspace, size_t workspace_bytes, void* stream,
+                                     int fill) {
   snapkv_status_t st = check_common(B, Hq, Hkv, L, d, W);
   if (st != SNAPKV_OK) return st;
   st = check_pool(pool_kernel, pool_type);
@@ -475,45 +629,29 @@ snapkv_status_t snapkv_compress_paged(const void* q_obs, const void* k_pool, con
   if (static_cast<long long>(pages_per_seq) * page_size < L) return SNAPKV_ERR_INVALID_ARG;
   KVStrides ks, vs;
   if (!strides_ok(k_strides, d, &ks) || !strides_ok(v_strides, d, &vs)) return SNAPKV_ERR_INVALID_ARG;
-  const PagedKV paged_all = {page_table, pages_per_seq, page_size, num_pages};
+  const PagedKV paged = {page_table, pages_per_seq, page_size, num_pages};
   if (!seq_lens)
     return compress_impl(q_obs, k_pool, v_pool, B, Hq, Hkv, L, d, W, pool_kernel, pool_type, budget,
                          out_k, out_v, out_idx, workspace, workspace_bytes, stream, false, lse_obs,
-                         &ks, &vs, false, &paged_all);
-  // per-sequence lengths: one single-sequence step each, as in snapkv_compress_varlen; every
-  // sequence and the workspace are checked before the first launch
-  for (int b = 0; b < B; ++b) {
-    if (seq_lens[b] < W || seq_lens[b] > L) return SNAPKV_ERR_INVALID_ARG;
-    if (!out_idx && seq_lens[b] > W) return SNAPKV_ERR_INVALID_ARG;
-  }
-  for (int b = 0; b < B; ++b) {
-    if (budget >= seq_lens[b]) continue;
-    const size_t need =
-        snapkv_workspace_size(1, Hq, Hkv, seq_lens[b], d, W, pool_kernel, pool_type, budget);
-    if (need == 0) return SNAPKV_ERR_INVALID_ARG;
-    if (!workspace_ok(workspace, workspace_bytes, need)) return SNAPKV_ERR_WORKSPACE;
-  }
-  if (workspace_ok(workspace, workspace_bytes, STATUS_BYTES) &&
-      clear_status(workspace, static_cast<cudaStream_t>(stream)) != cudaSuccess)
-    return SNAPKV_ERR_CUDA;
-  const size_t head_rows = static_cast<size_t>(Hq) * budget * d * 2;
-  int launches = 0;
-  for (int b = 0; b < B; ++b) {
-    const PagedKV one = {page_table + static_cast<size_t>(b) * pages_per_seq, pages_per_seq,
-                         page_size, num_pages};
-    st = compress_impl(static_cast<const uint8_t*>(q_obs) + static_cast<size_t>(b) * Hq * W * d * 2,
-                       k_pool, v_pool, 1, Hq, Hkv, seq_lens[b], d, W, pool_kernel, pool_type, budget,
-                       static_cast<uint8_t*>(out_k) + b * head_rows,
-                       static_cast<uint8_t*>(out_v) + b * head_rows,
-                       out_idx ? out_idx + static_cast<size_t>(b) * Hq * (budget - W) : nullptr,
-                       workspace, workspace_bytes, stream, /*keep_status=*/true,
-                       lse_obs ? lse_obs + static_cast<size_t>(b) * Hq * W : nullptr, &ks, &vs, false,
-                       &one);
-    if (st != SNAPKV_OK) return st;
-    launches += g_last_launches;
-  }
-  g_last_launches = launches;
-  return SNAPKV_OK;
+                         &ks, &vs, false, &paged);
+  const RaggedCall c = {q_obs, k_pool, v_pool, ks, vs, nullptr, nullptr, seq_lens, lse_obs, B, Hq, Hkv, d, W,
+                        pool_kernel, pool_type, budget, out_k, out_v, out_idx, workspace, workspace_bytes,
+                        static_cast<cudaStream_t>(stream), &paged, fill != 0};
+  st = ragged_check(c, L);
+  return st != SNAPKV_OK ? st : ragged_impl(c);
+}
+
+snapkv_status_t snapkv_compress_paged(const void* q_obs, const void* k_pool, const void* v_pool,
+                                      const int64_t* k_strides, const int64_t* v_strides,
+                                      const int32_t* page_table, int pages_per_seq, int page_size,
+                                      int num_pages, const int32_t* seq_lens, const float* lse_obs,
+                                      int B, int Hq, int Hkv, int L, int d, int W, int pool_kernel,
+                                      int pool_type, int budget, void* out_k, void* out_v,
+                                      int32_t* out_idx, void* workspace, size_t workspace_bytes,
+                                      void* stream) {
+  return snapkv_binding_paged(q_obs, k_pool, v_pool, k_strides, v_strides, page_table, pages_per_seq, page_size,
+                              num_pages, seq_lens, lse_obs, B, Hq, Hkv, L, d, W, pool_kernel, pool_type, budget,
+                              out_k, out_v, out_idx, workspace, workspace_bytes, stream, 0);
 }
 
 // ---- a prompt sharded along its length over several GPUs: the per-shard steps

@@ -1,0 +1,36 @@
+/*
+ * Entry points for the Python binding; not part of the interface in snapkv.h.  The ragged calls with
+ * one argument more: with `fill`, rows behind a sequence's end are zeroed and positions set to -1,
+ * so that the binding need not clear whole outputs first (two passes over them).
+ */
+#ifndef SNAPKV_BINDING_H_
+#define SNAPKV_BINDING_H_
+
+#include "../../include/snapkv.h"
+
+#ifdef __cplusplus
+extern "C" {
+#endif
+
+/* Workspace with which a ragged call needs the fewest launches (at least what it requires); 0 if
+ * the arguments are not acceptable or nothing needs scratch. */
+size_t snapkv_binding_ragged_workspace(const int32_t* lens, int B, int Hq, int Hkv, int d, int W, int pool_kernel,
+                                       int pool_type, int budget);
+snapkv_status_t snapkv_binding_varlen(const void* q_obs, const void* k, const void* v, const int64_t* k_strides,
+                                      const int64_t* v_strides, const int64_t* k_seq_offsets,
+                                      const int64_t* v_seq_offsets, const int32_t* seq_lens, const float* lse_obs,
+                                      int B, int Hq, int Hkv, int Lmax, int d, int W, int pool_kernel, int pool_type,
+                                      int budget, void* out_k, void* out_v, int32_t* out_idx, void* workspace,
+                                      size_t workspace_bytes, void* stream, int fill);
+snapkv_status_t snapkv_binding_paged(const void* q_obs, const void* k_pool, const void* v_pool,
+                                     const int64_t* k_strides, const int64_t* v_strides, const int32_t* page_table,
+                                     int pages_per_seq, int page_size, int num_pages, const int32_t* seq_lens,
+                                     const float* lse_obs, int B, int Hq, int Hkv, int L, int d, int W,
+                                     int pool_kernel, int pool_type, int budget, void* out_k, void* out_v,
+                                     int32_t* out_idx, void* workspace, size_t workspace_bytes, void* stream,
+                                     int fill);
+
+#ifdef __cplusplus
+}
+#endif
+#endif /* SNAPKV_BINDING_H_ */

@@ -106,6 +106,73 @@ gather_kernel(const uint4* __restrict__ k, const uint4* __restrict__ v, const Ga
     }
 }
 
+// The same for the sequences of a ragged batch (blockIdx.y = sequence * Hq + head): lengths and
+// first rows come with the launch.  A sequence no longer than the budget is copied through and
+// its position list written; with `fill` rows behind a sequence's end are zeroed.
+struct GatherSeqs {
+  int L[RAGGED_MAX];
+  long long k0[RAGGED_MAX], v0[RAGGED_MAX];  // first row, in 16-byte vectors
+  int b0, Hq, budget, fill;
+};
+template <int VPR, bool PAGED>
+__global__ void __launch_bounds__(GATHER_THREADS, GATHER_MIN_BLOCKS)
+ragged_gather_kernel(const uint4* __restrict__ k, const uint4* __restrict__ v, const GatherStrides st,
+                     const GatherPages pg, const __grid_constant__ GatherSeqs sq, int g, int W,
+                     int32_t* __restrict__ idx, uint4* __restrict__ out_k, uint4* __restrict__ out_v) {
+  constexpr int RPT = GATHER_THREADS / VPR;
+  constexpr int RPB = RPT * GATHER_UNROLL;
+  pdl_wait();
+  const int i = blockIdx.y / sq.Hq, h = blockIdx.y - i * sq.Hq;
+  const int L = sq.L[i], n = L - W, b = sq.b0 + i, c = h / g;
+  const int rows = min(sq.budget, L), ksel = rows - W, list = sq.budget - W;
+  const bool whole = sq.budget >= L;
+  const int vec = threadIdx.x % VPR;
+  const int t0 = blockIdx.x * RPB + threadIdx.x / VPR;
+  const uint4* k_head = k + (PAGED ? 0 : sq.k0[i]) + c * st.kh + vec;
+  const uint4* v_head = v + (PAGED ? 0 : sq.v0[i]) + c * st.vh + vec;
+  const int32_t* pages = PAGED ? pg.table + static_cast<size_t>(b) * pg.pages_per_seq : nullptr;
+  const size_t bh = static_cast<size_t>(b) * sq.Hq + h;
+  const size_t dst_head = bh * sq.budget * VPR + vec;
+  int32_t* idx_head = idx + bh * list;
+  int pos[GATHER_UNROLL];
+#pragma unroll
+  for (int uu = 0; uu < GATHER_UNROLL; ++uu) {
+    const int t = t0 + uu * RPT;
+    pos[uu] = -1;
+    if (t < rows) pos[uu] = t < ksel ? (whole ? t : __ldg(idx_head + t)) : n + (t - ksel);
+  }
+  uint4 kk[GATHER_UNROLL], vv[GATHER_UNROLL];
+#pragma unroll
+  for (int uu = 0; uu < GATHER_UNROLL; ++uu) {
+    kk[uu] = make_uint4(0u, 0u, 0u, 0u);
+    vv[uu] = make_uint4(0u, 0u, 0u, 0u);
+    if (pos[uu] >= 0) {
+      if (PAGED) {
+        const int slot = pos[uu] / pg.page_size;
+        const int row = pos[uu] - slot * pg.page_size;
+        const int page = __ldg(pages + slot);
+        if (static_cast<unsigned>(page) < static_cast<unsigned>(pg.num_pages)) {
+          kk[uu] = ld_stream(k_head + page * st.kb + row * st.kl);
+          vv[uu] = ld_stream(v_head + page * st.vb + row * st.vl);
+        }
+      } else {
+        kk[uu] = ld_stream(k_head + pos[uu] * st.kl);
+        vv[uu] = ld_stream(v_head + pos[uu] * st.vl);
+      }
+    }
+  }
+#pragma unroll
+  for (int uu = 0; uu < GATHER_UNROLL; ++uu) {
+    const int t = t0 + uu * RPT;
+    if (t < rows || (sq.fill && t < sq.budget)) {
+      const size_t dst = dst_head + static_cast<size_t>(t) * VPR;
+      st_stream(out_k + dst, kk[uu]);
+      st_stream(out_v + dst, vv[uu]);
+    }
+    if (whole && vec == 0 && t < list && (t < n || sq.fill)) idx_head[t] = t < n ? t : -1;
+  }
+}
+
 // A shard of a longer prompt holds positions [pos0, pos0 + L).  Of a head's ascending list of
 // selected positions, the entries inside that range form one contiguous segment.
 // seg_kernel finds it, one thread per head (two binary searches): seg[head] = {first entry of
@@ -197,6 +264,40 @@ cudaError_t launch_gather_range(const void* k, const void* v, const KVStrides& k
     gather_range_kernel<8><<<grid, GATHER_THREADS, 0, stream>>>(
         kp, vp, st, idx, Hq / Hkv, Hkv, L, pos0, ksel, append, out_rows_stride,
         static_cast<uint4*>(out_k), static_cast<uint4*>(out_v), seg);
+  *launches += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_ragged_gather(const void* k, const void* v, const KVStrides& ks, const KVStrides& vs,
+                                 const int* lens, const long long* k_off, const long long* v_off, int b0, int count,
+                                 int Hq, int Hkv, int d, int W, int budget, bool fill, int32_t* idx, void* out_k,
+                                 void* out_v, cudaStream_t stream, int* launches, const PagedKV* paged) {
+  if (static_cast<long long>(count) * Hq > 65535) return cudaErrorInvalidValue;
+  const int vpr = d * 2 / 16;
+  const int rpb = GATHER_THREADS / vpr * GATHER_UNROLL;
+  GatherSeqs sq = {};
+  sq.b0 = b0;
+  sq.Hq = Hq;
+  sq.budget = budget;
+  sq.fill = fill ? 1 : 0;
+  int rows = 0;
+  for (int i = 0; i < count; ++i) {
+    sq.L[i] = lens[i];
+    sq.k0[i] = paged ? 0 : k_off[i] / 8;
+    sq.v0[i] = paged ? 0 : v_off[i] / 8;
+    const int r = fill || lens[i] > budget ? budget : lens[i];
+    if (r > rows) rows = r;
+  }
+  const GatherStrides st = {ks.b / 8, ks.h / 8, ks.l / 8, vs.b / 8, vs.h / 8, vs.l / 8};
+  const GatherPages pg = paged ? GatherPages{paged->table, paged->pages_per_seq, paged->page_size, paged->num_pages}
+                               : GatherPages{nullptr, 0, 1, 0};
+  const dim3 grid(static_cast<unsigned>((rows + rpb - 1) / rpb), static_cast<unsigned>(count * Hq));
+  auto kernel = vpr == 16 ? (paged ? ragged_gather_kernel<16, true> : ragged_gather_kernel<16, false>)
+                          : (paged ? ragged_gather_kernel<8, true> : ragged_gather_kernel<8, false>);
+  const cudaError_t e = launch_pdl(kernel, grid, dim3(GATHER_THREADS), 0, stream, static_cast<const uint4*>(k),
+                                   static_cast<const uint4*>(v), st, pg, sq, Hq / Hkv, W, idx,
+                                   static_cast<uint4*>(out_k), static_cast<uint4*>(out_v));
+  if (e != cudaSuccess) return e;
   *launches += 1;
   return cudaGetLastError();
 }

@@ -29,6 +29,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <type_traits>
 
 #include "launch.cuh"
 #include "sm100_ptx.cuh"
@@ -101,6 +102,14 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t* warp_sums_s
   return warp_sums_s[warp] + inc - x;
 }
 
+struct OneLength {};
+struct RaggedRows {  // rows seq * heads + h: head h of the batch's sequence batch[seq]
+  int n[RAGGED_MAX], batch[RAGGED_MAX];
+  int2 want[RAGGED_MAX];
+  long long vote0[RAGGED_MAX];
+  int heads;
+};
+
 // Sliding pooling of eight positions: out[i] over a[i .. i + 2R].  The maximum is taken over
 // doubling spans (three or four operations per position instead of 2R + 1; a maximum is the same
 // in any order), the sum in ascending order.
@@ -139,11 +148,13 @@ __device__ __forceinline__ void pool8(const float* a, float (&out)[8], int r, in
 // R, PT >= 0: the pooling radius is exactly R and the type PT (0 max, 1 avg), no per-tap tests.
 // PT = -1: radius r <= R and pool_type are run-time values, and with `divisor` != 0 average pooling
 // divides the window sum by it (otherwise rows are ranked by the sum, which orders the same way up
-// to rounding).  `want`: the sample ranks (from the top) that bound the window.
-template <int THREADS, int EPT, int R, int PT>
+// to rounding).  `want`: the sample ranks (from the top) that bound the window.  ROWS: OneLength,
+// or RaggedRows when the rows come from sequences of different lengths (n and want are not used then).
+template <int THREADS, int EPT, int R, int PT, typename ROWS>
 __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 1024 / THREADS)
 pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r, int pool_type, float divisor,
-                         int ksel, int2 want, int32_t* __restrict__ out_idx, int ctas, int discard_votes) {
+                         int ksel, int2 want, int32_t* __restrict__ out_idx, int ctas, int discard_votes,
+                         const __grid_constant__ ROWS rows) {
   constexpr int CHUNK = THREADS * EPT;
   constexpr int BPT = CL_BINS / THREADS;      // bins a thread owns in the scans
   extern __shared__ __align__(16) uint32_t stage[];  // votes of the chunk, later the selected positions
@@ -157,11 +168,26 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
   __shared__ uint32_t scan_total, sel_bin, sel_above, sel_count, win_hi, win_lo, n_list, n_gt;
   __shared__ uint32_t thr_key, thr_eq, thr_all, before_gt, before_eq;
 
-  const uint32_t C = ctas, rank = blockIdx.x % ctas;
+  const uint32_t rank = blockIdx.x % ctas;
   const int row = blockIdx.x / ctas;
+  const float* vrow;
+  int32_t* orow;
+  uint32_t C = ctas;
+  if constexpr (std::is_same<ROWS, RaggedRows>::value) {
+    const int seq = row / rows.heads, h = row - seq * rows.heads;
+    n = rows.n[seq];
+    want = rows.want[seq];
+    vrow = vote + rows.vote0[seq] + static_cast<size_t>(h) * n;
+    orow = out_idx + (static_cast<size_t>(rows.batch[seq]) * rows.heads + h) * ksel;
+    // CTAs behind the end of a short row leave at once: cluster barriers do not count them
+    C = min(C, static_cast<uint32_t>((n + CHUNK - 1) / CHUNK));
+    if (rank >= C) return;
+  } else {
+    vrow = vote + static_cast<size_t>(row) * gsum * n;
+    orow = out_idx + static_cast<size_t>(row) * ksel;
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int c0 = static_cast<int>(rank) * CHUNK;  // first position of this CTA's chunk
-  const float* vrow = vote + static_cast<size_t>(row) * gsum * n;
   pdl_wait();
   if (C > 1) cluster_arrive();  // waited for before the first access to a peer's memory
 
@@ -545,7 +571,7 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
   }
   const uint32_t mine = (scan_total >> 16) + (all_eq ? 0u : min(eq0 + (scan_total & 0xffffu), need_eq) - kept0);
   __syncthreads();
-  int32_t* orow = out_idx + static_cast<size_t>(row) * ksel + gt0 + kept0;
+  orow += gt0 + kept0;
   for (uint32_t i = tid; i < mine; i += THREADS) orow[i] = static_cast<int32_t>(stage[i]);
 }
 
@@ -580,15 +606,33 @@ ClusterShape cluster_shape(int rows, int n) {
   return best;
 }
 
-template <int THREADS, int EPT, int R, int PT>
-cudaError_t launch_one(const float* vote, int rows, int n, int gsum, int r, int pool_type, float divisor, int ksel,
-                       int32_t* out_idx, int ctas, int discard, cudaStream_t stream) {
-  auto kernel = pool_topk_cluster_kernel<THREADS, EPT, R, PT>;
+// What a launch needs besides the shape.
+struct SelectCall {
+  const float* vote;
+  int rows, n, gsum, r, pool_type;
+  float divisor;
+  int ksel;
+  int32_t* out_idx;
+  int discard;
+  cudaStream_t stream;
+};
+
+// Sample ranks four standard deviations to either side of the rank that ksel maps to.
+int2 window_ranks(int ksel, int n) {
+  const double frac = static_cast<double>(ksel) / n;
+  const int delta = static_cast<int>(4.0 * sqrt(CL_SAMPLES * frac * (1.0 - frac))) + 2;
+  const int mid = static_cast<int>(frac * CL_SAMPLES);
+  return make_int2(mid - delta, mid + delta);
+}
+
+template <int THREADS, int EPT, int R, int PT, typename ROWS>
+cudaError_t launch_one(const SelectCall& c, int ctas, const ROWS& rows) {
+  auto kernel = pool_topk_cluster_kernel<THREADS, EPT, R, PT, ROWS>;
   // CTAs of this kernel take their places while the scoring CTAs leave the SMs one by one.  Asking
   // for so much shared memory that no SM takes more than its even share keeps them from crowding
   // on the SMs that come free first.
   constexpr int SMEM_MOST = 192 * 1024;
-  const int per_sm = (rows * ctas + sm_count() - 1) / sm_count();
+  const int per_sm = (c.rows * ctas + sm_count() - 1) / sm_count();
   int smem = slots_for(THREADS * EPT) * 4;
   if (smem < SMEM_MOST / per_sm) smem = SMEM_MOST / per_sm;
   static DeviceOnce once;
@@ -599,10 +643,10 @@ cudaError_t launch_one(const float* vote, int rows, int n, int gsum, int r, int 
     once.set();
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(rows) * ctas);
+  cfg.gridDim = dim3(static_cast<unsigned>(c.rows) * ctas);
   cfg.blockDim = dim3(THREADS);
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
+  cfg.stream = c.stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = ctas;
@@ -612,27 +656,29 @@ cudaError_t launch_one(const float* vote, int rows, int n, int gsum, int r, int 
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  // four standard deviations of a sample rank to either side of the rank that ksel maps to
-  const double frac = static_cast<double>(ksel) / n;
-  const int delta = static_cast<int>(4.0 * sqrt(CL_SAMPLES * frac * (1.0 - frac))) + 2;
-  const int mid = static_cast<int>(frac * CL_SAMPLES);
-  const int2 want = make_int2(mid - delta, mid + delta);
-  return cudaLaunchKernelEx(&cfg, kernel, vote, n, gsum, r, pool_type, divisor, ksel, want, out_idx, ctas, discard);
+  return cudaLaunchKernelEx(&cfg, kernel, c.vote, c.n, c.gsum, c.r, c.pool_type, c.divisor, c.ksel,
+                            window_ranks(c.ksel, c.n), c.out_idx, ctas, c.discard, rows);
 }
 
-template <int THREADS, int EPT>
-cudaError_t launch_shape(const float* vote, int rows, int n, int gsum, int r, int pool_type, float divisor, int ksel,
-                         int32_t* out_idx, int ctas, int discard, cudaStream_t stream) {
-  const bool mx = pool_type == 0;
-#define SNAPKV_CL(RR, PP) \
-  launch_one<THREADS, EPT, RR, PP>(vote, rows, n, gsum, r, pool_type, divisor, ksel, out_idx, ctas, discard, stream)
-  if (divisor != 0.f) return SNAPKV_CL(CL_RMAX, -1);
+template <int THREADS, int EPT, typename ROWS>
+cudaError_t launch_shape(const SelectCall& c, int ctas, const ROWS& rows) {
+  const bool mx = c.pool_type == 0;
+#define SNAPKV_CL(RR, PP) launch_one<THREADS, EPT, RR, PP, ROWS>(c, ctas, rows)
+  if (c.divisor != 0.f) return SNAPKV_CL(CL_RMAX, -1);
   // the paper's kernel sizes 5, 7 and 13 have instantiations of their own
-  if (r == 2) return mx ? SNAPKV_CL(2, 0) : SNAPKV_CL(2, 1);
-  if (r == 3) return mx ? SNAPKV_CL(3, 0) : SNAPKV_CL(3, 1);
-  if (r == 6) return mx ? SNAPKV_CL(6, 0) : SNAPKV_CL(6, 1);
+  if (c.r == 2) return mx ? SNAPKV_CL(2, 0) : SNAPKV_CL(2, 1);
+  if (c.r == 3) return mx ? SNAPKV_CL(3, 0) : SNAPKV_CL(3, 1);
+  if (c.r == 6) return mx ? SNAPKV_CL(6, 0) : SNAPKV_CL(6, 1);
   return SNAPKV_CL(CL_RMAX, -1);
 #undef SNAPKV_CL
+}
+
+template <typename ROWS>
+cudaError_t launch_rows(const ClusterShape& s, const SelectCall& c, const ROWS& rows) {
+  auto f = s.threads == 256 ? launch_shape<256, 8, ROWS>
+           : s.threads == 512 ? launch_shape<512, 8, ROWS>
+           : s.ept == 8 ? launch_shape<1024, 8, ROWS> : (s.ept == 16 ? launch_shape<1024, 16, ROWS> : launch_shape<1024, 32, ROWS>);
+  return f(c, s.ctas, rows);
 }
 
 }  // namespace
@@ -645,7 +691,7 @@ static bool cluster16_ok() {
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return false;
   int st = state[dev].load(std::memory_order_acquire);
   if (st == 0) {
-    auto kernel = pool_topk_cluster_kernel<1024, 32, CL_RMAX, -1>;
+    auto kernel = pool_topk_cluster_kernel<1024, 32, CL_RMAX, -1, OneLength>;
     constexpr int SMEM = slots_for(1024 * 32) * 4;
     int n_clusters = 0;
     bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
@@ -680,14 +726,53 @@ bool select_cluster_applies(int rows, int n, int pool_kernel) {
 cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int pool_kernel,
                                      int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream,
                                      int* launches, int gsum, bool vote_is_scratch) {
-  const ClusterShape s = cluster_shape(rows, n);
-  const int r = pool_kernel >> 1, discard = vote_is_scratch ? 1 : 0;
   // rows beyond 131072 positions rank average-pooled votes by the mean, shorter ones by the sum
   const float divisor = n > 131072 && pool_type == 1 ? static_cast<float>(pool_kernel) : 0.f;
-  auto f = s.threads == 256 ? launch_shape<256, 8>
-           : s.threads == 512 ? launch_shape<512, 8>
-           : s.ept == 8 ? launch_shape<1024, 8> : (s.ept == 16 ? launch_shape<1024, 16> : launch_shape<1024, 32>);
-  const cudaError_t e = f(vote, rows, n, gsum, r, pool_type, divisor, ksel, out_idx, s.ctas, discard, stream);
+  const SelectCall c = {vote, rows, n, gsum, pool_kernel >> 1, pool_type, divisor, ksel, out_idx,
+                        vote_is_scratch ? 1 : 0, stream};
+  const cudaError_t e = launch_rows(cluster_shape(rows, n), c, OneLength{});
+  if (e != cudaSuccess) return e;
+  *launches += 1;
+  return cudaGetLastError();
+}
+
+// Shape for the rows of a ragged batch (a cluster has as many CTAs as the longest row needs, those
+// that a shorter row does not need leave at once).
+static ClusterShape ragged_shape(int n) {
+  if (n <= 2048) return {256, 8, 1};
+  if (n <= 4096) return {512, 8, 1};
+  if (n <= 8192) return {1024, 8, 1};
+  if (n <= 8 * 16384) return {1024, 16, (n + 16383) / 16384};
+  return {1024, 32, (n + 32767) / 32768};
+}
+
+// Whether the rows of a ragged batch, the longest of n_max positions, can share a launch.
+bool ragged_select_applies(int n_max, int pool_kernel, int pool_type) {
+  if ((pool_kernel >> 1) > CL_RMAX || n_max > CL_MAX_CLUSTER * 1024 * 32) return false;
+  if (pool_type == 1 && n_max > 131072) return false;  // two ways of ranking in one launch
+  return ragged_shape(n_max).ctas <= 8 || cluster16_ok();
+}
+
+cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int Hq, int W, int pool_kernel,
+                                 int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream, int* launches) {
+  // longest rows first: the last CTAs to start should be short ones
+  int order[RAGGED_MAX];
+  for (int i = 0; i < rb.count; ++i) {
+    int at = i;
+    for (; at > 0 && rb.L[order[at - 1]] < rb.L[i]; --at) order[at] = order[at - 1];
+    order[at] = i;
+  }
+  RaggedRows rows = {};
+  rows.heads = Hq;
+  for (int i = 0; i < rb.count; ++i) {
+    const int o = order[i], n = rb.L[o] - W;
+    rows.n[i] = n;
+    rows.batch[i] = rb.batch[o];
+    rows.want[i] = window_ranks(ksel, n);
+    rows.vote0[i] = rb.vote0[o];
+  }
+  const SelectCall c = {vote, rb.count * Hq, rows.n[0], 1, pool_kernel >> 1, pool_type, 0.f, ksel, out_idx, 1, stream};
+  const cudaError_t e = launch_rows(ragged_shape(rows.n[0]), c, rows);
   if (e != cudaSuccess) return e;
   *launches += 1;
   return cudaGetLastError();

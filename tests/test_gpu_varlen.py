@@ -114,3 +114,37 @@ def test_status_block_is_clean_whichever_path_the_first_sequence_takes(use_lse):
     dev = {x: seqs[0][x].cuda() for x in ("q_obs", "k", "v")}
     sk.snapkv_compress(dev["q_obs"], dev["k"], dev["v"], kernel, sk.POOL_AVG, budget, workspace=ws)
     assert sk.snapkv_device_status(ws) == (sk.OK, 0)
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,d,W,kernel,ptype,budget,use_lse", [
+    ([300, 5000, 129, 2049, 700, 17], 8, 2, 128, 16, 5, "max", 200, False),   # copied through in between
+    ([1500] * 3 + [40, 9000, 641], 4, 4, 64, 32, 7, "max", 256, True),
+    ([2000, 300, 4097, 1025], 6, 2, 128, 24, 13, "avg", 128, False),          # window not a multiple of 16
+    ([900, 33000, 4000], 8, 1, 128, 64, 7, "max", 512, False),                # clusters of select CTAs
+    ([50000, 60000, 1000, 70000], 16, 8, 128, 32, 7, "max", 1024, False),     # more than one wave per sequence
+    ([150 + 37 * i for i in range(70)], 2, 1, 64, 32, 5, "avg", 140, False),  # more sequences than a launch takes
+    ([700, 1900, 800], 4, 2, 128, 32, 17, "max", 100, False),                 # radius 8: one sequence at a time
+])
+def test_ragged_batch_equals_the_calls_one_by_one(lens, Hq, Hkv, d, W, kernel, ptype, budget, use_lse):
+    # bit for bit: every sequence of the batch is scored in the order of a call of its own.  Once
+    # with the workspace the call picks and once with the least it must accept (groups of one).
+    g = torch.Generator(device="cuda").manual_seed(len(lens) + W)
+    seqs = [{x: torch.randn(*sh, generator=g, device="cuda").to(torch.bfloat16)
+             for x, sh in (("q", (1, Hq, W, d)), ("k", (1, Hkv, L, d)), ("v", (1, Hkv, L, d)))} for L in lens]
+    lses = [torch.randn(1, Hq, W, generator=g, device="cuda") + 7.0 for _ in lens] if use_lse else None
+    k, v = (torch.cat([s[x][0].permute(1, 0, 2) for s in seqs]).contiguous() for x in "kv")   # [T, Hkv, d]
+    q = torch.cat([s["q"] for s in seqs])
+    cu = [sum(lens[:b]) for b in range(len(lens))]
+    least = max([sk.snapkv_workspace_size(1, Hq, Hkv, L, d, W, kernel, PT[ptype], budget) for L in lens if L > budget])
+    for ws in (None, torch.full((least,), 0xFF, dtype=torch.uint8, device="cuda")):
+        out_k, out_v, out_idx, used = sk.snapkv_compress_varlen(
+            q, k, v, lens, kernel, PT[ptype], budget, cu_seqlens=cu, workspace=ws,
+            lse_obs=torch.cat(lses) if use_lse else None)
+        assert (used is ws) == (ws is not None) and sk.snapkv_device_status(used) == (sk.OK, 0)
+        for b, s in enumerate(seqs):
+            rows = min(budget, lens[b])
+            ok, ov, oi, _ = sk.snapkv_compress(s["q"], s["k"], s["v"], kernel, PT[ptype], budget,
+                                               lse_obs=lses[b] if use_lse else None)
+            assert torch.equal(out_idx[b, :, :rows - W], oi[0]) and bool((out_idx[b, :, rows - W:] == -1).all())
+            for got, want in ((out_k, ok), (out_v, ov)):
+                assert torch.equal(got[b, :, :rows], want[0]) and not bool(got[b, :, rows:].any())
