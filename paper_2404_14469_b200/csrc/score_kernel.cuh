@@ -63,16 +63,19 @@ constexpr int threads_for(bool split) { return split ? 640 : 384; }
 constexpr int WAVE_LAG = 2;           // waves that the statistics run ahead of the votes
 constexpr long long WAVE_BYTES = 64ll << 20;
 constexpr int RAGGED_AHEAD = 10;      // tiles per block, the same for the sequences of a ragged batch
+constexpr int MAX_RECORDS = 192;      // work items of a CTA that one launch can hold
 constexpr int NPB = 2;                // buffers for partial statistics (book-keeper queue)
 constexpr int NLB = 8;                // buffers for merged log-sum-exp rows
 constexpr int FOLD = 8;               // partials folded at a time
-constexpr int MERGE_SEGS = 40;        // partials staged in shared memory at a time
+constexpr int MERGE_SEGS = 36;        // partials staged in shared memory at a time
 
 struct ScoreArgs {
   int L, n, W, Hkv;
   int hpu, ncols, npad;
   int sub_per_kv, g;
-  int units, upw, nwaves;   // units per wave, number of waves
+  int units, upw, nwaves;   // units per wave, number of waves (of this launch, from wave0 on)
+  int wave0;
+  int per;                  // most work items of a CTA in one phase
   int T1, T2;               // tiles per unit in the statistics / vote pass
   int maxseg;               // partial slots per unit
   int pipelined;            // how many waves the statistics run ahead of the votes (>= 1)
@@ -105,7 +108,9 @@ struct Smem {
   static constexpr int OFF_PART = OFF_MISC + 16;              // float2 [NPB][2 sets][8][32]
   static constexpr int OFF_LSE = OFF_PART + NPB * 16 * 32 * 8; // float [NLB][128]
   static constexpr int OFF_MERGE = OFF_LSE + NLB * 128 * 4;   // float [MERGE_SEGS][128]
-  static constexpr int TOTAL = OFF_MERGE + MERGE_SEGS * 128 * 4;
+  static constexpr int OFF_ITEMS = OFF_MERGE + MERGE_SEGS * 128 * 4;  // ItemRecord [MAX_RECORDS]
+  static constexpr int OFF_ORDER = OFF_ITEMS + MAX_RECORDS * 16;      // uint16 [MAX_RECORDS]
+  static constexpr int TOTAL = OFF_ORDER + MAX_RECORDS * 2;
   static_assert(OFF_PART % 16 == 0 && OFF_LSE % 16 == 0 && OFF_MERGE % 16 == 0,
                 "float4 reads of the lse buffers, 16-byte copies into the merge buffer");
   static constexpr int DYN_BYTES = TOTAL + 1024;            // slack for 1024-byte alignment
@@ -184,26 +189,35 @@ __device__ __forceinline__ void copy16_async(uint32_t dst, const float* src) {
 }
 __device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Adds partials (log2-sum-exp each) to a running maximum M and sum S of exp2(. - M), in order.  The
-// maxima come first, so that the exponentials do not wait for one another: only the sums are a
-// chain, one fused multiply-add per partial.
+// Adds partials (log2-sum-exp each) to a running maximum M and sum S of exp2(. - M), in order.  With
+// Mn the new maximum, S = S exp2(M - Mn) + exp2(pv - Mn), and one of the two exponentials is
+// exp2(0) = 1: the other one is computed alone, since this warp shares its exponential unit with four
+// softmax warps.  The maxima come first, so that the exponentials do not wait for one another: only
+// the sums are a chain, one fused multiply-add per partial.
 __device__ __forceinline__ void fold_partials(const float (&pv)[FOLD], float& M, float& S) {
-  float scale[FOLD], term[FOLD];
+  float e[FOLD];
+  bool grows[FOLD];
 #pragma unroll
   for (int i = 0; i < FOLD; ++i) {
+    grows[i] = pv[i] > M;
     const float Mn = fmaxf(fmaxf(M, pv[i]), -1e30f);
-    scale[i] = ex2_approx(M - Mn);
-    term[i] = ex2_approx(pv[i] - Mn);
+    e[i] = ex2_approx(fminf(M, pv[i]) - Mn);
     M = Mn;
   }
 #pragma unroll
-  for (int i = 0; i < FOLD; ++i) S = fmaf(S, scale[i], term[i]);
+  for (int i = 0; i < FOLD; ++i) S = fmaf(S, grows[i] ? e[i] : 1.f, grows[i] ? 1.f : e[i]);
 }
 
 // One piece of work: tiles [t0, t1) of one unit in one pass.  `seq` and `flip` matter to ragged
 // batches alone: the sequence, and which set of softmax warps takes the first tile.
 struct Item {
   int unit, t0, t1, vote, slot, nseg, seq, flip;
+};
+// The same in shared memory: unit | seq << 24 | flip << 31, tiles, slot | nseg << 16.
+struct ItemRecord {
+  uint32_t what;
+  int t0, t1;
+  uint32_t seg;
 };
 
 // The sequences of a ragged batch, passed by value with the launch (in constant memory, no copies
@@ -224,126 +238,136 @@ struct RaggedSeqs {
   CUtensorMap maps[MAPS];
   RaggedSeq s[RAGGED_MAX];
   int nseq, units_per_seq;
+  int waves;           // of all sequences
 };
 struct NotRagged {};
 
-// The work items of CTA `cr` in one phase: the phase's TT = nu * T tiles (units u0 .. u0+nu-1,
-// T tiles each) are cut into G consecutive shares, CTA c owning tiles [c*TT/G, (c+1)*TT/G); a
-// share that crosses a unit boundary is one item per unit.  I is the integer type of the tile
-// arithmetic: every warp of a CTA walks the list, at every item, so the divisions are done in
-// 32 bits whenever the products fit (64-bit divisions cost about 0.1 us each here).
-template <typename I, typename F>
-__host__ __device__ __forceinline__ bool phase_items(int tiles_stats, int cr, int G, int u0,
-                                                     int nu, int T, int vote, F&& f) {
-  const I g = static_cast<I>(G);
-  const I TT = static_cast<I>(nu) * static_cast<I>(T);
-  const I lo = static_cast<I>(cr) * TT / g, hi = static_cast<I>(cr + 1) * TT / g;
-  // where this CTA's partial of a unit goes and how many partials the unit gets follow from
-  // the statistics-pass partition of the unit's wave (TT1 tiles)
-  const I T1 = static_cast<I>(tiles_stats);
-  const I TT1 = static_cast<I>(nu) * T1;
-  // the CTA whose share contains tile x: the largest c with c*TT1/G <= x
-  auto cta_of_tile = [&](I x) { return static_cast<int>(((x + 1) * g + TT1 - 1) / TT1) - 1; };
-  for (I pos = lo; pos < hi;) {
-    const I ul = pos / static_cast<I>(T);
-    Item it;
+// Quotients of tile arithmetic, in 32 bits whenever the dividend fits.
+__host__ __device__ __forceinline__ uint32_t quotient(unsigned long long x, uint32_t y) {
+  return (x >> 32) == 0 ? static_cast<uint32_t>(x) / y : static_cast<uint32_t>(x / y);
+}
+
+// The share of one CTA in one phase: the phase's TT = nu * T tiles (units u0 .. u0+nu-1, T tiles
+// each) are cut into G consecutive shares, the CTA playing part `cr` owning tiles
+// [cr*TT/G, (cr+1)*TT/G); a share that crosses a unit boundary is one item per unit.
+struct Share {
+  uint32_t lo, hi, pos;
+  int u0, nu, T, T1, cr, G;
+
+  __host__ __device__ __forceinline__ Share(int cr_, int G_, int u0_, int nu_, int T_, int T1_)
+      : u0(u0_), nu(nu_), T(T_), T1(T1_), cr(cr_), G(G_) {
+    const unsigned long long TT = static_cast<unsigned long long>(nu) * static_cast<uint32_t>(T);
+    lo = pos = quotient(static_cast<uint32_t>(cr) * TT, G);
+    hi = quotient(static_cast<uint32_t>(cr + 1) * TT, G);
+  }
+  // The next item; an empty one (t0 = t1) behind the last.
+  __host__ __device__ __forceinline__ Item take() {
+    Item it = {};
+    if (pos >= hi) return it;
+    const uint32_t ul = pos / static_cast<uint32_t>(T);
     it.unit = u0 + static_cast<int>(ul);
-    it.t0 = static_cast<int>(pos - ul * static_cast<I>(T));
-    const I t1 = static_cast<I>(it.t0) + (hi - pos);
-    it.t1 = t1 < static_cast<I>(T) ? static_cast<int>(t1) : T;
-    it.vote = vote;
-    it.seq = 0;
-    it.flip = static_cast<int>(pos - lo);  // tiles of this phase that this block has had before
-    if (TT1 >= g) {  // every CTA has tiles: a unit's owners are consecutive CTAs
-      const int cfirst = cta_of_tile(ul * T1);
-      const int clast = cta_of_tile((ul + 1) * T1 - 1);
-      it.slot = cr - cfirst;
-      it.nseg = clast - cfirst + 1;
-    } else {         // fewer tiles than CTAs: one tile per owner, one partial per tile
+    it.t0 = static_cast<int>(pos - ul * static_cast<uint32_t>(T));
+    const uint32_t t1 = static_cast<uint32_t>(it.t0) + (hi - pos);
+    it.t1 = t1 < static_cast<uint32_t>(T) ? static_cast<int>(t1) : T;
+    it.flip = static_cast<int>((pos - lo) & 1);  // tiles of this phase that this block has had before
+    pos += static_cast<uint32_t>(it.t1 - it.t0);
+    // where this CTA's partial of the unit goes and how many partials the unit gets follow from
+    // the statistics-pass partition of the unit's wave
+    const uint32_t T1u = static_cast<uint32_t>(T1), TT1 = static_cast<uint32_t>(nu) * T1u;
+    if (TT1 >= static_cast<uint32_t>(G)) {  // every CTA has tiles: a unit's owners are consecutive CTAs
+      // the CTA whose share contains tile x: the largest c with c*TT1/G <= x
+      auto owner = [&](uint32_t x) {
+        return static_cast<int>(quotient((x + 1ull) * static_cast<uint32_t>(G) + TT1 - 1, TT1)) - 1;
+      };
+      const int first = owner(ul * T1u);
+      it.slot = cr - first;
+      it.nseg = owner(ul * T1u + T1u - 1) - first + 1;
+    } else {  // fewer tiles than CTAs: one tile per owner, one partial per tile
       it.slot = it.t0;
-      it.nseg = tiles_stats;
+      it.nseg = T1;
     }
-    pos += static_cast<I>(it.t1 - it.t0);
-    if (!f(it)) return false;
+    return it;
   }
-  return true;
-}
+};
 
-// Calls f(item) for every work item of this CTA in schedule order; stops when f
-// returns false.  All warp roles walk the same list.
-template <typename F>
-__host__ __device__ __forceinline__ void for_each_item(const ScoreArgs& a, int cta, int G, int lag,
-                                                       F&& f) {
-  // Phase order: statistics run `lag` waves ahead of votes: S(0) .. S(lag-1) V(0) S(lag)
-  // V(1) ...; lag = 1 is the plain order S(0) V(0) S(1) V(1) ...
-  int s_next = a.votes_only ? a.nwaves : 0, v_next = a.stats_only ? a.nwaves : 0;
-  while (v_next < a.nwaves || s_next < a.nwaves) {
-    int w, vote;
-    if (s_next < a.nwaves && (v_next >= a.nwaves || s_next - v_next < lag)) { w = s_next++; vote = 0; }
-    else { w = v_next++; vote = 1; }
-    const int u0 = w * a.upw;
-    const int nu = a.upw < a.units - u0 ? a.upw : a.units - u0;
-    const int T = vote ? a.T2 : a.T1;
-    // TT is seldom a multiple of G, so some CTAs get one tile less than the others; which
-    // ones moves on by one CTA from phase to phase, so that over the phases of a launch no
-    // CTA carries the longer share every time
-    const int cr = (cta + 2 * w + vote) % G;
-    const long long tmax = static_cast<long long>(nu) * (a.T1 > T ? a.T1 : T);
-    const bool fits32 = (tmax + 1) * (G + 1) < (1ll << 32);
-    const bool go_on = fits32 ? phase_items<uint32_t>(a.T1, cr, G, u0, nu, T, vote, f)
-                              : phase_items<unsigned long long>(a.T1, cr, G, u0, nu, T, vote, f);
-    if (!go_on) return;
+// One phase: a wave (of a sequence) in one of the sweeps.  `ord` counts the waves of the launch.
+struct Phase {
+  int seq, wave, vote, ord;
+};
+
+// Phase p of the launch.  Statistics run `lag` waves ahead of votes: S(0) .. S(lag-1) V(0) S(lag)
+// V(1) ...; lag = 1 is the plain order S(0) V(0) S(1) V(1) ...
+__host__ __device__ __forceinline__ Phase phase_at(const ScoreArgs& a, NotRagged, int, int p) {
+  int s = a.votes_only ? a.nwaves : 0, v = 0;
+  Phase ph = {0, 0, 0, 0};
+  for (int i = 0; i <= p; ++i) {
+    ph.vote = !(s < a.nwaves && (a.stats_only || s - v < a.pipelined));
+    ph.ord = ph.vote ? v++ : s++;
   }
+  ph.wave = a.wave0 + ph.ord;
+  return ph;
 }
+__host__ __device__ __forceinline__ int phase_count(const ScoreArgs& a, NotRagged) {
+  return (a.votes_only || a.stats_only) ? a.nwaves : 2 * a.nwaves;
+}
+// CTA `cta`'s share of a phase.  TT is seldom a multiple of G, so some CTAs get one tile less than
+// the others; which ones moves on by one CTA from phase to phase, so that over the phases of a
+// launch no CTA carries the longer share every time.
+__host__ __device__ __forceinline__ Share share_of(const ScoreArgs& a, NotRagged, const Phase& ph, int cta, int G) {
+  const int u0 = ph.wave * a.upw;
+  return Share((cta + 2 * ph.wave + ph.vote) % G, G, u0, a.upw < a.units - u0 ? a.upw : a.units - u0,
+               ph.vote ? a.T2 : a.T1, a.T1);
+}
+__host__ __device__ __forceinline__ int tiles_before(const ScoreArgs&, NotRagged, const Phase&, int, int) { return 0; }
 
-// The same walk for a ragged batch.  Each sequence is cut as a call of its own would cut it (the
-// same shares, partials and order of additions, so its results do not depend on the batch), and
-// the waves of the sequences follow one another with the statistics at least `lag` waves and
+// The same for a ragged batch.  Each sequence is cut as a call of its own would cut it (the same
+// shares, partials and order of additions, so its results do not depend on the batch), and the
+// waves of the sequences follow one another with the statistics at least `lag` waves and
 // RAGGED_AHEAD tiles per block ahead: the hand-over of a wave's statistics takes some microseconds,
 // the tiles of a short sequence less than one.  Block c plays the part of block (c + rot) % G of
-// such a call, so that short sequences occupy different blocks; `flip` restores the parity with
-// which that block would have met the item's first tile.
-template <typename SEQS, typename F>
-__device__ __forceinline__ void for_each_item_ragged(const ScoreArgs& a, const SEQS& rs, int cta, int G, int lag,
-                                                     F&& f) {
-  int s_seq = a.votes_only ? rs.nseq : 0, s_lw = 0, v_seq = 0, v_lw = 0, ahead = 0, tiles_ahead = 0;
-  while (v_seq < rs.nseq) {
-    const int vote = !(s_seq < rs.nseq && (ahead < lag || tiles_ahead < RAGGED_AHEAD * G));
-    const int seq = vote ? v_seq : s_seq, w = vote ? v_lw : s_lw;
-    const RaggedSeq& q = rs.s[seq];
-    auto units_of = [&](int wave) { return min(q.upw, rs.units_per_seq - wave * q.upw); };
-    const int nu = units_of(w), T = vote ? q.T2 : q.T1;
-    const long long tmax = static_cast<long long>(nu) * max(q.T1, T);
-    const int wave_tiles = static_cast<int>(min(static_cast<long long>(nu) * q.T1, 1ll << 20));
-    if (vote) {
-      --ahead;
-      tiles_ahead -= wave_tiles;
-      if (++v_lw == q.nwaves) { v_lw = 0; ++v_seq; }
-    } else {
-      ++ahead;
-      tiles_ahead += wave_tiles;
-      if (++s_lw == q.nwaves) { s_lw = 0; ++s_seq; }
+// such a call, so that short sequences occupy different blocks; tiles_before restores the parity
+// with which that block would have met a statistics item's first tile.
+template <int MAPS>
+__device__ __forceinline__ Phase phase_at(const ScoreArgs& a, const RaggedSeqs<MAPS>& rs, int G, int p) {
+  int s_seq = a.votes_only ? rs.nseq : 0, s_wave = 0, v_seq = 0, v_wave = 0, s_ord = 0, v_ord = 0, tiles = 0;
+  Phase ph = {0, 0, 0, 0};
+  for (int i = 0; i <= p; ++i) {
+    ph.vote = !(s_seq < rs.nseq && (s_ord - v_ord < a.pipelined || tiles < RAGGED_AHEAD * G));
+    ph.seq = ph.vote ? v_seq : s_seq;
+    ph.wave = ph.vote ? v_wave : s_wave;
+    ph.ord = ph.vote ? v_ord++ : s_ord++;
+    const RaggedSeq& q = rs.s[ph.seq];
+    const int wave_tiles = min(q.T1, 1 << 16) * min(q.upw, rs.units_per_seq - ph.wave * q.upw);
+    int& wave = ph.vote ? v_wave : s_wave;
+    tiles += ph.vote ? -wave_tiles : wave_tiles;
+    if (++wave == q.nwaves) {
+      wave = 0;
+      ++(ph.vote ? v_seq : s_seq);
     }
-    const int me = (cta + q.rot) % G;
-    auto share = [&](int wave, int is_vote) {  // tiles of block `me` in an earlier phase of the sequence
-      const long long TT = static_cast<long long>(units_of(wave)) * (is_vote ? q.T2 : q.T1);
-      const int cr = (me + 2 * wave + is_vote) % G;
-      return static_cast<int>((cr + 1) * TT / G - cr * TT / G);
-    };
-    int before = 0;
-    if (!vote)
-      for (int e = 0; e < w; ++e) before += share(e, 0) + (e + WAVE_LAG <= w ? share(e, 1) : 0);
-    const int cr = (me + 2 * w + vote) % G;
-    auto g = [&](Item it) {
-      it.seq = seq;
-      it.flip += before;
-      return f(it);
-    };
-    const bool go_on = (tmax + 1) * (G + 1) < (1ll << 32)
-                           ? phase_items<uint32_t>(q.T1, cr, G, w * q.upw, nu, T, vote, g)
-                           : phase_items<unsigned long long>(q.T1, cr, G, w * q.upw, nu, T, vote, g);
-    if (!go_on) return;
   }
+  return ph;
+}
+template <int MAPS>
+__device__ __forceinline__ int phase_count(const ScoreArgs& a, const RaggedSeqs<MAPS>& rs) {
+  return a.votes_only ? rs.waves : 2 * rs.waves;
+}
+template <int MAPS>
+__device__ __forceinline__ Share share_of(const ScoreArgs&, const RaggedSeqs<MAPS>& rs, const Phase& ph, int cta, int G) {
+  const RaggedSeq& q = rs.s[ph.seq];
+  const int u0 = ph.wave * q.upw;
+  return Share((cta + q.rot + 2 * ph.wave + ph.vote) % G, G, u0, min(q.upw, rs.units_per_seq - u0), ph.vote ? q.T2 : q.T1,
+               q.T1);
+}
+template <int MAPS>
+__device__ __forceinline__ int tiles_before(const ScoreArgs& a, const RaggedSeqs<MAPS>& rs, const Phase& ph, int cta, int G) {
+  int before = 0;  // in earlier phases of the sequence
+  if (!ph.vote)
+    for (int e = 0; e < ph.wave; ++e)
+      for (int v = 0; v < (e + WAVE_LAG <= ph.wave ? 2 : 1); ++v) {
+        const Share earlier = share_of(a, rs, Phase{ph.seq, e, v, 0}, cta, G);
+        before += static_cast<int>(earlier.hi - earlier.lo);
+      }
+  return before;
 }
 
 // NCH = npad / 32: how many 32-column chunks of the accumulator a thread reads per tile.
@@ -414,6 +438,25 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     *reinterpret_cast<volatile unsigned long long*>(abort_s + 1) = a.wait_ns;
     mbar_fence_init();
   }
+  // The work items of this CTA, a phase per thread: `per` records for each wave in each sweep and
+  // the order of the phases.  (Walking the list cost a single thread 2500 cycles of divisions an
+  // item, in every role: a ragged batch of short prompts did little else.)
+  ItemRecord* items_s = reinterpret_cast<ItemRecord*>(smem + SM::OFF_ITEMS);
+  uint16_t* order_s = reinterpret_cast<uint16_t*>(smem + SM::OFF_ORDER);
+  const int nphase = phase_count(a, rs);
+  for (int p = threadIdx.x; p < nphase; p += threads_for(SPLIT)) {
+    const Phase ph = phase_at(a, rs, G, p);
+    order_s[p] = static_cast<uint16_t>(2 * ph.ord + ph.vote);
+    Share share = share_of(a, rs, ph, cta, G);
+    const int before = tiles_before(a, rs, ph, cta, G);
+    for (int m = 0; m < a.per; ++m) {
+      const Item it = share.take();
+      items_s[(2 * ph.ord + ph.vote) * a.per + m] =
+          ItemRecord{static_cast<uint32_t>(it.unit) | static_cast<uint32_t>(ph.seq) << 24 |
+                         static_cast<uint32_t>((it.flip + before) & 1) << 31,
+                     it.t0, it.t1, static_cast<uint32_t>(it.slot) | static_cast<uint32_t>(it.nseg) << 16};
+    }
+  }
   if (warp == 1) {
     tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_ptr_s)), TMEM_COLS);
     tmem_relinquish();
@@ -426,9 +469,30 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   tc_fence_after();
   const uint32_t tmem_base = *tmem_ptr_s;
 
-  auto each_item = [&](int lag, auto&& f) {
-    if constexpr (RAGGED) for_each_item_ragged(a, rs, cta, G, lag, f);
-    else for_each_item(a, cta, G, lag, f);
+  // Item m of phase 2 * wave + sweep.
+  auto item_at = [&](int phase, int m) {
+    const ItemRecord r = items_s[phase * a.per + m];
+    Item it;
+    it.unit = static_cast<int>(r.what & 0xffffffu);
+    it.seq = RAGGED ? static_cast<int>(r.what >> 24 & 0x7fu) : 0;
+    it.flip = static_cast<int>(r.what >> 31);
+    it.t0 = r.t0;
+    it.t1 = r.t1;
+    it.vote = phase & 1;
+    it.slot = static_cast<int>(r.seg & 0xffffu);
+    it.nseg = static_cast<int>(r.seg >> 16);
+    return it;
+  };
+  // Calls f(item) for the CTA's items in schedule order until it returns false.
+  auto each_item = [&](auto&& f) {
+    for (int p = 0, m = 0; p < nphase;) {
+      const Item it = item_at(order_s[p], m);
+      if (it.t0 < it.t1 && !f(it)) break;
+      if (++m == a.per) {
+        m = 0;
+        ++p;
+      }
+    }
   };
   // tile visited at step k of an item: ascending, except that the sequential schedule
   // sweeps the vote pass backwards (the keys read last are the likeliest to be in L2)
@@ -460,7 +524,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       const uint64_t pol_first = l2_policy_evict_first();
       int git = 0;      // tiles issued so far (ring position)
       int nitem = 0;    // items started so far (Q buffer position)
-      each_item(a.pipelined, [&](const Item& it) {
+      each_item([&](const Item& it) {
         int ukv;
         const int qrow0 = first_head(it, &ukv) * a.W;
         const CUtensorMap* mapK = &tmK;
@@ -529,7 +593,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       const uint32_t idesc_s = umma_idesc_bf16(128, 128);
       const uint32_t idesc_v = umma_idesc_bf16(128, NPAD);
       int git = 0, nitem = 0;
-      each_item(a.pipelined, [&](const Item& it) {
+      each_item([&](const Item& it) {
         const int qb = nitem & 1;
         if (!mbar_wait_thread(bar_qf(qb), (nitem >> 1) & 1, abort_s, WAIT_Q_FULL)) return false;
         ++nitem;
@@ -602,7 +666,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     const int gpw = a.W >> 4;  // 16-column groups per head (when W is a multiple of 16)
     const uint32_t te_arrivals = SPLIT ? 1 : 2;          // the barrier expects 8 per tile
     int git = 0, nstat = 0, nvote = 0;
-    each_item(a.pipelined, [&](const Item& it) {
+    each_item([&](const Item& it) {
       const int nt = it.t1 - it.t0;
       int ukv;
       const int hq0 = first_head(it, &ukv);
@@ -782,9 +846,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     // CTA and the fetcher runs as far ahead as its shared-memory buffers allow.
     const bool publisher = warp == 2 + EPI_WARPS;  // warp 10; warp 11 is the fetcher
     int nstat = 0, nvote = 0;
-    each_item(/*lag=*/1, [&](const Item& it) {
-      if ((it.vote != 0) == publisher) return true;  // the other warp's kind of item
-      if (!it.vote) {
+    auto keep = [&](const Item& it) {
+      if (publisher) {
         // merge the replicas and the two warpgroups (fixed order), publish, count
         const int pb = nstat % NPB;
         if (!mbar_wait_warp(bar_pf(pb), (nstat / NPB) & 1, abort_s, WAIT_PART_FULL)) return false;
@@ -825,6 +888,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       // bit-identical rows without a second hand-over through global memory.  No fence, no counter
       // and no staging copy: a write and a read through L2 are all that lies between the last
       // partial and the first vote.
+      // In a ragged batch one CTA per unit folds and leaves the row, a flag of its own as well, in
+      // global memory: a fold of 20 partials takes this warp 3-5 us beside the softmax warps, and
+      // with a vote item for every two or three tiles the folds would set the pace.
       const int lb = nvote % NLB;
       const int c0 = lane * NCH;  // this lane's NCH columns of the window rows
       float val[NCH];
@@ -841,27 +907,38 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         }
         return __shfl_sync(0xffffffffu, stop, 0) != 0;
       };
-      if (a.votes_only) {
+      float* const row = a.lse2 + static_cast<size_t>(unit_of(it)) * MAX_COLS + c0;
+      // whether one of this lane's columns is missing (columns behind the last one never come)
+      auto missing = [&](const float (&x)[NCH]) {
+        bool gap = false;
+#pragma unroll
+        for (int t = 0; t < NCH; ++t) gap |= c0 + t < a.ncols && __float_as_uint(x[t]) == NO_PARTIAL;
+        return __any_sync(0xffffffffu, gap);
+      };
+      if (RAGGED && !a.votes_only && it.vote) {
+        for (;;) {
+          ld_relaxed<NCH>(row, val);
+          if (!missing(val)) break;
+          if (give_up()) return false;
+          __nanosleep(100);
+        }
+#pragma unroll
+        for (int t = 0; t < NCH; ++t)
+          if (c0 + t >= a.ncols) val[t] = 0.f;
+      } else if (a.votes_only) {
         while (!__all_sync(0xffffffffu, ld_acquire(a.counters + unit_of(it)) > 0)) {
           if (give_up()) return false;
           __nanosleep(100);
         }
 #pragma unroll
         for (int t = 0; t < NCH; ++t)
-          if (c0 + t < a.ncols) val[t] = __ldcg(a.lse2 + static_cast<size_t>(unit_of(it)) * MAX_COLS + c0 + t);
+          if (c0 + t < a.ncols) val[t] = __ldcg(row + t);
       } else {
         const float* pp = slots_of(it);
         const uint32_t merge_addr = sbase + SM::OFF_MERGE;
         float M[NCH], S[NCH];
 #pragma unroll
         for (int t = 0; t < NCH; ++t) { M[t] = -INFINITY; S[t] = 0.f; }
-        // whether one of this lane's columns is missing (columns behind the last one never come)
-        auto missing = [&](const float (&x)[NCH]) {
-          bool gap = false;
-#pragma unroll
-          for (int t = 0; t < NCH; ++t) gap |= c0 + t < a.ncols && __float_as_uint(x[t]) == NO_PARTIAL;
-          return __any_sync(0xffffffffu, gap);
-        };
         // All slots at once, through shared memory: every round trip to L2 costs 0.8 us here, with
         // the other CTAs reading the same lines, and registers hold only a few slots.
         int s0 = 0;
@@ -907,6 +984,13 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
 #pragma unroll
         for (int t = 0; t < NCH; ++t)
           if (c0 + t < a.ncols) val[t] = -(M[t] + log2f(S[t]));
+        if (RAGGED) {
+#pragma unroll
+          for (int t = 0; t < NCH; ++t)
+            if (c0 + t < a.ncols)
+              st_relaxed(row + t, __float_as_uint(val[t]) == NO_PARTIAL ? __uint_as_float(0x7fffffffu) : val[t]);
+          return true;
+        }
       }
       // the softmax warps must be done with this buffer's previous row
       if (!mbar_wait_warp_relaxed(bar_le(lb), ((nvote / NLB) & 1) ^ 1, abort_s, WAIT_LSE_EMPTY))
@@ -917,7 +1001,24 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       if (lane == 0) mbar_arrive(bar_lf(lb));
       ++nvote;
       return true;
-    });
+    };
+    // The publisher goes through the statistics items, the fetcher through the vote items.
+    const int waves = (a.votes_only || a.stats_only) ? nphase : nphase / 2;
+    bool go = publisher ? !a.votes_only : !a.stats_only;
+    const bool folds = RAGGED && !publisher && !a.votes_only;
+    // In a ragged batch the fetcher folds the next wave's rows, where this CTA holds the unit's first
+    // slot, before it fetches those of a wave (the statistics are at least two waves ahead), so that
+    // nobody waits for a fold.
+    for (int w = folds ? -1 : 0; w < waves && go; ++w) {
+      for (int m = 0; m < a.per && go && folds && w + 1 < waves; ++m) {
+        const Item it = item_at(2 * (w + 1), m);
+        if (it.t0 < it.t1 && it.slot == 0) go = keep(it);
+      }
+      for (int m = 0; m < a.per && go && w >= 0; ++m) {
+        const Item it = item_at(2 * w + (publisher ? 0 : 1), m);
+        if (it.t0 < it.t1) go = keep(it);
+      }
+    }
   }
 
   tc_fence_before();
@@ -974,7 +1075,7 @@ static cudaError_t run_scores_for(int d, int W, int npad, const CUtensorMap& tmK
 
 }  // namespace score
 
-// The part of the kernel's arguments that fixes the schedule (what for_each_item reads).
+// The part of the kernel's arguments that fixes the schedule (what the work items follow from).
 score::ScoreArgs score_args(const ScorePlan& plan, int L, int W, int Hkv, int votes_only);
 
 }  // namespace snapkv

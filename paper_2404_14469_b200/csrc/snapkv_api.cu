@@ -422,11 +422,16 @@ static int ragged_group(const int32_t* lens, int B, int b, int Hq, int Hkv, int 
                         size_t workspace_bytes, RaggedBatch* rb) {
   rb->count = 0;
   rb->total = 0;
+  int waves = 0, upw = 1;
   for (; b < B; ++b) {
     if (budget >= lens[b]) continue;
     if (rb->count == RAGGED_MAX) break;
     const int i = rb->count;
     if (!make_score_plan(1, Hq, Hkv, lens[b], d, W, &rb->plan[i])) break;
+    // (with supplied normalisers a sequence is one wave of all its units)
+    if (rb->plan[i].units > upw) upw = rb->plan[i].units;
+    waves += rb->plan[i].nwaves;
+    if (waves > most_waves_per_launch(upw)) break;
     rb->L[i] = lens[b];
     rb->batch[i] = b;
     rb->count = i + 1;
@@ -480,8 +485,12 @@ static snapkv_status_t ragged_impl(const RaggedCall& c) {
   int longest = 0;
   for (int b = 0; b < c.B; ++b)
     if (c.lens[b] > longest) longest = c.lens[b];
+  // the longest sequence has the most waves
+  ScorePlan p;
+  const bool shares_launches = longest <= c.budget || (make_score_plan(1, c.Hq, c.Hkv, longest, c.d, c.W, &p) &&
+                                                       p.nwaves <= most_waves_per_launch(p.units));
   int launches = 0;
-  if (c.out_idx && c.Hq <= 65535 &&
+  if (shares_launches && c.out_idx && c.Hq <= 65535 &&
       ragged_select_applies(longest - c.W > 0 ? longest - c.W : 1, c.pool_kernel, c.pool_type)) {
     uint8_t* ws = static_cast<uint8_t*>(c.workspace);
     bool first = true;  // the first group's launches clear the status block, later ones leave it

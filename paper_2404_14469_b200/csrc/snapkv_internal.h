@@ -141,6 +141,12 @@ bool encode_tensor_map(CUtensorMap* m, const void* base, int rank, const unsigne
 // SM count of the current device (asked once per device).
 int sm_count();
 
+// CTAs of the scoring kernel; the most work items a CTA has in a phase of nu units; how many waves of
+// upw units fit one launch.
+int score_grid();
+int items_per_phase(int nu, int grid);
+int most_waves_per_launch(int upw);
+
 // `n_vote` < 0: the keys that get a vote are the L - W prefix keys (the whole prompt is here).
 bool make_score_plan(int B, int Hq, int Hkv, int L, int d, int W, ScorePlan* plan, int n_vote = -1);
 WorkspaceLayout make_layout(const ScorePlan& p, int B, int Hq, int n, bool need_vote,

@@ -109,7 +109,9 @@ __global__ void lse_finish_kernel(const float* __restrict__ partials, const int*
 
 }  // namespace
 
-// The part of the kernel's arguments that fixes the schedule (what for_each_item reads).
+int score_grid() { return sm_count() < MAX_GRID ? sm_count() : MAX_GRID; }
+
+// The part of the kernel's arguments that fixes the schedule (what the work items follow from).
 score::ScoreArgs score_args(const ScorePlan& plan, int L, int W, int Hkv, int votes_only) {
   score::ScoreArgs a = {};
   a.L = L;
@@ -131,9 +133,9 @@ score::ScoreArgs score_args(const ScorePlan& plan, int L, int W, int Hkv, int vo
   a.maxseg = plan.maxseg;
   a.pipelined = plan.pipelined;
   a.votes_only = votes_only;
-  if (votes_only) {  // nothing couples the units any more: one phase over all of them
-    a.upw = plan.units;
-    a.nwaves = 1;
+  if (votes_only) {  // nothing couples the units any more: one phase over all of them (over 4096 at most)
+    a.upw = plan.units < 4096 ? plan.units : 4096;
+    a.nwaves = (plan.units + a.upw - 1) / a.upw;
   }
   return a;
 }
@@ -142,16 +144,21 @@ int list_schedule_items(const ScorePlan& plan, int L, int W, int Hkv, int votes_
                         int cta, int32_t* out, int max_items) {
   const score::ScoreArgs a = score_args(plan, L, W, Hkv, votes_only);
   int count = 0;
-  score::for_each_item(a, cta, grid, a.pipelined, [&](const score::Item& it) {
-    if (count < max_items) {
+  for (int p = 0; p < score::phase_count(a, score::NotRagged{}); ++p) {
+    const score::Phase ph = score::phase_at(a, score::NotRagged{}, grid, p);
+    score::Share share = score::share_of(a, score::NotRagged{}, ph, cta, grid);
+    for (score::Item it = share.take(); it.t0 < it.t1; it = share.take(), ++count) {
+      if (count >= max_items) continue;
       int32_t* o = out + static_cast<size_t>(count) * 6;
-      o[0] = it.unit; o[1] = it.t0; o[2] = it.t1; o[3] = it.vote; o[4] = it.slot; o[5] = it.nseg;
+      o[0] = it.unit; o[1] = it.t0; o[2] = it.t1; o[3] = ph.vote; o[4] = it.slot; o[5] = it.nseg;
     }
-    ++count;
-    return true;
-  });
+  }
   return count;
 }
+
+// A share of a phase of nu units over `grid` CTAs has at most this many items.
+int items_per_phase(int nu, int grid) { return (nu + grid - 1) / grid + 1; }
+int most_waves_per_launch(int upw) { return score::MAX_RECORDS / (2 * items_per_phase(upw, score_grid())); }
 
 bool make_score_plan(int B, int Hq, int Hkv, int L, int d, int W, ScorePlan* plan, int n_vote) {
   if (B < 1 || Hq < 1 || Hkv < 1 || L < 1 || W < 1 || W > L || Hq % Hkv != 0) return false;
@@ -264,9 +271,17 @@ cudaError_t launch_window_scores(const void* q_obs, const void* k, const KVStrid
     if (e != cudaSuccess) return e;
     *launches += 1;
   }
-  int grid = sm_count();
-  if (grid > MAX_GRID) grid = MAX_GRID;
-  const cudaError_t e = score::run_scores_for(d, W, plan.npad, tmK, tmQ, a, score::NotRagged{}, grid, stream, launches);
+  const int grid = score_grid();
+  // a launch holds the items of so many waves; what has more (gigabytes of keys) takes a launch
+  // after the other
+  a.per = items_per_phase(a.upw, grid);
+  const int most = score::MAX_RECORDS / (2 * a.per), waves = a.nwaves;
+  if (most < 1) return cudaErrorInvalidValue;
+  cudaError_t e = cudaSuccess;
+  for (; a.wave0 < waves && e == cudaSuccess; a.wave0 += most) {
+    a.nwaves = waves - a.wave0 < most ? waves - a.wave0 : most;
+    e = score::run_scores_for(d, W, plan.npad, tmK, tmQ, a, score::NotRagged{}, grid, stream, launches);
+  }
   if (e != cudaSuccess || !a.stats_only) return e;
   lse_finish_kernel<<<plan.units, MAX_COLS, 0, stream>>>(partials, counters, shard->lse_out, plan.units,
                                                         plan.maxseg, plan.sub_per_kv, plan.g, plan.hpu,

@@ -24,7 +24,7 @@ __global__ void ragged_prep_kernel(const float* __restrict__ lse_obs, const Prep
   const int u = blockIdx.x, c = threadIdx.x;  // one block per unit, one thread per window column
   if (u == 0 && c < STATUS_BYTES / 4 && !keep_status) status[c] = 0;
   if (c == 0) counters[u] = lse_obs ? 1 : 0;  // supplied normalisers are ready
-  if (!lse_obs) {  // no partial is there yet
+  if (!lse_obs) {  // neither a partial nor a folded row is there yet
     for (long long i = static_cast<long long>(u) * MAX_COLS + c; i < slots16; i += static_cast<long long>(gridDim.x) * MAX_COLS)
       partials[i] = make_uint4(NO_PARTIAL, NO_PARTIAL, NO_PARTIAL, NO_PARTIAL);
     return;
@@ -50,6 +50,8 @@ cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, cons
   score::RaggedSeqs<MAPS> rs;
   rs.nseq = rb.count;
   rs.units_per_seq = units_per_seq;
+  rs.waves = 0;
+  int upw = 1;
   const u64 strides[3] = {static_cast<u64>(ks.l) * 2, static_cast<u64>(ks.h) * 2, static_cast<u64>(ks.b) * 2};
   const unsigned box[4] = {64, TILE_KEYS, 1, 1};
   for (int i = 0; i < rb.count; ++i) {
@@ -59,6 +61,8 @@ cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, cons
     q.n = p.n_vote;
     q.upw = lse_obs ? p.units : p.units_per_wave;  // votes alone: nothing couples the units
     q.nwaves = lse_obs ? 1 : p.nwaves;
+    rs.waves += q.nwaves;
+    if (q.upw > upw) upw = q.upw;
     q.T1 = p.tiles_stats;
     q.T2 = p.tiles_vote;
     q.maxseg = p.maxseg;
@@ -99,12 +103,13 @@ cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, cons
   for (int i = 0; i < rb.count; ++i) seqs.batch[i] = rb.batch[i];
   cudaError_t e = launch_pdl(ragged_prep_kernel, dim3(rb.count * units_per_seq), dim3(MAX_COLS), 0, stream, lse_obs,
                              seqs, a.lse2, a.counters, a.status, reinterpret_cast<uint4*>(a.partials),
-                             static_cast<long long>((rb.off_lse - rb.off_partials) / 16), keep_status ? 1 : 0,
+                             static_cast<long long>((rb.off_vote - rb.off_partials) / 16), keep_status ? 1 : 0,
                              units_per_seq, Hq, p0.sub_per_kv, p0.g, p0.hpu, W, p0.ncols);
   if (e != cudaSuccess) return e;
   *launches += 1;
-  int grid = sm_count();
-  if (grid > MAX_GRID) grid = MAX_GRID;
+  const int grid = score_grid();
+  a.per = items_per_phase(upw, grid);
+  if (rs.waves * 2 * a.per > score::MAX_RECORDS) return cudaErrorInvalidValue;  // (the callers' groups are small enough)
   return score::run_scores_for(d, W, p0.npad, tmQ, tmQ, a, rs, grid, stream, launches);
 }
 
