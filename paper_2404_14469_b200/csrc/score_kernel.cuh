@@ -62,12 +62,12 @@ constexpr int EPI_WARPS = 8;           // softmax warps per set (two warpgroups)
 constexpr int threads_for(bool split) { return split ? 640 : 384; }
 constexpr int WAVE_LAG = 2;           // waves that the statistics run ahead of the votes
 constexpr long long WAVE_BYTES = 64ll << 20;
-constexpr int RAGGED_AHEAD = 10;      // tiles per block, the same for the sequences of a ragged batch
+constexpr int RAGGED_AHEAD = 64;      // tiles per block, the same for the sequences of a ragged batch
 constexpr int MAX_RECORDS = 192;      // work items of a CTA that one launch can hold
 constexpr int NPB = 2;                // buffers for partial statistics (book-keeper queue)
 constexpr int NLB = 8;                // buffers for merged log-sum-exp rows
 constexpr int FOLD = 8;               // partials folded at a time
-constexpr int MERGE_SEGS = 36;        // partials staged in shared memory at a time
+constexpr int MERGE_SEGS = 32;        // partials staged in shared memory at a time (a multiple of FOLD)
 
 struct ScoreArgs {
   int L, n, W, Hkv;
@@ -183,29 +183,30 @@ __device__ __forceinline__ void lds(uint32_t addr, float (&v)[N]) {
                  : "memory");
 }
 
+__device__ __forceinline__ void sts4(uint32_t addr, float x) {
+  asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "f"(x) : "memory");
+}
+
 // 16 bytes from global memory (past L1) to shared memory, asynchronously.
 __device__ __forceinline__ void copy16_async(uint32_t dst, const float* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void copy_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// Adds partials (log2-sum-exp each) to a running maximum M and sum S of exp2(. - M), in order.  With
-// Mn the new maximum, S = S exp2(M - Mn) + exp2(pv - Mn), and one of the two exponentials is
-// exp2(0) = 1: the other one is computed alone, since this warp shares its exponential unit with four
-// softmax warps.  The maxima come first, so that the exponentials do not wait for one another: only
-// the sums are a chain, one fused multiply-add per partial.
+// Adds partials (log2-sum-exp each) to a running maximum M (at least -1e30) and sum S of
+// exp2(. - M), in order.  The maxima come first, so that the exponentials do not wait for one
+// another: only the sums are a chain, one fused multiply-add per partial.
 __device__ __forceinline__ void fold_partials(const float (&pv)[FOLD], float& M, float& S) {
-  float e[FOLD];
-  bool grows[FOLD];
+  float scale[FOLD], term[FOLD];
 #pragma unroll
   for (int i = 0; i < FOLD; ++i) {
-    grows[i] = pv[i] > M;
-    const float Mn = fmaxf(fmaxf(M, pv[i]), -1e30f);
-    e[i] = ex2_approx(fminf(M, pv[i]) - Mn);
+    const float Mn = fmaxf(M, pv[i]);
+    scale[i] = ex2_approx(M - Mn);
+    term[i] = ex2_approx(pv[i] - Mn);
     M = Mn;
   }
 #pragma unroll
-  for (int i = 0; i < FOLD; ++i) S = fmaf(S, grows[i] ? e[i] : 1.f, grows[i] ? 1.f : e[i]);
+  for (int i = 0; i < FOLD; ++i) S = fmaf(S, scale[i], term[i]);
 }
 
 // One piece of work: tiles [t0, t1) of one unit in one pass.  `seq` and `flip` matter to ragged
@@ -324,7 +325,9 @@ __host__ __device__ __forceinline__ int tiles_before(const ScoreArgs&, NotRagged
 // shares, partials and order of additions, so its results do not depend on the batch), and the
 // waves of the sequences follow one another with the statistics at least `lag` waves and
 // RAGGED_AHEAD tiles per block ahead: the hand-over of a wave's statistics takes some microseconds,
-// the tiles of a short sequence less than one.  Block c plays the part of block (c + rot) % G of
+// the tiles of a short sequence less than one.  (Waiting costs more than reading the keys again
+// from HBM: eight sequences of 822 to 24000 positions took 175 us with 10 tiles, 155 with 16,
+// 145 with 64 and 147 without a limit.)  Block c plays the part of block (c + rot) % G of
 // such a call, so that short sequences occupy different blocks; tiles_before restores the parity
 // with which that block would have met a statistics item's first tile.
 template <int MAPS>
@@ -444,7 +447,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   ItemRecord* items_s = reinterpret_cast<ItemRecord*>(smem + SM::OFF_ITEMS);
   uint16_t* order_s = reinterpret_cast<uint16_t*>(smem + SM::OFF_ORDER);
   const int nphase = phase_count(a, rs);
-  for (int p = threadIdx.x; p < nphase; p += threads_for(SPLIT)) {
+  // (warps 0 and 1 are busy with the barriers and the tensor memory)
+  for (int p = static_cast<int>(threadIdx.x) - 64; p >= 0 && p < nphase; p += threads_for(SPLIT) - 64) {
     const Phase ph = phase_at(a, rs, G, p);
     order_s[p] = static_cast<uint16_t>(2 * ph.ord + ph.vote);
     Share share = share_of(a, rs, ph, cta, G);
@@ -852,7 +856,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         const int pb = nstat % NPB;
         if (!mbar_wait_warp(bar_pf(pb), (nstat / NPB) & 1, abort_s, WAIT_PART_FULL)) return false;
         const float2* ps = part_s + pb * 16 * 32;
-        for (int c = lane; c < a.ncols; c += 32) {
+        for (int c = lane; c < NPAD; c += 32) {  // (padding columns too: a reader looks at all of them)
           float M = -INFINITY;
           for (int w2 = 0; w2 < 2 * NSET; ++w2)
             for (int r = 0; r < REPS; ++r) {
@@ -908,12 +912,12 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         return __shfl_sync(0xffffffffu, stop, 0) != 0;
       };
       float* const row = a.lse2 + static_cast<size_t>(unit_of(it)) * MAX_COLS + c0;
-      // whether one of this lane's columns is missing (columns behind the last one never come)
+      // whether a column of a row is missing
       auto missing = [&](const float (&x)[NCH]) {
-        bool gap = false;
+        uint32_t most = 0u;  // NO_PARTIAL is the largest of all bit patterns
 #pragma unroll
-        for (int t = 0; t < NCH; ++t) gap |= c0 + t < a.ncols && __float_as_uint(x[t]) == NO_PARTIAL;
-        return __any_sync(0xffffffffu, gap);
+        for (int t = 0; t < NCH; ++t) most = max(most, __float_as_uint(x[t]));
+        return __any_sync(0xffffffffu, most == NO_PARTIAL);
       };
       if (RAGGED && !a.votes_only && it.vote) {
         for (;;) {
@@ -922,9 +926,6 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
           if (give_up()) return false;
           __nanosleep(100);
         }
-#pragma unroll
-        for (int t = 0; t < NCH; ++t)
-          if (c0 + t >= a.ncols) val[t] = 0.f;
       } else if (a.votes_only) {
         while (!__all_sync(0xffffffffu, ld_acquire(a.counters + unit_of(it)) > 0)) {
           if (give_up()) return false;
@@ -938,7 +939,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         const uint32_t merge_addr = sbase + SM::OFF_MERGE;
         float M[NCH], S[NCH];
 #pragma unroll
-        for (int t = 0; t < NCH; ++t) { M[t] = -INFINITY; S[t] = 0.f; }
+        for (int t = 0; t < NCH; ++t) { M[t] = -1e30f; S[t] = 0.f; }
         // All slots at once, through shared memory: every round trip to L2 costs 0.8 us here, with
         // the other CTAs reading the same lines, and registers hold only a few slots.
         int s0 = 0;
@@ -948,24 +949,27 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
           for (int p = lane; p < ns * CPS; p += 32)
             copy16_async(merge_addr + (p / CPS) * (MAX_COLS * 4) + (p % CPS) * 16,
                          pp + static_cast<size_t>(s0 + p / CPS) * MAX_COLS + (p % CPS) * 4);
+          // slots up to the next multiple of FOLD add nothing
+          for (int p = ns * CPS + lane; p < (ns + FOLD - 1) / FOLD * FOLD * CPS; p += 32)
+            sts4(merge_addr + (p / CPS) * (MAX_COLS * 4) + (p % CPS) * 16, -INFINITY);
           copy_wait_all();
           __syncwarp();
           int at = 0;
           for (; at < ns; at += FOLD) {
             float x[FOLD][NCH];
-            bool gap = false;
+            uint32_t most = 0u;
 #pragma unroll
             for (int i = 0; i < FOLD; ++i) {
-              lds<NCH>(merge_addr + (min(at + i, ns - 1) * MAX_COLS + c0) * 4, x[i]);
+              lds<NCH>(merge_addr + ((at + i) * MAX_COLS + c0) * 4, x[i]);
 #pragma unroll
-              for (int t = 0; t < NCH; ++t) gap |= c0 + t < a.ncols && __float_as_uint(x[i][t]) == NO_PARTIAL;
+              for (int t = 0; t < NCH; ++t) most = max(most, __float_as_uint(x[i][t]));
             }
-            if (__any_sync(0xffffffffu, gap)) break;
+            if (__any_sync(0xffffffffu, most == NO_PARTIAL)) break;
 #pragma unroll
             for (int t = 0; t < NCH; ++t) {
               float pv[FOLD];
 #pragma unroll
-              for (int i = 0; i < FOLD; ++i) pv[i] = at + i < ns ? x[i][t] : -INFINITY;  // adds nothing
+              for (int i = 0; i < FOLD; ++i) pv[i] = x[i][t];
               fold_partials(pv, M[t], S[t]);
             }
           }
@@ -982,13 +986,11 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
           }
         }
 #pragma unroll
-        for (int t = 0; t < NCH; ++t)
-          if (c0 + t < a.ncols) val[t] = -(M[t] + log2f(S[t]));
+        for (int t = 0; t < NCH; ++t) val[t] = -(M[t] + log2f(S[t]));
         if (RAGGED) {
 #pragma unroll
           for (int t = 0; t < NCH; ++t)
-            if (c0 + t < a.ncols)
-              st_relaxed(row + t, __float_as_uint(val[t]) == NO_PARTIAL ? __uint_as_float(0x7fffffffu) : val[t]);
+            st_relaxed(row + t, __float_as_uint(val[t]) == NO_PARTIAL ? __uint_as_float(0x7fffffffu) : val[t]);
           return true;
         }
       }
