@@ -412,6 +412,47 @@ def test_compress_from_host_buffers_in_parts(B, Hq, Hkv, L, d, W, kernel, budget
         assert torch.equal(oi, ref[2].cpu())
 
 
+@pytest.mark.parametrize("threads", [2, 5])
+def test_compress_from_host_buffers_on_several_threads(threads):
+    # the calls share the library's side streams and events; each has buffers and a stream of its own
+    import threading
+    B, Hq, Hkv, L, d, W, kernel, budget = 2, 8, 4, 1500, 128, 16, 5, 200
+    work = []
+    for t in range(threads):
+        data = synth.make_random(B, Hq, Hkv, L, d, W, seed=40 + t)
+        dev = _to_dev(data)
+        ref = sk.snapkv_compress(dev["q_obs"], dev["k"], dev["v"], kernel, sk.POOL_MAX, budget)
+        need = sk.snapkv_host_staging_size(B, Hq, Hkv, L, d, W, kernel, 0, budget)
+        work.append(([data[x].pin_memory() for x in ("q_obs", "k", "v")],
+                     [torch.zeros(B, Hq, budget, d, dtype=torch.bfloat16).pin_memory(),
+                      torch.zeros(B, Hq, budget, d, dtype=torch.bfloat16).pin_memory(),
+                      torch.zeros(B, Hq, budget - W, dtype=torch.int32).pin_memory()],
+                     torch.empty(need, dtype=torch.uint8, device="cuda"), torch.cuda.Stream(),
+                     [x.cpu() for x in ref]))
+    torch.cuda.synchronize()
+    bad = []
+
+    def call(ins, outs, staging, stream, ref):
+        try:
+            with torch.cuda.stream(stream):
+                for _ in range(20):
+                    for o in outs:
+                        o.zero_()
+                    sk.snapkv_compress_host(*ins, kernel, sk.POOL_MAX, budget, *outs, staging)
+                    stream.synchronize()
+                    if not all(torch.equal(o, r) for o, r in zip(outs, ref)):
+                        bad.append("outputs differ")
+        except Exception as e:  # (an exception in a thread is not seen otherwise)
+            bad.append(repr(e))
+
+    ts = [threading.Thread(target=call, args=w) for w in work]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not bad
+
+
 # ------------------------------------------------------------------ full-size workloads, sampled heads
 def _sample_heads(B, Hq, count, seed):
     g = torch.Generator().manual_seed(seed)
