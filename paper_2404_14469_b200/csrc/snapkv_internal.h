@@ -180,11 +180,11 @@ cudaError_t launch_pool_topk(const float* vote, int rows, int n, int pool_kernel
                              bool vote_is_scratch = false);
 
 // The one-cluster-per-row select kernel: whether it takes rows of this length and pooling
-// kernel on the current device, and its launch (same contract as launch_pool_topk, no scratch).
+// kernel on the current device, and its launch (same contract as launch_pool_topk).
 bool select_cluster_applies(int rows, int n, int pool_kernel);
 cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int pool_kernel,
-                                     int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream,
-                                     int* launches, int gsum, bool vote_is_scratch);
+                                     int pool_type, int ksel, int32_t* out_idx, void* scratch,
+                                     cudaStream_t stream, int* launches, int gsum, bool vote_is_scratch);
 
 // The same two steps for the sequences of a ragged batch.
 cudaError_t launch_ragged_scores(const RaggedBatch& rb, const void* q_obs, const void* k, const KVStrides& ks,

@@ -487,8 +487,9 @@ cudaError_t launch_pool_topk(const float* vote, int rows, int n, int pool_kernel
     once.set();
   }
   if (select_cluster_applies(rows, n, pool_kernel))
-    return launch_pool_topk_cluster(vote, rows, n, pool_kernel, pool_type, ksel, out_idx, stream,
-                                    launches, gsum, vote_is_scratch);
+    return launch_pool_topk_cluster(vote, rows, n, pool_kernel, pool_type, ksel, out_idx,
+                                    select_needs_scratch(n) ? pooled_scratch : nullptr, stream, launches, gsum,
+                                    vote_is_scratch);
   if (!select_needs_scratch(n)) {  // fits one CTA, but the radius is beyond the fast path
     pool_topk_kernel<<<rows, SEL_THREADS, static_cast<size_t>(n) * 4, stream>>>(
         vote, n, gsum, pool_kernel, pool_type, ksel, out_idx, nullptr);

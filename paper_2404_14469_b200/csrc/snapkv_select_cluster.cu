@@ -22,8 +22,8 @@
 // Two cluster barriers on the usual path (a byte-wise radix select took five), one histogram
 // update for every sixth key.  Back to back: 4 rows of 992 in 6.0 us (one CTA per row with all keys
 // in shared memory and five passes over them: 12.4 us), 32 rows of 16352 in 11.6 us (14.4), 128 rows
-// of 32736 in 16.8 us (20.6), 32 rows of 131008 in 22.7 us (49.9), 32 rows of 379968 in 118 us (177:
-// eight launches with the keys in global memory).
+// of 32736 in 16.8 us (20.6), 32 rows of 131008 in 22.7 us (49.9).  Rows so long or so many that the
+// clusters come in several rounds are filtered first (long_filter_kernel).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -45,6 +45,8 @@ constexpr int CL_BINS = 1024;
 constexpr int CL_SAMPLES = 256;
 constexpr int CL_SAMPLE_BINS = 512;
 constexpr int CL_LIST = 2048;        // candidates in all of a cluster's lists
+constexpr int LONG_META = 256;       // words per row: threshold, whether it is done, keys listed per chunk
+constexpr int LONG_THRESHOLD = 0, LONG_DONE = 1, LONG_COUNTS = 2;
 constexpr uint32_t KEY_MIN = 0x80000000u;  // key of a vote of zero; below it: no position
 
 __device__ __forceinline__ uint32_t float_to_key(float x) {
@@ -154,7 +156,7 @@ template <int THREADS, int EPT, int R, int PT, typename ROWS>
 __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 1024 / THREADS)
 pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r, int pool_type, float divisor,
                          int ksel, int2 want, int32_t* __restrict__ out_idx, int ctas, int discard_votes,
-                         const __grid_constant__ ROWS rows) {
+                         const uint32_t* __restrict__ meta, const __grid_constant__ ROWS rows) {
   constexpr int CHUNK = THREADS * EPT;
   constexpr int BPT = CL_BINS / THREADS;      // bins a thread owns in the scans
   extern __shared__ __align__(16) uint32_t stage[];  // votes of the chunk, later the selected positions
@@ -189,6 +191,7 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int c0 = static_cast<int>(rank) * CHUNK;  // first position of this CTA's chunk
   pdl_wait();
+  if (meta != nullptr && meta[static_cast<size_t>(row) * LONG_META + LONG_DONE]) return;
   if (C > 1) cluster_arrive();  // waited for before the first access to a peer's memory
 
   // ---- 1. the sample (pooled values at 256 positions spread over the whole row), the chunk and its
@@ -575,8 +578,288 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
   for (uint32_t i = tid; i < mine; i += THREADS) orow[i] = static_cast<int32_t>(stage[i]);
 }
 
+// Long rows of which few positions are kept: a cluster that holds a row in registers needs so many
+// SMs that few clusters run at once (12 CTAs for a row of 379968: 7 rows).  But almost all keys
+// are out of the question, and a sample tells which:
+//   1. long_sample_kernel: a lower bound of the ksel-th largest key, four standard deviations
+//      below its rank among 2048 samples of the row;
+//   2. long_filter_kernel: a CTA per 4096 positions pools them and lists the keys that reach the
+//      bound, in order of position;
+//   3. long_finish_kernel: a CTA per row selects among its list (some 2 % of the row).
+// The counts are exact.  A row whose list does not hold ksel keys, or overflows, is left to the cluster
+// kernel, which follows and skips the rows that are done.
+// 32 rows of 379968, 4064 kept: 57 us (7 + 31 + 16 + 4 for the skipped clusters), 119 with clusters
+// alone; 32 rows of 262144: 48 (67); 128 rows of 131008: 69 (86).  What bounds it is the filter's
+// instructions (some eighty per position; the votes alone would take 8 us).
+constexpr int LONG_SAMPLES = 2048;
+constexpr int LONG_LIST = 16384;     // listed keys of a row that the last kernel takes
+constexpr int LONG_THREADS = 512, LONG_CHUNK = LONG_THREADS * 8;
+constexpr int LONG_PER_SM = 3;       // CTAs of the filter kernel on an SM
+constexpr int LONG_BINS = 2048;
+
+struct RankScratch {
+  uint32_t hist[LONG_BINS], warp_sums[32], total, sel_bin, sel_above, sel_count;
+};
+
+// One histogram round of 1024 threads over the keys lo .. lo + width: narrows lo, width to the bin
+// that holds the krem-th largest of them, takes the keys above the bin off krem and returns how many
+// keys the bin holds.  The keys must hold krem in that range.
+template <int EPT>
+__device__ __forceinline__ uint32_t rank_round(const uint32_t (&key)[EPT], RankScratch& rs, uint32_t& lo,
+                                               uint32_t& width, uint32_t& krem) {
+  const int shift = max(0, 21 - __clz(width));  // (width >> shift) < LONG_BINS
+  for (int b = threadIdx.x; b < LONG_BINS; b += 1024) rs.hist[b] = 0u;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < EPT; ++i) {
+    const uint32_t rel = key[i] - lo;  // wraps for keys below lo
+    if (rel <= width) atomicAdd(&rs.hist[rel >> shift], 1u);
+  }
+  __syncthreads();
+  const int b1 = LONG_BINS - 1 - 2 * static_cast<int>(threadIdx.x);  // this thread's bins, from the highest down
+  const uint32_t n1 = rs.hist[b1], n0 = rs.hist[b1 - 1];
+  const uint32_t above = block_scan<1024>(n0 + n1, rs.warp_sums, &rs.total);
+  if (above < krem && krem <= above + n1 + n0) {
+    const bool upper = krem <= above + n1;
+    rs.sel_bin = upper ? b1 : b1 - 1;
+    rs.sel_above = upper ? above : above + n1;
+    rs.sel_count = upper ? n1 : n0;
+  }
+  __syncthreads();
+  const uint32_t end = lo + width, bin = rs.sel_bin, count = rs.sel_count;
+  krem -= rs.sel_above;
+  lo += bin << shift;
+  width = min((1u << shift) - 1u, end - lo);
+  __syncthreads();  // all have read the results before the next round writes them
+  return count;
+}
+
+// `want`: the bound is the lower edge of the bin, two rounds of 2048 bins deep, that holds the want-th
+// largest sample.
+template <int R, int PT>
+__global__ void __launch_bounds__(1024) long_sample_kernel(const float* __restrict__ vote, int n, int gsum, int r,
+                                                           int pool_type, float divisor, int want,
+                                                           uint32_t* __restrict__ meta) {
+  __shared__ RankScratch rs;
+  __shared__ uint32_t key_max, key_min;
+  const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  const float* vrow = vote + static_cast<size_t>(row) * gsum * n;
+  if (tid == 0) {
+    key_max = 0u;
+    key_min = ~0u;
+  }
+  __syncthreads();
+  pdl_wait();
+  float tap[2][2 * R + 1];
+  int js[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    js[i] = static_cast<int>((static_cast<long long>(tid + 1024 * i) * n + n / 2) / LONG_SAMPLES);
+#pragma unroll
+    for (int t = 0; t <= 2 * R; ++t) {
+      const int j = js[i] + t - R;
+      tap[i][t] = static_cast<unsigned>(j) < static_cast<unsigned>(n) ? __ldg(vrow + j) : 0.f;
+    }
+  }
+  for (int g = 1; g < gsum; ++g)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int t = 0; t <= 2 * R; ++t) {
+        const int j = js[i] + t - R;
+        if (static_cast<unsigned>(j) < static_cast<unsigned>(n)) tap[i][t] += __ldg(vrow + static_cast<size_t>(g) * n + j);
+      }
+  uint32_t k[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    float p = 0.f;
+#pragma unroll
+    for (int t = 0; t <= 2 * R; ++t)
+      if (PT >= 0 || (t - R >= -r && t - R <= r))
+        p = (PT >= 0 ? PT == 0 : pool_type == 0) ? fmaxf(p, tap[i][t]) : p + tap[i][t];
+    if (PT < 0 && divisor != 0.f) p = p / divisor;
+    k[i] = float_to_key(p);
+  }
+  const uint32_t hi = __reduce_max_sync(0xffffffffu, max(k[0], k[1])), low = __reduce_min_sync(0xffffffffu, min(k[0], k[1]));
+  if (lane == 0) {
+    atomicMax(&key_max, hi);
+    atomicMin(&key_min, low);
+  }
+  __syncthreads();
+  uint32_t lo = key_min, width = key_max - lo, krem = static_cast<uint32_t>(want);
+  rank_round(k, rs, lo, width, krem);
+  if (width > 0u) rank_round(k, rs, lo, width, krem);
+  if (tid == 0) meta[static_cast<size_t>(row) * LONG_META + LONG_THRESHOLD] = max(lo, KEY_MIN);
+}
+
+// Persistent: the votes of a CTA's next chunk are on their way while it works on the present one.
+template <int R, int PT>
+__global__ void __launch_bounds__(LONG_THREADS, LONG_PER_SM)
+long_filter_kernel(const float* __restrict__ vote, int rows, int n, int gsum, int r, int pool_type, float divisor,
+                   int nchunk, int cap, uint32_t* __restrict__ meta, uint2* __restrict__ list) {
+  __shared__ __align__(16) uint32_t stage[slots_for(LONG_CHUNK)];
+  __shared__ float halo[2][CL_RMAX + 1];
+  __shared__ uint32_t warp_sums[32], scan_total;
+  const int tid = threadIdx.x, base = tid * 8, total = rows * nchunk;
+  const int h_i = tid - (LONG_THREADS - 2 * CL_RMAX);
+  float x[8], h;
+  uint32_t bound;
+  auto fetch = [&](int w) {
+    const int row = w / nchunk, c0 = (w - row * nchunk) * LONG_CHUNK;
+    const int h_j = h_i < CL_RMAX ? c0 - CL_RMAX + h_i : c0 + LONG_CHUNK + h_i - CL_RMAX;
+    const bool have_h = h_i >= 0 && static_cast<unsigned>(h_j) < static_cast<unsigned>(n);
+    const float* src = vote + static_cast<size_t>(row) * gsum * n;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int j = c0 + tid + LONG_THREADS * u;
+      x[u] = j < n ? __ldg(src + j) : 0.f;
+    }
+    h = have_h ? __ldg(src + h_j) : 0.f;
+    bound = __ldg(meta + static_cast<size_t>(row) * LONG_META + LONG_THRESHOLD);
+    for (int g = 1; g < gsum; ++g) {
+      src += n;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int j = c0 + tid + LONG_THREADS * u;
+        if (j < n) x[u] += __ldg(src + j);
+      }
+      if (have_h) h += __ldg(src + h_j);
+    }
+  };
+  pdl_wait();
+  int w = blockIdx.x;
+  if (w < total) fetch(w);
+#pragma unroll 1
+  for (; w < total; w += gridDim.x) {
+    const int row = w / nchunk, chunk = w - row * nchunk, c0 = chunk * LONG_CHUNK;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) stage[slot(tid + LONG_THREADS * u)] = __float_as_uint(x[u]);
+    if (h_i >= 0) halo[h_i >= CL_RMAX][h_i >= CL_RMAX ? h_i - CL_RMAX : h_i] = h;
+    const uint32_t least = bound;
+    __syncthreads();
+    if (w + static_cast<int>(gridDim.x) < total) fetch(w + gridDim.x);
+    auto at = [&](int t) {
+      return t < 0 ? halo[0][CL_RMAX + t]
+                   : (t >= LONG_CHUNK ? halo[1][t - LONG_CHUNK] : __uint_as_float(stage[slot(t)]));
+    };
+    float a[2 * R + 8], p[8];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      a[i] = at(base - R + i);
+      a[R + 8 + i] = at(base + 8 + i);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; q += 4) {
+      const uint4 v = *reinterpret_cast<const uint4*>(stage + slot(base + q));
+      a[R + q] = __uint_as_float(v.x);
+      a[R + q + 1] = __uint_as_float(v.y);
+      a[R + q + 2] = __uint_as_float(v.z);
+      a[R + q + 3] = __uint_as_float(v.w);
+    }
+    pool8<R, PT>(a, p, r, pool_type, divisor);
+    uint32_t key[8], in = 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      key[i] = c0 + base + i < n ? float_to_key(p[i]) : 0u;
+      in += key[i] >= least;
+    }
+    uint32_t to = block_scan<LONG_THREADS>(in, warp_sums, &scan_total);  // (two barriers: stage is free)
+    if (in) {
+      uint2* out = list + static_cast<size_t>(w) * cap;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (key[i] >= least) {
+          if (to < static_cast<uint32_t>(cap)) out[to] = make_uint2(key[i], static_cast<uint32_t>(c0 + base + i));
+          ++to;
+        }
+    }
+    if (tid == 0) meta[static_cast<size_t>(row) * LONG_META + LONG_COUNTS + chunk] = scan_total;
+  }
+}
+
+__global__ void __launch_bounds__(1024) long_finish_kernel(int ksel, int nchunk, int cap, uint32_t* __restrict__ meta,
+                                                           const uint2* __restrict__ list,
+                                                           int32_t* __restrict__ out_idx) {
+  constexpr int EPT = LONG_LIST / 1024;
+  constexpr uint32_t NONE = 0u;  // below every listed key
+  extern __shared__ __align__(16) uint32_t keys_s[];
+  uint32_t* pos_s = keys_s + slots_for(LONG_LIST);
+  __shared__ RankScratch rs;
+  __shared__ uint32_t first[LONG_META], overflow, key_max;
+  const int row = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  uint32_t* m = meta + static_cast<size_t>(row) * LONG_META;
+  if (tid == 0) overflow = key_max = 0u;
+  pdl_wait();
+  __syncthreads();
+  const uint32_t mine = tid < nchunk ? m[LONG_COUNTS + tid] : 0u;
+  if (mine > static_cast<uint32_t>(cap)) overflow = 1u;
+  const uint32_t before = block_scan<1024>(mine, rs.warp_sums, &rs.total);
+  if (tid < nchunk) first[tid] = before;
+  const uint32_t total = rs.total;
+  __syncthreads();
+  const bool ok = !overflow && total >= static_cast<uint32_t>(ksel) && total <= LONG_LIST;
+  if (tid == 0) m[LONG_DONE] = ok;
+  if (!ok) return;
+
+  // the list, compacted; slots behind its end are NONE
+  uint32_t top = 0u;
+#pragma unroll 8
+  for (int u = 0; u < EPT; ++u) {
+    const uint32_t e = tid + 1024 * u;
+    uint2 kp = make_uint2(NONE, 0u);
+    if (e < total) {
+      int c = 0;  // the last chunk whose first entry is at or before e
+#pragma unroll
+      for (int step = LONG_META / 4; step > 0; step >>= 1)
+        if (c + step < nchunk && first[c + step] <= e) c += step;
+      kp = __ldg(list + (static_cast<size_t>(row) * nchunk + c) * cap + (e - first[c]));
+    }
+    keys_s[slot(e)] = kp.x;
+    pos_s[slot(e)] = kp.y;
+    top = max(top, kp.x);
+  }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (lane == 0) atomicMax(&key_max, top);
+  __syncthreads();
+  const int base = tid * EPT;
+  uint32_t key[EPT];
+#pragma unroll
+  for (int i = 0; i < EPT; i += 4) {
+    const uint4 v = *reinterpret_cast<const uint4*>(keys_s + slot(base + i));
+    key[i] = v.x; key[i + 1] = v.y; key[i + 2] = v.z; key[i + 3] = v.w;
+  }
+
+  // until a bin is one key wide or all of it is kept (two rounds as a rule)
+  uint32_t lo = m[LONG_THRESHOLD], width = key_max - lo, krem = static_cast<uint32_t>(ksel), all;
+  do {
+    all = rank_round(key, rs, lo, width, krem);
+  } while (width > 0u && krem != all);
+  const uint32_t T = lo;
+  const bool all_eq = krem == all;  // every key from T on is kept
+  uint32_t m_keep = 0u, m_eq = 0u;
+#pragma unroll
+  for (int i = 0; i < EPT; ++i) {
+    m_keep |= static_cast<uint32_t>(key[i] > T || (all_eq && key[i] == T)) << i;
+    m_eq |= static_cast<uint32_t>(!all_eq && key[i] == T) << i;
+  }
+  const uint32_t packed =
+      block_scan<1024>((static_cast<uint32_t>(__popc(m_keep)) << 16) | __popc(m_eq), rs.warp_sums, &rs.total);
+  uint32_t eq_seen = packed & 0xffffu, at = (packed >> 16) + min(eq_seen, krem);
+  if (all_eq) at = packed >> 16;
+  while (m_eq && eq_seen < krem) {  // of the equal keys the lowest positions
+    m_keep |= m_eq & (0u - m_eq);
+    m_eq &= m_eq - 1;
+    ++eq_seen;
+  }
+  int32_t* orow = out_idx + static_cast<size_t>(row) * ksel;
+#pragma unroll
+  for (int i = 0; i < EPT; ++i)
+    if ((m_keep >> i) & 1u) orow[at++] = static_cast<int32_t>(pos_s[slot(base + i)]);
+}
+
 struct ClusterShape {
   int threads, ept, ctas;  // threads per CTA, keys per thread, CTAs per row
+  double us = 0.0;         // estimated time (of the shapes of 1024 threads)
 };
 
 // How rows of n positions are cut: the shape with the smallest estimated time.  Up to 4096
@@ -600,7 +883,7 @@ ClusterShape cluster_shape(int rows, int n) {
     const double us = static_cast<double>((rows + fit - 1) / fit) * (c == 1 ? alone[i] : shared[i] + 0.35 * c);
     if (us < best_us) {
       best_us = us;
-      best = {1024, ept[i], c};
+      best = {1024, ept[i], c, us};
     }
   }
   return best;
@@ -615,6 +898,7 @@ struct SelectCall {
   int32_t* out_idx;
   int discard;
   cudaStream_t stream;
+  const uint32_t* meta = nullptr;  // rows marked done here are skipped
 };
 
 // Sample ranks four standard deviations to either side of the rank that ksel maps to.
@@ -657,7 +941,7 @@ cudaError_t launch_one(const SelectCall& c, int ctas, const ROWS& rows) {
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kernel, c.vote, c.n, c.gsum, c.r, c.pool_type, c.divisor, c.ksel,
-                            window_ranks(c.ksel, c.n), c.out_idx, ctas, c.discard, rows);
+                            window_ranks(c.ksel, c.n), c.out_idx, ctas, c.discard, c.meta, rows);
 }
 
 template <int THREADS, int EPT, typename ROWS>
@@ -671,6 +955,49 @@ cudaError_t launch_shape(const SelectCall& c, int ctas, const ROWS& rows) {
   if (c.r == 6) return mx ? SNAPKV_CL(6, 0) : SNAPKV_CL(6, 1);
   return SNAPKV_CL(CL_RMAX, -1);
 #undef SNAPKV_CL
+}
+
+// The want-th of LONG_SAMPLES samples is the bound that rows of n are filtered with; 0: the list
+// would be too long (or the whole row).
+int long_want(int n, int ksel) {
+  const double p = static_cast<double>(ksel) / n;
+  const int want = static_cast<int>(LONG_SAMPLES * p + 4.0 * sqrt(LONG_SAMPLES * p * (1.0 - p))) + 2;
+  const double most = (want + 4.0 * sqrt(static_cast<double>(want))) / LONG_SAMPLES * n;
+  return most <= LONG_LIST ? want : 0;
+}
+
+template <int R, int PT>
+cudaError_t launch_filter(const SelectCall& c, int want, int nchunk, int cap, uint32_t* meta, uint2* list) {
+  cudaError_t e = launch_pdl(long_sample_kernel<R, PT>, dim3(c.rows), dim3(1024), 0, c.stream, c.vote, c.n, c.gsum,
+                             c.r, c.pool_type, c.divisor, want, meta);
+  if (e != cudaSuccess) return e;
+  const long long chunks = static_cast<long long>(c.rows) * nchunk;
+  const int most = LONG_PER_SM * sm_count();
+  return launch_pdl(long_filter_kernel<R, PT>, dim3(static_cast<unsigned>(chunks < most ? chunks : most)),
+                    dim3(LONG_THREADS), 0, c.stream, c.vote, c.rows, c.n, c.gsum, c.r, c.pool_type, c.divisor, nchunk, cap, meta, list);
+}
+
+// `list` holds rows * n * 4 bytes, `meta` LONG_META words per row.
+cudaError_t launch_long(const SelectCall& c, int want, uint32_t* meta, uint2* list) {
+  const int nchunk = (c.n + LONG_CHUNK - 1) / LONG_CHUNK;
+  const int cap = c.n / 2 / nchunk;
+  constexpr int SMEM = 2 * slots_for(LONG_LIST) * 4;
+  static DeviceOnce once;
+  if (!once.done()) {
+    const cudaError_t e = cudaFuncSetAttribute(long_finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+    if (e != cudaSuccess) return e;
+    once.set();
+  }
+  const bool mx = c.pool_type == 0;
+  auto f = c.divisor != 0.f ? launch_filter<CL_RMAX, -1>
+           : c.r == 2       ? (mx ? launch_filter<2, 0> : launch_filter<2, 1>)
+           : c.r == 3       ? (mx ? launch_filter<3, 0> : launch_filter<3, 1>)
+           : c.r == 6       ? (mx ? launch_filter<6, 0> : launch_filter<6, 1>)
+                            : launch_filter<CL_RMAX, -1>;
+  const cudaError_t e = f(c, want, nchunk, cap, meta, list);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(long_finish_kernel, dim3(c.rows), dim3(1024), SMEM, c.stream, c.ksel, nchunk, cap, meta, list,
+                    c.out_idx);
 }
 
 template <typename ROWS>
@@ -724,13 +1051,26 @@ bool select_cluster_applies(int rows, int n, int pool_kernel) {
 }
 
 cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int pool_kernel,
-                                     int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream,
-                                     int* launches, int gsum, bool vote_is_scratch) {
+                                     int pool_type, int ksel, int32_t* out_idx, void* scratch,
+                                     cudaStream_t stream, int* launches, int gsum, bool vote_is_scratch) {
   // rows beyond 131072 positions rank average-pooled votes by the mean, shorter ones by the sum
   const float divisor = n > 131072 && pool_type == 1 ? static_cast<float>(pool_kernel) : 0.f;
-  const SelectCall c = {vote, rows, n, gsum, pool_kernel >> 1, pool_type, divisor, ksel, out_idx,
-                        vote_is_scratch ? 1 : 0, stream};
-  const cudaError_t e = launch_rows(cluster_shape(rows, n), c, OneLength{});
+  SelectCall c = {vote, rows, n, gsum, pool_kernel >> 1, pool_type, divisor, ksel, out_idx,
+                  vote_is_scratch ? 1 : 0, stream};
+  const ClusterShape shape = cluster_shape(rows, n);
+  // The filter's four launches take 26 us and 2.6 us per million votes (within 10 % from 8 rows of
+  // 379968 to 128 of 65536); it is taken where that is clearly less than the rounds of the clusters.
+  const double filter_us = 26.0 + 2.6e-6 * static_cast<double>(rows) * n;
+  const int want = scratch != nullptr && filter_us < 0.9 * shape.us ? long_want(n, ksel) : 0;
+  if (want) {
+    uint8_t* p = static_cast<uint8_t*>(scratch);
+    uint32_t* meta = reinterpret_cast<uint32_t*>(p + ((static_cast<size_t>(rows) * n * 4 + 255) & ~static_cast<size_t>(255)));
+    const cudaError_t e = launch_long(c, want, meta, reinterpret_cast<uint2*>(p));
+    if (e != cudaSuccess) return e;
+    *launches += 3;
+    c.meta = meta;
+  }
+  const cudaError_t e = launch_rows(shape, c, OneLength{});
   if (e != cudaSuccess) return e;
   *launches += 1;
   return cudaGetLastError();

@@ -167,6 +167,30 @@ def test_pool_topk_at_the_edges_of_its_shapes(rows, n, kernel, ptype, ksel):
 
 
 @pytest.mark.parametrize("rows,n,kernel,ptype,ksel", [
+    (8, 524288, 7, "max", 4000), (16, 262145, 5, "avg", 1), (16, 266241, 13, "avg", 1500),
+    (17, 258048, 3, "max", 2000), (9, 400001, 15, "avg", 3000),
+])
+def test_pool_topk_of_filtered_long_rows(rows, n, kernel, ptype, ksel):
+    # row 0: few distinct values (the list overflows); 1: 60 octaves; 2: constant; 3: the best positions
+    # side by side (a chunk's list overflows); 4: the sample sees larger votes than there are elsewhere (too few
+    # keys reach the bound); the rest are ordinary
+    g = torch.Generator().manual_seed(n + ksel)
+    vote = torch.rand(rows, n, generator=g) ** 4
+    vote[0] = torch.floor(vote[0] * 3) / 4
+    vote[1] = torch.exp2(60 * (vote[1] - 0.5))
+    vote[2] = 0.25
+    vote[3, 8192:8192 + ksel] += 2
+    sampled = (torch.arange(2048) * n + n // 2) // 2048
+    vote[4, sampled[:max(1, ksel // 16)]] += 3
+    idx = sk.snapkv_pool_topk(vote.cuda(), kernel, PT[ptype], ksel).cpu().numpy()
+    for r in range(6):
+        pooled = orc.pool1d(vote[r].numpy().astype(np.float64), kernel, PT[ptype])
+        same = parity.check_indices(idx[r], pooled, ksel, orc.topk_positions(pooled, ksel))
+        if ptype == "max":
+            assert same
+
+
+@pytest.mark.parametrize("rows,n,kernel,ptype,ksel", [
     (2, 40960, 7, "max", 32767),    # one below / at the point where a 16-bit count reaches bit 15
     (2, 40960, 7, "max", 32768),
     (2, 40000, 5, "avg", 39000),
