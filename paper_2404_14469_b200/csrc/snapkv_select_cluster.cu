@@ -588,9 +588,10 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
 //   3. long_finish_kernel: a CTA per row selects among its list (some 2 % of the row).
 // The counts are exact.  A row whose list does not hold ksel keys, or overflows, is left to the cluster
 // kernel, which follows and skips the rows that are done.
-// 32 rows of 379968, 4064 kept: 57 us (7 + 31 + 16 + 4 for the skipped clusters), 119 with clusters
-// alone; 32 rows of 262144: 48 (67); 128 rows of 131008: 69 (86).  What bounds it is the filter's
-// instructions (some eighty per position; the votes alone would take 8 us).
+// 32 rows of 379968, 4064 kept: 47 us (7 + 21 + 16 + 5 for the skipped clusters), 119 with clusters
+// alone; 32 rows of 262144: 39 (67); 128 rows of 131008: 54 (86).  What bounds it is the filter's
+// instructions (some thirty per position; the votes alone would take 8 us) and, in the last kernel, the
+// chain of steps that one CTA per row takes.
 constexpr int LONG_SAMPLES = 2048;
 constexpr int LONG_LIST = 16384;     // listed keys of a row that the last kernel takes
 constexpr int LONG_THREADS = 512, LONG_CHUNK = LONG_THREADS * 8;
@@ -606,12 +607,13 @@ struct RankScratch {
 // keys the bin holds.  The keys must hold krem in that range.
 template <int EPT>
 __device__ __forceinline__ uint32_t rank_round(const uint32_t (&key)[EPT], RankScratch& rs, uint32_t& lo,
-                                               uint32_t& width, uint32_t& krem) {
+                                               uint32_t& width, uint32_t& krem, int run = EPT) {
   const int shift = max(0, 21 - __clz(width));  // (width >> shift) < LONG_BINS
   for (int b = threadIdx.x; b < LONG_BINS; b += 1024) rs.hist[b] = 0u;
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < EPT; ++i) {
+    if (i >= run) break;  // (the first `run` keys, the same in all threads)
     const uint32_t rel = key[i] - lo;  // wraps for keys below lo
     if (rel <= width) atomicAdd(&rs.hist[rel >> shift], 1u);
   }
@@ -693,87 +695,104 @@ __global__ void __launch_bounds__(1024) long_sample_kernel(const float* __restri
 }
 
 // Persistent: the votes of a CTA's next chunk are on their way while it works on the present one.
+// Few instructions per position are what counts here: the halo lies in front of and behind the chunk in
+// the same array (so a thread reads its run and its neighbours' as aligned vectors), whole chunks
+// skip the checks of the row's end, the pooled values are compared as numbers, and only warps that
+// have something to list scan (32 rows of 379968: 31 us with a scan of the block, element-wise
+// neighbours and a division per chunk, 21 so).
 template <int R, int PT>
 __global__ void __launch_bounds__(LONG_THREADS, LONG_PER_SM)
 long_filter_kernel(const float* __restrict__ vote, int rows, int n, int gsum, int r, int pool_type, float divisor,
                    int nchunk, int cap, uint32_t* __restrict__ meta, uint2* __restrict__ list) {
-  __shared__ __align__(16) uint32_t stage[slots_for(LONG_CHUNK)];
-  __shared__ float halo[2][CL_RMAX + 1];
-  __shared__ uint32_t warp_sums[32], scan_total;
-  const int tid = threadIdx.x, base = tid * 8, total = rows * nchunk;
-  const int h_i = tid - (LONG_THREADS - 2 * CL_RMAX);
-  float x[8], h;
+  constexpr int PAD = 8;             // halo positions staged on either side
+  constexpr int NV = (R + 3) / 4;    // vectors of neighbours read on either side
+  constexpr int STEP = LONG_THREADS + LONG_THREADS / 8;  // slot(t + LONG_THREADS) - slot(t)
+  static_assert(CL_RMAX <= PAD && LONG_THREADS % 32 == 0, "the halo holds the largest radius");
+  __shared__ __align__(16) uint32_t stage[slots_for(LONG_CHUNK + 2 * PAD)];
+  __shared__ uint32_t warp_sums[LONG_THREADS / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  uint32_t* const put = stage + slot(tid + PAD);
+  const int h_at = tid < PAD ? tid - PAD : LONG_CHUNK + tid - PAD;  // halo position of the first 2 * PAD threads
+  float x[8], h = 0.f;
   uint32_t bound;
-  auto fetch = [&](int w) {
-    const int row = w / nchunk, c0 = (w - row * nchunk) * LONG_CHUNK;
-    const int h_j = h_i < CL_RMAX ? c0 - CL_RMAX + h_i : c0 + LONG_CHUNK + h_i - CL_RMAX;
-    const bool have_h = h_i >= 0 && static_cast<unsigned>(h_j) < static_cast<unsigned>(n);
-    const float* src = vote + static_cast<size_t>(row) * gsum * n;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int j = c0 + tid + LONG_THREADS * u;
-      x[u] = j < n ? __ldg(src + j) : 0.f;
-    }
-    h = have_h ? __ldg(src + h_j) : 0.f;
+  auto fetch = [&](int row, int c0) {
+    const bool have_h = tid < 2 * PAD && static_cast<unsigned>(c0 + h_at) < static_cast<unsigned>(n);
+    const float* src = vote + static_cast<size_t>(row) * gsum * n + c0;
+    const int left = n - c0 - tid;  // positions from this thread's first one to the row's end
     bound = __ldg(meta + static_cast<size_t>(row) * LONG_META + LONG_THRESHOLD);
+    if (n - c0 >= LONG_CHUNK) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = __ldg(src + tid + LONG_THREADS * u);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] = LONG_THREADS * u < left ? __ldg(src + tid + LONG_THREADS * u) : 0.f;
+    }
+    if (tid < 2 * PAD) h = have_h ? __ldg(src + h_at) : 0.f;
     for (int g = 1; g < gsum; ++g) {
       src += n;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int j = c0 + tid + LONG_THREADS * u;
-        if (j < n) x[u] += __ldg(src + j);
-      }
-      if (have_h) h += __ldg(src + h_j);
+      for (int u = 0; u < 8; ++u)
+        if (LONG_THREADS * u < left) x[u] += __ldg(src + tid + LONG_THREADS * u);
+      if (have_h) h += __ldg(src + h_at);
     }
   };
   pdl_wait();
-  int w = blockIdx.x;
-  if (w < total) fetch(w);
+  const int row_step = gridDim.x / nchunk, chunk_step = gridDim.x - row_step * nchunk;
+  int next_row = blockIdx.x / nchunk, next_chunk = blockIdx.x - next_row * nchunk;
+  if (next_row < rows) fetch(next_row, next_chunk * LONG_CHUNK);
 #pragma unroll 1
-  for (; w < total; w += gridDim.x) {
-    const int row = w / nchunk, chunk = w - row * nchunk, c0 = chunk * LONG_CHUNK;
+  while (next_row < rows) {
+    const int row = next_row, chunk = next_chunk;
+    next_row += row_step;
+    next_chunk += chunk_step;
+    if (next_chunk >= nchunk) {
+      next_chunk -= nchunk;
+      ++next_row;
+    }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) stage[slot(tid + LONG_THREADS * u)] = __float_as_uint(x[u]);
-    if (h_i >= 0) halo[h_i >= CL_RMAX][h_i >= CL_RMAX ? h_i - CL_RMAX : h_i] = h;
-    const uint32_t least = bound;
+    for (int u = 0; u < 8; ++u) put[STEP * u] = __float_as_uint(x[u]);
+    if (tid < 2 * PAD) stage[slot(h_at + PAD)] = __float_as_uint(h);
+    const float least = __uint_as_float(bound & 0x7fffffffu);  // (bounds are keys of values from zero on)
     __syncthreads();
-    if (w + static_cast<int>(gridDim.x) < total) fetch(w + gridDim.x);
-    auto at = [&](int t) {
-      return t < 0 ? halo[0][CL_RMAX + t]
-                   : (t >= LONG_CHUNK ? halo[1][t - LONG_CHUNK] : __uint_as_float(stage[slot(t)]));
-    };
-    float a[2 * R + 8], p[8];
+    if (next_row < rows) fetch(next_row, next_chunk * LONG_CHUNK);
+    float v[8 * NV + 8], p[8];
 #pragma unroll
-    for (int i = 0; i < R; ++i) {
-      a[i] = at(base - R + i);
-      a[R + 8 + i] = at(base + 8 + i);
+    for (int q = 0; q < 2 * NV + 2; ++q) {
+      const uint4 y = *reinterpret_cast<const uint4*>(stage + slot(tid * 8 + PAD + 4 * (q - NV)));
+      v[4 * q] = __uint_as_float(y.x);
+      v[4 * q + 1] = __uint_as_float(y.y);
+      v[4 * q + 2] = __uint_as_float(y.z);
+      v[4 * q + 3] = __uint_as_float(y.w);
     }
+    pool8<R, PT>(v + 4 * NV - R, p, r, pool_type, divisor);
+    const int base = chunk * LONG_CHUNK + tid * 8;
+    uint32_t m_in = 0u;
 #pragma unroll
-    for (int q = 0; q < 8; q += 4) {
-      const uint4 v = *reinterpret_cast<const uint4*>(stage + slot(base + q));
-      a[R + q] = __uint_as_float(v.x);
-      a[R + q + 1] = __uint_as_float(v.y);
-      a[R + q + 2] = __uint_as_float(v.z);
-      a[R + q + 3] = __uint_as_float(v.w);
-    }
-    pool8<R, PT>(a, p, r, pool_type, divisor);
-    uint32_t key[8], in = 0u;
+    for (int i = 0; i < 8; ++i) m_in |= static_cast<uint32_t>(p[i] >= least) << i;
+    if (base + 8 > n) m_in &= base < n ? (1u << (n - base)) - 1u : 0u;
+    const uint32_t in = __popc(m_in), of_warp = __reduce_add_sync(0xffffffffu, in);
+    if (lane == 0) warp_sums[warp] = of_warp;
+    __syncthreads();  // (and stage is free)
+    if (of_warp || warp == LONG_THREADS / 32 - 1) {
+      uint32_t to = __reduce_add_sync(0xffffffffu, lane < warp ? warp_sums[lane] : 0u);
+      if (warp == LONG_THREADS / 32 - 1 && lane == 0)
+        meta[static_cast<size_t>(row) * LONG_META + LONG_COUNTS + chunk] = to + of_warp;
+      uint32_t inc = in;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      key[i] = c0 + base + i < n ? float_to_key(p[i]) : 0u;
-      in += key[i] >= least;
-    }
-    uint32_t to = block_scan<LONG_THREADS>(in, warp_sums, &scan_total);  // (two barriers: stage is free)
-    if (in) {
-      uint2* out = list + static_cast<size_t>(w) * cap;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      to += inc - in;
+      uint2* out = list + (static_cast<size_t>(row) * nchunk + chunk) * cap + to;
+      int room = cap - static_cast<int>(to);
 #pragma unroll
       for (int i = 0; i < 8; ++i)
-        if (key[i] >= least) {
-          if (to < static_cast<uint32_t>(cap)) out[to] = make_uint2(key[i], static_cast<uint32_t>(c0 + base + i));
-          ++to;
+        if ((m_in >> i) & 1u) {
+          if (room-- > 0) *out = make_uint2(__float_as_uint(p[i]) | KEY_MIN, static_cast<uint32_t>(base + i));
+          ++out;
         }
     }
-    if (tid == 0) meta[static_cast<size_t>(row) * LONG_META + LONG_COUNTS + chunk] = scan_total;
   }
 }
 
@@ -803,8 +822,9 @@ __global__ void __launch_bounds__(1024) long_finish_kernel(int ksel, int nchunk,
 
   // the list, compacted; slots behind its end are NONE
   uint32_t top = 0u;
+  const int run = static_cast<int>((total + 4095) / 4096) * 4;  // slots a thread owns, up to EPT
 #pragma unroll 8
-  for (int u = 0; u < EPT; ++u) {
+  for (int u = 0; u < run; ++u) {
     const uint32_t e = tid + 1024 * u;
     uint2 kp = make_uint2(NONE, 0u);
     if (e < total) {
@@ -821,10 +841,13 @@ __global__ void __launch_bounds__(1024) long_finish_kernel(int ksel, int nchunk,
   top = __reduce_max_sync(0xffffffffu, top);
   if (lane == 0) atomicMax(&key_max, top);
   __syncthreads();
-  const int base = tid * EPT;
+  const int base = tid * run;
   uint32_t key[EPT];
 #pragma unroll
+  for (int i = 0; i < EPT; ++i) key[i] = NONE;
+#pragma unroll
   for (int i = 0; i < EPT; i += 4) {
+    if (i >= run) break;
     const uint4 v = *reinterpret_cast<const uint4*>(keys_s + slot(base + i));
     key[i] = v.x; key[i + 1] = v.y; key[i + 2] = v.z; key[i + 3] = v.w;
   }
@@ -832,7 +855,7 @@ __global__ void __launch_bounds__(1024) long_finish_kernel(int ksel, int nchunk,
   // until a bin is one key wide or all of it is kept (two rounds as a rule)
   uint32_t lo = m[LONG_THRESHOLD], width = key_max - lo, krem = static_cast<uint32_t>(ksel), all;
   do {
-    all = rank_round(key, rs, lo, width, krem);
+    all = rank_round(key, rs, lo, width, krem, run);
   } while (width > 0u && krem != all);
   const uint32_t T = lo;
   const bool all_eq = krem == all;  // every key from T on is kept
@@ -1058,9 +1081,9 @@ cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int poo
   SelectCall c = {vote, rows, n, gsum, pool_kernel >> 1, pool_type, divisor, ksel, out_idx,
                   vote_is_scratch ? 1 : 0, stream};
   const ClusterShape shape = cluster_shape(rows, n);
-  // The filter's four launches take 26 us and 2.6 us per million votes (within 10 % from 8 rows of
-  // 379968 to 128 of 65536); it is taken where that is clearly less than the rounds of the clusters.
-  const double filter_us = 26.0 + 2.6e-6 * static_cast<double>(rows) * n;
+  // The filter's four launches take 24 us and 1.85 us per million votes (within 5 % from 32 rows of
+  // 262144 to 128 of 131008); it is taken where that is clearly less than the rounds of the clusters.
+  const double filter_us = 24.0 + 1.85e-6 * static_cast<double>(rows) * n;
   const int want = scratch != nullptr && filter_us < 0.9 * shape.us ? long_want(n, ksel) : 0;
   if (want) {
     uint8_t* p = static_cast<uint8_t*>(scratch);
