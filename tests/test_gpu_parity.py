@@ -395,6 +395,23 @@ def test_runs_are_bit_identical():
         assert all(torch.equal(first[i], again[i]) for i in range(3))
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,L,d,W", [(900, 32, 32, 160, 64, 16), (450, 64, 32, 257, 128, 32)])
+def test_more_work_items_than_a_launch_holds(B, Hq, Hkv, L, d, W):
+    # so many short sequences that the scoring kernel's item lists fill: the waves go in several launches
+    g = torch.Generator(device="cuda").manual_seed(L)
+    q = torch.randn(B, Hq, W, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    k = torch.randn(B, Hkv, L, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    v = torch.randn(B, Hkv, L, d, generator=g, device="cuda", dtype=torch.bfloat16)
+    whole = sk.snapkv_compress(q, k, v, 5, sk.POOL_MAX, W + 24)
+    assert sk.snapkv_last_launch_count() > 4
+    for b in (0, 1, B // 3, B // 2, B - 2, B - 1):
+        one = sk.snapkv_compress(q[b:b + 1], k[b:b + 1], v[b:b + 1], 5, sk.POOL_MAX, W + 24)
+        # (another cut of the statistics: votes may differ by an ulp, positions hardly ever)
+        same = (one[2][0] == whole[2][b]).all(dim=1)
+        assert same.float().mean() > 0.9
+        assert torch.equal(one[0][0][same], whole[0][b][same]) and torch.equal(one[1][0][same], whole[1][b][same])
+
+
 def test_compress_from_host_buffers():
     w = synth.WORKLOADS[0]
     data = synth.make_layer(w, 0)
