@@ -198,6 +198,7 @@ bool make_score_plan(int B, int Hq, int Hkv, int L, int d, int W, ScorePlan* pla
   // bounds the work items per phase (the book-keeper's buffers are sized for that)
   if (upw > 128) upw = 128 / p.sub_per_kv * p.sub_per_kv;
   if (upw < p.sub_per_kv) upw = p.sub_per_kv;
+  if (upw > 4096) upw = 4096;  // (thousands of sub-groups per KV head: a CTA's item list holds 192)
   if (upw > units) upw = units;
   // the bigger waves must not leave a single wave where two of the plain size were possible:
   // with one wave the votes start right behind the statistics and wait for the hand-over
