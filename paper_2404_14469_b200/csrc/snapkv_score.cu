@@ -36,9 +36,19 @@ bool encode_tensor_map(CUtensorMap* m, const void* base, int rank, const unsigne
   cuuint64_t d64[5] = {}, s64[5] = {};
   for (int i = 0; i < rank; ++i) d64[i] = dims[i];
   for (int i = 0; i + 1 < rank; ++i) s64[i] = strides_bytes[i];
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), d64, s64, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  auto encode = [&] {
+    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), d64, s64, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = encode();
+  if (r != CUDA_SUCCESS && r != CUDA_ERROR_INVALID_VALUE) {
+    // A driver call needs a context, and a thread gets its device's only with the first runtime call
+    // that touches the device: for a thread that starts with a decode step, this is before any.
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaSetDevice(dev) == cudaSuccess) r = encode();
+  }
+  return r == CUDA_SUCCESS;
 }
 
 int sm_count() {
