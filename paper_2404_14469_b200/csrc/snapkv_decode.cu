@@ -413,20 +413,22 @@ cudaError_t launch_decode_shape(const void* q, const void* ck, const void* cv, i
   if (dev < 0 || dev >= MAX_DEV) return cudaErrorInvalidDevice;
   if (!known[dev].load(std::memory_order_acquire)) {
     std::lock_guard<std::mutex> lock(mu);
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    active[dev][1] = SHAPE::CTAS * sm_count();
-    for (int c = 2; c <= DEC_MAX_CLUSTER; ++c) {
-      cfg.gridDim = dim3(c);
-      attr[0].val.clusterDim.x = c;
-      cfg.numAttrs = 1;
-      if (cudaOccupancyMaxActiveClusters(&active[dev][c], kernel, &cfg) != cudaSuccess) {
-        active[dev][c] = 0;
-        (void)cudaGetLastError();  // a refusal here is an answer, not an error of the call
+    if (!known[dev].load(std::memory_order_relaxed)) {  // (another thread may have done it meanwhile)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+      active[dev][1] = SHAPE::CTAS * sm_count();
+      for (int c = 2; c <= DEC_MAX_CLUSTER; ++c) {
+        cfg.gridDim = dim3(c);
+        attr[0].val.clusterDim.x = c;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&active[dev][c], kernel, &cfg) != cudaSuccess) {
+          active[dev][c] = 0;
+          (void)cudaGetLastError();  // a refusal here is an answer, not an error of the call
+        }
       }
+      known[dev].store(true, std::memory_order_release);
     }
-    known[dev].store(true, std::memory_order_release);
   }
   CUtensorMap tmK, tmV;
   const unsigned long long dims[3] = {static_cast<unsigned long long>(D), static_cast<unsigned long long>(rows),

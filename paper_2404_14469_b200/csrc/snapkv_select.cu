@@ -14,6 +14,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/snapkv.h"
 #include "launch.cuh"
 #include "snapkv_internal.h"
@@ -551,19 +553,20 @@ static __device__ __align__(256) uint32_t g_static_keys[SNAPKV_STATIC_MAX_KEYS];
 namespace snapkv {
 namespace {
 constexpr int MAX_DEVICES = 64;
-uint32_t* g_static_keys_addr[MAX_DEVICES] = {nullptr};
+std::atomic<uint32_t*> g_static_keys_addr[MAX_DEVICES] = {};
 
 // The array's name is only a handle on the host; the device address has to be asked for,
 // once per device, with that device current.
 snapkv_status_t static_keys_address(uint32_t** out) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return SNAPKV_ERR_CUDA;
-  if (g_static_keys_addr[dev] == nullptr) {
+  *out = g_static_keys_addr[dev].load(std::memory_order_relaxed);
+  if (*out == nullptr) {
     void* p = nullptr;
     if (cudaGetSymbolAddress(&p, g_static_keys) != cudaSuccess || p == nullptr) return SNAPKV_ERR_CUDA;
-    g_static_keys_addr[dev] = static_cast<uint32_t*>(p);
+    *out = static_cast<uint32_t*>(p);
+    g_static_keys_addr[dev].store(*out, std::memory_order_relaxed);
   }
-  *out = g_static_keys_addr[dev];
   return SNAPKV_OK;
 }
 }  // namespace
