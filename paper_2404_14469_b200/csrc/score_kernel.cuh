@@ -892,6 +892,15 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       // bit-identical rows without a second hand-over through global memory.  No fence, no counter
       // and no staging copy: a write and a read through L2 are all that lies between the last
       // partial and the first vote.
+      // The slots are read with cp.async, which the PTX memory model counts as a weak access: against
+      // the publishers' relaxed stores it promises nothing.  What the reading relies on is how this
+      // GPU carries it out: `.cg` passes L1 by and reads L2, the point of coherence, where an aligned
+      // 4-byte element is old or new, never a mixture; every element carries its own flag and is
+      // looked at by itself; and each attempt is a new copy (volatile, memory clobber), so an old
+      // element is read again until it is new.  Relaxed loads instead keep within the model, but the
+      // slots on their way are then held in registers: 8 to 16 slots at a time, with or without the
+      // next ones behind them, took 43.9-47 us against 43.5 for a prompt of 13K and 149-155 against
+      // 146.5 for eight sequences of 1353 to 24000 positions.
       // In a ragged batch one CTA per unit folds and leaves the row, a flag of its own as well, in
       // global memory: a fold of 20 partials takes this warp 3-5 us beside the softmax warps, and
       // with a vote item for every two or three tiles the folds would set the pace.
