@@ -242,7 +242,8 @@ snapkv_status_t snapkv_compress_grouped(const void* q_obs, const void* k, const 
  * The whole step (Listing 1) on a batch whose prompts differ in length.  Listing 1 has one
  * q_len for the batch; the sequences are independent of one another (Sec. 4.1), so each is
  * compressed as a single-sequence step of its own length.  Up to 32 of them share each launch when
- * the workspace has room for them all (the more it holds, the fewer launches).
+ * the workspace has room for them all (snapkv_varlen_workspace_size); with less they go through in
+ * as many sets of launches as the workspace makes necessary.
  *   seq_lens       HOST int32 [B]: L_b, W <= L_b <= Lmax.  Sequence b's window is its last W
  *                  positions, its prefix the L_b - W before them.
  *   k, v           as in snapkv_compress_strided (k_strides / v_strides NULL: dense
@@ -261,6 +262,12 @@ snapkv_status_t snapkv_compress_grouped(const void* q_obs, const void* k, const 
  * largest snapkv_workspace_size(1, Hq, Hkv, L_b, ...) over the sequences with L_b > budget);
  * the status block keeps the first error of any sequence.  Each sequence's result is that of snapkv_compress on that sequence alone.
  */
+/* Bytes of scratch with which snapkv_compress_varlen (or snapkv_compress_paged with seq_lens) takes
+ * the fewest launches for these lengths on the current device: one set for every 32 sequences longer
+ * than the budget (fewer where they have gigabytes of keys, or with a pooling kernel above 15).
+ * seq_lens: HOST int32 [B].  0 if the arguments are not acceptable.  Enqueues nothing. */
+size_t snapkv_varlen_workspace_size(const int32_t* seq_lens, int B, int Hq, int Hkv, int d, int W,
+                                    int pool_kernel, int pool_type, int budget);
 snapkv_status_t snapkv_compress_varlen(const void* q_obs, const void* k, const void* v,
                                        const int64_t* k_strides, const int64_t* v_strides,
                                        const int64_t* k_seq_offsets, const int64_t* v_seq_offsets,

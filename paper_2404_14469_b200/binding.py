@@ -31,7 +31,7 @@ SYMBOLS = [
     "snapkv_host_staging_size", "snapkv_compress_host", "snapkv_device_status",
     "snapkv_last_launch_count", "snapkv_pool_topk_static",
     "snapkv_window_scores_lse", "snapkv_compress_lse", "snapkv_compress_strided",
-    "snapkv_compress_grouped", "snapkv_compress_varlen",
+    "snapkv_compress_grouped", "snapkv_compress_varlen", "snapkv_varlen_workspace_size",
     "snapkv_hit_counts", "snapkv_decode_workspace_size", "snapkv_decode_attention",
     "snapkv_set_wait_limit_ns", "snapkv_selftest_stalled_scores", "snapkv_schedule_items",
     "snapkv_compress_paged",
@@ -39,7 +39,7 @@ SYMBOLS = [
 ]
 
 # entry points for the extension alone (csrc/snapkv_binding.h)
-BINDING_SYMBOLS = ["snapkv_binding_ragged_workspace", "snapkv_binding_varlen", "snapkv_binding_paged"]
+BINDING_SYMBOLS = ["snapkv_binding_varlen", "snapkv_binding_paged"]
 
 _lib = None
 _native = None
@@ -83,6 +83,8 @@ def lib() -> ctypes.CDLL:
     L.snapkv_compress_varlen.restype = c_int
     L.snapkv_compress_varlen.argtypes = ([c_vp] * 3 + [p64] * 4 + [p32, c_vp] + [c_int] * 9 + [c_vp] * 3
                                          + [c_vp, c_sz, c_vp])
+    L.snapkv_varlen_workspace_size.restype = c_sz
+    L.snapkv_varlen_workspace_size.argtypes = [p32] + [c_int] * 8
     L.snapkv_compress_paged.restype = c_int
     L.snapkv_compress_paged.argtypes = ([c_vp] * 3 + [p64] * 2 + [c_vp] + [c_int] * 3 + [p32, c_vp]
                                         + [c_int] * 9 + [c_vp] * 3 + [c_vp, c_sz, c_vp])
@@ -217,6 +219,12 @@ def snapkv_compress(q_obs, k, v, pool_kernel: int, pool_type: int, budget: int,
                                                 out_idx, workspace, lse_obs, grouped)
 
 
+def snapkv_varlen_workspace_size(seq_lens, Hq, Hkv, d, W, pool_kernel, pool_type, budget) -> int:
+    """Bytes of scratch with which a batch of these lengths takes the fewest launches."""
+    lens = (ctypes.c_int32 * len(seq_lens))(*seq_lens)
+    return lib().snapkv_varlen_workspace_size(lens, len(seq_lens), Hq, Hkv, d, W, pool_kernel, pool_type, budget)
+
+
 def snapkv_compress_varlen(q_obs, k, v, seq_lens, pool_kernel: int, pool_type: int, budget: int,
                            cu_seqlens=None, lse_obs=None, workspace=None):
     """Batch of prompts of different lengths.  seq_lens: list of B lengths.
@@ -226,6 +234,11 @@ def snapkv_compress_varlen(q_obs, k, v, seq_lens, pool_kernel: int, pool_type: i
     [total_tokens, Hkv, d] tensor.  Returns (out_k, out_v [B, Hq, budget, d] zero-filled,
     out_idx [B, Hq, budget - W] filled with -1, workspace); a sequence with budget >= its
     length fills only its first rows.
+
+    The returned workspace may be handed to the next call.  A workspace that a call has allocated is
+    replaced by a larger one when the batch would need more launches with it; one of the caller's own
+    is used as it is if it holds the largest single sequence (snapkv_varlen_workspace_size says
+    what the whole batch needs).
     """
     return (_native or _load_native()).varlen(q_obs, k, v, seq_lens, pool_kernel, pool_type, budget, cu_seqlens,
                                               lse_obs, workspace)

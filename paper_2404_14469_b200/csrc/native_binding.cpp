@@ -34,7 +34,7 @@ struct Library {
   decltype(&snapkv_compress_lse) compress_lse;
   decltype(&snapkv_compress_strided) compress_strided;
   decltype(&snapkv_compress_grouped) compress_grouped;
-  decltype(&snapkv_binding_ragged_workspace) binding_ragged_workspace;
+  decltype(&snapkv_varlen_workspace_size) varlen_workspace_size;
   decltype(&snapkv_binding_varlen) binding_varlen;
   decltype(&snapkv_binding_paged) binding_paged;
   decltype(&snapkv_decode_workspace_size) decode_workspace_size;
@@ -87,9 +87,13 @@ void check(int code, const char* what) {
   if (code != SNAPKV_OK) throw Fail{std::string(what) + " failed: " + g_lib.status_string(code)};
 }
 
+// Attribute of the workspaces that were allocated here, as opposed to the caller's own.
+constexpr const char* ALLOCATED = "snapkv_allocated";
+
 // A tensor the caller may have passed in: its own object is handed back, else a new one.
 struct Out {
   PyObject* given = nullptr;
+  bool workspace = false;
   at::Tensor t;
   void* data() const { return t.data_ptr(); }
   PyObject* release() {
@@ -97,7 +101,12 @@ struct Out {
       Py_INCREF(given);
       return given;
     }
-    return THPVariable_Wrap(t);
+    PyObject* o = THPVariable_Wrap(t);
+    if (o && workspace && PyObject_SetAttrString(o, ALLOCATED, Py_True) != 0) {
+      Py_DECREF(o);
+      return nullptr;
+    }
+    return o;
   }
 };
 
@@ -115,6 +124,7 @@ Out workspace_for(PyObject* o, size_t need, const at::Device& dev) {
   Out w = given_or(o, "workspace");
   if (!w.given || static_cast<size_t>(w.t.numel()) < need) {
     w.given = nullptr;
+    w.workspace = true;
     w.t = empty({static_cast<int64_t>(need > 256 ? need : 256)}, at::kByte, dev);
   }
   return w;
@@ -228,21 +238,28 @@ PyObject* py_compress(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
   });
 }
 
-// The caller's workspace if it meets the requirement (the largest single sequence), else a new one
-// with which the whole batch goes through in one set of launches.
+// The workspace of a ragged batch.  The call requires room for its largest single sequence, and with
+// no more it takes the sequences one after the other; with `want` all go through in one set of launches.
+// A caller's own workspace is used as it is when it meets the requirement.  One that an earlier call
+// allocated, for a smaller batch perhaps, gives way to a larger one where it would cost launches.
 Out ragged_workspace(PyObject* given, const std::vector<int32_t>& lens, int Hq, int Hkv, int d, int W, int pk, int pt,
                      int budget, const at::Device& dev) {
+  const size_t want =
+      g_lib.varlen_workspace_size(lens.data(), static_cast<int>(lens.size()), Hq, Hkv, d, W, pk, pt, budget);
   if (given != Py_None) {
-    size_t need = 256;
-    for (int32_t x : lens)
-      if (x > budget) {
-        const size_t one = g_lib.workspace_size(1, Hq, Hkv, x, d, W, pk, pt, budget);
-        if (one > need) need = one;
-      }
-    if (static_cast<size_t>(tensor(given, "workspace").numel()) >= need) return workspace_for(given, need, dev);
+    const size_t have = static_cast<size_t>(tensor(given, "workspace").numel());
+    if (have >= want) return workspace_for(given, 0, dev);
+    if (!PyObject_HasAttrString(given, ALLOCATED)) {
+      size_t least = 256;
+      for (int32_t x : lens)
+        if (x > budget) {
+          const size_t one = g_lib.workspace_size(1, Hq, Hkv, x, d, W, pk, pt, budget);
+          if (one > least) least = one;
+        }
+      if (have >= least) return workspace_for(given, least, dev);
+    }
   }
-  const int B = static_cast<int>(lens.size());
-  return workspace_for(Py_None, g_lib.binding_ragged_workspace(lens.data(), B, Hq, Hkv, d, W, pk, pt, budget), dev);
+  return workspace_for(Py_None, want, dev);
 }
 
 struct RaggedOut {
@@ -420,7 +437,7 @@ PyObject* py_bind(PyObject*, PyObject* const* a, Py_ssize_t nargs) {
     SNAPKV_BIND(compress_lse);
     SNAPKV_BIND(compress_strided);
     SNAPKV_BIND(compress_grouped);
-    SNAPKV_BIND(binding_ragged_workspace);
+    SNAPKV_BIND(varlen_workspace_size);
     SNAPKV_BIND(binding_varlen);
     SNAPKV_BIND(binding_paged);
     SNAPKV_BIND(decode_workspace_size);

@@ -448,6 +448,19 @@ static int ragged_group(const int32_t* lens, int B, int b, int Hq, int Hkv, int 
   return b;
 }
 
+// Whether sequences of these lengths can share launches at all (one too long, or a pooling radius that
+// the cluster kernel does not take, and each goes through by itself).
+static bool ragged_shares_launches(const int32_t* lens, int B, int Hq, int Hkv, int d, int W, int pool_kernel,
+                                   int pool_type, int budget) {
+  int longest = 0;
+  for (int b = 0; b < B; ++b)
+    if (lens[b] > longest) longest = lens[b];
+  if (Hq > 65535 || !ragged_select_applies(longest - W > 0 ? longest - W : 1, pool_kernel, pool_type)) return false;
+  ScorePlan p;  // the longest sequence has the most waves
+  return longest <= budget ||
+         (make_score_plan(1, Hq, Hkv, longest, d, W, &p) && p.nwaves <= most_waves_per_launch(p.units));
+}
+
 struct RaggedCall {
   const void *q_obs, *k, *v;
   KVStrides ks, vs;
@@ -485,16 +498,8 @@ static snapkv_status_t ragged_check(const RaggedCall& c, int Lmax) {
 static snapkv_status_t ragged_impl(const RaggedCall& c) {
   const size_t head_rows = static_cast<size_t>(c.Hq) * c.budget * c.d * 2;  // bytes of one sequence's out_k
   const bool have_ws = workspace_ok(c.workspace, c.workspace_bytes, STATUS_BYTES);
-  int longest = 0;
-  for (int b = 0; b < c.B; ++b)
-    if (c.lens[b] > longest) longest = c.lens[b];
-  // the longest sequence has the most waves
-  ScorePlan p;
-  const bool shares_launches = longest <= c.budget || (make_score_plan(1, c.Hq, c.Hkv, longest, c.d, c.W, &p) &&
-                                                       p.nwaves <= most_waves_per_launch(p.units));
   int launches = 0;
-  if (shares_launches && c.out_idx && c.Hq <= 65535 &&
-      ragged_select_applies(longest - c.W > 0 ? longest - c.W : 1, c.pool_kernel, c.pool_type)) {
+  if (c.out_idx && ragged_shares_launches(c.lens, c.B, c.Hq, c.Hkv, c.d, c.W, c.pool_kernel, c.pool_type, c.budget)) {
     uint8_t* ws = static_cast<uint8_t*>(c.workspace);
     bool first = true;  // the first group's launches clear the status block, later ones leave it
     for (int b = 0; b < c.B;) {
@@ -562,18 +567,21 @@ static snapkv_status_t ragged_impl(const RaggedCall& c) {
   return SNAPKV_OK;
 }
 
-size_t snapkv_binding_ragged_workspace(const int32_t* lens, int B, int Hq, int Hkv, int d, int W, int pool_kernel,
-                                       int pool_type, int budget) {
-  size_t need = 0;
+size_t snapkv_varlen_workspace_size(const int32_t* seq_lens, int B, int Hq, int Hkv, int d, int W, int pool_kernel,
+                                    int pool_type, int budget) {
+  if (!seq_lens || B < 1 || check_pool(pool_kernel, pool_type) != SNAPKV_OK || budget <= W) return 0;
+  size_t need = STATUS_BYTES;
   for (int b = 0; b < B; ++b) {
-    if (lens[b] <= budget) continue;
-    const size_t one = snapkv_workspace_size(1, Hq, Hkv, lens[b], d, W, pool_kernel, pool_type, budget);
+    if (check_common(1, Hq, Hkv, seq_lens[b], d, W) != SNAPKV_OK) return 0;
+    if (seq_lens[b] <= budget) continue;
+    const size_t one = snapkv_workspace_size(1, Hq, Hkv, seq_lens[b], d, W, pool_kernel, pool_type, budget);
     if (one == 0) return 0;
     if (one > need) need = one;
   }
+  if (!ragged_shares_launches(seq_lens, B, Hq, Hkv, d, W, pool_kernel, pool_type, budget)) return need;
   for (int b = 0; b < B;) {
     RaggedBatch rb;
-    b = ragged_group(lens, B, b, Hq, Hkv, d, W, budget, ~static_cast<size_t>(0), &rb);
+    b = ragged_group(seq_lens, B, b, Hq, Hkv, d, W, budget, ~static_cast<size_t>(0), &rb);
     if (rb.count == 0) break;
     if (rb.total > need) need = rb.total;
   }

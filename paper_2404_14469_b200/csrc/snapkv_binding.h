@@ -12,10 +12,6 @@
 extern "C" {
 #endif
 
-/* Workspace with which a ragged call needs the fewest launches (at least what it requires); 0 if
- * the arguments are not acceptable or nothing needs scratch. */
-size_t snapkv_binding_ragged_workspace(const int32_t* lens, int B, int Hq, int Hkv, int d, int W, int pool_kernel,
-                                       int pool_type, int budget);
 snapkv_status_t snapkv_binding_varlen(const void* q_obs, const void* k, const void* v, const int64_t* k_strides,
                                       const int64_t* v_strides, const int64_t* k_seq_offsets,
                                       const int64_t* v_seq_offsets, const int32_t* seq_lens, const float* lse_obs,

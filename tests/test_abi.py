@@ -195,3 +195,21 @@ def test_product_package_does_not_import_the_oracle():
             elif f.endswith((".cu", ".cuh", ".h")):
                 assert "oracle" not in open(os.path.join(dirpath, f)).read(), f
     assert "paper_2404_14469_b200" not in open(os.path.join(ROOT, "oracle", "snapkv_oracle.py")).read()
+
+
+def test_varlen_workspace_size(L):
+    size = sk.snapkv_varlen_workspace_size
+    one = lambda x: sk.snapkv_workspace_size(1, 8, 2, x, 128, 32, 7, 0, 256)
+    assert size([3000], 8, 2, 128, 32, 7, 0, 256) >= one(3000)
+    # every further sequence beyond the budget takes its votes' room, one that is copied through none
+    three, four = size([3000, 900, 2000], 8, 2, 128, 32, 7, 0, 256), size([3000, 900, 2000, 700], 8, 2, 128, 32, 7, 0, 256)
+    assert four - three >= 8 * (700 - 32) * 4 and three > max(one(3000), one(2000))
+    assert size([3000, 900, 2000, 256], 8, 2, 128, 32, 7, 0, 256) == three
+    # more than 32 share launches in groups of 32: the largest group counts
+    assert size([900] * 32 + [500], 8, 2, 128, 32, 7, 0, 256) == size([900] * 32, 8, 2, 128, 32, 7, 0, 256)
+    assert size([100, 256], 8, 2, 128, 32, 7, 0, 256) == 256          # the status block alone
+    for bad in [([31, 900], 8, 2, 128, 32, 7, 0, 256), ([900], 8, 3, 128, 32, 7, 0, 256), ([900], 8, 2, 96, 32, 7, 0, 256),
+                ([900], 8, 2, 128, 32, 6, 0, 256), ([900], 8, 2, 128, 32, 7, 2, 256), ([900], 8, 2, 128, 32, 7, 0, 32),
+                ([], 8, 2, 128, 32, 7, 0, 256)]:
+        assert size(*bad) == 0, bad
+    assert L.snapkv_varlen_workspace_size(None, 1, 8, 2, 128, 32, 7, 0, 256) == 0

@@ -148,3 +148,31 @@ def test_ragged_batch_equals_the_calls_one_by_one(lens, Hq, Hkv, d, W, kernel, p
             assert torch.equal(out_idx[b, :, :rows - W], oi[0]) and bool((out_idx[b, :, rows - W:] == -1).all())
             for got, want in ((out_k, ok), (out_v, ov)):
                 assert torch.equal(got[b, :, :rows], want[0]) and not bool(got[b, :, rows:].any())
+
+
+def test_a_workspace_from_a_smaller_batch_does_not_cost_launches():
+    Hq, Hkv, d, W, kernel, budget = 4, 2, 128, 32, 5, 200
+    g = torch.Generator(device="cuda").manual_seed(9)
+    k = torch.randn(16, Hkv, 1500, d, generator=g, device="cuda").to(torch.bfloat16)
+    q = torch.randn(16, Hq, W, d, generator=g, device="cuda").to(torch.bfloat16)
+    small, large = [900, 1500, 640], [300 + 80 * i for i in range(16)]
+
+    def call(lens, ws):
+        out = sk.snapkv_compress_varlen(q[:len(lens)], k[:len(lens)], k[:len(lens)], lens, kernel, sk.POOL_MAX, budget,
+                                        workspace=ws)
+        assert sk.snapkv_device_status(out[3]) == (sk.OK, 0)
+        return out, sk.snapkv_last_launch_count()
+
+    want, fewest = call(large, None)
+    (_, _, _, ws), _ = call(small, None)
+    got, launches = call(large, ws)                       # handed on, as a serving loop does
+    assert launches == fewest and all(torch.equal(x, y) for x, y in zip(got[:3], want[:3]))
+    again, launches = call(small, got[3])                 # and kept from then on
+    assert again[3] is got[3] and launches == fewest
+    # a workspace of the caller's own is used as it is: of the size the library names, one set of launches
+    size = sk.snapkv_varlen_workspace_size(large, Hq, Hkv, d, W, kernel, sk.POOL_MAX, budget)
+    for nbytes, sets in ((size, 1), (size - 256, 2)):
+        own = torch.full((nbytes,), 0xFF, dtype=torch.uint8, device="cuda")
+        got, launches = call(large, own)
+        assert got[3] is own and all(torch.equal(x, y) for x, y in zip(got[:3], want[:3]))
+        assert (launches - fewest) // 3 == sets - 1       # preparation, scores, selection per set; one gather
