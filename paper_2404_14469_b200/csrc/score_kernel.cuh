@@ -60,7 +60,6 @@ constexpr int EPI_WARPS = 8;           // softmax warps per set (two warpgroups)
 // Warps: 0 producer, 1 MMA issuer, 2-9 softmax set 0, 10 publisher, 11 lse fetcher and, in
 // split mode, 12-19 softmax set 1.
 constexpr int threads_for(bool split) { return split ? 640 : 384; }
-constexpr int WAVE_LAG = 2;           // waves that the statistics run ahead of the votes
 constexpr long long WAVE_BYTES = 64ll << 20;
 constexpr int RAGGED_AHEAD = 64;      // tiles per block, the same for the sequences of a ragged batch
 constexpr int MAX_RECORDS = 192;      // work items of a CTA that one launch can hold
@@ -78,7 +77,6 @@ struct ScoreArgs {
   int per;                  // most work items of a CTA in one phase
   int T1, T2;               // tiles per unit in the statistics / vote pass
   int maxseg;               // partial slots per unit
-  int pipelined;            // how many waves the statistics run ahead of the votes (>= 1)
   int mask_n;               // window row i sees keys j <= mask_n + i (n, or n minus a shard's first position)
   int stats_only;           // 1: statistics pass alone (a shard's partial log-sum-exp), no votes
   int votes_only;           // 1: lse2 and the counters are already set, no statistics pass
@@ -296,13 +294,12 @@ struct Phase {
   int seq, wave, vote, ord;
 };
 
-// Phase p of the launch.  Statistics run `lag` waves ahead of votes: S(0) .. S(lag-1) V(0) S(lag)
-// V(1) ...; lag = 1 is the plain order S(0) V(0) S(1) V(1) ...
+// Phase p of the launch.  Statistics run WAVE_LAG waves ahead of votes: S(0) S(1) V(0) S(2) V(1) ...
 __host__ __device__ __forceinline__ Phase phase_at(const ScoreArgs& a, NotRagged, int, int p) {
   int s = a.votes_only ? a.nwaves : 0, v = 0;
   Phase ph = {0, 0, 0, 0};
   for (int i = 0; i <= p; ++i) {
-    ph.vote = !(s < a.nwaves && (a.stats_only || s - v < a.pipelined));
+    ph.vote = !(s < a.nwaves && (a.stats_only || s - v < WAVE_LAG));
     ph.ord = ph.vote ? v++ : s++;
   }
   ph.wave = a.wave0 + ph.ord;
@@ -323,7 +320,7 @@ __host__ __device__ __forceinline__ int tiles_before(const ScoreArgs&, NotRagged
 
 // The same for a ragged batch.  Each sequence is cut as a call of its own would cut it (the same
 // shares, partials and order of additions, so its results do not depend on the batch), and the
-// waves of the sequences follow one another with the statistics at least `lag` waves and
+// waves of the sequences follow one another with the statistics at least WAVE_LAG waves and
 // RAGGED_AHEAD tiles per block ahead: the hand-over of a wave's statistics takes some microseconds,
 // the tiles of a short sequence less than one.  (Waiting costs more than reading the keys again
 // from HBM: eight sequences of 822 to 24000 positions took 175 us with 10 tiles, 155 with 16,
@@ -335,7 +332,7 @@ __device__ __forceinline__ Phase phase_at(const ScoreArgs& a, const RaggedSeqs<M
   int s_seq = a.votes_only ? rs.nseq : 0, s_wave = 0, v_seq = 0, v_wave = 0, s_ord = 0, v_ord = 0, tiles = 0;
   Phase ph = {0, 0, 0, 0};
   for (int i = 0; i <= p; ++i) {
-    ph.vote = !(s_seq < rs.nseq && (s_ord - v_ord < a.pipelined || tiles < RAGGED_AHEAD * G));
+    ph.vote = !(s_seq < rs.nseq && (s_ord - v_ord < WAVE_LAG || tiles < RAGGED_AHEAD * G));
     ph.seq = ph.vote ? v_seq : s_seq;
     ph.wave = ph.vote ? v_wave : s_wave;
     ph.ord = ph.vote ? v_ord++ : s_ord++;
@@ -498,11 +495,6 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       }
     }
   };
-  // tile visited at step k of an item: ascending, except that the sequential schedule
-  // sweeps the vote pass backwards (the keys read last are the likeliest to be in L2)
-  auto tile_of = [&](const Item& it, int k) {
-    return (it.vote && a.pipelined == 1) ? (it.t1 - 1 - k) : (it.t0 + k);
-  };
   auto first_head = [&](const Item& it, int* ukv) {
     *ukv = it.unit / a.sub_per_kv;
     const int sub = it.unit - *ukv * a.sub_per_kv;
@@ -548,13 +540,12 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         }
         ++nitem;
         const int kb = ukv / a.Hkv, kh = ukv - kb * a.Hkv;  // the K map is (d, L, Hkv, B); ragged: B = 1
-        const int nt = it.t1 - it.t0;
-        for (int k = 0; k < nt; ++k, ++git) {
+        for (int t = it.t0; t < it.t1; ++t, ++git) {
           const int s = git % STAGES;
           const uint32_t ph = (git / STAGES) & 1;
           if (!mbar_wait_thread(bar_empty(s), ph ^ 1, abort_s, WAIT_PRODUCER_EMPTY)) return false;
           mbar_expect_tx(bar_full(s), SM::STAGE_BYTES);
-          int key0 = tile_of(it, k) * TILE_KEYS;
+          int key0 = t * TILE_KEYS;
           int kslab = RAGGED ? 0 : kb;  // outermost coordinate of the K map: the batch, or the page of the pool
           if (a.page_table) {
             // a page holds a whole number of tiles: the tile's 128 keys sit in one page
@@ -671,7 +662,6 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     const uint32_t te_arrivals = SPLIT ? 1 : 2;          // the barrier expects 8 per tile
     int git = 0, nstat = 0, nvote = 0;
     each_item([&](const Item& it) {
-      const int nt = it.t1 - it.t0;
       int ukv;
       const int hq0 = first_head(it, &ukv);
       int flip = 0;
@@ -693,13 +683,13 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         // ---------------------------------------------------------- statistics
         float m2 = -INFINITY;  // running max, log2 domain
         float l = 0.f;         // running sum of exp2(x - m2)
-        for (int k = 0; k < nt; ++k, ++git) {
+        for (int t = it.t0; t < it.t1; ++t, ++git) {
           if (((git ^ flip) & 1) != (SPLIT ? set : wg)) continue;
           const int buf = git & (NBUF - 1);
           const uint32_t ub = (git / NBUF) & 1;
           if (!mbar_wait_warp(bar_tf(buf), ub, abort_s, WAIT_EPI_TMEM_FULL)) return false;
           tc_fence_after();
-          const int key0 = tile_of(it, k) * TILE_KEYS;
+          const int key0 = t * TILE_KEYS;
           // this thread's slice of its window row: CPT key columns
           float v[VCH][32];
           const uint32_t taddr = tmem_base + lane_sel + buf * 128 + rep * NPAD + coff;
@@ -758,13 +748,13 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       const int lb = nvote % NLB;
       if (!mbar_wait_warp(bar_lf(lb), (nvote / NLB) & 1, abort_s, WAIT_LSE_FULL)) return false;
       const float* lse_b = lse_s + lb * MAX_COLS;
-      for (int k = 0; k < nt; ++k, ++git) {
+      for (int t = it.t0; t < it.t1; ++t, ++git) {
         if ((git & 1) != (SPLIT ? set : wg)) continue;
         const int buf = git & (NBUF - 1);
         const uint32_t ub = (git / NBUF) & 1;
         if (!mbar_wait_warp(bar_tf(buf), ub, abort_s, WAIT_EPI_TMEM_FULL)) return false;
         tc_fence_after();
-        const int j = tile_of(it, k) * TILE_KEYS + 32 * q + lane;
+        const int j = t * TILE_KEYS + 32 * q + lane;
         const uint32_t taddr = tmem_base + lane_sel + buf * 128 + coff;
         float g16[VCH * 2];
         float v[SPLIT ? 1 : VCH][32];
@@ -1018,8 +1008,10 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     bool go = publisher ? !a.votes_only : !a.stats_only;
     const bool folds = RAGGED && !publisher && !a.votes_only;
     // In a ragged batch the fetcher folds the next wave's rows, where this CTA holds the unit's first
-    // slot, before it fetches those of a wave (the statistics are at least two waves ahead), so that
-    // nobody waits for a fold.
+    // slot, before it fetches those of a wave, so that nobody waits for a fold.  With a lag of one
+    // wave this would never end: the next wave's statistics would stand behind the votes that wait
+    // for this very fetch.
+    static_assert(!RAGGED || WAVE_LAG >= 2, "a wave's statistics come before the votes of the wave before it");
     for (int w = folds ? -1 : 0; w < waves && go; ++w) {
       for (int m = 0; m < a.per && go && folds && w + 1 < waves; ++m) {
         const Item it = item_at(2 * (w + 1), m);

@@ -897,7 +897,7 @@ int snapkv_schedule_items(int B, int Hq, int Hkv, int L, int d, int W, int votes
     out_plan[3] = p.tiles_stats;
     out_plan[4] = p.tiles_vote;
     out_plan[5] = p.maxseg;
-    out_plan[6] = p.pipelined;
+    out_plan[6] = WAVE_LAG;
     out_plan[7] = p.ncols;
   }
   return list_schedule_items(p, L, W, Hkv, votes_only ? 1 : 0, grid, cta, out_items, max_items);

@@ -16,6 +16,7 @@ constexpr int SM_COUNT_HINT = 148;  // B200
 constexpr int MAX_GRID = 192;       // the scoring kernel runs one CTA per SM, at most this many
 
 constexpr uint32_t NO_PARTIAL = 0xffffffffu;  // a partial-statistics slot that has not been written
+constexpr int WAVE_LAG = 2;         // waves that the scoring kernel's statistics run ahead of the votes
 constexpr int RAGGED_MAX = 32;      // sequences of a ragged batch that share a launch
 
 // Codes stored in the workspace status block's second word when a wait gives up.
@@ -49,7 +50,6 @@ struct ScorePlan {
   int units_per_wave;
   int nwaves;
   int maxseg;       // partial-statistics slots per unit
-  int pipelined;    // how many waves the statistics pass runs ahead of the vote pass (>= 1)
 };
 
 // Where a K or V tensor's rows are: element strides between consecutive batches, KV heads and

@@ -141,7 +141,6 @@ score::ScoreArgs score_args(const ScorePlan& plan, int L, int W, int Hkv, int vo
   a.T1 = plan.tiles_stats;
   a.T2 = plan.tiles_vote;
   a.maxseg = plan.maxseg;
-  a.pipelined = plan.pipelined;
   a.votes_only = votes_only;
   if (votes_only) {  // nothing couples the units any more: one phase over all of them (over 4096 at most)
     a.upw = plan.units < 4096 ? plan.units : 4096;
@@ -201,7 +200,6 @@ bool make_score_plan(int B, int Hq, int Hkv, int L, int d, int W, ScorePlan* pla
   long long kv_per_wave = wave_bytes / kbytes;
   // units bigger than a wave run one per wave: their second sweep comes from HBM, but the
   // statistics of the next unit still hide the hand-over between the two passes
-  p.pipelined = score::WAVE_LAG;
   if (kv_per_wave < 1) kv_per_wave = 1;
   long long upw = kv_per_wave * p.sub_per_kv;
   // at most 128 units per wave: a CTA's share of a phase then spans few units, which
