@@ -453,8 +453,8 @@ int snapkv_schedule_items(int B, int Hq, int Hkv, int L, int d, int W, int votes
 unsigned long long snapkv_set_wait_limit_ns(unsigned long long limit_ns);
 
 /*
- * Self-test of the time-out path (no counterpart in the paper).  Same arguments as
- * snapkv_window_scores, but only the vote sweep is launched and nothing ever supplies the
+ * Self-test of the time-out path (no counterpart in the paper), here of the wait for supplied
+ * normalisers.  Same arguments as snapkv_window_scores, but only the vote sweep is launched and nothing ever supplies the
  * softmax statistics it waits for: every block's wait runs into the limit, the blocks drain
  * their copies, release tensor memory and return; out_vote is left unwritten.  Afterwards
  * snapkv_device_status(workspace) reports SNAPKV_ERR_TIMEOUT with detail 7 (the wait for a
@@ -467,6 +467,19 @@ snapkv_status_t snapkv_selftest_stalled_scores(const void* q_obs, const void* k,
                                                float* out_vote,
                                                void* workspace, size_t workspace_bytes,
                                                void* stream);
+
+/*
+ * Self-test of the waits between the two sweeps (no counterpart in the paper).  Both sweeps are
+ * launched as snapkv_compress launches them on a dense cache (seq_lens NULL) or, with HOST int32 [B]
+ * lengths in (W, L], as snapkv_compress_varlen does (B <= 32), the votes going to the workspace; but
+ * no block publishes its share of the softmax statistics, so every wait for one runs into the limit.
+ * The votes are left unwritten, and snapkv_device_status(workspace) reports SNAPKV_ERR_TIMEOUT with
+ * detail 7, as after snapkv_selftest_stalled_scores.  Workspace: snapkv_workspace_size or
+ * snapkv_varlen_workspace_size with budget W + 1.  Lower the limit first and restore it afterwards.
+ */
+snapkv_status_t snapkv_selftest_withheld_partials(const void* q_obs, const void* k, const int32_t* seq_lens,
+                                                  int B, int Hq, int Hkv, int L, int d, int W,
+                                                  void* workspace, size_t workspace_bytes, void* stream);
 
 /* Number of kernel launches the last successful snapkv_compress /
  * snapkv_window_scores call of this thread enqueued (for accounting in benchmarks).

@@ -34,6 +34,7 @@ SYMBOLS = [
     "snapkv_compress_grouped", "snapkv_compress_varlen", "snapkv_varlen_workspace_size",
     "snapkv_hit_counts", "snapkv_decode_workspace_size", "snapkv_decode_attention",
     "snapkv_set_wait_limit_ns", "snapkv_selftest_stalled_scores", "snapkv_schedule_items",
+    "snapkv_selftest_withheld_partials",
     "snapkv_compress_paged",
     "snapkv_shard_lse", "snapkv_lse_merge", "snapkv_shard_votes", "snapkv_gather_range",
 ]
@@ -125,6 +126,8 @@ def lib() -> ctypes.CDLL:
     L.snapkv_set_wait_limit_ns.argtypes = [ctypes.c_ulonglong]
     L.snapkv_selftest_stalled_scores.restype = c_int
     L.snapkv_selftest_stalled_scores.argtypes = L.snapkv_window_scores.argtypes
+    L.snapkv_selftest_withheld_partials.restype = c_int
+    L.snapkv_selftest_withheld_partials.argtypes = [c_vp, c_vp, p32] + [c_int] * 6 + [c_vp, c_sz, c_vp]
     _lib = L
     return L
 
@@ -400,6 +403,17 @@ def snapkv_selftest_stalled_scores(q_obs, k, out_vote=None, workspace=None):
                                              workspace.numel(), _stream_ptr())
     _check(code, "snapkv_selftest_stalled_scores")
     return out_vote, workspace
+
+
+def snapkv_selftest_withheld_partials(q_obs, k, workspace, seq_lens=None):
+    """Launches both sweeps with statistics that are never published (time-out self-test), for one
+    length or, with seq_lens, as a ragged batch.  The votes are in the last bytes of the workspace."""
+    _dev_bf16(q_obs, "q_obs"), _dev_bf16(k, "k")
+    B, Hq, Hkv, L, d, W = _shapes(q_obs, k)
+    lens = None if seq_lens is None else (ctypes.c_int32 * B)(*seq_lens)
+    code = lib().snapkv_selftest_withheld_partials(q_obs.data_ptr(), k.data_ptr(), lens, B, Hq, Hkv, L, d, W,
+                                                   workspace.data_ptr(), workspace.numel(), _stream_ptr())
+    _check(code, "snapkv_selftest_withheld_partials")
 
 
 def snapkv_pool_topk(vote, pool_kernel: int, pool_type: int, ksel: int, out_idx=None,

@@ -80,6 +80,7 @@ struct ScoreArgs {
   int mask_n;               // window row i sees keys j <= mask_n + i (n, or n minus a shard's first position)
   int stats_only;           // 1: statistics pass alone (a shard's partial log-sum-exp), no votes
   int votes_only;           // 1: lse2 and the counters are already set, no statistics pass
+  int withhold;             // 1: nothing is published (self-test of the waits for it)
   unsigned long long wait_ns;  // time limit of every device-side wait
   const int32_t* page_table;   // paged K: [batch][pages_per_seq] page numbers, else nullptr
   int pages_per_seq, page_size;
@@ -863,8 +864,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
             }
           // log2 of this CTA's share of the row's softmax normaliser (-inf if it saw no key)
           const float part = M + log2f(S);
-          st_relaxed(slots_of(it) + static_cast<size_t>(it.slot) * MAX_COLS + c,
-                     __float_as_uint(part) == NO_PARTIAL ? __uint_as_float(0x7fffffffu) : part);
+          if (!a.withhold)
+            st_relaxed(slots_of(it) + static_cast<size_t>(it.slot) * MAX_COLS + c,
+                       __float_as_uint(part) == NO_PARTIAL ? __uint_as_float(0x7fffffffu) : part);
         }
         __syncwarp();  // every lane is done with the buffer
         if (lane == 0) {

@@ -939,6 +939,43 @@ snapkv_status_t snapkv_selftest_stalled_scores(const void* q_obs, const void* k,
   return SNAPKV_OK;
 }
 
+snapkv_status_t snapkv_selftest_withheld_partials(const void* q_obs, const void* k, const int32_t* seq_lens, int B,
+                                                  int Hq, int Hkv, int L, int d, int W, void* workspace,
+                                                  size_t workspace_bytes, void* stream) {
+  snapkv_status_t st = check_common(B, Hq, Hkv, L, d, W);
+  if (st != SNAPKV_OK) return st;
+  if (W >= L || !q_obs || !k || !aligned16(q_obs) || !aligned16(k)) return SNAPKV_ERR_INVALID_ARG;
+  const KVStrides ks = dense_strides(Hkv, L, d);
+  uint8_t* ws = static_cast<uint8_t*>(workspace);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  int launches = 0;
+  if (seq_lens) {
+    for (int b = 0; b < B; ++b)
+      if (seq_lens[b] <= W || seq_lens[b] > L) return SNAPKV_ERR_INVALID_ARG;
+    RaggedBatch rb;
+    ragged_group(seq_lens, B, 0, Hq, Hkv, d, W, W, workspace_bytes, &rb);
+    if (rb.count != B || !workspace_ok(workspace, workspace_bytes, rb.total)) return SNAPKV_ERR_WORKSPACE;
+    for (int i = 0; i < B; ++i) rb.k_off[i] = i * ks.b;
+    if (launch_ragged_scores(rb, q_obs, k, ks, B, Hq, Hkv, d, W, ws, s, &launches, nullptr, false, nullptr,
+                             /*withhold=*/true) != cudaSuccess)
+      return SNAPKV_ERR_CUDA;
+  } else {
+    ScorePlan p;
+    if (!make_score_plan(B, Hq, Hkv, L, d, W, &p)) return SNAPKV_ERR_UNSUPPORTED;
+    const WorkspaceLayout w = make_layout(p, B, Hq, L - W, true, false);
+    if (!workspace_ok(workspace, workspace_bytes, w.total)) return SNAPKV_ERR_WORKSPACE;
+    if (launch_clear(ws, w, s) != cudaSuccess) return SNAPKV_ERR_CUDA;
+    launches = 1;
+    if (launch_window_scores(q_obs, k, ks, B, Hq, Hkv, L, d, W, p, reinterpret_cast<float*>(ws + w.off_vote),
+                             reinterpret_cast<int*>(ws + w.off_status), reinterpret_cast<int*>(ws + w.off_counters),
+                             reinterpret_cast<float*>(ws + w.off_partials), reinterpret_cast<float*>(ws + w.off_lse), s,
+                             &launches, nullptr, false, false, nullptr, nullptr, /*withhold=*/true) != cudaSuccess)
+      return SNAPKV_ERR_CUDA;
+  }
+  g_last_launches = launches;
+  return SNAPKV_OK;
+}
+
 snapkv_status_t snapkv_device_status(const void* workspace, void* stream, int* detail) {
   if (!workspace) return SNAPKV_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);

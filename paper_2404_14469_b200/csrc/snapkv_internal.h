@@ -160,14 +160,16 @@ size_t select_scratch_bytes(int rows, int n);  // 0 when the rows fit one CTA
 // skipped: a small kernel converts the rows first, then only the vote pass runs; that kernel
 // also zeroes the status block unless `keep_status` is set.  `never_ready` (self-test of the
 // time-out path): the vote pass alone is launched and nothing marks the units' statistics as
-// present, so its wait for them must run out.
+// present, so its wait for them must run out.  `withhold` (another): both passes run, but no
+// partial is written.
 cudaError_t launch_window_scores(const void* q_obs, const void* k, const KVStrides& ks, int B,
                                  int Hq, int Hkv, int L, int d, int W, const ScorePlan& plan,
                                  float* vote, int* status,
                                  int* counters, float* partials, float* lse2, cudaStream_t stream,
                                  int* launches, const float* lse_obs = nullptr,
                                  bool keep_status = false, bool never_ready = false,
-                                 const PagedKV* paged = nullptr, const ShardMode* shard = nullptr);
+                                 const PagedKV* paged = nullptr, const ShardMode* shard = nullptr,
+                                 bool withhold = false);
 
 // Pool + top-k over `rows` rows of fp32 votes.  `pooled_scratch` (select_scratch_bytes bytes)
 // is only touched when select_needs_scratch(n).  With gsum > 1 a selection row is the sum of
@@ -189,7 +191,8 @@ cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int poo
 // The same two steps for the sequences of a ragged batch.
 cudaError_t launch_ragged_scores(const RaggedBatch& rb, const void* q_obs, const void* k, const KVStrides& ks,
                                  int B, int Hq, int Hkv, int d, int W, uint8_t* ws, cudaStream_t stream,
-                                 int* launches, const float* lse_obs, bool keep_status, const PagedKV* paged);
+                                 int* launches, const float* lse_obs, bool keep_status, const PagedKV* paged,
+                                 bool withhold = false);
 bool ragged_select_applies(int n_max, int pool_kernel, int pool_type);
 cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int Hq, int W, int pool_kernel,
                                  int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream, int* launches);

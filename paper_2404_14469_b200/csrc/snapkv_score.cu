@@ -236,7 +236,7 @@ cudaError_t launch_window_scores(const void* q_obs, const void* k, const KVStrid
                                  float* vote, int* status,
                                  int* counters, float* partials, float* lse2, cudaStream_t stream,
                                  int* launches, const float* lse_obs, bool keep_status,
-                                 bool never_ready, const PagedKV* paged, const ShardMode* shard) {
+                                 bool never_ready, const PagedKV* paged, const ShardMode* shard, bool withhold) {
   CUtensorMap tmK, tmQ;
   {
     // (d, position, KV head, batch) with the caller's strides: any layout whose rows of d
@@ -259,6 +259,7 @@ cudaError_t launch_window_scores(const void* q_obs, const void* k, const KVStrid
   }
   score::ScoreArgs a = score_args(plan, L, W, Hkv, (lse_obs || never_ready) ? 1 : 0);
   a.wait_ns = wait_limit_setting();
+  a.withhold = withhold ? 1 : 0;
   if (shard) {
     a.mask_n = shard->mask_n;
     a.stats_only = shard->lse_out ? 1 : 0;

@@ -43,7 +43,7 @@ __global__ void ragged_prep_kernel(const float* __restrict__ lse_obs, const Prep
 template <int MAPS>
 cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, const KVStrides& ks, int B, int Hq,
                    int Hkv, int d, int W, uint8_t* ws, cudaStream_t stream, int* launches, const float* lse_obs,
-                   bool keep_status, const PagedKV* paged) {
+                   bool keep_status, const PagedKV* paged, bool withhold) {
   using u64 = unsigned long long;
   const ScorePlan& p0 = rb.plan[0];  // head grouping and columns are the same for all sequences
   const int units_per_seq = Hkv * p0.sub_per_kv;
@@ -90,6 +90,7 @@ cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, cons
   }
   score::ScoreArgs a = score_args(p0, rb.L[0], W, Hkv, lse_obs ? 1 : 0);
   a.wait_ns = wait_limit_setting();
+  a.withhold = withhold ? 1 : 0;
   a.page_table = paged ? paged->table : nullptr;
   a.pages_per_seq = paged ? paged->pages_per_seq : 0;
   a.page_size = paged ? paged->page_size : 1;
@@ -117,9 +118,9 @@ cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, cons
 
 cudaError_t launch_ragged_scores(const RaggedBatch& rb, const void* q_obs, const void* k, const KVStrides& ks, int B,
                                  int Hq, int Hkv, int d, int W, uint8_t* ws, cudaStream_t stream, int* launches,
-                                 const float* lse_obs, bool keep_status, const PagedKV* paged) {
+                                 const float* lse_obs, bool keep_status, const PagedKV* paged, bool withhold) {
   auto f = paged ? launch<1> : launch<RAGGED_MAX>;
-  return f(rb, q_obs, k, ks, B, Hq, Hkv, d, W, ws, stream, launches, lse_obs, keep_status, paged);
+  return f(rb, q_obs, k, ks, B, Hq, Hkv, d, W, ws, stream, launches, lse_obs, keep_status, paged, withhold);
 }
 
 }  // namespace snapkv

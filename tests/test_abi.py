@@ -213,3 +213,13 @@ def test_varlen_workspace_size(L):
                 ([], 8, 2, 128, 32, 7, 0, 256)]:
         assert size(*bad) == 0, bad
     assert L.snapkv_varlen_workspace_size(None, 1, 8, 2, 128, 32, 7, 0, 256) == 0
+
+
+def test_withheld_partials_selftest_checks_its_arguments(L):
+    lens = (ctypes.c_int32 * 2)(1024, 32)
+    call = lambda lens, W=32, ws=(FAKE, 1 << 30): L.snapkv_selftest_withheld_partials(
+        FAKE, FAKE, lens, 2, 4, 4, 1024, 64, W, ws[0], ws[1], None)
+    assert call(lens) == 1                                       # a sequence without a prefix
+    assert call((ctypes.c_int32 * 2)(1024, 1025)) == 1
+    assert call(None, W=1024) == 1
+    assert call(None, ws=(None, 0)) == 3 and call((ctypes.c_int32 * 2)(1024, 500), ws=(0x10000, 4096)) == 3
