@@ -217,9 +217,9 @@ def test_varlen_workspace_size(L):
 
 def test_withheld_partials_selftest_checks_its_arguments(L):
     lens = (ctypes.c_int32 * 2)(1024, 32)
-    call = lambda lens, W=32, ws=(FAKE, 1 << 30): L.snapkv_selftest_withheld_partials(
-        FAKE, FAKE, lens, 2, 4, 4, 1024, 64, W, ws[0], ws[1], None)
+    call = lambda lens, ws=(FAKE, 1 << 30): L.snapkv_selftest_withheld_partials(
+        FAKE, FAKE, lens, 2, 4, 4, 1024, 64, 32, ws[0], ws[1], None)
     assert call(lens) == 1                                       # a sequence without a prefix
     assert call((ctypes.c_int32 * 2)(1024, 1025)) == 1
-    assert call(None, W=1024) == 1
+    assert L.snapkv_selftest_withheld_partials(FAKE, FAKE, None, 2, 4, 4, 32, 64, 32, FAKE, 1 << 30, None) == 1  # W == L
     assert call(None, ws=(None, 0)) == 3 and call((ctypes.c_int32 * 2)(1024, 500), ws=(0x10000, 4096)) == 3
