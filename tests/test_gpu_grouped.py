@@ -93,3 +93,21 @@ def test_grouped_full_size_gqa_workload_on_sampled_kv_heads():
     w = synth.WORKLOADS[2]
     dev = synth.make_layer(w, 7, device="cuda")
     _check_grouped(dev, w.W, w.pool_kernel, w.pool_type, w.budgets[0], kv_heads=[(0, 3), (2, 0), (3, 7)])
+
+
+@pytest.mark.parametrize("flat", [False, True])
+def test_grouped_rows_that_are_filtered_first(flat):
+    # 8 rows of 262144 positions, each the sum of two heads: sample, filter and finish kernels ahead of
+    # the clusters.  With equal votes everywhere the list overflows, the clusters take the rows after
+    # all and the lowest positions win.
+    B, Hq, Hkv, L, d, W, kernel, budget = 1, 16, 8, 262160, 64, 16, 7, 1000
+    w = synth.Workload(72, "t", B, Hq, Hkv, d, L, W, kernel, "max", (budget,), 1, 40)
+    dev = synth.make_layer(w, 3, device="cuda")
+    if flat:
+        dev["q_obs"].zero_()
+        _, _, out_idx, ws = sk.snapkv_compress_grouped(dev["q_obs"], dev["k"], dev["v"], kernel, sk.POOL_MAX, budget)
+        assert sk.snapkv_device_status(ws) == (sk.OK, 0)
+        assert torch.equal(out_idx.cpu(), torch.arange(budget - W, dtype=torch.int32).expand(B, Hkv, budget - W))
+    else:
+        _check_grouped(dev, W, kernel, "max", budget, kv_heads=[(0, 0), (0, 5)])
+    assert sk.snapkv_last_launch_count() == 7   # clear, score, sample, filter, finish, clusters, gather

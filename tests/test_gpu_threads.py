@@ -82,3 +82,55 @@ print("same")
 def test_first_calls_of_several_threads_at_once():
     r = subprocess.run([sys.executable, "-c", FIRST_CALLS], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip() == "same", r.stdout + r.stderr
+
+
+def _batches(n):
+    g = torch.Generator(device="cuda").manual_seed(6)
+    out = []
+    for i in range(n):
+        lens = [400 + 311 * i, 150, 2000 - 97 * i, 129]
+        out.append((lens, [torch.randn(4, h, r, 128, generator=g, device="cuda").to(torch.bfloat16)
+                           for h, r in ((4, 32), (2, 2400), (2, 2400))]))
+    return out
+
+
+@pytest.mark.parametrize("own_streams", [False, True])
+def test_ragged_batches_of_several_threads(own_streams):
+    # Each thread has its workspace.  On one stream their launches interleave as they come; on streams
+    # of their own the calls are ordered by events, since two may not overlap on one device.
+    batches, rounds = _batches(4), 3
+    call = lambda lens, x, ws=None: sk.snapkv_compress_varlen(*x, lens, 5, sk.POOL_MAX, 200, workspace=ws)
+    want = [call(lens, x) for lens, x in batches]
+    torch.cuda.synchronize()
+    got, bad, turn, last = [[] for _ in batches], [], threading.Lock(), [None]
+
+    def work(i):
+        try:
+            lens, x = batches[i]
+            ws = None
+            stream = torch.cuda.Stream() if own_streams else torch.cuda.current_stream()
+            with torch.cuda.stream(stream):
+                for _ in range(rounds):
+                    if own_streams:
+                        with turn:
+                            if last[0] is not None:
+                                stream.wait_event(last[0])
+                            got[i].append(call(lens, x, ws))
+                            last[0] = stream.record_event()
+                    else:
+                        got[i].append(call(lens, x, ws))
+                    ws = got[i][-1][3]
+        except Exception as e:
+            bad.append(repr(e))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(batches))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not bad, bad
+    for i, ref in enumerate(want):
+        for out in got[i]:
+            assert sk.snapkv_device_status(out[3]) == (sk.OK, 0)
+            assert all(torch.equal(x, y) for x, y in zip(out[:3], ref[:3]))
