@@ -97,10 +97,10 @@ def test_grouped_full_size_gqa_workload_on_sampled_kv_heads():
 
 @pytest.mark.parametrize("flat", [False, True])
 def test_grouped_rows_that_are_filtered_first(flat):
-    # 8 rows of 262144 positions, each the sum of two heads: sample, filter and finish kernels ahead of
-    # the clusters.  With equal votes everywhere the list overflows, the clusters take the rows after
+    # 8 rows of 360448 positions, each the sum of two heads: sample, filter and finish kernels ahead of
+    # the clusters (of 11 CTAs, of which 7 find a place at once).  With equal votes everywhere the list overflows, the clusters take the rows after
     # all and the lowest positions win.
-    B, Hq, Hkv, L, d, W, kernel, budget = 1, 16, 8, 262160, 64, 16, 7, 1000
+    B, Hq, Hkv, L, d, W, kernel, budget = 1, 16, 8, 360464, 64, 16, 7, 1000
     w = synth.Workload(72, "t", B, Hq, Hkv, d, L, W, kernel, "max", (budget,), 1, 40)
     dev = synth.make_layer(w, 3, device="cuda")
     if flat:
