@@ -39,8 +39,8 @@ SYMBOLS = [
     "snapkv_shard_lse", "snapkv_lse_merge", "snapkv_shard_votes", "snapkv_gather_range",
 ]
 
-# entry points for the extension alone (csrc/snapkv_binding.h)
-BINDING_SYMBOLS = ["snapkv_binding_varlen", "snapkv_binding_paged"]
+# entry points for the extension and the tests alone (csrc/snapkv_binding.h)
+BINDING_SYMBOLS = ["snapkv_binding_varlen", "snapkv_binding_paged", "snapkv_binding_ragged_items"]
 
 _lib = None
 _native = None
@@ -122,6 +122,8 @@ def lib() -> ctypes.CDLL:
     L.snapkv_schedule_items.restype = c_int
     L.snapkv_schedule_items.argtypes = [c_int] * 9 + [ctypes.POINTER(ctypes.c_int32), c_int,
                                                       ctypes.POINTER(ctypes.c_int32)]
+    L.snapkv_binding_ragged_items.restype = c_int
+    L.snapkv_binding_ragged_items.argtypes = [p32] + [c_int] * 8 + [p32, c_int]
     L.snapkv_set_wait_limit_ns.restype = ctypes.c_ulonglong
     L.snapkv_set_wait_limit_ns.argtypes = [ctypes.c_ulonglong]
     L.snapkv_selftest_stalled_scores.restype = c_int
@@ -380,6 +382,18 @@ def snapkv_schedule_items(B, Hq, Hkv, L, d, W, grid, cta, votes_only=False):
     items = [tuple(buf[6 * i:6 * i + 6]) for i in range(n)]
     names = ("units", "units_per_wave", "waves", "tiles_stats", "tiles_vote", "maxseg", "lag", "ncols")
     return items, dict(zip(names, plan))
+
+
+def ragged_schedule_items(seq_lens, Hq, Hkv, d, W, grid, cta, votes_only=False):
+    """The same for a ragged batch: a list of (unit, t0, t1, vote, slot, nseg, sequence, wave)."""
+    L_ = lib()
+    args = ((ctypes.c_int32 * len(seq_lens))(*seq_lens), len(seq_lens), Hq, Hkv, d, W, int(votes_only), grid, cta)
+    n = L_.snapkv_binding_ragged_items(*args, None, 0)
+    if n < 0:
+        raise SnapKVError("ragged_schedule_items: arguments not acceptable")
+    buf = (ctypes.c_int32 * (8 * max(n, 1)))()
+    L_.snapkv_binding_ragged_items(*args, buf, n)
+    return [tuple(buf[8 * i:8 * i + 8]) for i in range(n)]
 
 
 def snapkv_set_wait_limit_ns(limit_ns: int) -> int:

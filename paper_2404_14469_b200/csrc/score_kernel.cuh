@@ -329,7 +329,7 @@ __host__ __device__ __forceinline__ int tiles_before(const ScoreArgs&, NotRagged
 // such a call, so that short sequences occupy different blocks; tiles_before restores the parity
 // with which that block would have met a statistics item's first tile.
 template <int MAPS>
-__device__ __forceinline__ Phase phase_at(const ScoreArgs& a, const RaggedSeqs<MAPS>& rs, int G, int p) {
+__host__ __device__ __forceinline__ Phase phase_at(const ScoreArgs& a, const RaggedSeqs<MAPS>& rs, int G, int p) {
   int s_seq = a.votes_only ? rs.nseq : 0, s_wave = 0, v_seq = 0, v_wave = 0, s_ord = 0, v_ord = 0, tiles = 0;
   Phase ph = {0, 0, 0, 0};
   for (int i = 0; i <= p; ++i) {
@@ -338,7 +338,8 @@ __device__ __forceinline__ Phase phase_at(const ScoreArgs& a, const RaggedSeqs<M
     ph.wave = ph.vote ? v_wave : s_wave;
     ph.ord = ph.vote ? v_ord++ : s_ord++;
     const RaggedSeq& q = rs.s[ph.seq];
-    const int wave_tiles = min(q.T1, 1 << 16) * min(q.upw, rs.units_per_seq - ph.wave * q.upw);
+    const int left = rs.units_per_seq - ph.wave * q.upw;
+    const int wave_tiles = (q.T1 < 1 << 16 ? q.T1 : 1 << 16) * (q.upw < left ? q.upw : left);
     int& wave = ph.vote ? v_wave : s_wave;
     tiles += ph.vote ? -wave_tiles : wave_tiles;
     if (++wave == q.nwaves) {
@@ -349,18 +350,18 @@ __device__ __forceinline__ Phase phase_at(const ScoreArgs& a, const RaggedSeqs<M
   return ph;
 }
 template <int MAPS>
-__device__ __forceinline__ int phase_count(const ScoreArgs& a, const RaggedSeqs<MAPS>& rs) {
+__host__ __device__ __forceinline__ int phase_count(const ScoreArgs& a, const RaggedSeqs<MAPS>& rs) {
   return a.votes_only ? rs.waves : 2 * rs.waves;
 }
 template <int MAPS>
-__device__ __forceinline__ Share share_of(const ScoreArgs&, const RaggedSeqs<MAPS>& rs, const Phase& ph, int cta, int G) {
+__host__ __device__ __forceinline__ Share share_of(const ScoreArgs&, const RaggedSeqs<MAPS>& rs, const Phase& ph, int cta, int G) {
   const RaggedSeq& q = rs.s[ph.seq];
-  const int u0 = ph.wave * q.upw;
-  return Share((cta + q.rot + 2 * ph.wave + ph.vote) % G, G, u0, min(q.upw, rs.units_per_seq - u0), ph.vote ? q.T2 : q.T1,
+  const int u0 = ph.wave * q.upw, left = rs.units_per_seq - u0;
+  return Share((cta + q.rot + 2 * ph.wave + ph.vote) % G, G, u0, q.upw < left ? q.upw : left, ph.vote ? q.T2 : q.T1,
                q.T1);
 }
 template <int MAPS>
-__device__ __forceinline__ int tiles_before(const ScoreArgs& a, const RaggedSeqs<MAPS>& rs, const Phase& ph, int cta, int G) {
+__host__ __device__ __forceinline__ int tiles_before(const ScoreArgs& a, const RaggedSeqs<MAPS>& rs, const Phase& ph, int cta, int G) {
   int before = 0;  // in earlier phases of the sequence
   if (!ph.vote)
     for (int e = 0; e < ph.wave; ++e)

@@ -903,6 +903,17 @@ int snapkv_schedule_items(int B, int Hq, int Hkv, int L, int d, int W, int votes
   return list_schedule_items(p, L, W, Hkv, votes_only ? 1 : 0, grid, cta, out_items, max_items);
 }
 
+int snapkv_binding_ragged_items(const int32_t* seq_lens, int B, int Hq, int Hkv, int d, int W, int votes_only,
+                                int grid, int cta, int32_t* out_items, int max_items) {
+  if (!seq_lens || B < 1 || max_items < 0 || (max_items > 0 && !out_items)) return -1;
+  if (grid < 1 || grid > MAX_GRID || cta < 0 || cta >= grid) return -1;
+  for (int b = 0; b < B; ++b)
+    if (check_common(1, Hq, Hkv, seq_lens[b], d, W) != SNAPKV_OK || seq_lens[b] <= W) return -1;
+  RaggedBatch rb;
+  ragged_group(seq_lens, B, 0, Hq, Hkv, d, W, W, ~static_cast<size_t>(0), &rb);
+  return rb.count == B ? list_ragged_items(rb, W, Hkv, votes_only ? 1 : 0, grid, cta, out_items, max_items) : -1;
+}
+
 unsigned long long snapkv_set_wait_limit_ns(unsigned long long limit_ns) {
   // at least a millisecond: a limit near the length of an ordinary wait would turn a busy
   // memory system into an error

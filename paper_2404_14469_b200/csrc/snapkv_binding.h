@@ -1,6 +1,6 @@
 /*
- * Entry points for the Python binding; not part of the interface in snapkv.h.  The ragged calls with
- * one argument more: with `fill`, rows behind a sequence's end are zeroed and positions set to -1,
+ * Entry points for the Python binding and the tests; not part of the interface in snapkv.h.  The ragged
+ * calls with one argument more: with `fill`, rows behind a sequence's end are zeroed and positions set to -1,
  * so that the binding need not clear whole outputs first (two passes over them).
  */
 #ifndef SNAPKV_BINDING_H_
@@ -12,6 +12,10 @@
 extern "C" {
 #endif
 
+/* snapkv_schedule_items for a ragged batch (at most 32 lengths above W that share a launch): records
+ * of eight int32, {unit, t0, t1, vote, slot, nseg, sequence, wave of the launch}. */
+int snapkv_binding_ragged_items(const int32_t* seq_lens, int B, int Hq, int Hkv, int d, int W, int votes_only,
+                                int grid, int cta, int32_t* out_items, int max_items);
 snapkv_status_t snapkv_binding_varlen(const void* q_obs, const void* k, const void* v, const int64_t* k_strides,
                                       const int64_t* v_strides, const int64_t* k_seq_offsets,
                                       const int64_t* v_seq_offsets, const int32_t* seq_lens, const float* lse_obs,

@@ -129,6 +129,10 @@ struct WorkspaceLayout {
 int list_schedule_items(const ScorePlan& plan, int L, int W, int Hkv, int votes_only, int grid,
                         int cta, int32_t* out, int max_items);
 
+// The same for a ragged batch: records of eight, with the sequence and the wave behind the six.
+int list_ragged_items(const RaggedBatch& rb, int W, int Hkv, int votes_only, int grid, int cta, int32_t* out,
+                      int max_items);
+
 // Time limit, in nanoseconds, that kernels launched from now on give each of their device-side
 // waits (process-wide; one second unless snapkv_set_wait_limit_ns changed it).
 unsigned long long wait_limit_setting();

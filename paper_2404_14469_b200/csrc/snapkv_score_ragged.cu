@@ -40,28 +40,21 @@ __global__ void ragged_prep_kernel(const float* __restrict__ lse_obs, const Prep
   lse2[static_cast<size_t>(u) * MAX_COLS + c] = out;
 }
 
+// The sequences as the kernel gets them, without their tensor maps; returns the most units of a wave.
 template <int MAPS>
-cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, const KVStrides& ks, int B, int Hq,
-                   int Hkv, int d, int W, uint8_t* ws, cudaStream_t stream, int* launches, const float* lse_obs,
-                   bool keep_status, const PagedKV* paged, bool withhold) {
-  using u64 = unsigned long long;
-  const ScorePlan& p0 = rb.plan[0];  // head grouping and columns are the same for all sequences
-  const int units_per_seq = Hkv * p0.sub_per_kv;
-  score::RaggedSeqs<MAPS> rs;
-  rs.nseq = rb.count;
-  rs.units_per_seq = units_per_seq;
-  rs.waves = 0;
+int describe(const RaggedBatch& rb, bool votes_only, bool paged, score::RaggedSeqs<MAPS>* rs) {
   int upw = 1;
-  const u64 strides[3] = {static_cast<u64>(ks.l) * 2, static_cast<u64>(ks.h) * 2, static_cast<u64>(ks.b) * 2};
-  const unsigned box[4] = {64, TILE_KEYS, 1, 1};
+  rs->nseq = rb.count;
+  rs->units_per_seq = rb.plan[0].units;
+  rs->waves = 0;
   for (int i = 0; i < rb.count; ++i) {
     const ScorePlan& p = rb.plan[i];
-    score::RaggedSeq& q = rs.s[i];
+    score::RaggedSeq& q = rs->s[i];
     q.L = rb.L[i];
     q.n = p.n_vote;
-    q.upw = lse_obs ? p.units : p.units_per_wave;  // votes alone: nothing couples the units
-    q.nwaves = lse_obs ? 1 : p.nwaves;
-    rs.waves += q.nwaves;
+    q.upw = votes_only ? p.units : p.units_per_wave;  // votes alone: nothing couples the units
+    q.nwaves = votes_only ? 1 : p.nwaves;
+    rs->waves += q.nwaves;
     if (q.upw > upw) upw = q.upw;
     q.T1 = p.tiles_stats;
     q.T2 = p.tiles_vote;
@@ -71,7 +64,22 @@ cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, cons
     q.map = paged ? 0 : i;
     q.part0 = rb.part0[i];
     q.vote0 = rb.vote0[i];
-    if (paged) continue;
+  }
+  return upw;
+}
+
+template <int MAPS>
+cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, const KVStrides& ks, int B, int Hq,
+                   int Hkv, int d, int W, uint8_t* ws, cudaStream_t stream, int* launches, const float* lse_obs,
+                   bool keep_status, const PagedKV* paged, bool withhold) {
+  using u64 = unsigned long long;
+  const ScorePlan& p0 = rb.plan[0];  // head grouping and columns are the same for all sequences
+  const int units_per_seq = Hkv * p0.sub_per_kv;
+  score::RaggedSeqs<MAPS> rs;
+  const int upw = describe(rb, lse_obs != nullptr, paged != nullptr, &rs);
+  const u64 strides[3] = {static_cast<u64>(ks.l) * 2, static_cast<u64>(ks.h) * 2, static_cast<u64>(ks.b) * 2};
+  const unsigned box[4] = {64, TILE_KEYS, 1, 1};
+  for (int i = 0; i < rb.count && !paged; ++i) {
     const u64 dims[4] = {static_cast<u64>(d), static_cast<u64>(rb.L[i]), static_cast<u64>(Hkv), 1};
     if (!encode_tensor_map(&rs.maps[i], static_cast<const uint8_t*>(k) + rb.k_off[i] * 2, 4, dims, strides, box))
       return cudaErrorInvalidValue;
@@ -115,6 +123,25 @@ cudaError_t launch(const RaggedBatch& rb, const void* q_obs, const void* k, cons
 }
 
 }  // namespace
+
+int list_ragged_items(const RaggedBatch& rb, int W, int Hkv, int votes_only, int grid, int cta, int32_t* out,
+                      int max_items) {
+  score::RaggedSeqs<1> rs;
+  describe(rb, votes_only != 0, true, &rs);
+  const score::ScoreArgs a = score_args(rb.plan[0], rb.L[0], W, Hkv, votes_only);
+  int count = 0;
+  for (int p = 0; p < score::phase_count(a, rs); ++p) {
+    const score::Phase ph = score::phase_at(a, rs, grid, p);
+    score::Share share = score::share_of(a, rs, ph, cta, grid);
+    for (score::Item it = share.take(); it.t0 < it.t1; it = share.take(), ++count) {
+      if (count >= max_items) continue;
+      int32_t* o = out + static_cast<size_t>(count) * 8;
+      o[0] = it.unit; o[1] = it.t0; o[2] = it.t1; o[3] = ph.vote; o[4] = it.slot; o[5] = it.nseg;
+      o[6] = ph.seq; o[7] = ph.ord;
+    }
+  }
+  return count;
+}
 
 cudaError_t launch_ragged_scores(const RaggedBatch& rb, const void* q_obs, const void* k, const KVStrides& ks, int B,
                                  int Hq, int Hkv, int d, int W, uint8_t* ws, cudaStream_t stream, int* launches,

@@ -2,12 +2,15 @@
 statistics between its blocks (Eq. 1 needs each window row's normaliser over ALL keys before
 any probability can be summed, so blocks that share a unit exchange partial log-sum-exps).
 
-The item lists come from the library itself (snapkv_schedule_items runs the kernel's own item
-walk on the host).  The hand-over is modelled with one CPU thread per block: publish a
-partial and count it; before a vote item, wait (with a time limit) until the unit's count
-says that all partials are there, then fold them in slot order.  The model shows that the
-schedule cannot deadlock, that every block folds the same value whatever the thread timing,
-and that a block which never arrives turns into time-outs, not into a hang."""
+The item lists come from the library itself (snapkv_schedule_items and its counterpart for ragged
+batches run the kernel's own item walk on the host).  The hand-over is modelled with two CPU threads
+per block, as the kernel has warps: one walks the items, computes statistics and writes partials (a
+written slot is its own flag) and adds up votes; the other fetches, for every vote item, the unit's row:
+it looks until every slot is written, with a time limit, and folds them in slot order.  In a ragged
+batch the block with slot 0 folds, one wave ahead of the votes, and the others wait for its row.  The
+model shows that the schedule cannot deadlock, that every block gets the same row whatever the thread
+timing, and that a block which never arrives turns into time-outs, not into a hang."""
+import queue
 import threading
 import time
 
@@ -93,45 +96,127 @@ def test_votes_only_schedule_is_one_phase_without_statistics():
     assert tiles == plan["units"] * plan["tiles_vote"]
 
 
+RAGGED = [
+    # lens, Hq, Hkv, d, W, grid
+    ([24000, 5012, 1353, 9000, 600, 2047], 32, 8, 128, 32, 148),
+    ([300, 129, 700, 17], 8, 2, 128, 16, 148),          # fewer tiles than blocks in every sequence
+    ([60000, 1000, 70000, 50000], 16, 8, 128, 32, 148),  # several waves in a sequence
+    ([900, 5000, 33], 8, 1, 64, 32, 7),                  # two head sub-groups, small grid
+]
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,d,W,grid", RAGGED)
+def test_a_ragged_batch_is_cut_as_the_calls_one_by_one(lens, Hq, Hkv, d, W, grid):
+    # block c has, of sequence i, what block (c + 53 i) % grid has in a call on that sequence alone: the
+    # same tiles, slots and counts of slots, so that results do not depend on the batch
+    ragged = [sk.ragged_schedule_items(lens, Hq, Hkv, d, W, grid, c) for c in range(grid)]
+    for i, L in enumerate(lens):
+        alone, _ = _all_items(1, Hq, Hkv, L, d, W, grid)
+        for c in range(grid):
+            assert [x[:6] for x in ragged[c] if x[6] == i and x[3] == 0] == \
+                [x for x in alone[(c + 53 * i) % grid] if x[3] == 0]
+            assert [x[:6] for x in ragged[c] if x[6] == i and x[3] == 1] == \
+                [x for x in alone[(c + 53 * i) % grid] if x[3] == 1]
+
+
+@pytest.mark.parametrize("lens,Hq,Hkv,d,W,grid", RAGGED)
+def test_statistics_of_the_next_wave_come_before_a_waves_votes(lens, Hq, Hkv, d, W, grid):
+    # what the folding blocks of a ragged batch rely on; waves are numbered through the launch
+    waves = {}
+    for c in range(grid):
+        items = sk.ragged_schedule_items(lens, Hq, Hkv, d, W, grid, c)
+        done = [-1, -1]
+        for unit, t0, t1, vote, slot, nseg, seq, wave in items:
+            assert wave >= done[vote]                       # each sweep in the order of the waves
+            done[vote] = wave
+            if vote == 0:
+                waves.setdefault(wave, seq)
+                assert waves[wave] == seq
+        order = [(x[7], x[3]) for x in items]
+        for at, (wave, vote) in enumerate(order):
+            if vote:                                        # none of waves 0 .. wave + 1 is still to come
+                assert not any(v == 0 and w <= wave + 1 for w, v in order[at:])
+
+
 class _Model:
-    """One thread per block; `absent` blocks never run."""
+    """Two threads per block; `absent` blocks never run.  Items are (unit key, vote, slot, nseg, wave)."""
 
-    def __init__(self, per_cta, units, limit_s):
-        self.per_cta, self.limit = per_cta, limit_s
-        self.partials = [dict() for _ in range(units)]
-        self.count = [0] * units
-        self.lock = threading.Lock()
+    def __init__(self, per_cta, limit_s, ragged):
+        self.per_cta, self.limit, self.ragged = per_cta, limit_s, ragged
+        self.slots, self.rows = {}, {}                    # (key, slot) -> partial; key -> row
         self.abort = [0] * len(per_cta)
-        self.folds = [[] for _ in per_cta]
+        self.got = [[] for _ in per_cta]
 
-    def run_block(self, c, jitter):
-        for k, (unit, t0, t1, vote, slot, nseg) in enumerate(self.per_cta[c]):
+    def _wait(self, c, ready):
+        t_end = time.monotonic() + self.limit / 2         # a wait on other blocks: half the limit
+        while not ready():
+            if self.abort[c]:
+                return False
+            if time.monotonic() > t_end:
+                self.abort[c] = 7                         # the code of the wait for a unit's statistics
+                return False
+            time.sleep(1e-4)
+        return True
+
+    def _fold(self, c, key, nseg):
+        if not self._wait(c, lambda: all((key, s) in self.slots for s in range(nseg))):
+            return None
+        acc = 0
+        for s in range(nseg):                             # slot order: the same in every block
+            acc = acc * 31 + self.slots[key, s]
+        return acc
+
+    def _items(self, c, vote, wave):
+        return [x for x in self.per_cta[c] if x[1] == vote and x[4] == wave]
+
+    def fetcher(self, c, out):
+        waves = 1 + max(x[4] for items in self.per_cta for x in items)
+        for w in range(-1 if self.ragged else 0, waves):
+            if self.ragged:
+                for key, _, slot, nseg, _ in self._items(c, 0, w + 1):
+                    if slot == 0:
+                        row = self._fold(c, key, nseg)
+                        if row is None:
+                            return
+                        self.rows[key] = row
+            for key, _, _, nseg, _ in self._items(c, 1, w):
+                if self.ragged:
+                    row = self.rows[key] if self._wait(c, lambda: key in self.rows) else None
+                else:
+                    row = self._fold(c, key, nseg)
+                if row is None:
+                    return
+                while not self.abort[c]:
+                    try:
+                        out.put((key, row), timeout=0.01)  # eight buffers
+                        break
+                    except queue.Full:
+                        pass
+
+    def softmax(self, c, rows, jitter):
+        for k, (key, vote, slot, nseg, wave) in enumerate(self.per_cta[c]):
             if jitter:
                 time.sleep(((c * 7 + k * 3) % 5) * 1e-4)
             if not vote:
-                value = (unit + 1) * 1000 + slot        # stands for the block's partial
-                self.partials[unit][slot] = value        # the data first ...
-                with self.lock:
-                    self.count[unit] += 1                # ... then the count (release)
-            else:
-                t_end = time.monotonic() + self.limit / 2   # a wait on other blocks: half the limit
-                while True:
-                    with self.lock:
-                        ready = self.count[unit] >= nseg
-                    if ready:
-                        break
-                    if time.monotonic() > t_end:
-                        self.abort[c] = 7                # the code of the wait for a unit's statistics
+                self.slots[key, slot] = (hash(key) % 1009 + 1) * 1000 + slot   # stands for the block's partial
+                continue
+            while True:
+                try:
+                    got = rows.get(timeout=0.01)
+                    break
+                except queue.Empty:
+                    if self.abort[c]:
                         return
-                    time.sleep(1e-4)
-                acc = 0
-                for s in range(nseg):                    # slot order: the same in every block
-                    acc = acc * 31 + self.partials[unit][s]
-                self.folds[c].append((unit, acc))
+            assert got[0] == key, "rows come in the order of the items"
+            self.got[c].append(got)
 
     def run(self, absent=(), jitter=True):
-        threads = [threading.Thread(target=self.run_block, args=(c, jitter))
-                   for c in range(len(self.per_cta)) if c not in absent]
+        threads = []
+        for c in range(len(self.per_cta)):
+            if c not in absent:
+                rows = queue.Queue(maxsize=8)
+                threads += [threading.Thread(target=self.fetcher, args=(c, rows)),
+                            threading.Thread(target=self.softmax, args=(c, rows, jitter))]
         t0 = time.monotonic()
         for t in threads:
             t.start()
@@ -141,30 +226,46 @@ class _Model:
         return time.monotonic() - t0
 
 
-@pytest.mark.parametrize("shape", [(2, 8, 2, 3000, 128, 32, 24), (1, 4, 4, 1024, 64, 32, 40)])
-def test_hand_over_completes_and_every_block_folds_the_same_value(shape):
+def _model(shape, limit_s):
+    """Of one length (B, Hq, Hkv, L, d, W, grid) or of a ragged batch ([lengths], Hq, Hkv, d, W, grid)."""
+    if isinstance(shape[0], list):
+        items = [[((x[6], x[0]), x[3], x[4], x[5], x[7]) for x in sk.ragged_schedule_items(*shape, c)]
+                 for c in range(shape[-1])]
+        return _Model(items, limit_s, True)
     per_cta, plan = _all_items(*shape)
-    m = _Model(per_cta, plan["units"], limit_s=5.0)
+    return _Model([[(x[0], x[3], x[4], x[5], x[0] // plan["units_per_wave"]) for x in items] for items in per_cta],
+                  limit_s, False)
+
+
+HAND_OVER = [
+    (2, 8, 2, 3000, 128, 32, 24), (1, 4, 4, 1024, 64, 32, 40),
+    ([3000, 700, 150, 1200, 90], 8, 2, 128, 32, 24), ([60000, 50000], 16, 8, 128, 32, 16),
+]
+
+
+@pytest.mark.parametrize("shape", HAND_OVER)
+def test_hand_over_completes_and_every_block_folds_the_same_value(shape):
+    m = _model(shape, limit_s=10.0)
     m.run()
     assert not any(m.abort)
     by_unit = {}
-    for folds in m.folds:
-        for unit, acc in folds:
-            by_unit.setdefault(unit, set()).add(acc)
-    assert set(by_unit) == set(range(plan["units"]))
+    for got in m.got:
+        for key, row in got:
+            by_unit.setdefault(key, set()).add(row)
+    assert set(by_unit) == {x[0] for items in m.per_cta for x in items if x[1] == 1}
     assert all(len(v) == 1 for v in by_unit.values())
+    assert [len(g) for g in m.got] == [sum(x[1] for x in items) for items in m.per_cta]
 
 
-def test_a_block_that_never_arrives_becomes_time_outs_not_a_hang():
-    shape = (2, 8, 2, 3000, 128, 32, 24)
-    per_cta, plan = _all_items(*shape)
-    m = _Model(per_cta, plan["units"], limit_s=0.4)
+@pytest.mark.parametrize("shape", HAND_OVER[::2])
+def test_a_block_that_never_arrives_becomes_time_outs_not_a_hang(shape):
+    m = _model(shape, limit_s=0.4)
     took = m.run(absent={5})
-    # blocks that share a unit with block 5 give up at half the limit with the code of that
-    # wait; nobody waits longer than the limit
-    units_of_5 = {u for (u, _, _, v, _, _) in per_cta[5] if v == 0}
-    waiting = [c for c, items in enumerate(per_cta)
-               if c != 5 and any(v == 1 and u in units_of_5 for (u, _, _, v, _, _) in items)]
+    # blocks that need a unit which block 5 has a share of give up at half the limit with the code of
+    # that wait; nobody waits longer than the limit
+    units_of_5 = {x[0] for x in m.per_cta[5] if x[1] == 0}
+    waiting = [c for c, items in enumerate(m.per_cta)
+               if c != 5 and any(x[1] == 1 and x[0] in units_of_5 for x in items)]
     assert waiting and all(m.abort[c] == 7 for c in waiting)
     assert took < 5.0
 
