@@ -29,6 +29,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 #include <type_traits>
 
 #include "launch.cuh"
@@ -885,29 +886,73 @@ struct ClusterShape {
   double us = 0.0;         // estimated time (of the shapes of 1024 threads)
 };
 
+// How many clusters of c CTAs of 1024 threads (one per SM) run at once on the current device, which is
+// asked once: a B200 answers 148, 74, 45, 33, 26, 22, 15, 15, 15, 11 for c = 1 .. 10 and 7 for more.
+// When the clusters come in rounds fewer find a place than on an empty device: 52 clusters of five
+// take three rounds, eight of nine two.  So sizes above 8 count as 16, and up to 8 the SMs that the
+// GPCs leave over (16 with clusters of three or four, 28 with larger ones) are not counted on.
+int clusters_at_once(int c) {
+  constexpr int MAX_DEV = 64;
+  static std::mutex mu;
+  static int fit[MAX_DEV][CL_MAX_CLUSTER + 1];
+  static std::atomic<bool> known[MAX_DEV];
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return c <= 8 ? sm_count() / c : 0;
+  if (!known[dev].load(std::memory_order_acquire)) {
+    std::lock_guard<std::mutex> lock(mu);
+    if (!known[dev].load(std::memory_order_relaxed)) {
+      auto kernel = pool_topk_cluster_kernel<1024, 32, CL_RMAX, -1, OneLength>;
+      constexpr int SMEM = slots_for(1024 * 32) * 4;
+      const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) == cudaSuccess;
+      fit[dev][1] = sm_count();
+      for (int i = 2; i <= CL_MAX_CLUSTER; ++i) {
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = i;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(i);
+        cfg.blockDim = dim3(1024);
+        cfg.dynamicSmemBytes = SMEM;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (!ok || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+          n = i <= 8 ? 1 : 0;       // (a size that every device takes, or none)
+          (void)cudaGetLastError();  // a refusal here is an answer, not an error of the call
+        }
+        fit[dev][i] = n;
+      }
+      known[dev].store(true, std::memory_order_release);
+    }
+  }
+  if (c > 8) return fit[dev][CL_MAX_CLUSTER];
+  const int in_rounds = (fit[dev][1] - (c <= 2 ? 0 : (c <= 4 ? 16 : 28))) / c;
+  return fit[dev][c] < in_rounds ? fit[dev][c] : in_rounds;
+}
+
 // How rows of n positions are cut: the shape with the smallest estimated time.  Up to 4096
 // positions small CTAs have the shortest chain, and clusters of them while every CTA has an SM to
 // itself (79.6 against 84.2 us for the whole step of 32 rows of 16352).  Beyond, CTAs of 1024 threads
 // (one per SM) with 8, 16 or 32 keys a thread take about 8, 10.5 and 16.5 us, 2 to 4 us more when a
-// cluster shares a row, and come in rounds when they do not all find a place at once (clusters fit
-// less well the larger they are).
+// cluster shares a row, and come in rounds when they do not all find a place at once.  No CTAs: the
+// device holds no cluster that is large enough.
 ClusterShape cluster_shape(int rows, int n) {
   if (n <= 2048) return {256, 8, 1};
   const int small = (n + 4095) / 4096;
-  if (small <= 8 && rows * small <= 148) return {512, 8, small};
+  if (small <= 8 && rows * small <= sm_count()) return {512, 8, small};
   const int ept[3] = {8, 16, 32};
   const double alone[3] = {8.0, 10.5, 16.5}, shared[3] = {10.2, 12.5, 20.0};
-  ClusterShape best = {1024, 32, (n + 32767) / 32768};
-  double best_us = 1e30;
+  ClusterShape best = {1024, 32, 0, 1e30};
   for (int i = 0; i < 3; ++i) {
     const int c = (n + 1024 * ept[i] - 1) / (1024 * ept[i]);
     if (c > CL_MAX_CLUSTER) continue;
-    const int fit = c == 1 ? 148 : (c <= 2 ? 74 : (c <= 4 ? 132 / c : (c <= 8 ? 120 / c : 7)));  // clusters at once
+    const int fit = clusters_at_once(c);
+    if (fit < 1) continue;
     const double us = static_cast<double>((rows + fit - 1) / fit) * (c == 1 ? alone[i] : shared[i] + 0.35 * c);
-    if (us < best_us) {
-      best_us = us;
-      best = {1024, ept[i], c, us};
-    }
+    if (us < best.us) best = {1024, ept[i], c, us};
   }
   return best;
 }
@@ -1033,44 +1078,10 @@ cudaError_t launch_rows(const ClusterShape& s, const SelectCall& c, const ROWS& 
 
 }  // namespace
 
-// Whether this device can hold a cluster of 16 CTAs of the largest shape (asked once per device).
-static bool cluster16_ok() {
-  constexpr int MAX_DEV = 64;
-  static std::atomic<int> state[MAX_DEV] = {};  // 0 unknown, 1 yes, 2 no
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEV) return false;
-  int st = state[dev].load(std::memory_order_acquire);
-  if (st == 0) {
-    auto kernel = pool_topk_cluster_kernel<1024, 32, CL_RMAX, -1, OneLength>;
-    constexpr int SMEM = slots_for(1024 * 32) * 4;
-    int n_clusters = 0;
-    bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-              cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM) == cudaSuccess;
-    if (ok) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(16);
-      cfg.blockDim = dim3(1024);
-      cfg.dynamicSmemBytes = SMEM;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeClusterDimension;
-      attr[0].val.clusterDim.x = 16;
-      attr[0].val.clusterDim.y = 1;
-      attr[0].val.clusterDim.z = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      ok = cudaOccupancyMaxActiveClusters(&n_clusters, kernel, &cfg) == cudaSuccess && n_clusters >= 1;
-    }
-    if (!ok) (void)cudaGetLastError();  // a refusal here is an answer, not an error of the call
-    st = ok ? 1 : 2;
-    state[dev].store(st, std::memory_order_release);
-  }
-  return st == 1;
-}
-
 bool select_cluster_applies(int rows, int n, int pool_kernel) {
   if ((pool_kernel >> 1) > CL_RMAX || n > CL_MAX_CLUSTER * 1024 * 32) return false;
   const int ctas = cluster_shape(rows, n).ctas;
-  return static_cast<long long>(rows) * ctas < 2147483647ll && (ctas <= 8 || cluster16_ok());
+  return ctas > 0 && static_cast<long long>(rows) * ctas < 2147483647ll;
 }
 
 cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int pool_kernel,
@@ -1113,7 +1124,8 @@ static ClusterShape ragged_shape(int n) {
 bool ragged_select_applies(int n_max, int pool_kernel, int pool_type) {
   if ((pool_kernel >> 1) > CL_RMAX || n_max > CL_MAX_CLUSTER * 1024 * 32) return false;
   if (pool_type == 1 && n_max > 131072) return false;  // two ways of ranking in one launch
-  return ragged_shape(n_max).ctas <= 8 || cluster16_ok();
+  const int ctas = ragged_shape(n_max).ctas;
+  return ctas <= 8 || clusters_at_once(ctas) > 0;
 }
 
 cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int Hq, int W, int pool_kernel,

@@ -564,3 +564,11 @@ def test_extreme_prompt_keeps_the_needle():
     vote, _ = sk.snapkv_window_scores(dev["q_obs"][:, :2].contiguous(), dev["k"][:, :2].contiguous())
     ref = _oracle_head(_bits(dev["q_obs"][:, :2]), _bits(dev["k"][:, :2]), 0, 1, 1)
     parity.check_votes(vote[0, 1].cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("rows,n,kernel,ptype,ksel", [
+    (16, 53000, 7, "max", 2000), (17, 106500, 5, "avg", 999),   # more rows than there is room for clusters of seven
+    (34, 107000, 13, "max", 1000), (16, 210000, 7, "max", 4000),  # these are filtered first
+])
+def test_pool_topk_of_rows_that_took_clusters_of_seven(rows, n, kernel, ptype, ksel):
+    test_pool_topk_at_the_edges_of_its_shapes(rows, n, kernel, ptype, ksel)
