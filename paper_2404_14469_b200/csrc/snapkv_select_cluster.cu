@@ -439,11 +439,14 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
     }
     __syncthreads();
     const uint32_t b = sel_bin;
-    if (b == ~0u) {  // above the guessed window or below it: the whole range decides
+    if (b == ~0u) {
+      // Above the guessed window or below it: the whole range decides, and all of it, so that a bin is
+      // found whatever the votes are (the 0 of the positions outside the row is its lowest key, and
+      // those positions come last).
       guess = false;
-      lo = KEY_MIN;
-      width = ~KEY_MIN;
-      shift = 21;
+      lo = 0u;
+      width = ~0u;
+      shift = 22;
       __syncthreads();  // everybody has read sel_bin before it is written again
       continue;
     }
@@ -451,7 +454,7 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
     krem -= sel_above;
     in_bin = sel_count;
     bin_lo = lo + (b << shift);
-    bin_w = (1u << shift) - 1u;
+    bin_w = min((1u << shift) - 1u, lo + width - bin_lo);  // keys behind the window's end count as above it
     if (shift == 0 || in_bin <= cap) break;
     lo = bin_lo;
     width = bin_w;

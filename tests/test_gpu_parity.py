@@ -572,3 +572,45 @@ def test_extreme_prompt_keeps_the_needle():
 ])
 def test_pool_topk_of_rows_that_took_clusters_of_seven(rows, n, kernel, ptype, ksel):
     test_pool_topk_at_the_edges_of_its_shapes(rows, n, kernel, ptype, ksel)
+
+
+@pytest.mark.parametrize("n,kernel,ptype", [
+    (60, 5, "avg"), (1004, 7, "max"), (1500, 13, "max"),          # 256 threads per row
+    (3001, 5, "max"), (13000, 7, "avg"), (16352, 7, "max"),       # 512 threads, clusters of up to 4
+    (24001, 3, "max"), (40000, 15, "max"), (150000, 5, "avg"),    # 1024 threads
+])
+def test_pool_topk_that_drops_few_positions(n, kernel, ptype):
+    # The window of keys then starts at zero, its bins are wide, and the ksel-th key tends to lie in the
+    # last of them, which reaches beyond the window's end.  Rows spread over a few and over many octaves.
+    g = torch.Generator().manual_seed(n)
+    spread = torch.tensor([0.1, 1.0, 1.0, 3.0])[:, None]
+    vote = torch.exp(spread * torch.randn(4, n, generator=g))
+    for gap in sorted({1, 3, 12, n // 40 + 1, n // 12, n // 7}):
+        ksel = n - gap
+        idx = sk.snapkv_pool_topk(vote.cuda(), kernel, PT[ptype], ksel).cpu().numpy()
+        for r in range(4):
+            pooled = orc.pool1d(vote[r].numpy().astype(np.float64), kernel, PT[ptype])
+            same = parity.check_indices(idx[r], pooled, ksel, orc.topk_positions(pooled, ksel))
+            if ptype == "max":
+                assert same
+
+
+def test_prompts_a_little_longer_than_the_budget():
+    # a batch as a server gets it: one prompt far longer than the budget, the others hardly
+    Hq, Hkv, d, W, kernel, budget = 8, 2, 128, 32, 7, 1024
+    lens = [1036, 1030, 1100, 1200, 6000]
+    data = [synth.make_layer(synth.Workload(60, "t", 1, Hq, Hkv, d, L, W, kernel, "max", (budget,), 1, 3), L) for L in lens]
+    q = torch.cat([x["q_obs"] for x in data]).cuda()
+    k, v = (torch.zeros(len(lens), Hkv, max(lens), d, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    for b, x in enumerate(data):
+        k[b, :, :lens[b]], v[b, :, :lens[b]] = x["k"][0], x["v"][0]
+    ok, ov, oi, ws = sk.snapkv_compress_varlen(q, k, v, lens, kernel, sk.POOL_MAX, budget)
+    assert sk.snapkv_device_status(ws) == (sk.OK, 0)
+    for b, L in enumerate(lens):
+        one = sk.snapkv_compress(q[b:b + 1], k[b:b + 1, :, :L].contiguous(), v[b:b + 1, :, :L].contiguous(), kernel,
+                                 sk.POOL_MAX, budget)
+        assert torch.equal(oi[b], one[2][0]) and torch.equal(ok[b], one[0][0]) and torch.equal(ov[b], one[1][0])
+        if b < 4:
+            ref = orc.compress(*(_bits(data[b][x]) for x in ("q_obs", "k", "v")), kernel, orc.POOL_MAX, budget)
+            for h in range(Hq):
+                parity.check_indices(oi[b, h].cpu().numpy(), ref["pooled"][0, h], budget - W, ref["out_idx"][0, h])
