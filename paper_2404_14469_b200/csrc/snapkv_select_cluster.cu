@@ -983,16 +983,10 @@ int2 window_ranks(int ksel, int n) {
 template <int THREADS, int EPT, int R, int PT, typename ROWS>
 cudaError_t launch_one(const SelectCall& c, int ctas, const ROWS& rows) {
   auto kernel = pool_topk_cluster_kernel<THREADS, EPT, R, PT, ROWS>;
-  // CTAs of this kernel take their places while the scoring CTAs leave the SMs one by one.  Asking
-  // for so much shared memory that no SM takes more than its even share keeps them from crowding
-  // on the SMs that come free first.
-  constexpr int SMEM_MOST = 192 * 1024;
-  const int per_sm = (c.rows * ctas + sm_count() - 1) / sm_count();
-  int smem = slots_for(THREADS * EPT) * 4;
-  if (smem < SMEM_MOST / per_sm) smem = SMEM_MOST / per_sm;
+  constexpr int SMEM = slots_for(THREADS * EPT) * 4;
   static DeviceOnce once;
   if (!once.done()) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MOST);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     once.set();
@@ -1000,7 +994,7 @@ cudaError_t launch_one(const SelectCall& c, int ctas, const ROWS& rows) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(c.rows) * ctas);
   cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = SMEM;
   cfg.stream = c.stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
