@@ -18,7 +18,7 @@
  *   - The caller owns every buffer the entry points read or write.  The library itself
  *     holds, for the life of the process: one fixed 16 MiB device array on every GPU
  *     that loads it (the scratch of snapkv_pool_topk_static), and, per device and
- *     created on the first snapkv_compress_host call there, one side stream and a
+ *     created on the first snapkv_compress_host call there, two side streams and a
  *     handful of events.  It caches driver entry points, the SM count and "attribute
  *     set" flags per device.  Nothing else is allocated and no per-call state is kept.
  *   - One call at a time per device.  The scoring kernel behind snapkv_compress*,
@@ -31,8 +31,9 @@
  *     unwritten and SNAPKV_ERR_TIMEOUT is recorded in the status block.  So do not let
  *     two scoring/compress calls, or such a call and other large kernels, overlap on one
  *     GPU; calls on one stream never do.  snapkv_compress_host in addition shares its
- *     side stream and events among all calls on a device: one caller per device at a
- *     time.
+ *     side streams and events among all calls on a device: one caller per device at a
+ *     time.  A second caller waits on the host until the first has enqueued its work,
+ *     which with pageable host buffers includes the copies.
  *   - Work is enqueued on `stream` (a cudaStream_t passed as void*; NULL is the
  *     default stream).  Calls return without synchronising unless stated.  Several of
  *     the kernels are launched with programmatic dependent launch: their blocks may
@@ -284,11 +285,12 @@ snapkv_status_t snapkv_compress_varlen(const void* q_obs, const void* k, const v
  * `staging` is DEVICE scratch of at least snapkv_host_staging_size(...) bytes,
  * 256-byte aligned, holding the device copies and the workspace.  Copies in,
  * compresses, copies out; returns after enqueueing (synchronise `stream` before
- * reading the outputs).  The (batch, KV head) pairs are independent (Sec. 4.1: every
- * head selects on its own), so they go through in up to eight parts: a part's
- * results are copied back on a side stream of the library while the next part's
- * inputs are still arriving on `stream`, and `stream` waits for the last copy back
- * before the call's work counts as complete.  The side stream and its events are
+ * reading the outputs; with pageable buffers the copies block the call).  The (batch, KV head) pairs are independent (Sec. 4.1: every
+ * head selects on its own), so they go through in up to eight parts, the copies in
+ * and the copies back on a side stream of the library each: a part's results leave
+ * while the next part computes on `stream` and the inputs of the one after arrive.
+ * `stream` waits for the last copy back before the call's work counts as complete.
+ * The side streams and their events are
  * created on the first call on a device and kept for the life of the process (make
  * that first call outside any stream capture); if they cannot be created everything
  * runs on `stream`.  The status block (snapkv_device_status on the workspace part of
@@ -329,7 +331,8 @@ snapkv_status_t snapkv_hit_counts(const float* a_cur, const int32_t* idx, int ro
  * bf16 products accumulated in fp32; the rows are split over many blocks and merged in a
  * fixed order, so results are reproducible run to run.  `workspace`: device memory of
  * snapkv_decode_workspace_size(B, Hq, rows, d) bytes, 256-byte aligned (0 from the size
- * query means unacceptable arguments); checked, not written.  Enqueued on `stream`: one kernel,
+ * query means unacceptable arguments); checked for callers' sake who sized it so, not
+ * written any more.  Enqueued on `stream`: one kernel,
  * no allocation.  Should a wait of the kernel exceed its time limit, the affected outputs are NaN.
  * d must be 64 or 128 (SNAPKV_ERR_UNSUPPORTED otherwise), B * Hq <= 65535.
  */
@@ -362,14 +365,14 @@ snapkv_status_t snapkv_device_status(const void* workspace, void* stream, int* d
  *   page_size       positions per page: a multiple of 128, so that a tile of 128 keys lies in
  *                   one page (SNAPKV_ERR_INVALID_ARG otherwise); pages_per_seq * page_size >= L.
  *   seq_lens        host int32[B] or NULL.  NULL: every sequence has L positions.  Otherwise
- *                   sequence b has seq_lens[b] in [W, L] positions and the call does one
- *                   single-sequence step per prompt (as snapkv_compress_varlen does), a
+ *                   sequence b has seq_lens[b] in [W, L] positions and is compressed as by
+ *                   snapkv_compress_varlen (up to 32 sequences share the launches), a
  *                   sequence with budget >= its length being copied through.
  *   lse_obs         optional, as in snapkv_compress_lse.
  * What lies in a page behind a sequence's last position is never used (it may be anything).
  * Outputs and workspace as for snapkv_compress (with seq_lens: as for
  * snapkv_compress_varlen; the workspace must hold snapkv_workspace_size(1, Hq, Hkv, L_b, ...)
- * of the longest sequence).  Results are bit-identical to snapkv_compress on a dense copy.
+ * of the longest sequence, snapkv_varlen_workspace_size bytes save launches).  Results are bit-identical to snapkv_compress on a dense copy.
  */
 snapkv_status_t snapkv_compress_paged(const void* q_obs, const void* k_pool, const void* v_pool,
                                       const int64_t* k_strides, const int64_t* v_strides,

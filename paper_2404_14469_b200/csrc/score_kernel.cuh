@@ -8,15 +8,15 @@
 //      When the unit has fewer than 128 window rows the rows are replicated along M and
 //      each replica takes a different slice of the tile's keys, so all four epilogue
 //      warps of a warpgroup stay busy.  Each CTA publishes one log2-sum-exp per window row
-//      for the keys it saw (its "partial") and bumps the unit's counter.
+//      for the keys it saw (its "partial") in a slot of the unit that is its own flag.
 //  pass V (votes)       S tile = K_tile[128 x d] . Q[ncols x d]^T : keys on TMEM lanes,
-//      window rows on columns.  Once the unit's counter shows that every partial has been
-//      published, the CTA folds them, in slot order, into one log2-sum-exp per window row;
+//      window rows on columns.  Once every slot of the unit has been written, the CTA folds
+//      the partials, in slot order, into one log2-sum-exp per window row;
 //      then each thread owns one key and adds exp2(s*c - lse) over the W columns of each
 //      head: the sum over the window is a serial add per thread.
 //
 // Units (batch, KV head, head sub-group) are grouped into waves small enough for L2; the
-// kernel walks the phases  S(0), S(1), V(0), S(2), V(1), ...  so that the second sweep
+// kernel walks the phases  S(0), S(1), V(0), S(2), V(1), ...  so that part of the second sweep
 // over a wave's keys is served by L2 and the partials a vote phase needs were published
 // a whole phase earlier.  Within a phase the wave's tiles are split evenly over the CTAs.
 // One CTA per SM and no more CTAs than SMs, so all of them are resident and waiting on
@@ -87,7 +87,7 @@ struct ScoreArgs {
   float c2;                 // log2(e) / sqrt(d)
   float* partials;          // [units][maxseg][MAX_COLS] log2-sum-exp of one CTA's share
   float* lse2;              // [units][MAX_COLS] minus the log2-sum-exp per window row, when supplied
-  int* counters;            // [units] published partials (a large value when lse2 was supplied)
+  int* counters;            // [units] partials of a statistics-only launch; above zero when lse2 was supplied
   int* status;
   float* vote;
 };
@@ -584,8 +584,8 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     // ------------------------------------------------------------ MMA issuer
     // One key tile per instruction.  Two tiles as one 128 x 256 x 16 instruction complete together:
     // both sets of softmax warps then wait for the tensor pipe at the same time and the
-    // exponentials stand still; tile by tile they take turns (198.1 -> 194.6 us per layer on the
-    // 32K GQA workload, 78.3 -> 76.7 us on the 16K MHA one).
+    // exponentials stand still; tile by tile they take turns (78.3 -> 76.7 us on the 16K MHA
+    // workload; the gain on the 32K GQA one is within its spread).
     if (elect_one()) {
       const uint32_t idesc_s = umma_idesc_bf16(128, 128);
       const uint32_t idesc_v = umma_idesc_bf16(128, NPAD);
@@ -844,7 +844,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     int nstat = 0, nvote = 0;
     auto keep = [&](const Item& it) {
       if (publisher) {
-        // merge the replicas and the two warpgroups (fixed order), publish, count
+        // merge the replicas and the two warpgroups (fixed order), publish
         const int pb = nstat % NPB;
         if (!mbar_wait_warp(bar_pf(pb), (nstat / NPB) & 1, abort_s, WAIT_PART_FULL)) return false;
         const float2* ps = part_s + pb * 16 * 32;
