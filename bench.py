@@ -26,29 +26,37 @@ if ROOT not in sys.path:
 import torch  # noqa: E402
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the committed ncu summaries
-# (profiles/): (stage, workload id) -> (bytes, source file of the kernel, first 12 hex digits of
-# that file's SHA-256 when the counters were taken).  A figure is reported only while the
-# kernel's source is unchanged; after any edit it reads null until the capture is redone.
+# (profiles/): (stage, workload id) -> (bytes, the source files that decide it, first 12 hex digits
+# of their SHA-256 when the counters were taken).  For the scoring kernel that is the plan on the host
+# side too: wave size and lag say how much of the second sweep comes from L2.  A figure is reported
+# only while the sources are unchanged; after any edit it reads null until the capture is redone.
+SCORE_SOURCES = ("score_kernel.cuh", "sm100_ptx.cuh", "snapkv_score.cu", "snapkv_internal.h")
 NCU_TRAFFIC = {
-    ("score", 2): (472.64e6, "score_kernel.cuh", "09728ac2de52"),
-    ("score-lse", 2): (274.65e6, "score_kernel.cuh", "09728ac2de52"),
-    ("gather", 2): (334.96e6, "snapkv_gather.cu", "ad8a2fd28b3e"),
+    ("score", 2): (475.75e6, SCORE_SOURCES, "1deb67de3738"),
+    ("score-lse", 2): (275.86e6, SCORE_SOURCES, "1deb67de3738"),
+    ("gather", 2): (335.18e6, ("snapkv_gather.cu",), "ad8a2fd28b3e"),
 }
 
 
-def ncu_traffic(stage, wid):
+def sources_digest(sources):
     import hashlib
+    h = hashlib.sha256()
+    for src in sources:
+        with open(os.path.join(ROOT, "paper_2404_14469_b200", "csrc", src), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:12]
+
+
+def ncu_traffic(stage, wid):
     ent = NCU_TRAFFIC.get((stage, wid))
     if ent is None:
         return None
-    nbytes, src, digest = ent
-    path = os.path.join(ROOT, "paper_2404_14469_b200", "csrc", src)
+    nbytes, sources, digest = ent
     try:
-        with open(path, "rb") as f:
-            now = hashlib.sha256(f.read()).hexdigest()[:12]
+        return nbytes if sources_digest(sources) == digest else None
     except OSError:
         return None
-    return nbytes if now == digest else None
+
 
 METRIC = "prompt_tokens_compressed_per_s"
 UNIT = "prompt tokens/s"
