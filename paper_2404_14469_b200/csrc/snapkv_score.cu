@@ -194,8 +194,9 @@ bool make_score_plan(int B, int Hq, int Hkv, int L, int d, int W, ScorePlan* pla
   // With 128 window columns on one unit per KV head a vote tile costs the same from L2 as from
   // HBM (the softmax warps are its bound), so nothing is lost by waves too big for L2, and fewer,
   // longer phases split more evenly over the CTAs: such shapes take waves of twice the size
-  // (191.6 vs 193.6 us per layer on the 32K GQA workload; narrower units and KV heads with
-  // two sub-groups, whose vote tiles do gain from L2, are 3-5 % slower that way).
+  // (191.6 vs 193.6 us per layer on the 32K GQA workload when the hand-over took longer, 193.1 vs
+  // 192.6 with the present one; narrower units and KV heads with two sub-groups, whose vote tiles
+  // do gain from L2, are 3-5 % slower that way).
   const long long wave_bytes = (p.ncols == 128 && p.sub_per_kv == 1) ? 2 * score::WAVE_BYTES : score::WAVE_BYTES;
   long long kv_per_wave = wave_bytes / kbytes;
   // units bigger than a wave run one per wave: their second sweep comes from HBM, but the
