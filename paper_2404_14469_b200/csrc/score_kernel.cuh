@@ -386,6 +386,11 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   constexpr int NPAD = NCH * 32;
   constexpr int REPS = 128 / NPAD;
   constexpr int NSET = SPLIT ? 2 : 1;  // sets of softmax warps
+  // In split mode the fetcher folds the columns in two halves, and the publisher takes one of them.
+  constexpr int HALVES = SPLIT && !RAGGED ? 2 : 1;
+  // (with more vote items in a phase than row buffers, the publisher would wait for the softmax warps
+  // to use up rows while they wait for it to publish)
+  const bool both_fold = HALVES == 2 && !a.votes_only && !a.stats_only && a.per <= NLB;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -434,7 +439,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       mbar_init(bar_pe(b), 1);
     }
     for (int b = 0; b < NLB; ++b) {
-      mbar_init(bar_lf(b), 1);
+      mbar_init(bar_lf(b), both_fold ? 2 : 1);
       mbar_init(bar_le(b), EPI_WARPS * NSET);
     }
     mbar_init(bar_drain, 1);
@@ -844,46 +849,50 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   } else {
     // ------------------------------------------------------------ book-keeper warps
     // Warp 10 publishes this CTA's statistics partials; warp 11 fetches the unit's partials
-    // for every vote item and folds them into the log-sum-exp row the item needs.  Each
-    // walks its own kind of item in schedule order, so publishing never waits for another
-    // CTA and the fetcher runs as far ahead as its shared-memory buffers allow.
+    // for every vote item and folds them into the log-sum-exp row the item needs, as far ahead
+    // as its shared-memory buffers allow.  A fold of 37 partials of 128 columns took one warp 5 us
+    // beside the softmax warps, which keep the special-function units busy, longer than a wave of a 13K
+    // prompt lasts; so it takes one exponential per partial, not two, and in split mode warp 10 folds
+    // the upper half of the columns once it has published a wave's partials.  All CTAs publish a wave
+    // before they fold it, so this wait too is for something that does not wait for it.
     const bool publisher = warp == 2 + EPI_WARPS;  // warp 10; warp 11 is the fetcher
+    constexpr int CPL = NCH / HALVES;              // columns per lane
     int nstat = 0, nvote = 0;
-    auto keep = [&](const Item& it) {
-      if (publisher) {
-        // merge the replicas and the two warpgroups (fixed order), publish
-        const int pb = nstat % NPB;
-        if (!mbar_wait_warp(bar_pf(pb), (nstat / NPB) & 1, abort_s, WAIT_PART_FULL)) return false;
-        const float2* ps = part_s + pb * 16 * 32;
-        for (int c = lane; c < NPAD; c += 32) {  // (padding columns too: a reader looks at all of them)
-          float M = -INFINITY;
-          for (int w2 = 0; w2 < 2 * NSET; ++w2)
-            for (int r = 0; r < REPS; ++r) {
-              const int row = r * NPAD + c;
-              M = fmaxf(M, ps[(w2 * 4 + (row >> 5)) * 32 + (row & 31)].x);
-            }
-          M = fmaxf(M, -1e30f);
-          float S = 0.f;
-          for (int w2 = 0; w2 < 2 * NSET; ++w2)
-            for (int r = 0; r < REPS; ++r) {
-              const int row = r * NPAD + c;
-              const float2 p = ps[(w2 * 4 + (row >> 5)) * 32 + (row & 31)];
-              S += p.y * ex2_approx(p.x - M);
-            }
-          // log2 of this CTA's share of the row's softmax normaliser (-inf if it saw no key)
-          const float part = M + log2f(S);
-          if (!a.withhold)
-            st_relaxed(slots_of(it) + static_cast<size_t>(it.slot) * MAX_COLS + c,
-                       __float_as_uint(part) == NO_PARTIAL ? __uint_as_float(0x7fffffffu) : part);
-        }
-        __syncwarp();  // every lane is done with the buffer
-        if (lane == 0) {
-          if (a.stats_only) atomicAdd(a.counters + unit_of(it), 1);  // for the kernel that folds a shard's partials
-          mbar_arrive(bar_pe(pb));
-        }
-        ++nstat;
-        return true;
+    auto publish = [&](const Item& it) {
+      // merge the replicas and the two warpgroups (fixed order), publish
+      const int pb = nstat % NPB;
+      if (!mbar_wait_warp(bar_pf(pb), (nstat / NPB) & 1, abort_s, WAIT_PART_FULL)) return false;
+      const float2* ps = part_s + pb * 16 * 32;
+      for (int c = lane; c < NPAD; c += 32) {  // (padding columns too: a reader looks at all of them)
+        float M = -INFINITY;
+        for (int w2 = 0; w2 < 2 * NSET; ++w2)
+          for (int r = 0; r < REPS; ++r) {
+            const int row = r * NPAD + c;
+            M = fmaxf(M, ps[(w2 * 4 + (row >> 5)) * 32 + (row & 31)].x);
+          }
+        M = fmaxf(M, -1e30f);
+        float S = 0.f;
+        for (int w2 = 0; w2 < 2 * NSET; ++w2)
+          for (int r = 0; r < REPS; ++r) {
+            const int row = r * NPAD + c;
+            const float2 p = ps[(w2 * 4 + (row >> 5)) * 32 + (row & 31)];
+            S += p.y * ex2_approx(p.x - M);
+          }
+        // log2 of this CTA's share of the row's softmax normaliser (-inf if it saw no key)
+        const float part = M + log2f(S);
+        if (!a.withhold)
+          st_relaxed(slots_of(it) + static_cast<size_t>(it.slot) * MAX_COLS + c,
+                     __float_as_uint(part) == NO_PARTIAL ? __uint_as_float(0x7fffffffu) : part);
       }
+      __syncwarp();  // every lane is done with the buffer
+      if (lane == 0) {
+        if (a.stats_only) atomicAdd(a.counters + unit_of(it), 1);  // for the kernel that folds a shard's partials
+        mbar_arrive(bar_pe(pb));
+      }
+      ++nstat;
+      return true;
+    };
+    auto fetch_half = [&](const Item& it, int half) {
       // Fetcher.  A vote item needs minus the log2-sum-exp of every window row of its unit.
       // With a supplied normaliser that row is in global memory already (its counter says so).
       // Otherwise it is the fold of the unit's partials.  A partial is its own flag: the slots hold
@@ -905,10 +914,10 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       // global memory: a fold of 20 partials takes this warp 3-5 us beside the softmax warps, and
       // with a vote item for every two or three tiles the folds would set the pace.
       const int lb = nvote % NLB;
-      const int c0 = lane * NCH;  // this lane's NCH columns of the window rows
-      float val[NCH];
+      const int c0 = (half * 32 + lane) * CPL;  // this lane's columns of the window rows
+      float val[CPL];
 #pragma unroll
-      for (int t = 0; t < NCH; ++t) val[t] = 0.f;
+      for (int t = 0; t < CPL; ++t) val[t] = 0.f;
       const unsigned long long t0 = globaltimer_ns();
       // half the limit: the roles of this CTA that wait for this row then still see the abort
       // flag, not their own time-out, and the status names the wait that failed
@@ -922,15 +931,15 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       };
       float* const row = a.lse2 + static_cast<size_t>(unit_of(it)) * MAX_COLS + c0;
       // whether a column of a row is missing
-      auto missing = [&](const float (&x)[NCH]) {
+      auto missing = [&](const float (&x)[CPL]) {
         uint32_t most = 0u;  // NO_PARTIAL is the largest of all bit patterns
 #pragma unroll
-        for (int t = 0; t < NCH; ++t) most = max(most, __float_as_uint(x[t]));
+        for (int t = 0; t < CPL; ++t) most = max(most, __float_as_uint(x[t]));
         return __any_sync(0xffffffffu, most == NO_PARTIAL);
       };
       if (RAGGED && !a.votes_only && it.vote) {
         for (;;) {
-          ld_relaxed<NCH>(row, val);
+          ld_relaxed<CPL>(row, val);
           if (!missing(val)) break;
           if (give_up()) return false;
           __nanosleep(100);
@@ -941,41 +950,42 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
           __nanosleep(100);
         }
 #pragma unroll
-        for (int t = 0; t < NCH; ++t)
+        for (int t = 0; t < CPL; ++t)
           if (c0 + t < a.ncols) val[t] = __ldcg(row + t);
       } else {
         const float* pp = slots_of(it);
         const uint32_t merge_addr = sbase + SM::OFF_MERGE;
-        float M[NCH], S[NCH];
+        float M[CPL], S[CPL];
 #pragma unroll
-        for (int t = 0; t < NCH; ++t) { M[t] = -1e30f; S[t] = 0.f; }
+        for (int t = 0; t < CPL; ++t) { M[t] = -1e30f; S[t] = 0.f; }
         // All slots at once, through shared memory: every round trip to L2 costs 0.8 us here, with
         // the other CTAs reading the same lines, and registers hold only a few slots.
         int s0 = 0;
         while (s0 < it.nseg) {
           const int ns = min(MERGE_SEGS, it.nseg - s0);
-          constexpr int CPS = NPAD / 4;  // 16-byte pieces per slot
+          constexpr int CPS = NPAD / 4 / HALVES;  // 16-byte pieces of this warp's columns per slot
+          const uint32_t mine = merge_addr + half * (CPS * 16);
           for (int p = lane; p < ns * CPS; p += 32)
-            copy16_async(merge_addr + (p / CPS) * (MAX_COLS * 4) + (p % CPS) * 16,
-                         pp + static_cast<size_t>(s0 + p / CPS) * MAX_COLS + (p % CPS) * 4);
+            copy16_async(mine + (p / CPS) * (MAX_COLS * 4) + (p % CPS) * 16,
+                         pp + static_cast<size_t>(s0 + p / CPS) * MAX_COLS + (half * CPS + p % CPS) * 4);
           // slots up to the next multiple of FOLD add nothing
           for (int p = ns * CPS + lane; p < (ns + FOLD - 1) / FOLD * FOLD * CPS; p += 32)
-            sts4(merge_addr + (p / CPS) * (MAX_COLS * 4) + (p % CPS) * 16, -INFINITY);
+            sts4(mine + (p / CPS) * (MAX_COLS * 4) + (p % CPS) * 16, -INFINITY);
           copy_wait_all();
           __syncwarp();
           int at = 0;
           for (; at < ns; at += FOLD) {
-            float x[FOLD][NCH];
+            float x[FOLD][CPL];
             uint32_t most = 0u;
 #pragma unroll
             for (int i = 0; i < FOLD; ++i) {
-              lds<NCH>(merge_addr + ((at + i) * MAX_COLS + c0) * 4, x[i]);
+              lds<CPL>(merge_addr + ((at + i) * MAX_COLS + c0) * 4, x[i]);
 #pragma unroll
-              for (int t = 0; t < NCH; ++t) most = max(most, __float_as_uint(x[i][t]));
+              for (int t = 0; t < CPL; ++t) most = max(most, __float_as_uint(x[i][t]));
             }
             if (__any_sync(0xffffffffu, most == NO_PARTIAL)) break;
 #pragma unroll
-            for (int t = 0; t < NCH; ++t) {
+            for (int t = 0; t < CPL; ++t) {
               float pv[FOLD];
 #pragma unroll
               for (int i = 0; i < FOLD; ++i) pv[i] = x[i][t];
@@ -988,17 +998,17 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
           // usually), then fetch again from the first that was missing.
           while (at < ns) {
             if (give_up()) return false;
-            float x[NCH];
-            ld_relaxed<NCH>(pp + static_cast<size_t>(it.nseg - 1) * MAX_COLS + c0, x);
+            float x[CPL];
+            ld_relaxed<CPL>(pp + static_cast<size_t>(it.nseg - 1) * MAX_COLS + c0, x);
             if (!missing(x)) break;
             __nanosleep(100);
           }
         }
 #pragma unroll
-        for (int t = 0; t < NCH; ++t) val[t] = -(M[t] + log2f(S[t]));
+        for (int t = 0; t < CPL; ++t) val[t] = -(M[t] + log2f(S[t]));
         if (RAGGED) {
 #pragma unroll
-          for (int t = 0; t < NCH; ++t)
+          for (int t = 0; t < CPL; ++t)
             st_relaxed(row + t, __float_as_uint(val[t]) == NO_PARTIAL ? __uint_as_float(0x7fffffffu) : val[t]);
           return true;
         }
@@ -1007,13 +1017,22 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       if (!mbar_wait_warp_relaxed(bar_le(lb), ((nvote / NLB) & 1) ^ 1, abort_s, WAIT_LSE_EMPTY))
         return false;
 #pragma unroll
-      for (int t = 0; t < NCH; ++t) lse_s[lb * MAX_COLS + c0 + t] = val[t];
+      for (int t = 0; t < CPL; ++t) lse_s[lb * MAX_COLS + c0 + t] = val[t];
+      return true;
+    };
+    auto fetch = [&](const Item& it) {  // this warp's columns
+      if (publisher || !both_fold) {
+        if (!fetch_half(it, HALVES - 1)) return false;
+      }
+      if (HALVES == 2 && !publisher) {
+        if (!fetch_half(it, 0)) return false;
+      }
+      if (RAGGED && !a.votes_only && !it.vote) return true;  // (a folded row went to global memory)
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar_lf(lb));
+      if (lane == 0) mbar_arrive(bar_lf(nvote % NLB));
       ++nvote;
       return true;
     };
-    // The publisher goes through the statistics items, the fetcher through the vote items.
     const int waves = (a.votes_only || a.stats_only) ? nphase : nphase / 2;
     bool go = publisher ? !a.votes_only : !a.stats_only;
     const bool folds = RAGGED && !publisher && !a.votes_only;
@@ -1025,11 +1044,15 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     for (int w = folds ? -1 : 0; w < waves && go; ++w) {
       for (int m = 0; m < a.per && go && folds && w + 1 < waves; ++m) {
         const Item it = item_at(2 * (w + 1), m);
-        if (it.t0 < it.t1 && it.slot == 0) go = keep(it);
+        if (it.t0 < it.t1 && it.slot == 0) go = fetch(it);
       }
-      for (int m = 0; m < a.per && go && w >= 0; ++m) {
-        const Item it = item_at(2 * w + (publisher ? 0 : 1), m);
-        if (it.t0 < it.t1) go = keep(it);
+      for (int m = 0; m < a.per && go && w >= 0 && publisher; ++m) {
+        const Item it = item_at(2 * w, m);
+        if (it.t0 < it.t1) go = publish(it);
+      }
+      for (int m = 0; m < a.per && go && w >= 0 && (!publisher || both_fold); ++m) {
+        const Item it = item_at(2 * w + 1, m);
+        if (it.t0 < it.t1) go = fetch(it);
       }
     }
   }
