@@ -390,7 +390,10 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   constexpr int HALVES = SPLIT && !RAGGED ? 2 : 1;
   // (with more vote items in a phase than row buffers, the publisher would wait for the softmax warps
   // to use up rows while they wait for it to publish)
-  const bool both_fold = HALVES == 2 && !a.votes_only && !a.stats_only && a.per <= NLB;
+  // With few partials per unit one warp is fast enough, and the publisher is better left alone: four
+  // prompts of 5316 with some 10 partials take 42.7 us so, 44.4 with both warps; one of 13013 with 37
+  // takes 40.1 and 38.7.
+  const bool both_fold = HALVES == 2 && !a.votes_only && !a.stats_only && a.per <= NLB && a.maxseg > 16;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -856,7 +859,6 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     // the upper half of the columns once it has published a wave's partials.  All CTAs publish a wave
     // before they fold it, so this wait too is for something that does not wait for it.
     const bool publisher = warp == 2 + EPI_WARPS;  // warp 10; warp 11 is the fetcher
-    constexpr int CPL = NCH / HALVES;              // columns per lane
     int nstat = 0, nvote = 0;
     auto publish = [&](const Item& it) {
       // merge the replicas and the two warpgroups (fixed order), publish
@@ -892,7 +894,10 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       ++nstat;
       return true;
     };
-    auto fetch_half = [&](const Item& it, int half) {
+    // Part `part` of the columns of a vote item's row, the whole row cut into as many as the constant says.
+    auto fetch_part = [&](const Item& it, auto parts, int part) {
+      constexpr int PARTS = decltype(parts)::value;
+      constexpr int CPL = NCH / PARTS;  // columns per lane
       // Fetcher.  A vote item needs minus the log2-sum-exp of every window row of its unit.
       // With a supplied normaliser that row is in global memory already (its counter says so).
       // Otherwise it is the fold of the unit's partials.  A partial is its own flag: the slots hold
@@ -914,7 +919,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       // global memory: a fold of 20 partials takes this warp 3-5 us beside the softmax warps, and
       // with a vote item for every two or three tiles the folds would set the pace.
       const int lb = nvote % NLB;
-      const int c0 = (half * 32 + lane) * CPL;  // this lane's columns of the window rows
+      const int c0 = (part * 32 + lane) * CPL;  // this lane's columns of the window rows
       float val[CPL];
 #pragma unroll
       for (int t = 0; t < CPL; ++t) val[t] = 0.f;
@@ -963,11 +968,11 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
         int s0 = 0;
         while (s0 < it.nseg) {
           const int ns = min(MERGE_SEGS, it.nseg - s0);
-          constexpr int CPS = NPAD / 4 / HALVES;  // 16-byte pieces of this warp's columns per slot
-          const uint32_t mine = merge_addr + half * (CPS * 16);
+          constexpr int CPS = NPAD / 4 / PARTS;  // 16-byte pieces of this warp's columns per slot
+          const uint32_t mine = merge_addr + part * (CPS * 16);
           for (int p = lane; p < ns * CPS; p += 32)
             copy16_async(mine + (p / CPS) * (MAX_COLS * 4) + (p % CPS) * 16,
-                         pp + static_cast<size_t>(s0 + p / CPS) * MAX_COLS + (half * CPS + p % CPS) * 4);
+                         pp + static_cast<size_t>(s0 + p / CPS) * MAX_COLS + (part * CPS + p % CPS) * 4);
           // slots up to the next multiple of FOLD add nothing
           for (int p = ns * CPS + lane; p < (ns + FOLD - 1) / FOLD * FOLD * CPS; p += 32)
             sts4(mine + (p / CPS) * (MAX_COLS * 4) + (p % CPS) * 16, -INFINITY);
@@ -1021,11 +1026,10 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
       return true;
     };
     auto fetch = [&](const Item& it) {  // this warp's columns
-      if (publisher || !both_fold) {
-        if (!fetch_half(it, HALVES - 1)) return false;
-      }
-      if (HALVES == 2 && !publisher) {
-        if (!fetch_half(it, 0)) return false;
+      if (HALVES == 2 && both_fold) {
+        if (!fetch_part(it, std::integral_constant<int, HALVES>{}, publisher ? 1 : 0)) return false;
+      } else {
+        if (!fetch_part(it, std::integral_constant<int, 1>{}, 0)) return false;
       }
       if (RAGGED && !a.votes_only && !it.vote) return true;  // (a folded row went to global memory)
       __syncwarp();
