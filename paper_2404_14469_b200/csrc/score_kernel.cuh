@@ -253,26 +253,26 @@ __host__ __device__ __forceinline__ uint32_t quotient(unsigned long long x, uint
 // each) are cut into G consecutive shares, the CTA playing part `cr` owning tiles
 // [cr*TT/G, (cr+1)*TT/G); a share that crosses a unit boundary is one item per unit.
 struct Share {
-  uint32_t lo, hi, pos;
+  uint32_t lo, hi;
   int u0, nu, T, T1, cr, G;
 
   __host__ __device__ __forceinline__ Share(int cr_, int G_, int u0_, int nu_, int T_, int T1_)
       : u0(u0_), nu(nu_), T(T_), T1(T1_), cr(cr_), G(G_) {
     const unsigned long long TT = static_cast<unsigned long long>(nu) * static_cast<uint32_t>(T);
-    lo = pos = quotient(static_cast<uint32_t>(cr) * TT, G);
+    lo = quotient(static_cast<uint32_t>(cr) * TT, G);
     hi = quotient(static_cast<uint32_t>(cr + 1) * TT, G);
   }
-  // The next item; an empty one (t0 = t1) behind the last.
-  __host__ __device__ __forceinline__ Item take() {
+  // Item m of the share, which ends where its unit does; an empty one (t0 = t1) behind the last.
+  __host__ __device__ __forceinline__ Item item(int m) const {
     Item it = {};
+    const uint32_t ul = lo / static_cast<uint32_t>(T) + static_cast<uint32_t>(m);
+    const uint32_t pos = m == 0 ? lo : ul * static_cast<uint32_t>(T);
     if (pos >= hi) return it;
-    const uint32_t ul = pos / static_cast<uint32_t>(T);
     it.unit = u0 + static_cast<int>(ul);
     it.t0 = static_cast<int>(pos - ul * static_cast<uint32_t>(T));
     const uint32_t t1 = static_cast<uint32_t>(it.t0) + (hi - pos);
     it.t1 = t1 < static_cast<uint32_t>(T) ? static_cast<int>(t1) : T;
     it.flip = static_cast<int>((pos - lo) & 1);  // tiles of this phase that this block has had before
-    pos += static_cast<uint32_t>(it.t1 - it.t0);
     // where this CTA's partial of the unit goes and how many partials the unit gets follow from
     // the statistics-pass partition of the unit's wave
     const uint32_t T1u = static_cast<uint32_t>(T1), TT1 = static_cast<uint32_t>(nu) * T1u;
@@ -425,6 +425,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   const int G = gridDim.x;
 
   if (threadIdx.x == 0) {
+    // (the descriptors come with the launch: no need to wait for the previous kernel)
+    if constexpr (!RAGGED) tma_prefetch_desc(&tmK);
+    tma_prefetch_desc(&tmQ);
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(bar_full(s), 1);
       mbar_init(bar_empty(s), 1);
@@ -450,25 +453,24 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     *reinterpret_cast<volatile unsigned long long*>(abort_s + 1) = a.wait_ns;
     mbar_fence_init();
   }
-  // The work items of this CTA, a phase per thread: `per` records for each wave in each sweep and
+  // The work items of this CTA, one per thread: `per` records for each wave in each sweep and
   // the order of the phases.  (Walking the list cost a single thread 2500 cycles of divisions an
   // item, in every role: a ragged batch of short prompts did little else.)
   ItemRecord* items_s = reinterpret_cast<ItemRecord*>(smem + SM::OFF_ITEMS);
   uint16_t* order_s = reinterpret_cast<uint16_t*>(smem + SM::OFF_ORDER);
   const int nphase = phase_count(a, rs);
   // (warps 0 and 1 are busy with the barriers and the tensor memory)
-  for (int p = static_cast<int>(threadIdx.x) - 64; p >= 0 && p < nphase; p += threads_for(SPLIT) - 64) {
+  for (int i = static_cast<int>(threadIdx.x) - 64; i >= 0 && i < nphase * a.per; i += threads_for(SPLIT) - 64) {
+    const int m = i / nphase, p = i - m * nphase;
     const Phase ph = phase_at(a, rs, G, p);
-    order_s[p] = static_cast<uint16_t>(2 * ph.ord + ph.vote);
-    Share share = share_of(a, rs, ph, cta, G);
+    if (m == 0) order_s[p] = static_cast<uint16_t>(2 * ph.ord + ph.vote);
+    const Share share = share_of(a, rs, ph, cta, G);
     const int before = tiles_before(a, rs, ph, cta, G);
-    for (int m = 0; m < a.per; ++m) {
-      const Item it = share.take();
-      items_s[(2 * ph.ord + ph.vote) * a.per + m] =
-          ItemRecord{static_cast<uint32_t>(it.unit) | static_cast<uint32_t>(ph.seq) << 24 |
-                         static_cast<uint32_t>((it.flip + before) & 1) << 31,
-                     it.t0, it.t1, static_cast<uint32_t>(it.slot) | static_cast<uint32_t>(it.nseg) << 16};
-    }
+    const Item it = share.item(m);
+    items_s[(2 * ph.ord + ph.vote) * a.per + m] =
+        ItemRecord{static_cast<uint32_t>(it.unit) | static_cast<uint32_t>(ph.seq) << 24 |
+                       static_cast<uint32_t>((it.flip + before) & 1) << 31,
+                   it.t0, it.t1, static_cast<uint32_t>(it.slot) | static_cast<uint32_t>(it.nseg) << 16};
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_ptr_s)), TMEM_COLS);
@@ -527,8 +529,6 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (elect_one()) {
-      if constexpr (!RAGGED) tma_prefetch_desc(&tmK);
-      tma_prefetch_desc(&tmQ);
       const uint64_t pol_first = l2_policy_evict_first();
       int git = 0;      // tiles issued so far (ring position)
       int nitem = 0;    // items started so far (Q buffer position)

@@ -132,8 +132,9 @@ int list_ragged_items(const RaggedBatch& rb, int W, int Hkv, int votes_only, int
   int count = 0;
   for (int p = 0; p < score::phase_count(a, rs); ++p) {
     const score::Phase ph = score::phase_at(a, rs, grid, p);
-    score::Share share = score::share_of(a, rs, ph, cta, grid);
-    for (score::Item it = share.take(); it.t0 < it.t1; it = share.take(), ++count) {
+    const score::Share share = score::share_of(a, rs, ph, cta, grid);
+    int m = 0;
+    for (score::Item it = share.item(0); it.t0 < it.t1; it = share.item(++m), ++count) {
       if (count >= max_items) continue;
       int32_t* o = out + static_cast<size_t>(count) * 8;
       o[0] = it.unit; o[1] = it.t0; o[2] = it.t1; o[3] = ph.vote; o[4] = it.slot; o[5] = it.nseg;
