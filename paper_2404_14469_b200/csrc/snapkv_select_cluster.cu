@@ -106,11 +106,17 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t* warp_sums_s
 }
 
 struct OneLength {};
-struct RaggedRows {  // rows seq * heads + h: head h of the batch's sequence batch[seq]
+// Rows seq * heads + h: head h of the batch's sequence batch[seq].  A batch's long and short rows may be
+// two launches with CTAs of different sizes, side by side: the first (`lets_in`) lets the second in
+// as soon as its own wait for the votes is over, so the second finds them complete and does not wait
+// for the first until it ends itself (`after`); the gather kernel, which waits for the second, then
+// finds both complete.
+struct RaggedRows {
   int n[RAGGED_MAX], batch[RAGGED_MAX];
   int2 want[RAGGED_MAX];
   long long vote0[RAGGED_MAX];
   int heads;
+  bool lets_in, after;
 };
 
 // Sliding pooling of eight positions: out[i] over a[i .. i + 2R].  The maximum is taken over
@@ -191,7 +197,12 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
   }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int c0 = static_cast<int>(rank) * CHUNK;  // first position of this CTA's chunk
-  pdl_wait();
+  if constexpr (std::is_same<ROWS, RaggedRows>::value) {
+    if (!rows.after) pdl_wait();
+    if (rows.lets_in) pdl_launch_dependents();
+  } else {
+    pdl_wait();
+  }
   if (meta != nullptr && meta[static_cast<size_t>(row) * LONG_META + LONG_DONE]) return;
   if (C > 1) cluster_arrive();  // waited for before the first access to a peer's memory
 
@@ -580,6 +591,9 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
   __syncthreads();
   orow += gt0 + kept0;
   for (uint32_t i = tid; i < mine; i += THREADS) orow[i] = static_cast<int32_t>(stage[i]);
+  if constexpr (std::is_same<ROWS, RaggedRows>::value) {
+    if (rows.after) pdl_wait();
+  }
 }
 
 // Long rows of which few positions are kept: a cluster that holds a row in registers needs so many
@@ -1107,22 +1121,36 @@ cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int poo
   return cudaGetLastError();
 }
 
-// Shape for the rows of a ragged batch (a cluster has as many CTAs as the longest row needs, those
-// that a shorter row does not need leave at once).
-static ClusterShape ragged_shape(int n) {
-  if (n <= 2048) return {256, 8, 1};
-  if (n <= 4096) return {512, 8, 1};
-  if (n <= 8192) return {1024, 8, 1};
-  if (n <= 8 * 16384) return {1024, 16, (n + 16383) / 16384};
-  return {1024, 32, (n + 32767) / 32768};
+// Shape for rows of a ragged batch, `heads` of each of the lengths n, the longest first (a cluster has
+// as many CTAs as that one needs, those that a shorter row does not need leave at once): the smallest
+// estimated time, as for rows of one length.  128 rows of 8046 to 23968 take one round of CTAs with 32
+// keys a thread (16 us) where clusters of two with 16 keys a thread took two (22 us).
+constexpr int RAGGED_SHORT = 4096;  // rows up to here take a CTA of 256 or 512 threads
+static ClusterShape ragged_shape(const int* n, int count, int heads) {
+  if (n[0] <= 2048) return {256, 8, 1};
+  if (n[0] <= RAGGED_SHORT) return {512, 8, 1};
+  const int ept[3] = {8, 16, 32};
+  const double alone[3] = {8.0, 10.5, 16.5}, shared[3] = {10.2, 12.5, 20.0};
+  ClusterShape best = {1024, 32, 0, 1e30};
+  for (int i = 0; i < 3; ++i) {
+    const int chunk = 1024 * ept[i], c = (n[0] + chunk - 1) / chunk;
+    if (c > CL_MAX_CLUSTER) continue;
+    const int fit = clusters_at_once(c);
+    if (fit < 1) continue;
+    long long ctas = 0;
+    for (int j = 0; j < count; ++j) ctas += static_cast<long long>(heads) * ((n[j] + chunk - 1) / chunk);
+    const long long at_once = static_cast<long long>(fit) * c;
+    const double us = static_cast<double>((ctas + at_once - 1) / at_once) * (c == 1 ? alone[i] : shared[i] + 0.35 * c);
+    if (us < best.us) best = {1024, ept[i], c, us};
+  }
+  return best;
 }
 
 // Whether the rows of a ragged batch, the longest of n_max positions, can share a launch.
 bool ragged_select_applies(int n_max, int pool_kernel, int pool_type) {
   if ((pool_kernel >> 1) > CL_RMAX || n_max > CL_MAX_CLUSTER * 1024 * 32) return false;
   if (pool_type == 1 && n_max > 131072) return false;  // two ways of ranking in one launch
-  const int ctas = ragged_shape(n_max).ctas;
-  return ctas <= 8 || clusters_at_once(ctas) > 0;
+  return ragged_shape(&n_max, 1, 1).ctas > 0;
 }
 
 cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int Hq, int W, int pool_kernel,
@@ -1134,19 +1162,35 @@ cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int H
     for (; at > 0 && rb.L[order[at - 1]] < rb.L[i]; --at) order[at] = order[at - 1];
     order[at] = i;
   }
-  RaggedRows rows = {};
-  rows.heads = Hq;
-  for (int i = 0; i < rb.count; ++i) {
-    const int o = order[i], n = rb.L[o] - W;
-    rows.n[i] = n;
-    rows.batch[i] = rb.batch[o];
-    rows.want[i] = window_ranks(ksel, n);
-    rows.vote0[i] = rb.vote0[o];
+  // Where the long rows alone are estimated to take less time, because they come in fewer rounds or can
+  // have more CTAs each, the short ones are a launch of their own behind them: a CTA of 1024 threads has an SM to itself and takes 10 us however short its row is,
+  // and the small CTAs fit where the long rows' last round leaves SMs over.  (Eight sequences of 822
+  // to 24000: 143 us in one launch, 132 in two; sixteen of 300 to 20000 with 8 heads 104.7 and 97.0.
+  // Four of 400 to 12283, which take one round either way: 52.4 and 53.4.)
+  int n[RAGGED_MAX], longer = 0;
+  for (int i = 0; i < rb.count; ++i) n[i] = rb.L[order[i]] - W;
+  while (longer < rb.count && n[longer] > RAGGED_SHORT) ++longer;
+  if (longer > 0 && longer < rb.count && ragged_shape(n, longer, Hq).us + 1.0 >= ragged_shape(n, rb.count, Hq).us) longer = 0;
+  for (int first = 0; first < rb.count;) {
+    const int last = first < longer ? longer : rb.count;
+    RaggedRows rows = {};
+    rows.heads = Hq;
+    rows.lets_in = last < rb.count;
+    rows.after = first > 0;
+    for (int i = first; i < last; ++i) {
+      rows.n[i - first] = n[i];
+      rows.batch[i - first] = rb.batch[order[i]];
+      rows.want[i - first] = window_ranks(ksel, n[i]);
+      rows.vote0[i - first] = rb.vote0[order[i]];
+    }
+    const ClusterShape shape = ragged_shape(rows.n, last - first, Hq);
+    if (shape.ctas < 1) return cudaErrorInvalidValue;  // (callers ask ragged_select_applies)
+    const SelectCall c = {vote, (last - first) * Hq, rows.n[0], 1, pool_kernel >> 1, pool_type, 0.f, ksel, out_idx, 1, stream};
+    const cudaError_t e = launch_rows(shape, c, rows);
+    if (e != cudaSuccess) return e;
+    *launches += 1;
+    first = last;
   }
-  const SelectCall c = {vote, rb.count * Hq, rows.n[0], 1, pool_kernel >> 1, pool_type, 0.f, ksel, out_idx, 1, stream};
-  const cudaError_t e = launch_rows(ragged_shape(rows.n[0]), c, rows);
-  if (e != cudaSuccess) return e;
-  *launches += 1;
   return cudaGetLastError();
 }
 

@@ -176,3 +176,40 @@ def test_a_workspace_from_a_smaller_batch_does_not_cost_launches():
         got, launches = call(large, own)
         assert got[3] is own and all(torch.equal(x, y) for x, y in zip(got[:3], want[:3]))
         assert (launches - fewest) // 3 == sets - 1       # preparation, scores, selection per set; one gather
+
+
+@pytest.mark.parametrize("lens,ptype,kernel,selects", [
+    # rows of 4097 and more, and up to 4096 and 2048, in two launches side by side; the last ones all long or all in one
+    ([700, 20000, 4128, 2081, 9000, 4129, 2080, 4127], "max", 7, 2),
+    ([24000, 1400, 23000, 8000, 1500, 21000], "avg", 5, 2),
+    ([12283, 900, 2990, 2867], "max", 5, 1),
+    ([17000, 16416, 8225, 8224, 33000], "max", 13, 1),
+])
+def test_rows_of_a_ragged_batch_in_one_or_two_select_launches(lens, ptype, kernel, selects):
+    Hq, Hkv, d, W, budget = 32, 8, 64, 32, 512
+    g = torch.Generator(device="cuda").manual_seed(sum(lens))
+    seqs = [{x: torch.randn(*sh, generator=g, device="cuda").to(torch.bfloat16)
+             for x, sh in (("q", (1, Hq, W, d)), ("k", (1, Hkv, L, d)), ("v", (1, Hkv, L, d)))} for L in lens]
+    k, v = (torch.cat([s[x][0].permute(1, 0, 2) for s in seqs]).contiguous() for x in "kv")
+    q = torch.cat([s["q"] for s in seqs])
+    cu = [sum(lens[:b]) for b in range(len(lens))]
+    want = [sk.snapkv_compress(s["q"], s["k"], s["v"], kernel, PT[ptype], budget)[:3] for s in seqs]
+
+    def call(ws):
+        return sk.snapkv_compress_varlen(q, k, v, lens, kernel, PT[ptype], budget, cu_seqlens=cu, workspace=ws)
+
+    got = call(None)
+    assert sk.snapkv_last_launch_count() == 3 + selects  # preparation, scores, selection, gather
+    runs = [got] + [call(got[3]) for _ in range(3)]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        captured = call(got[3])
+    for _ in range(3):
+        for x in captured[:3]:
+            x.zero_()
+        graph.replay()
+    runs.append(captured)
+    for run in runs:
+        for b in range(len(lens)):
+            assert all(torch.equal(x[b], y[0]) for x, y in zip(run[:3], want[b]))
