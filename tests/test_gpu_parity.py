@@ -614,3 +614,26 @@ def test_prompts_a_little_longer_than_the_budget():
             ref = orc.compress(*(_bits(data[b][x]) for x in ("q_obs", "k", "v")), kernel, orc.POOL_MAX, budget)
             for h in range(Hq):
                 parity.check_indices(oi[b, h].cpu().numpy(), ref["pooled"][0, h], budget - W, ref["out_idx"][0, h])
+
+
+@pytest.mark.parametrize("rows,n,kernel,ptype", [
+    (128, 32736, 5, "avg"), (100, 32768, 7, "max"), (140, 17001, 13, "max"),   # 32 keys a thread
+    (128, 16384, 7, "max"), (120, 16383, 5, "avg"), (148, 8193, 3, "max"),     # 16 keys a thread
+    (3, 131001, 7, "max"), (40, 65537, 5, "max"),                              # clusters of several such blocks
+])
+def test_select_with_many_keys_per_thread(rows, n, kernel, ptype):
+    # votes that are small multiples of 1/64: every sum is exact, ties abound and go to the lower position
+    g = torch.Generator(device="cuda").manual_seed(rows + n)
+    r = kernel // 2
+    for levels in (64, 4096):
+        vote = torch.randint(0, levels, (rows, n), generator=g, device="cuda").float() / 64
+        if levels == 64:
+            vote[:, : n // 2] = 0  # half of a row equal: blocks and lanes that keep all or nothing
+        pad = torch.nn.functional.pad(vote, (r, r))
+        taps = torch.stack([pad[:, t:t + n] for t in range(kernel)])
+        pooled = taps.amax(0) if ptype == "max" else taps.sum(0)
+        order = torch.sort(pooled, dim=1, descending=True, stable=True)[1]
+        for ksel in (1, n // 8, n // 2 + n // 3, n - 1, n):
+            want = torch.sort(order[:, :ksel], dim=1)[0].int()
+            got = sk.snapkv_pool_topk(vote, kernel, sk.POOL_MAX if ptype == "max" else sk.POOL_AVG, ksel)
+            assert torch.equal(got.view(rows, ksel), want)
