@@ -221,22 +221,15 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
       const int j = js + t - R;
       tap[t] = static_cast<unsigned>(j) < static_cast<unsigned>(n) ? __ldg(vrow + j) : 0.f;
     }
-    for (int g = 1; g < gsum; ++g) {
-      const float* src = vrow + static_cast<size_t>(g) * n;
-#pragma unroll
-      for (int t = 0; t <= 2 * R; ++t) {
-        const int j = js + t - R;
-        if (static_cast<unsigned>(j) < static_cast<unsigned>(n)) tap[t] += __ldg(src + j);
-      }
-    }
   }
   float h_val = 0.f;
+  int h_at = -1;  // the halo position this thread fetches
   if (tid >= THREADS - 2 * CL_RMAX) {
     const int i = tid - (THREADS - 2 * CL_RMAX);
     const int j = i < CL_RMAX ? c0 - CL_RMAX + i : c0 + CHUNK + i - CL_RMAX;
     if (static_cast<unsigned>(j) < static_cast<unsigned>(n)) {
+      h_at = j;
       h_val = __ldg(vrow + j);
-      for (int g = 1; g < gsum; ++g) h_val += __ldg(vrow + static_cast<size_t>(g) * n + j);
     }
   }
   {
@@ -251,10 +244,33 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
         x[u] = j < n ? __ldg(vrow + j) : 0.f;
       }
     }
+    // Of each further head the sample, the halo and the first keys are requested before any is added:
+    // one round trip a head, not one for the sample and one for the chunk.
     for (int g = 1; g < gsum; ++g) {
       const float* src = vrow + static_cast<size_t>(g) * n;
+      float t2[2 * R + 1], y[8], h2 = 0.f;
+      if (tid < CL_SAMPLES) {
 #pragma unroll
-      for (int u = 0; u < EPT; ++u) {
+        for (int t = 0; t <= 2 * R; ++t) {
+          const int j = js + t - R;
+          t2[t] = static_cast<unsigned>(j) < static_cast<unsigned>(n) ? __ldg(src + j) : 0.f;
+        }
+      }
+      if (h_at >= 0) h2 = __ldg(src + h_at);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int j = c0 + tid + THREADS * u;
+        y[u] = j < n ? __ldg(src + j) : 0.f;
+      }
+      if (tid < CL_SAMPLES) {
+#pragma unroll
+        for (int t = 0; t <= 2 * R; ++t) tap[t] += t2[t];
+      }
+      h_val += h2;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) x[u] += y[u];
+#pragma unroll
+      for (int u = 8; u < EPT; ++u) {
         const int j = c0 + tid + THREADS * u;
         if (j < n) x[u] += __ldg(src + j);
       }
