@@ -392,8 +392,11 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   // to use up rows while they wait for it to publish)
   // With few partials per unit one warp is fast enough, and the publisher is better left alone: four
   // prompts of 5316 with some 10 partials take 42.7 us so, 44.4 with both warps; one of 13013 with 37
-  // takes 40.1 and 38.7.
-  const bool both_fold = HALVES == 2 && !a.votes_only && !a.stats_only && a.per <= NLB && a.maxseg > 16;
+  // takes 40.1 and 38.7.  A single unit is left to one warp too: alone it would take 22.8 us instead of
+  // 24.8 (8192 positions), but the parts of a call on host buffers are such launches, and between the
+  // copies they cost more than they gain (966-988 us against 932-940).
+  const bool both_fold =
+      HALVES == 2 && !a.votes_only && !a.stats_only && a.per <= NLB && a.maxseg > 16 && a.units > 1;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
