@@ -3,13 +3,16 @@ statistics between its blocks (Eq. 1 needs each window row's normaliser over ALL
 any probability can be summed, so blocks that share a unit exchange partial log-sum-exps).
 
 The item lists come from the library itself (snapkv_schedule_items and its counterpart for ragged
-batches run the kernel's own item walk on the host).  The hand-over is modelled with two CPU threads
-per block, as the kernel has warps: one walks the items, computes statistics and writes partials (a
-written slot is its own flag) and adds up votes; the other fetches, for every vote item, the unit's row:
-it looks until every slot is written, with a time limit, and folds them in slot order.  In a ragged
-batch the block with slot 0 folds, one wave ahead of the votes, and the others wait for its row.  The
-model shows that the schedule cannot deadlock, that every block gets the same row whatever the thread
-timing, and that a block which never arrives turns into time-outs, not into a hang."""
+batches run the kernel's own item walk on the host).  The hand-over is modelled with three CPU threads
+per block, as the kernel has warps: one walks the items, leaves its statistics in two buffers and adds up
+votes; the publisher takes them from there and writes the partials (a written slot is its own flag); the
+fetcher provides, for every vote item, the unit's row, eight rows ahead at most: it looks until every slot
+is written, with a time limit, and folds them in slot order.  Where the fold is shared the publisher folds
+the upper half of each row of a wave once it has published the wave's partials, and a row is there when
+both halves are.  In a ragged batch the block with slot 0 folds, one wave ahead of the votes, and the
+others wait for its row.  The model shows that the schedule cannot deadlock, that every block gets the
+same row whatever the thread timing, that a block which never arrives turns into time-outs, not into a
+hang, and that a phase with more vote items than row buffers must not share the fold."""
 import queue
 import threading
 import time
@@ -138,30 +141,43 @@ def test_statistics_of_the_next_wave_come_before_a_waves_votes(lens, Hq, Hkv, d,
                 assert not any(v == 0 and w <= wave + 1 for w, v in order[at:])
 
 
-class _Model:
-    """Two threads per block; `absent` blocks never run.  Items are (unit key, vote, slot, nseg, wave)."""
+PARTIAL_BUFFERS, ROW_BUFFERS = 2, 8
 
-    def __init__(self, per_cta, limit_s, ragged):
-        self.per_cta, self.limit, self.ragged = per_cta, limit_s, ragged
+
+class _Model:
+    """Three threads per block; `absent` blocks never run.  Items are (unit key, vote, slot, nseg, wave).
+    `shared`: the publisher folds the upper halves."""
+
+    def __init__(self, per_cta, limit_s, ragged, shared):
+        self.per_cta, self.limit, self.ragged, self.shared = per_cta, limit_s, ragged, shared
         self.slots, self.rows = {}, {}                    # (key, slot) -> partial; key -> row
         self.abort = [0] * len(per_cta)
         self.got = [[] for _ in per_cta]
+        self.waves = 1 + max(x[4] for items in per_cta for x in items)
 
-    def _wait(self, c, ready):
-        t_end = time.monotonic() + self.limit / 2         # a wait on other blocks: half the limit
+    def _wait(self, c, ready, limit, code):
+        t_end = time.monotonic() + limit
         while not ready():
             if self.abort[c]:
                 return False
             if time.monotonic() > t_end:
-                self.abort[c] = 7                         # the code of the wait for a unit's statistics
+                self.abort[c] = self.abort[c] or code
                 return False
             time.sleep(1e-4)
         return True
 
-    def _fold(self, c, key, nseg):
-        if not self._wait(c, lambda: all((key, s) in self.slots for s in range(nseg))):
+    # waits inside a block; the codes are the kernel's
+    def _put(self, c, q, x, code):
+        return self._wait(c, lambda: not q.full(), self.limit, code) and (q.put(x) or True)
+
+    def _get(self, c, q, code):
+        return q.get() if self._wait(c, lambda: not q.empty(), self.limit, code) else None
+
+    # waits for other blocks: half the limit, and the code of the wait for a unit's statistics
+    def _fold(self, c, key, nseg, half):
+        if not self._wait(c, lambda: all((key, s) in self.slots for s in range(nseg)), self.limit / 2, 7):
             return None
-        acc = 0
+        acc = half
         for s in range(nseg):                             # slot order: the same in every block
             acc = acc * 31 + self.slots[key, s]
         return acc
@@ -169,54 +185,62 @@ class _Model:
     def _items(self, c, vote, wave):
         return [x for x in self.per_cta[c] if x[1] == vote and x[4] == wave]
 
-    def fetcher(self, c, out):
-        waves = 1 + max(x[4] for items in self.per_cta for x in items)
-        for w in range(-1 if self.ragged else 0, waves):
+    def publisher(self, c, partials, upper):
+        for w in range(self.waves):
+            for key, _, slot, _, _ in self._items(c, 0, w):
+                got = self._get(c, partials, 9)
+                if got is None:
+                    return
+                assert got[0] == (key, slot), "partials come in the order of the items"
+                self.slots[got[0]] = got[1]
+            for key, _, _, nseg, _ in self._items(c, 1, w) if self.shared else ():
+                row = self._fold(c, key, nseg, 1)
+                if row is None or not self._put(c, upper, (key, row), 11):
+                    return
+
+    def fetcher(self, c, lower):
+        for w in range(-1 if self.ragged else 0, self.waves):
             if self.ragged:
                 for key, _, slot, nseg, _ in self._items(c, 0, w + 1):
                     if slot == 0:
-                        row = self._fold(c, key, nseg)
+                        row = self._fold(c, key, nseg, 0)
                         if row is None:
                             return
                         self.rows[key] = row
             for key, _, _, nseg, _ in self._items(c, 1, w):
                 if self.ragged:
-                    row = self.rows[key] if self._wait(c, lambda: key in self.rows) else None
+                    row = self.rows[key] if self._wait(c, lambda: key in self.rows, self.limit / 2, 7) else None
                 else:
-                    row = self._fold(c, key, nseg)
-                if row is None:
+                    row = self._fold(c, key, nseg, 0)
+                if row is None or not self._put(c, lower, (key, row), 11):
                     return
-                while not self.abort[c]:
-                    try:
-                        out.put((key, row), timeout=0.01)  # eight buffers
-                        break
-                    except queue.Full:
-                        pass
 
-    def softmax(self, c, rows, jitter):
+    def softmax(self, c, partials, halves, jitter):
         for k, (key, vote, slot, nseg, wave) in enumerate(self.per_cta[c]):
             if jitter:
                 time.sleep(((c * 7 + k * 3) % 5) * 1e-4)
-            if not vote:
-                self.slots[key, slot] = (hash(key) % 1009 + 1) * 1000 + slot   # stands for the block's partial
+            if not vote:                                  # (the number stands for the block's partial)
+                if not self._put(c, partials, ((key, slot), (hash(key) % 1009 + 1) * 1000 + slot), 8):
+                    return
                 continue
-            while True:
-                try:
-                    got = rows.get(timeout=0.01)
-                    break
-                except queue.Empty:
-                    if self.abort[c]:
-                        return
-            assert got[0] == key, "rows come in the order of the items"
-            self.got[c].append(got)
+            row = ()
+            for half in halves:                           # a row is there when all its parts are
+                got = self._get(c, half, 10)
+                if got is None:
+                    return
+                assert got[0] == key, "rows come in the order of the items"
+                row += (got[1],)
+            self.got[c].append((key, row))
 
     def run(self, absent=(), jitter=True):
         threads = []
         for c in range(len(self.per_cta)):
             if c not in absent:
-                rows = queue.Queue(maxsize=8)
-                threads += [threading.Thread(target=self.fetcher, args=(c, rows)),
-                            threading.Thread(target=self.softmax, args=(c, rows, jitter))]
+                partials = queue.Queue(maxsize=PARTIAL_BUFFERS)
+                halves = [queue.Queue(maxsize=ROW_BUFFERS) for _ in range(2 if self.shared else 1)]
+                threads += [threading.Thread(target=self.fetcher, args=(c, halves[0])),
+                            threading.Thread(target=self.publisher, args=(c, partials, halves[-1])),
+                            threading.Thread(target=self.softmax, args=(c, partials, halves, jitter))]
         t0 = time.monotonic()
         for t in threads:
             t.start()
@@ -226,26 +250,30 @@ class _Model:
         return time.monotonic() - t0
 
 
-def _model(shape, limit_s):
+def _model(shape, limit_s, shared=False):
     """Of one length (B, Hq, Hkv, L, d, W, grid) or of a ragged batch ([lengths], Hq, Hkv, d, W, grid)."""
     if isinstance(shape[0], list):
         items = [[((x[6], x[0]), x[3], x[4], x[5], x[7]) for x in sk.ragged_schedule_items(*shape, c)]
                  for c in range(shape[-1])]
-        return _Model(items, limit_s, True)
+        return _Model(items, limit_s, True, shared)
     per_cta, plan = _all_items(*shape)
     return _Model([[(x[0], x[3], x[4], x[5], x[0] // plan["units_per_wave"]) for x in items] for items in per_cta],
-                  limit_s, False)
+                  limit_s, False, shared)
 
 
+# (shape, whether the fold is shared)
 HAND_OVER = [
-    (2, 8, 2, 3000, 128, 32, 24), (1, 4, 4, 1024, 64, 32, 40),
-    ([3000, 700, 150, 1200, 90], 8, 2, 128, 32, 24), ([60000, 50000], 16, 8, 128, 32, 16),
+    ((2, 8, 2, 3000, 128, 32, 24), False), ((1, 4, 4, 1024, 64, 32, 40), False),
+    (([3000, 700, 150, 1200, 90], 8, 2, 128, 32, 24), False), (([60000, 50000], 16, 8, 128, 32, 16), False),
+    ((2, 8, 2, 3000, 128, 32, 24), True),
+    ((1, 8, 4, 250000, 128, 32, 24), True),   # four waves, 24 partials per unit
+    ((48, 32, 8, 300, 128, 32, 19), True),    # three waves, phases with as many vote items as row buffers
 ]
 
 
-@pytest.mark.parametrize("shape", HAND_OVER)
-def test_hand_over_completes_and_every_block_folds_the_same_value(shape):
-    m = _model(shape, limit_s=10.0)
+@pytest.mark.parametrize("shape,shared", HAND_OVER)
+def test_hand_over_completes_and_every_block_folds_the_same_value(shape, shared):
+    m = _model(shape, limit_s=10.0, shared=shared)
     m.run()
     assert not any(m.abort)
     by_unit = {}
@@ -257,9 +285,30 @@ def test_hand_over_completes_and_every_block_folds_the_same_value(shape):
     assert [len(g) for g in m.got] == [sum(x[1] for x in items) for items in m.per_cta]
 
 
-@pytest.mark.parametrize("shape", HAND_OVER[::2])
-def test_a_block_that_never_arrives_becomes_time_outs_not_a_hang(shape):
-    m = _model(shape, limit_s=0.4)
+def test_the_shapes_of_the_shared_fold_have_what_they_are_for():
+    many = _model(HAND_OVER[5][0], 1.0)
+    assert many.waves == 4 and {x[3] for items in many.per_cta for x in items} == {24}
+    full = _model(HAND_OVER[6][0], 1.0)
+    assert full.waves == 3
+    assert max(len(full._items(c, 1, w)) for c in range(19) for w in range(3)) == ROW_BUFFERS
+
+
+def test_more_vote_items_in_a_phase_than_row_buffers_must_not_share_the_fold():
+    # the publisher waits for a free row while the softmax warps wait for it to publish the next wave:
+    # a cycle, which ends in time-outs.  With one warp that folds the same shape goes through.
+    shape = (48, 32, 8, 300, 128, 32, 8)
+    alone = _model(shape, limit_s=10.0)
+    assert max(len(alone._items(c, 1, w)) for c in range(8) for w in range(alone.waves)) > ROW_BUFFERS
+    alone.run(jitter=False)
+    assert not any(alone.abort)
+    shared = _model(shape, limit_s=0.5, shared=True)
+    shared.run(jitter=False)
+    assert any(shared.abort)
+
+
+@pytest.mark.parametrize("shape,shared", HAND_OVER[::2])
+def test_a_block_that_never_arrives_becomes_time_outs_not_a_hang(shape, shared):
+    m = _model(shape, limit_s=0.4 if not shared else 2.0, shared=shared)
     took = m.run(absent={5})
     # blocks that need a unit which block 5 has a share of give up at half the limit with the code of
     # that wait; nobody waits longer than the limit
