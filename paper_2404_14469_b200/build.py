@@ -44,22 +44,24 @@ def _run(cmd, what: str, verbose: bool):
         raise RuntimeError(f"{what} failed:\n" + res.stdout + res.stderr)
     if verbose:
         sys.stderr.write(res.stdout + res.stderr)
+    return res.stdout + res.stderr
 
 
 def _build_lib(force: bool, verbose: bool):
-    """One object per source, compiled side by side, then one shared library."""
+    """One object per source, compiled side by side, then one shared library.  What ptxas says of each
+    kernel's registers and spills stays beside the object (build/<source>.ptxas)."""
     if not force and not _older(LIB, SOURCES + HEADERS):
         return
     os.makedirs(OBJ, exist_ok=True)
     flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
-             "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC,-O3,-Wall"]
-    if verbose:
-        flags += ["-Xptxas", "-v"]
+             "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC,-O3,-Wall", "-Xptxas", "-v"]
 
     def compile_one(src):
         obj = os.path.join(OBJ, src + ".o")
         if force or _older(obj, [src] + HEADERS):
-            _run([_nvcc(), "-c", *flags, "-o", obj, os.path.join(CSRC, src)], "nvcc " + src, verbose)
+            said = _run([_nvcc(), "-c", *flags, "-o", obj, os.path.join(CSRC, src)], "nvcc " + src, verbose)
+            with open(os.path.join(OBJ, src + ".ptxas"), "w") as f:
+                f.write(said)
         return obj
 
     with ThreadPoolExecutor(max_workers=min(len(SOURCES), os.cpu_count() or 1)) as pool:

@@ -106,6 +106,10 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t* warp_sums_s
 }
 
 struct OneLength {};
+// Rows of one length that are sums of gsum consecutive vote rows.  A kind of its own: the sums need a second
+// set of registers for the loads in flight, and kernels that never make one would spill for it (with 32 keys
+// a thread 96 to 224 bytes where it is 0 to 88 without).
+struct GroupedRows {};
 // Rows seq * heads + h: head h of the batch's sequence batch[seq].  A batch's long and short rows may be
 // two launches with CTAs of different sizes, side by side: the first (`lets_in`) lets the second in
 // as soon as its own wait for the votes is over, so the second finds them complete and does not wait
@@ -157,8 +161,9 @@ __device__ __forceinline__ void pool8(const float* a, float (&out)[8], int r, in
 // R, PT >= 0: the pooling radius is exactly R and the type PT (0 max, 1 avg), no per-tap tests.
 // PT = -1: radius r <= R and pool_type are run-time values, and with `divisor` != 0 average pooling
 // divides the window sum by it (otherwise rows are ranked by the sum, which orders the same way up
-// to rounding).  `want`: the sample ranks (from the top) that bound the window.  ROWS: OneLength,
-// or RaggedRows when the rows come from sequences of different lengths (n and want are not used then).
+// to rounding).  `want`: the sample ranks (from the top) that bound the window.  ROWS: OneLength (gsum = 1),
+// GroupedRows, or RaggedRows when the rows come from sequences of different lengths (gsum = 1, n and want are
+// not used then).
 template <int THREADS, int EPT, int R, int PT, typename ROWS>
 __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 1024 / THREADS)
 pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r, int pool_type, float divisor,
@@ -232,6 +237,25 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
       h_val = __ldg(vrow + j);
     }
   }
+  // Of each further head of a group the sample, the halo and the first eight keys of a thread are requested
+  // before any is added: one round trip a head where a thread has eight, not one for the sample and one
+  // for the chunk.  With 32 keys and a wide sample the registers do not hold both (96 and 196 bytes of
+  // spills with radius 6 and with any radius): there the sample is summed before the chunk is loaded.
+  constexpr bool GROUPED = std::is_same<ROWS, GroupedRows>::value;
+  constexpr bool TOGETHER = EPT < 32 || R <= 3;
+  if constexpr (GROUPED && !TOGETHER) {
+    for (int g = 1; g < gsum; ++g) {
+      const float* src = vrow + static_cast<size_t>(g) * n;
+      if (tid < CL_SAMPLES) {
+#pragma unroll
+        for (int t = 0; t <= 2 * R; ++t) {
+          const int j = js + t - R;
+          if (static_cast<unsigned>(j) < static_cast<unsigned>(n)) tap[t] += __ldg(src + j);
+        }
+      }
+      if (h_at >= 0) h_val += __ldg(src + h_at);
+    }
+  }
   {
     float x[EPT];
     if (EPT > 8 && c0 + CHUNK <= n) {
@@ -244,33 +268,33 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
         x[u] = j < n ? __ldg(vrow + j) : 0.f;
       }
     }
-    // Of each further head the sample, the halo and the first keys are requested before any is added:
-    // one round trip a head, not one for the sample and one for the chunk.
-    for (int g = 1; g < gsum; ++g) {
+    for (int g = 1; GROUPED && g < gsum; ++g) {
       const float* src = vrow + static_cast<size_t>(g) * n;
-      float t2[2 * R + 1], y[8], h2 = 0.f;
-      if (tid < CL_SAMPLES) {
+      if constexpr (TOGETHER) {
+        float t2[2 * R + 1], y[8], h2 = 0.f;
+        if (tid < CL_SAMPLES) {
 #pragma unroll
-        for (int t = 0; t <= 2 * R; ++t) {
-          const int j = js + t - R;
-          t2[t] = static_cast<unsigned>(j) < static_cast<unsigned>(n) ? __ldg(src + j) : 0.f;
+          for (int t = 0; t <= 2 * R; ++t) {
+            const int j = js + t - R;
+            t2[t] = static_cast<unsigned>(j) < static_cast<unsigned>(n) ? __ldg(src + j) : 0.f;
+          }
         }
+        if (h_at >= 0) h2 = __ldg(src + h_at);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int j = c0 + tid + THREADS * u;
+          y[u] = j < n ? __ldg(src + j) : 0.f;
+        }
+        if (tid < CL_SAMPLES) {
+#pragma unroll
+          for (int t = 0; t <= 2 * R; ++t) tap[t] += t2[t];
+        }
+        h_val += h2;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) x[u] += y[u];
       }
-      if (h_at >= 0) h2 = __ldg(src + h_at);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int j = c0 + tid + THREADS * u;
-        y[u] = j < n ? __ldg(src + j) : 0.f;
-      }
-      if (tid < CL_SAMPLES) {
-#pragma unroll
-        for (int t = 0; t <= 2 * R; ++t) tap[t] += t2[t];
-      }
-      h_val += h2;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) x[u] += y[u];
-#pragma unroll
-      for (int u = 8; u < EPT; ++u) {
+      for (int u = TOGETHER ? 8 : 0; u < EPT; ++u) {
         const int j = c0 + tid + THREADS * u;
         if (j < n) x[u] += __ldg(src + j);
       }
@@ -1158,7 +1182,7 @@ cudaError_t launch_pool_topk_cluster(const float* vote, int rows, int n, int poo
     *launches += 3;
     c.meta = meta;
   }
-  const cudaError_t e = launch_rows(shape, c, OneLength{});
+  const cudaError_t e = gsum > 1 ? launch_rows(shape, c, GroupedRows{}) : launch_rows(shape, c, OneLength{});
   if (e != cudaSuccess) return e;
   *launches += 1;
   return cudaGetLastError();

@@ -111,3 +111,30 @@ def test_grouped_rows_that_are_filtered_first(flat):
     else:
         _check_grouped(dev, W, kernel, "max", budget, kv_heads=[(0, 0), (0, 5)])
     assert sk.snapkv_last_launch_count() == 7   # clear, score, sample, filter, finish, clusters, gather
+
+
+@pytest.mark.parametrize("B,Hkv,L,kernel,ptype", [
+    (1, 64, 16033, 7, "max"),      # 64 rows of 16001: 16 keys a thread, the last ones missing
+    (2, 50, 30033, 5, "avg"),      # 100 rows of 30001: 32 keys a thread, a CTA per row
+    (2, 50, 32768, 13, "max"),     # the same with a wide sample
+    (1, 32, 78033, 9, "max"),      # 32 rows of 78001: clusters of three, a radius without a kernel of its own
+    (1, 32, 78033, 13, "avg"),
+])
+def test_grouped_rows_with_many_keys_per_thread(B, Hkv, L, kernel, ptype):
+    # against the votes of the same scoring kernel, summed and pooled in the same order: every
+    # addition is the same fp32 addition, so the positions are the same
+    W, d, budget, r = 32, 64, 512, kernel // 2
+    g = torch.Generator(device="cuda").manual_seed(L + kernel)
+    q, k, v = (torch.randn(B, h, x, d, generator=g, device="cuda").to(torch.bfloat16)
+               for h, x in ((2 * Hkv, W), (Hkv, L), (Hkv, L)))
+    vote, _ = sk.snapkv_window_scores(q, k)
+    got = sk.snapkv_compress_grouped(q, k, v, kernel, PT[ptype], budget)[2]
+    vote = vote.view(B * Hkv, 2, L - W)
+    pad = torch.nn.functional.pad(vote[:, 0] + vote[:, 1], (r, r))
+    pooled = pad[:, :L - W].clone()
+    for t in range(1, kernel):
+        tap = pad[:, t:t + L - W]
+        pooled = torch.maximum(pooled, tap) if ptype == "max" else pooled + tap
+    order = torch.sort(pooled, dim=1, descending=True, stable=True)[1]
+    want = torch.sort(order[:, :budget - W], dim=1)[0].int()
+    assert torch.equal(got.view(B * Hkv, budget - W), want)
