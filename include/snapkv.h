@@ -38,8 +38,10 @@
  *     default stream).  Calls return without synchronising unless stated.  Several of
  *     the kernels are launched with programmatic dependent launch: their blocks may
  *     become resident while the stream's previous kernel - the caller's included - is
- *     still running, but they read and write nothing before that kernel has completed
- *     and its writes are visible, so stream order holds for every buffer.
+ *     still running, but they read and write nothing of the caller's before that kernel
+ *     has completed and its writes are visible, so stream order holds for every buffer.
+ *     (Inside a call on prompts of different lengths two selection kernels may run side
+ *     by side; what the call is given was complete before the first of them started.)
  *   - Errors come back as a snapkv_status_t; nothing aborts or throws.  Argument
  *     errors are found on the host before anything is launched.
  *   - A device-side wait that exceeds its time limit stops the kernel early and

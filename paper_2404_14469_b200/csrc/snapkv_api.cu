@@ -515,7 +515,8 @@ static snapkv_status_t ragged_impl(const RaggedCall& c) {
                                c.lse_obs, !first, c.paged) != cudaSuccess)
         return SNAPKV_ERR_CUDA;
       if (launch_ragged_select(rb, reinterpret_cast<const float*>(ws + rb.off_vote), c.Hq, c.W, c.pool_kernel,
-                               c.pool_type, c.budget - c.W, c.out_idx, c.stream, &launches) != cudaSuccess)
+                               c.pool_type, c.budget - c.W, c.out_idx, reinterpret_cast<int*>(ws) + STATUS_READY, c.stream,
+                               &launches) != cudaSuccess)
         return SNAPKV_ERR_CUDA;
       first = false;
     }

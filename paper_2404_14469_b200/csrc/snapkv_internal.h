@@ -15,6 +15,8 @@ constexpr int STATUS_BYTES = 256;   // status block at the start of every worksp
 constexpr int SM_COUNT_HINT = 148;  // B200
 constexpr int MAX_GRID = 192;       // the scoring kernel runs one CTA per SM, at most this many
 
+constexpr int STATUS_READY = 2;     // its word (0: status, 1: detail) for launch_ragged_select
+
 constexpr uint32_t NO_PARTIAL = 0xffffffffu;  // a partial-statistics slot that has not been written
 constexpr int WAVE_LAG = 2;         // waves that the scoring kernel's statistics run ahead of the votes
 constexpr int RAGGED_MAX = 32;      // sequences of a ragged batch that share a launch
@@ -198,8 +200,10 @@ cudaError_t launch_ragged_scores(const RaggedBatch& rb, const void* q_obs, const
                                  int* launches, const float* lse_obs, bool keep_status, const PagedKV* paged,
                                  bool withhold = false);
 bool ragged_select_applies(int n_max, int pool_kernel, int pool_type);
+// `ready`: a word that is zero when the scoring kernel ends (the first of two launches sets it).
 cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int Hq, int W, int pool_kernel,
-                                 int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream, int* launches);
+                                 int pool_type, int ksel, int32_t* out_idx, int* ready, cudaStream_t stream,
+                                 int* launches);
 
 // Gather + append for `count` (up to RAGGED_MAX) consecutive sequences of a batch, from sequence b0
 // on; lens, k_off and v_off begin with that sequence.  A sequence with budget >= its length is

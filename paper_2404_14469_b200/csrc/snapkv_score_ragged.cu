@@ -22,7 +22,7 @@ __global__ void ragged_prep_kernel(const float* __restrict__ lse_obs, const Prep
   pdl_launch_dependents();
   pdl_wait();
   const int u = blockIdx.x, c = threadIdx.x;  // one block per unit, one thread per window column
-  if (u == 0 && c < STATUS_BYTES / 4 && !keep_status) status[c] = 0;
+  if (u == 0 && c < STATUS_BYTES / 4 && (!keep_status || c == STATUS_READY)) status[c] = 0;
   if (c == 0) counters[u] = lse_obs ? 1 : 0;  // supplied normalisers are ready
   if (!lse_obs) {  // neither a partial nor a folded row is there yet
     for (long long i = static_cast<long long>(u) * MAX_COLS + c; i < slots16; i += static_cast<long long>(gridDim.x) * MAX_COLS)

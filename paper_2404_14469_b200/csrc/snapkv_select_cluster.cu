@@ -111,17 +111,42 @@ struct OneLength {};
 // a thread 96 to 224 bytes where it is 0 to 88 without).
 struct GroupedRows {};
 // Rows seq * heads + h: head h of the batch's sequence batch[seq].  A batch's long and short rows may be
-// two launches with CTAs of different sizes, side by side: the first (`lets_in`) lets the second in
-// as soon as its own wait for the votes is over, so the second finds them complete and does not wait
-// for the first until it ends itself (`after`); the gather kernel, which waits for the second, then
-// finds both complete.
+// two launches with CTAs of different sizes, side by side.  A CTA of the first one lets the second in
+// once its own wait for the votes is over; the first CTA before that stores a flag (`ready`) with release
+// semantics.  The second launch (`after`) reads the flag with acquire semantics and then the votes: what
+// the first had visible is visible to it by that pair, not by the early start, which promises nothing.  A
+// thread that does not find the flag set waits for the first launch to end.  Every CTA of the second
+// launch waits for that before it ends itself, so the gather kernel, which waits for the second, finds both
+// complete.
 struct RaggedRows {
   int n[RAGGED_MAX], batch[RAGGED_MAX];
   int2 want[RAGGED_MAX];
   long long vote0[RAGGED_MAX];
   int heads;
-  bool lets_in, after;
+  int* ready;  // zero when the first of two launches starts; nullptr: one launch
+  bool after;
 };
+
+__device__ __forceinline__ void st_release(int* p, int v) {
+  asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ int ld_acquire(const int* p) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// A vote.  Rows of a ragged batch may be read by a kernel that starts while the one before it runs, so the
+// load is an ordinary one, behind the acquire; others may take the read-only path.
+template <typename ROWS>
+__device__ __forceinline__ float ld_vote(const float* p) {
+  if constexpr (std::is_same<ROWS, RaggedRows>::value) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+  } else {
+    return __ldg(p);
+  }
+}
 
 // Sliding pooling of eight positions: out[i] over a[i .. i + 2R].  The maximum is taken over
 // doubling spans (three or four operations per position instead of 2R + 1; a maximum is the same
@@ -199,7 +224,10 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
     orow = out_idx + (static_cast<size_t>(rows.batch[seq]) * rows.heads + h) * ksel;
     // CTAs behind the end of a short row leave at once: cluster barriers do not count them
     C = min(C, static_cast<uint32_t>((n + CHUNK - 1) / CHUNK));
-    if (rank >= C) return;
+    if (rank >= C) {
+      if (rows.after) pdl_wait();
+      return;
+    }
   } else {
     vrow = vote + static_cast<size_t>(row) * gsum * n;
     orow = out_idx + static_cast<size_t>(row) * ksel;
@@ -207,8 +235,11 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int c0 = static_cast<int>(rank) * CHUNK;  // first position of this CTA's chunk
   if constexpr (std::is_same<ROWS, RaggedRows>::value) {
-    if (!rows.after) pdl_wait();
-    if (rows.lets_in) pdl_launch_dependents();
+    if (!rows.after || ld_acquire(rows.ready) == 0) pdl_wait();
+    if (rows.ready != nullptr && !rows.after) {
+      if (blockIdx.x == 0 && tid == 0) st_release(rows.ready, 1);
+      pdl_launch_dependents();
+    }
   } else {
     pdl_wait();
   }
@@ -224,7 +255,7 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
 #pragma unroll
     for (int t = 0; t <= 2 * R; ++t) {
       const int j = js + t - R;
-      tap[t] = static_cast<unsigned>(j) < static_cast<unsigned>(n) ? __ldg(vrow + j) : 0.f;
+      tap[t] = static_cast<unsigned>(j) < static_cast<unsigned>(n) ? ld_vote<ROWS>(vrow + j) : 0.f;
     }
   }
   float h_val = 0.f;
@@ -234,7 +265,7 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
     const int j = i < CL_RMAX ? c0 - CL_RMAX + i : c0 + CHUNK + i - CL_RMAX;
     if (static_cast<unsigned>(j) < static_cast<unsigned>(n)) {
       h_at = j;
-      h_val = __ldg(vrow + j);
+      h_val = ld_vote<ROWS>(vrow + j);
     }
   }
   // Of each further head of a group the sample, the halo and the first eight keys of a thread are requested
@@ -260,12 +291,12 @@ pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r,
     float x[EPT];
     if (EPT > 8 && c0 + CHUNK <= n) {
 #pragma unroll
-      for (int u = 0; u < EPT; ++u) x[u] = __ldg(vrow + c0 + tid + THREADS * u);
+      for (int u = 0; u < EPT; ++u) x[u] = ld_vote<ROWS>(vrow + c0 + tid + THREADS * u);
     } else {
 #pragma unroll
       for (int u = 0; u < EPT; ++u) {
         const int j = c0 + tid + THREADS * u;
-        x[u] = j < n ? __ldg(vrow + j) : 0.f;
+        x[u] = j < n ? ld_vote<ROWS>(vrow + j) : 0.f;
       }
     }
     for (int g = 1; GROUPED && g < gsum; ++g) {
@@ -1221,7 +1252,7 @@ bool ragged_select_applies(int n_max, int pool_kernel, int pool_type) {
 }
 
 cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int Hq, int W, int pool_kernel,
-                                 int pool_type, int ksel, int32_t* out_idx, cudaStream_t stream, int* launches) {
+                                 int pool_type, int ksel, int32_t* out_idx, int* ready, cudaStream_t stream, int* launches) {
   // longest rows first: the last CTAs to start should be short ones
   int order[RAGGED_MAX];
   for (int i = 0; i < rb.count; ++i) {
@@ -1242,7 +1273,7 @@ cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int H
     const int last = first < longer ? longer : rb.count;
     RaggedRows rows = {};
     rows.heads = Hq;
-    rows.lets_in = last < rb.count;
+    rows.ready = longer > 0 && longer < rb.count ? ready : nullptr;
     rows.after = first > 0;
     for (int i = first; i < last; ++i) {
       rows.n[i - first] = n[i];

@@ -213,3 +213,47 @@ def test_rows_of_a_ragged_batch_in_one_or_two_select_launches(lens, ptype, kerne
     for run in runs:
         for b in range(len(lens)):
             assert all(torch.equal(x[b], y[0]) for x, y in zip(run[:3], want[b]))
+
+
+def test_two_select_launches_read_the_votes_of_their_own_call():
+    # Calls on different inputs follow one another on one workspace without a synchronisation: the second
+    # select launch of each reads votes while the first one runs, and must find this call's.
+    lens, Hq, Hkv, d, W, budget = [700, 20000, 4128, 2081, 9000, 4129, 2080, 4127], 32, 8, 64, 32, 512
+    inputs, want = [], []
+    for i in range(4):
+        g = torch.Generator(device="cuda").manual_seed(i)
+        x = [torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+             for s in ((len(lens), Hq, W, d), (sum(lens), Hkv, d), (sum(lens), Hkv, d))]
+        inputs.append(x)
+        at = 0
+        for b, L in enumerate(lens):
+            one = [t[at:at + L].permute(1, 0, 2)[None].contiguous() for t in x[1:]]
+            want.append(sk.snapkv_compress(x[0][b:b + 1].contiguous(), *one, 7, sk.POOL_MAX, budget)[2])
+            at += L
+    cu = [sum(lens[:b]) for b in range(len(lens))]
+    ws, got = None, []
+    for _ in range(5):
+        for x in inputs:
+            *out, ws = sk.snapkv_compress_varlen(*x, lens, 7, sk.POOL_MAX, budget, cu_seqlens=cu, workspace=ws)
+            got.append(out[2])
+            assert sk.snapkv_last_launch_count() == 5  # preparation, scores, two selections, gather
+    for c, idx in enumerate(got):
+        for b in range(len(lens)):
+            assert torch.equal(idx[b], want[c % 4 * len(lens) + b][0])
+
+
+def test_two_groups_of_sequences_with_two_select_launches_each():
+    lens = [19000 + 37 * b if b % 4 == 0 else 300 + 29 * b for b in range(40)]
+    Hq, Hkv, d, W, budget = 16, 4, 64, 32, 128
+    g = torch.Generator(device="cuda").manual_seed(40)
+    q, k, v = (torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+               for s in ((len(lens), Hq, W, d), (sum(lens), Hkv, d), (sum(lens), Hkv, d)))
+    cu = [sum(lens[:b]) for b in range(len(lens))]
+    ws = None
+    for _ in range(2):  # the second time on a workspace that the first one left
+        *out, ws = sk.snapkv_compress_varlen(q, k, v, lens, 7, sk.POOL_MAX, budget, cu_seqlens=cu, workspace=ws)
+        assert sk.snapkv_last_launch_count() == 2 * 4 + 2  # two groups, and a gather for 32 and for 8 sequences
+        for b, L in enumerate(lens):
+            one = [t[cu[b]:cu[b] + L].permute(1, 0, 2)[None].contiguous() for t in (k, v)]
+            want = sk.snapkv_compress(q[b:b + 1].contiguous(), *one, 7, sk.POOL_MAX, budget)[:3]
+            assert all(torch.equal(x[b], y[0]) for x, y in zip(out, want))
