@@ -40,7 +40,8 @@ SYMBOLS = [
 ]
 
 # entry points for the extension and the tests alone (csrc/snapkv_binding.h)
-BINDING_SYMBOLS = ["snapkv_binding_varlen", "snapkv_binding_paged", "snapkv_binding_ragged_items"]
+BINDING_SYMBOLS = ["snapkv_binding_varlen", "snapkv_binding_paged", "snapkv_binding_ragged_items",
+                   "snapkv_binding_shared_fold"]
 
 _lib = None
 _native = None
@@ -124,6 +125,8 @@ def lib() -> ctypes.CDLL:
                                                       ctypes.POINTER(ctypes.c_int32)]
     L.snapkv_binding_ragged_items.restype = c_int
     L.snapkv_binding_ragged_items.argtypes = [p32] + [c_int] * 8 + [p32, c_int]
+    L.snapkv_binding_shared_fold.restype = c_int
+    L.snapkv_binding_shared_fold.argtypes = [c_int] * 7
     L.snapkv_set_wait_limit_ns.restype = ctypes.c_ulonglong
     L.snapkv_set_wait_limit_ns.argtypes = [ctypes.c_ulonglong]
     L.snapkv_selftest_stalled_scores.restype = c_int
@@ -394,6 +397,14 @@ def ragged_schedule_items(seq_lens, Hq, Hkv, d, W, grid, cta, votes_only=False):
     buf = (ctypes.c_int32 * (8 * max(n, 1)))()
     L_.snapkv_binding_ragged_items(*args, buf, n)
     return [tuple(buf[8 * i:8 * i + 8]) for i in range(n)]
+
+
+def shared_fold(B, Hq, Hkv, L, d, W, host_part=False) -> bool:
+    """Whether the scoring kernel folds a call's partial statistics with two warps (host only)."""
+    r = lib().snapkv_binding_shared_fold(B, Hq, Hkv, L, d, W, int(host_part))
+    if r < 0:
+        raise SnapKVError("shared_fold: arguments not acceptable")
+    return r == 1
 
 
 def snapkv_set_wait_limit_ns(limit_ns: int) -> int:

@@ -81,6 +81,7 @@ struct ScoreArgs {
   int stats_only;           // 1: statistics pass alone (a shard's partial log-sum-exp), no votes
   int votes_only;           // 1: lse2 and the counters are already set, no statistics pass
   int withhold;             // 1: nothing is published (self-test of the waits for it)
+  int both_fold;            // 1: the publisher folds half of the columns (shared_fold)
   unsigned long long wait_ns;  // time limit of every device-side wait
   const int32_t* page_table;   // paged K: [batch][pages_per_seq] page numbers, else nullptr
   int pages_per_seq, page_size;
@@ -388,15 +389,7 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
   constexpr int NSET = SPLIT ? 2 : 1;  // sets of softmax warps
   // In split mode the fetcher folds the columns in two halves, and the publisher takes one of them.
   constexpr int HALVES = SPLIT && !RAGGED ? 2 : 1;
-  // (with more vote items in a phase than row buffers, the publisher would wait for the softmax warps
-  // to use up rows while they wait for it to publish)
-  // With few partials per unit one warp is fast enough, and the publisher is better left alone: four
-  // prompts of 5316 with some 10 partials take 42.7 us so, 44.4 with both warps; one of 13013 with 37
-  // takes 40.1 and 38.7.  A single unit is left to one warp too: alone it would take 22.8 us instead of
-  // 24.8 (8192 positions), but the parts of a call on host buffers are such launches, and between the
-  // copies they cost more than they gain (966-988 us against 932-940).
-  const bool both_fold =
-      HALVES == 2 && !a.votes_only && !a.stats_only && a.per <= NLB && a.maxseg > 16 && a.units > 1;
+  const bool both_fold = HALVES == 2 && a.both_fold;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -1099,13 +1092,15 @@ static cudaError_t run_scores(const CUtensorMap& tmK, const CUtensorMap& tmQ, co
   return cudaSuccess;
 }
 
-// The instantiation for a plan: columns padded to 32, 64 or 128, and the column-split epilogue when
-// each warpgroup's half of the columns is whole heads.
+// The column-split epilogue: each warpgroup's half of the columns is whole heads.
+inline bool split_columns(int npad, int W) { return npad >= 64 && (W % 16) == 0 && ((npad / 2) % W) == 0; }
+
+// The instantiation for a plan: columns padded to 32, 64 or 128, split or not.
 template <typename SEQS>
 static cudaError_t run_scores_for(int d, int W, int npad, const CUtensorMap& tmK, const CUtensorMap& tmQ,
                                   const ScoreArgs& a, const SEQS& rs, int grid, cudaStream_t stream, int* launches) {
   const int nch = npad >> 5;
-  const bool split = nch >= 2 && (W % 16) == 0 && ((npad / 2) % W) == 0;
+  const bool split = split_columns(npad, W);
 #define SNAPKV_SCORES(DD, NN, SS) run_scores<DD, NN, SS, SEQS>(tmK, tmQ, a, rs, grid, stream, launches)
 #define SNAPKV_SCORES_D(DD)                                                                                  \
   (nch == 1 ? SNAPKV_SCORES(DD, 1, false)                                                                    \

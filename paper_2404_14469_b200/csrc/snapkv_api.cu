@@ -269,7 +269,7 @@ static snapkv_status_t compress_impl(const void* q_obs, const void* k, const voi
                                      bool keep_status, const float* lse_obs = nullptr,
                                      const KVStrides* k_str = nullptr,
                                      const KVStrides* v_str = nullptr, bool grouped = false,
-                                     const PagedKV* paged = nullptr) {
+                                     const PagedKV* paged = nullptr, bool host_part = false) {
   snapkv_status_t st = check_common(B, Hq, Hkv, L, d, W);
   if (st != SNAPKV_OK) return st;
   st = check_pool(pool_kernel, pool_type);
@@ -320,7 +320,7 @@ static snapkv_status_t compress_impl(const void* q_obs, const void* k, const voi
                            reinterpret_cast<int*>(ws + w.off_counters),
                            reinterpret_cast<float*>(ws + w.off_partials),
                            reinterpret_cast<float*>(ws + w.off_lse), s, &launches, lse_obs,
-                           keep_status, false, paged) != cudaSuccess)
+                           keep_status, false, paged, nullptr, false, host_part) != cudaSuccess)
     return SNAPKV_ERR_CUDA;
   if (launch_pool_topk(vote, B * Ho, n, pool_kernel, pool_type, ksel, out_idx,
                        scratch ? reinterpret_cast<float*>(ws + w.off_pooled) : nullptr, s,
@@ -870,7 +870,7 @@ snapkv_status_t snapkv_compress_host(const void* q_obs, const void* k, const voi
     st = compress_impl(
         dq + qo, dk + ko, dv + ko, 1, np * g, np, L, d, W, pool_kernel, pool_type, budget,
         dok + oo, dov + oo, reinterpret_cast<int32_t*>(di + io), dws, ws_bytes, stream,
-        /*keep_status=*/true);
+        /*keep_status=*/true, nullptr, nullptr, nullptr, false, nullptr, /*host_part=*/true);
     if (st != SNAPKV_OK) break;
     launches += g_last_launches;
     if ((side && !order(s, side->computed[c], back)) || !to_host(out_k, dok, oo, np * o_pair) ||
@@ -902,6 +902,12 @@ int snapkv_schedule_items(int B, int Hq, int Hkv, int L, int d, int W, int votes
     out_plan[7] = p.ncols;
   }
   return list_schedule_items(p, L, W, Hkv, votes_only ? 1 : 0, grid, cta, out_items, max_items);
+}
+
+int snapkv_binding_shared_fold(int B, int Hq, int Hkv, int L, int d, int W, int host_part) {
+  ScorePlan p;
+  if (check_common(B, Hq, Hkv, L, d, W) != SNAPKV_OK || !make_score_plan(B, Hq, Hkv, L, d, W, &p)) return -1;
+  return shared_fold(p, W, items_per_phase(p.units_per_wave, score_grid()), host_part != 0) ? 1 : 0;
 }
 
 int snapkv_binding_ragged_items(const int32_t* seq_lens, int B, int Hq, int Hkv, int d, int W, int votes_only,

@@ -16,6 +16,9 @@ extern "C" {
  * of eight int32, {unit, t0, t1, vote, slot, nseg, sequence, wave of the launch}. */
 int snapkv_binding_ragged_items(const int32_t* seq_lens, int B, int Hq, int Hkv, int d, int W, int votes_only,
                                 int grid, int cta, int32_t* out_items, int max_items);
+/* Whether the scoring kernel of such a call (host_part: of a part of a call on host buffers) folds the
+ * partial statistics with both of its book-keeping warps; -1: arguments not acceptable. */
+int snapkv_binding_shared_fold(int B, int Hq, int Hkv, int L, int d, int W, int host_part);
 snapkv_status_t snapkv_binding_varlen(const void* q_obs, const void* k, const void* v, const int64_t* k_strides,
                                       const int64_t* v_strides, const int64_t* k_seq_offsets,
                                       const int64_t* v_seq_offsets, const int32_t* seq_lens, const float* lse_obs,

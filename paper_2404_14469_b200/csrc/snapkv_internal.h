@@ -153,6 +153,10 @@ int score_grid();
 int items_per_phase(int nu, int grid);
 int most_waves_per_launch(int upw);
 
+// Whether the publisher of the scoring kernel shares the folds; `per` as from items_per_phase.
+constexpr int SHARED_FOLD_ABOVE = 16;  // partials per unit
+bool shared_fold(const ScorePlan& plan, int W, int per, bool host_part);
+
 // `n_vote` < 0: the keys that get a vote are the L - W prefix keys (the whole prompt is here).
 bool make_score_plan(int B, int Hq, int Hkv, int L, int d, int W, ScorePlan* plan, int n_vote = -1);
 WorkspaceLayout make_layout(const ScorePlan& p, int B, int Hq, int n, bool need_vote,
@@ -167,7 +171,7 @@ size_t select_scratch_bytes(int rows, int n);  // 0 when the rows fit one CTA
 // also zeroes the status block unless `keep_status` is set.  `never_ready` (self-test of the
 // time-out path): the vote pass alone is launched and nothing marks the units' statistics as
 // present, so its wait for them must run out.  `withhold` (another): both passes run, but no
-// partial is written.
+// partial is written.  `host_part`: the launch is a part of a call on host buffers (see shared_fold).
 cudaError_t launch_window_scores(const void* q_obs, const void* k, const KVStrides& ks, int B,
                                  int Hq, int Hkv, int L, int d, int W, const ScorePlan& plan,
                                  float* vote, int* status,
@@ -175,7 +179,7 @@ cudaError_t launch_window_scores(const void* q_obs, const void* k, const KVStrid
                                  int* launches, const float* lse_obs = nullptr,
                                  bool keep_status = false, bool never_ready = false,
                                  const PagedKV* paged = nullptr, const ShardMode* shard = nullptr,
-                                 bool withhold = false);
+                                 bool withhold = false, bool host_part = false);
 
 // Pool + top-k over `rows` rows of fp32 votes.  `pooled_scratch` (select_scratch_bytes bytes)
 // is only touched when select_needs_scratch(n).  With gsum > 1 a selection row is the sum of

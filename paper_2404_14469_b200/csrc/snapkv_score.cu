@@ -170,6 +170,25 @@ int list_schedule_items(const ScorePlan& plan, int L, int W, int Hkv, int votes_
 int items_per_phase(int nu, int grid) { return (nu + grid - 1) / grid + 1; }
 int most_waves_per_launch(int upw) { return score::MAX_RECORDS / (2 * items_per_phase(upw, score_grid())); }
 
+// Whether the publisher folds half of the columns of a launch's vote rows (us per call, one warp and both;
+// 32 query heads on 8 KV heads unless stated).
+//  - Not with more vote items in a phase than row buffers: the publisher would wait for the softmax warps
+//    to use up rows while they wait for it to publish.
+//  - Not with few partials per unit: with 14 the two are level (four prompts of 8192 73.2 and 73.0, of 16000
+//    104.2 and 104.9, of 32768 169.2 and 169.6), and then the publisher is better left alone.  From 17 on
+//    both are level or faster: 17 partials 60.1 and 59.1 (three of 8192), 25 22.9 and 22.3 (one of 3001, 16-row
+//    windows), 28 68.9 and 68.5 (two of 20011), 33 46.5 and 46.7 (two of 8192), 52 39.3 and 37.2 (one of 13013),
+//    64 24.8 and 23.0 (one KV head of 8192), 192 32.8 and 28.8 (one KV head of 30000).
+//  - Not in a part of a call on host buffers that is one KV head.  The part alone gains as above, but the
+//    call, which PCIe bounds, does not: 8192 positions 955-959 and 968-988, with 64-row windows 951 and 954-1008;
+//    other lengths differ by 1 % at most, either way, and with two KV heads a part the call is faster
+//    with both warps (two prompts of 8192: 2026-2079 and 2008-2016).  Why is not known: the copies of one
+//    part fall differently against those of the next.
+bool shared_fold(const ScorePlan& plan, int W, int per, bool host_part) {
+  return !(host_part && plan.units == plan.sub_per_kv) && score::split_columns(plan.npad, W) &&
+         per <= score::NLB && plan.maxseg > SHARED_FOLD_ABOVE;
+}
+
 bool make_score_plan(int B, int Hq, int Hkv, int L, int d, int W, ScorePlan* plan, int n_vote) {
   if (B < 1 || Hq < 1 || Hkv < 1 || L < 1 || W < 1 || W > L || Hq % Hkv != 0) return false;
   if (n_vote > L) return false;
@@ -238,7 +257,8 @@ cudaError_t launch_window_scores(const void* q_obs, const void* k, const KVStrid
                                  float* vote, int* status,
                                  int* counters, float* partials, float* lse2, cudaStream_t stream,
                                  int* launches, const float* lse_obs, bool keep_status,
-                                 bool never_ready, const PagedKV* paged, const ShardMode* shard, bool withhold) {
+                                 bool never_ready, const PagedKV* paged, const ShardMode* shard, bool withhold,
+                                 bool host_part) {
   CUtensorMap tmK, tmQ;
   {
     // (d, position, KV head, batch) with the caller's strides: any layout whose rows of d
@@ -289,6 +309,7 @@ cudaError_t launch_window_scores(const void* q_obs, const void* k, const KVStrid
   a.per = items_per_phase(a.upw, grid);
   const int most = score::MAX_RECORDS / (2 * a.per), waves = a.nwaves;
   if (most < 1) return cudaErrorInvalidValue;
+  a.both_fold = !a.votes_only && !a.stats_only && shared_fold(plan, W, a.per, host_part);
   cudaError_t e = cudaSuccess;
   for (; a.wave0 < waves && e == cudaSuccess; a.wave0 += most) {
     a.nwaves = waves - a.wave0 < most ? waves - a.wave0 : most;

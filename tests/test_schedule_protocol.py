@@ -319,6 +319,18 @@ def test_a_block_that_never_arrives_becomes_time_outs_not_a_hang(shape, shared):
     assert took < 5.0
 
 
+def test_which_calls_share_the_fold():
+    # one unit or many, where a unit has many partials; not where it has few, where a warpgroup's half of the
+    # columns is not whole heads, or in a part of a call on host buffers that is one KV head, however many units
+    # that has
+    for shape in ((1, 4, 1, 8192, 128, 32), (1, 32, 8, 13013, 128, 32), (1, 32, 8, 131072, 128, 64)):
+        assert sk.shared_fold(*shape)
+    for shape in ((4, 32, 8, 5316, 128, 32), (1, 32, 32, 380000, 128, 32)):
+        assert not sk.shared_fold(*shape)
+    for part in ((1, 4, 1, 8192, 128, 32), (1, 4, 1, 8192, 128, 64), (1, 8, 2, 8192, 128, 32)):
+        assert sk.shared_fold(*part) and sk.shared_fold(*part, host_part=True) == (part[2] > 1)
+
+
 def test_wait_limit_setter_returns_the_previous_value_and_has_a_floor():
     prev = sk.snapkv_set_wait_limit_ns(5)            # raised to one millisecond
     try:
