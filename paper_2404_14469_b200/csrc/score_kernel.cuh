@@ -670,8 +670,9 @@ score_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CU
     const uint32_t te_arrivals = SPLIT ? 1 : 2;          // the barrier expects 8 per tile
     // Two columns per instruction wherever the arithmetic is not an exponential: an element then
     // takes one multiply-add and one add for every two of what the special-function unit does, the
-    // results are the same, and the registers no longer spill (one sweep of 2 x 20K keys with the
-    // rest of the call 42.6 -> 41.1 us, 128K keys with 64-row windows 265 -> 258).
+    // results are the same (one sweep of 2 x 20K keys with the rest of the call 42.6 -> 41.1 us, 128K
+    // keys with 64-row windows 265 -> 258).  The kernels for one length no longer spill; those for
+    // ragged batches with 128 columns in split mode are three registers short (12 bytes).
     const unsigned long long scale2 = pack2(a.c2, a.c2);
     int git = 0, nstat = 0, nvote = 0;
     each_item([&](const Item& it) {
