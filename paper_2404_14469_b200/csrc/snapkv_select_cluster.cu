@@ -20,10 +20,11 @@
 // window the histogram is taken over the whole key range, and a bin with more keys than the list
 // holds is refined by a further histogram; ties go to the lower position by construction.
 // Two cluster barriers on the usual path (a byte-wise radix select took five), one histogram
-// update for every sixth key.  Back to back: 4 rows of 992 in 6.0 us (one CTA per row with all keys
-// in shared memory and five passes over them: 12.4 us), 32 rows of 16352 in 11.6 us (14.4), 128 rows
-// of 32736 in 16.8 us (20.6), 32 rows of 131008 in 22.7 us (49.9).  Rows so long or so many that the
-// clusters come in several rounds are filtered first (long_filter_kernel).
+// update for every sixth key.  Back to back in a graph: 4 rows of 992 in 4.7 us, 32 rows of 16352 in
+// 9.1, 128 rows of 32736 in 13.8, 32 rows of 131008 in 17.  (Single launches back to back, when the kernel
+// was new: 6.0, 11.6, 16.8 and 22.7; with one CTA per row, all keys in shared memory and five passes over them
+// 12.4, 14.4, 20.6 and 49.9.)  Rows so long or so many that the clusters come in several rounds are
+// filtered first (long_filter_kernel).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -1048,6 +1049,37 @@ int clusters_at_once(int c) {
   return fit[dev][c] < in_rounds ? fit[dev][c] : in_rounds;
 }
 
+// What a round of CTAs of 1024 threads takes, in us, by the keys a thread holds: rows that have a CTA to
+// themselves, and rows that a cluster shares (0.35 us more for each CTA of it).  Measured in a graph, rows that
+// fill the device, kernel size 7 (5: up to two less, 13: two more), an eighth of the positions kept: 8.3,
+// 11.0 and 16.4 alone; clusters of two, three and four 10.4, 10.8, 11.3 with 8 keys, 12.4, 12.9, 13.9 with 16,
+// 18.1, 18.1, 19.8 with 32.  So the last entry is two to three us high, and 91 to 132 rows of 33000 to 49000
+// take three rounds with 16 keys (34) where two with 32 are shorter (31).  With 18.7 there they would take
+// those, but rows that are filtered now would come to the clusters, whose time depends on the sample
+// (64 rows of 115000: 31 to 35 filtered, 34 to 43 in clusters; 56 of 131008: 36 to 40, and 33 to 43).
+struct RoundCost {
+  int ept;
+  double alone, shared;
+};
+constexpr RoundCost ROUND_COST[3] = {{8, 8.0, 10.2}, {16, 10.5, 12.5}, {32, 16.5, 20.0}};
+
+// The shape with the smallest estimated time for rows of which the longest has n positions;
+// rounds(chunk, c, fit): in how many rounds clusters of c CTAs, of which `fit` find a place at once, come
+// when a CTA takes `chunk` positions.  No CTAs: the device holds no cluster that is large enough.
+template <typename Rounds>
+ClusterShape cheapest_shape(int n, Rounds&& rounds) {
+  ClusterShape best = {1024, 32, 0, 1e30};
+  for (const RoundCost& cost : ROUND_COST) {
+    const int chunk = 1024 * cost.ept, c = (n + chunk - 1) / chunk;
+    if (c > CL_MAX_CLUSTER) continue;
+    const int fit = clusters_at_once(c);
+    if (fit < 1) continue;
+    const double us = static_cast<double>(rounds(chunk, c, fit)) * (c == 1 ? cost.alone : cost.shared + 0.35 * c);
+    if (us < best.us) best = {1024, cost.ept, c, us};
+  }
+  return best;
+}
+
 // How rows of n positions are cut: the shape with the smallest estimated time.  Up to 4096
 // positions small CTAs have the shortest chain, and clusters of them while every CTA has an SM to
 // itself (79.6 against 84.2 us for the whole step of 32 rows of 16352).  Beyond, CTAs of 1024 threads
@@ -1058,18 +1090,7 @@ ClusterShape cluster_shape(int rows, int n) {
   if (n <= 2048) return {256, 8, 1};
   const int small = (n + 4095) / 4096;
   if (small <= 8 && rows * small <= sm_count()) return {512, 8, small};
-  const int ept[3] = {8, 16, 32};
-  const double alone[3] = {8.0, 10.5, 16.5}, shared[3] = {10.2, 12.5, 20.0};
-  ClusterShape best = {1024, 32, 0, 1e30};
-  for (int i = 0; i < 3; ++i) {
-    const int c = (n + 1024 * ept[i] - 1) / (1024 * ept[i]);
-    if (c > CL_MAX_CLUSTER) continue;
-    const int fit = clusters_at_once(c);
-    if (fit < 1) continue;
-    const double us = static_cast<double>((rows + fit - 1) / fit) * (c == 1 ? alone[i] : shared[i] + 0.35 * c);
-    if (us < best.us) best = {1024, ept[i], c, us};
-  }
-  return best;
+  return cheapest_shape(n, [&](int, int, int fit) { return (rows + fit - 1) / fit; });
 }
 
 // What a launch needs besides the shape.
@@ -1227,21 +1248,12 @@ constexpr int RAGGED_SHORT = 4096;  // rows up to here take a CTA of 256 or 512 
 static ClusterShape ragged_shape(const int* n, int count, int heads) {
   if (n[0] <= 2048) return {256, 8, 1};
   if (n[0] <= RAGGED_SHORT) return {512, 8, 1};
-  const int ept[3] = {8, 16, 32};
-  const double alone[3] = {8.0, 10.5, 16.5}, shared[3] = {10.2, 12.5, 20.0};
-  ClusterShape best = {1024, 32, 0, 1e30};
-  for (int i = 0; i < 3; ++i) {
-    const int chunk = 1024 * ept[i], c = (n[0] + chunk - 1) / chunk;
-    if (c > CL_MAX_CLUSTER) continue;
-    const int fit = clusters_at_once(c);
-    if (fit < 1) continue;
+  return cheapest_shape(n[0], [&](int chunk, int c, int fit) {
     long long ctas = 0;
     for (int j = 0; j < count; ++j) ctas += static_cast<long long>(heads) * ((n[j] + chunk - 1) / chunk);
     const long long at_once = static_cast<long long>(fit) * c;
-    const double us = static_cast<double>((ctas + at_once - 1) / at_once) * (c == 1 ? alone[i] : shared[i] + 0.35 * c);
-    if (us < best.us) best = {1024, ept[i], c, us};
-  }
-  return best;
+    return (ctas + at_once - 1) / at_once;
+  });
 }
 
 // Whether the rows of a ragged batch, the longest of n_max positions, can share a launch.
@@ -1261,8 +1273,9 @@ cudaError_t launch_ragged_select(const RaggedBatch& rb, const float* vote, int H
     order[at] = i;
   }
   // Where the long rows alone are estimated to take less time, because they come in fewer rounds or can
-  // have more CTAs each, the short ones are a launch of their own behind them: a CTA of 1024 threads has an SM to itself and takes 10 us however short its row is,
-  // and the small CTAs fit where the long rows' last round leaves SMs over.  (Eight sequences of 822
+  // have more CTAs each, the short ones are a launch of their own behind them: a CTA of 1024 threads has an
+  // SM to itself and takes 10 us however short its row is, and the small CTAs fit where the long rows' last
+  // round leaves SMs over.  (Eight sequences of 822
   // to 24000: 143 us in one launch, 132 in two; sixteen of 300 to 20000 with 8 heads 104.7 and 97.0.
   // Four of 400 to 12283, which take one round either way: 52.4 and 53.4.)
   int n[RAGGED_MAX], longer = 0;
