@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 1024 ? 1 : 1024 / THREADS)
 pool_topk_cluster_kernel(const float* __restrict__ vote, int n, int gsum, int r, int pool_type, float divisor,
                          int ksel, int2 want, int32_t* __restrict__ out_idx, int ctas, int discard_votes,
                          const uint32_t* __restrict__ meta, const __grid_constant__ ROWS rows) {
-  // With 16 and 32 keys a thread the instructions per key count (72 with 32 keys: the schedulers issued in
+  // With 16 and 32 keys a thread the instructions per key count (72 with 32 keys, 58 now: the schedulers issued in
   // 55 to 60 % of the cycles), so whole chunks skip the checks of the row's end, the keys are compared
   // with the bin once, and the positions are picked by set bits (128 rows of 32736: 3 us less).  With
   // eight it is the chain of steps: there the forms that need the fewest steps in a row stay.
